@@ -147,12 +147,12 @@ extern "C" pd_status pd_autotune(pd_ctx* cx, const pd_diagram* A, const pd_diagr
                 h.walk = kWalks[q % NW];
                 if (h.block > 4 * M) continue;
             } else {
-                h.block = std::max<int64_t>(8 * NS_THREADS, (int64_t)sqrt((double)M));
+                h.block = ns_default_block(h);
                 h.walk = kDefaultWalk;
             }
             NSInst res{};
             c->last_ns_ms = 0.f;
-            PD_TRY(ns_run(c, &h, 1, w.ns.smem, d, &res, st));
+            PD_TRY(ns_run(c, &h, 1, d, &res, st));
             PD_TRY(ns_status(c, res));
             if (opt >= 0 && res.opt != opt) return fail(c, PD_ECUDA, "tuner: the optimum changed with the parameters");
             opt = res.opt;

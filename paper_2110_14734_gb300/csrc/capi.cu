@@ -617,7 +617,7 @@ static pd_status warm_start(Ctx* c, Ctx* tc, const Front& f, W1Prep* w, const pd
         NSInst* d = bufT<NSInst>(c, B_NS_INST, 1);
         if (!d) return PD_ENOMEM;
         NSInst r{};
-        PD_TRY(ns_run(c, &w->ns.h, 1, w->ns.smem, d, &r, st));
+        PD_TRY(ns_run(c, &w->ns.h, 1, d, &r, st));
         PD_TRY(ns_status(c, r));
         const int64_t nt = w->nt;
         std::vector<int64_t> pi((size_t)nt);
@@ -674,7 +674,7 @@ extern "C" pd_status pd_w1_approx(pd_ctx* c, pd_diagram A, pd_diagram B, double 
             if (!d) return PD_ENOMEM;
             NSInst r{};
             if (o.warm_start == 2) c->last_ns_ms = 0.f;  // report the warm solve only
-            PD_TRY(ns_run(c, &w.ns.h, 1, w.ns.smem, d, &r, st));
+            PD_TRY(ns_run(c, &w.ns.h, 1, d, &r, st));
             PD_TRY(ns_finish_w1(c, f.tree, f.s, nullptr, o, w, d, r, &ss, st));
         }
         if (!w.ns.ready || ss.method == -1) {
@@ -915,7 +915,6 @@ pd_status batch_solve(Ctx* c, const pd_diagram* A, const pd_diagram* B, int64_t 
         // certificate in one launch, records and certificate counts down
         hin.clear();
         jobs.clear();
-        size_t smem = 0;
         for (int64_t j = 0; j < nw; j++) {
             BatchPair& p = bp[(size_t)j];
             if (p.done) continue;
@@ -926,12 +925,11 @@ pd_status batch_solve(Ctx* c, const pd_diagram* A, const pd_diagram* B, int64_t 
             J.S = p.w.S;
             J.T = p.w.T;
             J.nS = p.w.nS;
-            J.nT = p.w.nT;
+            J.ld = p.w.ld;
             J.s = p.f.s;
             J.tree = p.tree;
             J.dc = diag_cost(o);
             jobs.push_back(J);
-            smem = std::max(smem, p.w.ns.smem);
         }
         hout.assign(hin.size(), NSInst{});
         cert.assign(2 * hin.size(), 0ull);
@@ -939,7 +937,7 @@ pd_status batch_solve(Ctx* c, const pd_diagram* A, const pd_diagram* B, int64_t 
         const auto tl = std::chrono::steady_clock::now();
         const long long lw = launch_count_ref();
         if (!hin.empty()) {
-            status = ns_run_wave(c, hin.data(), (int)hin.size(), smem, jobs.data(), hout.data(), cert.data(), st);
+            status = ns_run_wave(c, hin.data(), (int)hin.size(), jobs.data(), hout.data(), cert.data(), st);
             if (status != PD_OK) break;
         }
         const float wave_ms = elapsed_ms(tl), wave_ns = c->last_ns_ms;
@@ -1048,7 +1046,7 @@ extern "C" pd_status pd_ws_train(pd_ctx* c, const pd_diagram* A, const pd_diagra
         std::vector<double> base;
         PD_TRY(ws_coarse_potentials(c, f, w, o, &base, st));
         NSInst rec{};
-        PD_TRY(ns_run(c, &w.ns.h, 1, w.ns.smem, d, &rec, st));
+        PD_TRY(ns_run(c, &w.ns.h, 1, d, &rec, st));
         PD_TRY(ns_status(c, rec));
         const int64_t cmax = (rec.big - 1) / (int64_t)(rec.n + 1) - 1;
         PD_TRY(ws_collect(c, f.nodes, w, d, rec, cmax, base.empty() ? nullptr : &base, st));

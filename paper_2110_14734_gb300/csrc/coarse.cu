@@ -142,7 +142,7 @@ pd_status ws_coarse_potentials(Ctx* c, const Front& f, const W1Prep& w, const pd
     NSInst* d = bufT<NSInst>(cc, B_NS_INST, 1);
     if (!d) return fail(c, PD_ENOMEM, "coarse solve: " + cc->err);
     NSInst r{};
-    e = ns_run(cc, &wc.ns.h, 1, wc.ns.smem, d, &r, st);
+    e = ns_run(cc, &wc.ns.h, 1, d, &r, st);
     if (e == PD_OK) e = ns_status(cc, r);
     if (e != PD_OK) return fail(c, e, "coarse solve: " + cc->err);
     const int64_t nt = w.nt;

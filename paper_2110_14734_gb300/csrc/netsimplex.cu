@@ -24,6 +24,10 @@
 // and the leaving arc is the last blocking arc met when the cycle is walked
 // from the apex in the direction of the entering arc, which rules out cycling.
 // An instance may instead carry its own strongly feasible start (warm start).
+//
+// Instances whose potentials fit 32 bits go to simplex32.cu; this kernel takes
+// the others (more than 65,533 nodes, arc costs above 2^25 quanta, ...) and the
+// few that simplex32.cu hands back.
 #include <algorithm>
 #include <mutex>
 #include <vector>
@@ -42,12 +46,18 @@ PD_D uint64_t ns_now() {
 
 PD_D void arc_ends(const NSInst& I, int64_t a, int32_t* t, int32_t* h) {
     if (a < I.mst) {  // m + n < 2^31, so 32-bit division is exact
-        int32_t i = (int32_t)a / (int32_t)I.nT;
+        int32_t i = (int32_t)a / (int32_t)I.ld;
         *t = i;
-        *h = (int32_t)I.nS + ((int32_t)a - i * (int32_t)I.nT);
+        *h = (int32_t)I.nS + ((int32_t)a - i * (int32_t)I.ld);
     } else if (a < I.m) {
-        *t = I.tail[a - I.mst];
-        *h = I.head[a - I.mst];
+        if (I.th) {
+            const uint32_t w = I.th[a - I.mst];
+            *t = (int32_t)(w >> 16);
+            *h = (int32_t)(w & 0xffffu);
+        } else {
+            *t = I.tail[a - I.mst];
+            *h = I.head[a - I.mst];
+        }
     } else {
         int32_t i = (int32_t)(a - I.m);
         if (I.supply[i] >= 0) {
@@ -189,8 +199,8 @@ __device__ __forceinline__ void ns_body(NSInst& G, NSInst& I, Tree<IX>& T) {
             // and the sink potentials pi(nS + j) they read are consecutive
             // 8-byte words of shared memory (no bank conflicts)
             const int32_t iend = (int32_t)(aend < I.mst ? aend : I.mst);
-            const int32_t nT = (int32_t)I.nT, nS = (int32_t)I.nS;
-            const int32_t step_i = NS_THREADS / nT, step_j = NS_THREADS - step_i * nT;
+            const int32_t nT = (int32_t)I.nT, ld = (int32_t)I.ld, nS = (int32_t)I.nS;
+            const int32_t step_i = NS_THREADS / ld, step_j = NS_THREADS - step_i * ld;
             for (int32_t base = (int32_t)a0; base < iend; base += NS_PR * NS_THREADS) {
                 int32_t cv[NS_PR];
 #pragma unroll
@@ -200,11 +210,11 @@ __device__ __forceinline__ void ns_body(NSInst& G, NSInst& I, Tree<IX>& T) {
                 }
                 // row i and column j of arc base + tid, then NS_THREADS arcs further per step
                 const int32_t a1 = base + tid;
-                int32_t i = a1 / nT, j = a1 - i * nT;
+                int32_t i = a1 / ld, j = a1 - i * ld;
 #pragma unroll
                 for (int q = 0; q < NS_PR; q++) {
                     const int32_t a = a1 + q * NS_THREADS;
-                    if (a < iend) {
+                    if (a < iend && j < nT) {
                         const int64_t r = (int64_t)cv[q] - T.pi[i] + T.pi[nS + j];
                         if (r < lb) {
                             lb = r;
@@ -213,8 +223,8 @@ __device__ __forceinline__ void ns_body(NSInst& G, NSInst& I, Tree<IX>& T) {
                     }
                     i += step_i;
                     j += step_j;
-                    if (j >= nT) {
-                        j -= nT;
+                    if (j >= ld) {
+                        j -= ld;
                         ++i;
                     }
                 }
@@ -697,6 +707,13 @@ __device__ __forceinline__ void ns_body(NSInst& G, NSInst& I, Tree<IX>& T) {
 
 __device__ __forceinline__ void ns_instance(NSInst& G) {
     NSInst I = G;
+    if (I.lay32) {
+        // handed back by simplex32.cu: a cold start with costs that its 32 bits could not hold
+        if (I.status != S32_REDO) return;
+        I.big = I.big64;
+        I.init_tree = 0;
+        I.art = nullptr;
+    }
     const int32_t N1 = I.n + 1;
     if (I.smem_nodes) {
         // 1: every node array in shared memory (24 B a node); 2: pred and the
@@ -831,22 +848,24 @@ __global__ void k_abs_sum(const int64_t* __restrict__ s, int64_t n, unsigned lon
 
 // One network simplex instance on an arc list, ready to launch (buffers of
 // this context; nothing is launched).  cmax = largest arc cost.
-pd_status ns_prepare_arcs(Ctx* c, int32_t n, int64_t m, int64_t mst, int64_t nS, int64_t nT, const int32_t* cmat,
-                          const int32_t* tail, const int32_t* head, const int32_t* cost, const int64_t* supply,
-                          int64_t cmax, const pd_opts& o, NSPrep* p, cudaStream_t st) {
+pd_status ns_prepare_arcs(Ctx* c, int32_t n, const NSArcs& a, const int64_t* supply, int64_t cmax, const pd_opts& o,
+                          NSPrep* p, cudaStream_t st) {
     *p = NSPrep{};
     if (n <= 0) return PD_OK;
     int64_t N1 = (int64_t)n + 1;
+    const int64_t m = a.m;
     NSInst& h = p->h;
     h.n = n;
     h.m = m;
-    h.mst = mst;
-    h.nS = nS;
-    h.nT = nT > 0 ? nT : 1;
-    h.cmat = cmat;
-    h.tail = tail;
-    h.head = head;
-    h.cost = cost;
+    h.mst = a.mst;
+    h.nS = a.nS;
+    h.nT = std::max<int64_t>(a.nT, 1);
+    h.ld = std::max<int64_t>(a.ld, 1);
+    h.cmat = a.cmat;
+    h.th = a.th;
+    h.tail = a.tail;
+    h.head = a.head;
+    h.cost = a.cost;
     h.supply = supply;
     h.pi = bufT<int64_t>(c, B_NS_PI, N1);
     h.parent = bufT<int32_t>(c, B_NS_PARENT, N1);
@@ -866,12 +885,6 @@ pd_status ns_prepare_arcs(Ctx* c, int32_t n, int64_t m, int64_t mst, int64_t nS,
     // arc ids, plus one pricing step past the last arc, stay below 2^31
     if (M >= (int64_t(1) << 31) - 1 - 8 * NS_THREADS)
         return fail(c, PD_ECAPACITY, "network simplex needs fewer than 2^31 - 8193 arcs");
-    // default block: one pass of the CTA (8 arcs per thread), more for very
-    // large networks; blocks start at multiples of 8 (vector loads)
-    int64_t blk = o.ns_block > 0 ? o.ns_block : tuned_block(c, M);
-    if (blk <= 0) blk = std::max<int64_t>(8 * NS_THREADS, (int64_t)sqrt((double)M));
-    blk = (blk + 7) & ~(int64_t)7;
-    h.block = blk;
     h.walk = o.ns_walk >= 0 ? std::min<int32_t>(o.ns_walk, NS_LMAX) : tuned_walk(c, M);
     h.max_pivots = o.max_rounds > 0 ? o.max_rounds : (int64_t(1) << 40);
     h.time_limit_ns = (o.time_limit_ms > 0 ? (uint64_t)o.time_limit_ms : 60000ull) * 1000000ull;
@@ -888,48 +901,129 @@ pd_status ns_prepare_arcs(Ctx* c, int32_t n, int64_t m, int64_t mst, int64_t nS,
     }
     // big-M: more than any path cost; |potentials| stay below ~3 big
     if (cmax > (INT64_MAX / 8) / N1) return fail(c, PD_EOVERFLOW, "network simplex big-M would overflow");
-    h.big = N1 * (cmax + 1) + 1;
     int max_optin = 0;
     PD_TRY_CUDA(c, cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-    h.smem_nodes = o.ns_smem != 0 ? ns_smem_layout(N1, max_optin) : 0;
-    p->smem = h.smem_nodes ? ns_smem_bytes(N1, h.smem_nodes) : 0;
+    ns_choose_kernel(&h, cmax, a.complete, o.ns_smem != 0, max_optin);
+    const int64_t blk = o.ns_block > 0 ? o.ns_block : tuned_block(c, M);
+    h.block = blk > 0 ? (blk + 7) & ~(int64_t)7 : ns_default_block(h);  // whole 32-byte steps
     p->ready = true;
     return PD_OK;
 }
 
-pd_status ns_run(Ctx* c, const NSInst* h, int count, size_t smem, NSInst* d, NSInst* r, cudaStream_t st) {
-    if (count <= 0) return PD_OK;
+// Pricing block where neither the caller nor the tuner names one.  A matrix in
+// simplex32.cu: 16384 arcs, its whole stage, priced in the pivot's shadow
+// (100,000 lower-star points, cold: 278 ms against 296 with 8192; 2,000 uniform
+// points: 25.7 / 26.8 ms).  Otherwise one pass of the CTA (8 arcs per thread),
+// more for very large networks.
+int64_t ns_default_block(const NSInst& h) {
+    if (h.lay32 && h.mst > 0) return 16384;
+    return (std::max<int64_t>(8 * NS_THREADS, (int64_t)sqrt((double)(h.m + h.n))) + 7) & ~(int64_t)7;
+}
+
+// 32-bit potentials (simplex32.cu) whenever costs, node ids and the matrix's
+// rows allow: it is the faster kernel at every size both take.  Artificial
+// arcs then cost just enough instead of more than any path.  With an arc from
+// every supply node to every demand node, cmax + 1 is enough: a unit on two
+// artificial arcs could be sent directly for less than 2 (cmax + 1).  On an
+// arc list a shortest route can be longer than S32_MAX_BIG; an optimum that
+// then keeps artificial flow proves nothing and goes to the 64-bit kernel.
+void ns_choose_kernel(NSInst* h, int64_t cmax, bool complete, bool smem, int max_optin) {
+    const int64_t N1 = (int64_t)h->n + 1;
+    h->big = h->big64 = N1 * (cmax + 1) + 1;
+    h->smem_nodes = smem ? ns_smem_layout(N1, max_optin) : 0;
+    h->lay32 = 0;
+    h->big_safe = 1;
+    if (!smem || cmax > S32_MAX_COST || (h->m > h->mst && !h->th) || (h->mst > 0 && h->ld % 8 != 0)) return;
+    h->lay32 = s32_layout(N1);
+    if (h->lay32 == 0) return;
+    if (complete) {
+        h->big = cmax + 1;
+    } else if (h->big64 > S32_MAX_BIG) {
+        h->big = S32_MAX_BIG;
+        h->big_safe = 0;
+    }
+}
+
+// How `count` instances are launched: a kernel per 32-bit class present, over
+// its stretch of the order, then k_netsimplex over all of them (it takes its own
+// and those handed back).
+struct NSLaunch {
+    int first[S32_CLASSES] = {}, num[S32_CLASSES] = {};  // stretches of the order
+    int own64 = 0;                                       // instances of k_netsimplex
+    size_t smem64 = 0;
+    int grid64 = 0;
+};
+constexpr int NS_COUNTERS = S32_CLASSES + 1;  // instance counters behind the order
+
+// Fills order (count indices, by class, largest instances first -- nodes, then
+// arcs, ties by index -- and the zeroed counters) and *L.
+static pd_status ns_plan(Ctx* c, const NSInst* h, int count, int32_t* order, NSLaunch* L) {
     PD_TRY_CUDA(c, ns_kernel_setup());
-    int per_sm = 0;
-    PD_TRY_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_netsimplex, NS_THREADS, smem));
-    if (per_sm < 1) return fail(c, PD_ECAPACITY, "network simplex kernel does not fit on an SM");
-    const int grid = std::min(count, per_sm * std::max(c->sm_count, 1));
-    // largest instances first (nodes, then arcs), ties by position
-    std::vector<int32_t> order((size_t)count);
-    for (int q = 0; q < count; q++) order[(size_t)q] = q;
-    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+    PD_TRY_CUDA(c, s32_kernel_setup());
+    *L = NSLaunch{};
+    for (int q = 0; q < count; q++) {
+        order[q] = q;
+        const int k = s32_class(h[q]);
+        if (k < 0) L->own64++;
+        else L->num[k]++;
+        if (h[q].smem_nodes) L->smem64 = std::max(L->smem64, ns_smem_bytes((int64_t)h[q].n + 1, h[q].smem_nodes));
+    }
+    for (int k = 1; k < S32_CLASSES; k++) L->first[k] = L->first[k - 1] + L->num[k - 1];
+    std::stable_sort(order, order + count, [&](int32_t x, int32_t y) {
+        const unsigned cx = (unsigned)s32_class(h[x]), cy = (unsigned)s32_class(h[y]);  // -1 sorts last
+        if (cx != cy) return cx < cy;
         return h[x].n != h[y].n ? h[x].n > h[y].n : h[x].m > h[y].m;
     });
-    int32_t* dord = bufT<int32_t>(c, B_NS_ORDER, count + 1);
+    for (int q = 0; q < NS_COUNTERS; q++) order[count + q] = 0;
+    int per_sm = 0;
+    PD_TRY_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_netsimplex, NS_THREADS, L->smem64));
+    if (per_sm < 1) return fail(c, PD_ECAPACITY, "network simplex kernel does not fit on an SM");
+    L->grid64 = std::min(count, per_sm * std::max(c->sm_count, 1));
+    return PD_OK;
+}
+
+pd_status ns_run(Ctx* c, const NSInst* h, int count, NSInst* d, NSInst* r, cudaStream_t st) {
+    if (count <= 0) return PD_OK;
+    std::vector<int32_t> order((size_t)count + NS_COUNTERS);
+    NSLaunch L;
+    PD_TRY(ns_plan(c, h, count, order.data(), &L));
+    bool any64 = L.own64 > 0;
+    int32_t* dord = bufT<int32_t>(c, B_NS_ORDER, count + NS_COUNTERS);
     if (!dord) return PD_ENOMEM;
     PD_TRY_CUDA(c, cudaMemcpyAsync(d, h, sizeof(NSInst) * count, cudaMemcpyHostToDevice, st));
-    PD_TRY_CUDA(c, cudaMemcpyAsync(dord, order.data(), sizeof(int32_t) * count, cudaMemcpyHostToDevice, st));
-    PD_TRY_CUDA(c, cudaMemsetAsync(dord + count, 0, sizeof(int32_t), st));
+    PD_TRY_CUDA(c, cudaMemcpyAsync(dord, order.data(), sizeof(int32_t) * order.size(), cudaMemcpyHostToDevice, st));
     cudaEvent_t e0, e1;
     PD_TRY_CUDA(c, cudaEventCreate(&e0));
     PD_TRY_CUDA(c, cudaEventCreate(&e1));
-    PD_TRY_CUDA(c, cudaEventRecord(e0, st));
-    k_netsimplex<<<grid, NS_THREADS, smem, st>>>(d, dord, count, dord + count); pd::count_launch();
-    cudaError_t le = cudaGetLastError();
-    if (le == cudaSuccess) le = cudaEventRecord(e1, st);
-    if (le == cudaSuccess) le = cudaMemcpyAsync(r, d, sizeof(NSInst) * count, cudaMemcpyDeviceToHost, st);
-    if (le == cudaSuccess) le = cudaStreamSynchronize(st);
-    float nms = 0.f;
-    if (le == cudaSuccess) le = cudaEventElapsedTime(&nms, e0, e1);
+    // the 32-bit kernels, then the 64-bit one over its own instances and those handed back
+    cudaError_t le = cudaSuccess;
+    for (int pass = 0; pass < 2 && le == cudaSuccess; pass++) {
+        if (pass == 0 ? L.own64 == count : !any64) continue;
+        le = cudaEventRecord(e0, st);
+        if (pass == 0) {
+            for (int k = 0; k < S32_CLASSES; k++)
+                if (L.num[k] > 0) {
+                    s32_launch(k, std::min(L.num[k], std::max(c->sm_count, 1)), d, dord + L.first[k], L.num[k],
+                               dord + count + k, st);
+                    pd::count_launch();
+                }
+        } else {
+            k_netsimplex<<<L.grid64, NS_THREADS, L.smem64, st>>>(d, dord, count, dord + count + S32_CLASSES);
+            pd::count_launch();
+        }
+        if (le == cudaSuccess) le = cudaGetLastError();
+        if (le == cudaSuccess) le = cudaEventRecord(e1, st);
+        if (le == cudaSuccess) le = cudaMemcpyAsync(r, d, sizeof(NSInst) * count, cudaMemcpyDeviceToHost, st);
+        if (le == cudaSuccess) le = cudaStreamSynchronize(st);
+        float nms = 0.f;
+        if (le == cudaSuccess) le = cudaEventElapsedTime(&nms, e0, e1);
+        c->last_ns_ms += nms;
+        if (pass == 0)
+            for (int q = 0; q < count; q++) any64 |= r[q].lay32 != 0 && r[q].status == S32_REDO;
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (le != cudaSuccess) return cuda_fail(c, le, "k_netsimplex");
-    c->last_ns_ms += nms;
+    if (le != cudaSuccess) return cuda_fail(c, le, "network simplex");
     return PD_OK;
 }
 
@@ -942,7 +1036,7 @@ struct WaveLayout {
         in = 0;
         out = in + al(sizeof(NSInst) * count);
         ord = out + al(sizeof(NSInst) * count);
-        jobs = ord + al(sizeof(int32_t) * (count + 1));
+        jobs = ord + al(sizeof(int32_t) * (count + NS_COUNTERS));
         cert = jobs + al(sizeof(CertJob) * count);
         total = cert + al(2 * sizeof(unsigned long long) * count);
     }
@@ -950,14 +1044,9 @@ struct WaveLayout {
 
 constexpr int WAVE_CERT_BLOCKS = 8;  // blocks per pair of the batched certificate (grid-stride)
 
-pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, size_t smem, const CertJob* jobs, NSInst* r,
+pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, const CertJob* jobs, NSInst* r,
                       unsigned long long* cert, cudaStream_t st) {
     if (count <= 0) return PD_OK;
-    PD_TRY_CUDA(c, ns_kernel_setup());
-    int per_sm = 0;
-    PD_TRY_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_netsimplex, NS_THREADS, smem));
-    if (per_sm < 1) return fail(c, PD_ECAPACITY, "network simplex kernel does not fit on an SM");
-    const int grid = std::min(count, per_sm * std::max(c->sm_count, 1));
     const WaveLayout L(count);
     if (c->wave_pin_bytes < L.total) {
         if (c->wave_exec) cudaGraphExecDestroy(c->wave_exec);
@@ -978,18 +1067,15 @@ pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, size_t smem, const Cer
     CertJob* p_jobs = (CertJob*)(pin + L.jobs);
     unsigned long long* p_cert = (unsigned long long*)(pin + L.cert);
     NSInst* d = bufT<NSInst>(c, B_NS_INST, count);
-    int32_t* dord = bufT<int32_t>(c, B_NS_ORDER, count + 1);
+    int32_t* dord = bufT<int32_t>(c, B_NS_ORDER, count + NS_COUNTERS);
     CertJob* djobs = bufT<CertJob>(c, B_NS_JOBS, count);
     unsigned long long* dcert = bufT<unsigned long long>(c, B_NS_CERT, 2 * count);
     if (!d || !dord || !djobs || !dcert) return PD_ENOMEM;
     // this wave's contents into the pinned staging the graph copies from;
     // largest instances first (nodes, then arcs), ties by position
     memcpy(p_in, h, sizeof(NSInst) * count);
-    for (int q = 0; q < count; q++) p_ord[q] = q;
-    std::stable_sort(p_ord, p_ord + count, [&](int32_t x, int32_t y) {
-        return h[x].n != h[y].n ? h[x].n > h[y].n : h[x].m > h[y].m;
-    });
-    p_ord[count] = 0;
+    NSLaunch NL;
+    PD_TRY(ns_plan(c, h, count, p_ord, &NL));
     for (int q = 0; q < count; q++) {
         if (jobs[q].rec < 0 || jobs[q].rec >= count) return fail(c, PD_EINVAL, "certificate job without a record");
         p_jobs[q] = jobs[q];
@@ -999,8 +1085,9 @@ pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, size_t smem, const Cer
     uint64_t key = 1469598103934665603ull;
     auto mix = [&](uint64_t v) { key = (key ^ v) * 1099511628211ull; };
     mix((uint64_t)count);
-    mix((uint64_t)grid);
-    mix((uint64_t)smem);
+    for (int k = 0; k < S32_CLASSES; k++) mix((uint64_t)NL.num[k]);
+    mix((uint64_t)NL.grid64);
+    mix((uint64_t)NL.smem64);
     mix((uint64_t)(uintptr_t)pin);
     mix((uint64_t)(uintptr_t)d);
     mix((uint64_t)(uintptr_t)dord);
@@ -1012,10 +1099,14 @@ pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, size_t smem, const Cer
         c->wave_exec = nullptr;
         PD_TRY_CUDA(c, cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal));
         cudaMemcpyAsync(d, p_in, sizeof(NSInst) * count, cudaMemcpyHostToDevice, gs);
-        cudaMemcpyAsync(dord, p_ord, sizeof(int32_t) * (count + 1), cudaMemcpyHostToDevice, gs);
+        cudaMemcpyAsync(dord, p_ord, sizeof(int32_t) * (count + NS_COUNTERS), cudaMemcpyHostToDevice, gs);
         cudaMemcpyAsync(djobs, p_jobs, sizeof(CertJob) * count, cudaMemcpyHostToDevice, gs);
         cudaMemsetAsync(dcert, 0, 2 * sizeof(unsigned long long) * count, gs);
-        k_netsimplex<<<grid, NS_THREADS, smem, gs>>>(d, dord, count, dord + count);
+        for (int k = 0; k < S32_CLASSES; k++)
+            if (NL.num[k] > 0)
+                s32_launch(k, std::min(NL.num[k], std::max(c->sm_count, 1)), d, dord + NL.first[k], NL.num[k],
+                           dord + count + k, gs);
+        k_netsimplex<<<NL.grid64, NS_THREADS, NL.smem64, gs>>>(d, dord, count, dord + count + S32_CLASSES);
         k_certify_batch<<<dim3(WAVE_CERT_BLOCKS, count), 256, 0, gs>>>(djobs, dcert);
         cudaMemcpyAsync(p_out, d, sizeof(NSInst) * count, cudaMemcpyDeviceToHost, gs);
         cudaMemcpyAsync(p_cert, dcert, 2 * sizeof(unsigned long long) * count, cudaMemcpyDeviceToHost, gs);
@@ -1036,7 +1127,9 @@ pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, size_t smem, const Cer
     PD_TRY_CUDA(c, cudaEventRecord(c->wave_ev[0], gs));
     PD_TRY_CUDA(c, cudaGraphLaunch(c->wave_exec, gs));
     PD_TRY_CUDA(c, cudaEventRecord(c->wave_ev[1], gs));
-    pd::count_launch();  // the persistent simplex
+    for (int k = 0; k < S32_CLASSES; k++)
+        if (NL.num[k] > 0) pd::count_launch();  // the persistent simplex on 32-bit potentials
+    pd::count_launch();                         // ... on 64-bit ones
     pd::count_launch();  // the batched certificate
     c->wave_launches++;
     PD_TRY_CUDA(c, cudaStreamSynchronize(gs));
@@ -1058,17 +1151,15 @@ pd_status ns_status(Ctx* c, const NSInst& r) {
 
 // Network simplex on an arc list (one CTA), result in this context's
 // instance record.
-static pd_status ns_solve_arcs(Ctx* c, int32_t n, int64_t m, int64_t mst, int64_t nS, int64_t nT,
-                               const int32_t* cmat, const int32_t* tail, const int32_t* head, const int32_t* cost,
-                               const int64_t* supply, int64_t cmax, const pd_opts& o, NSInst* out,
-                               cudaStream_t st) {
+static pd_status ns_solve_arcs(Ctx* c, int32_t n, const NSArcs& a, const int64_t* supply, int64_t cmax,
+                               const pd_opts& o, NSInst* out, cudaStream_t st) {
     *out = NSInst{};
     NSPrep p;
-    PD_TRY(ns_prepare_arcs(c, n, m, mst, nS, nT, cmat, tail, head, cost, supply, cmax, o, &p, st));
+    PD_TRY(ns_prepare_arcs(c, n, a, supply, cmax, o, &p, st));
     if (!p.ready) return PD_OK;
     NSInst* d = bufT<NSInst>(c, B_NS_INST, 1);
     if (!d) return PD_ENOMEM;
-    PD_TRY(ns_run(c, &p.h, 1, p.smem, d, out, st));
+    PD_TRY(ns_run(c, &p.h, 1, d, out, st));
     return ns_status(c, *out);
 }
 
@@ -1100,43 +1191,85 @@ __global__ void k_side_lists(const int64_t* __restrict__ cntA, const int64_t* __
     }
 }
 
-// Arc i*nT + j: source i -> sink j at min(l2, diag(i) + diag(j)) (the route
-// through the diagonal node has unbounded capacity); then the arcs of the
-// diagonal node if its supply |B| - |A| is not 0.
+// Arc i*ld + j: source i -> sink j at min(l2, diag(i) + diag(j)) (the route
+// through the diagonal node has unbounded capacity), rows padded to ld columns;
+// then the arcs of the diagonal node if its supply |B| - |A| is not 0 (th, when
+// given, with their ends packed and padded to a multiple of four arcs).
+// stat[0] += costs that do not fit 31 bits, stat[1] = the largest cost.
 __global__ void k_transport_arcs(const int32_t* __restrict__ S, const int32_t* __restrict__ T, int64_t nS,
-                                 int64_t nT, int dside, const int32_t* __restrict__ X, const int32_t* __restrict__ Y,
-                                 int32_t* __restrict__ cmat, int32_t* __restrict__ tail, int32_t* __restrict__ head,
-                                 int32_t* __restrict__ cost, unsigned long long* __restrict__ bad, DiagCost dc) {
-    int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t mst = nS * nT;
-    int64_t D = nS + nT;
-    int64_t c;
+                                 int64_t nT, int64_t ld, int dside, const int32_t* __restrict__ X,
+                                 const int32_t* __restrict__ Y, int32_t* __restrict__ cmat, int32_t* __restrict__ tail,
+                                 int32_t* __restrict__ head, int32_t* __restrict__ cost, uint32_t* __restrict__ th,
+                                 unsigned long long* __restrict__ stat, DiagCost dc) {
+    const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t mst = nS * ld, D = nS + nT, mx = dside < 0 ? nS : dside > 0 ? nT : 0;
+    int64_t c = 0;
     if (a < mst) {
-        int64_t i = a / nT, j = a - i * nT;
-        int32_t u = S[i], v = T[j];
-        int64_t d = cost_l2(X[u], Y[u], X[v], Y[v]);
-        int64_t g = cost_make(X[u], Y[u], dc) + cost_make(X[v], Y[v], dc);
-        c = d < g ? d : g;
-        if (c >= (int64_t(1) << 31)) atomicAdd(bad, 1ull);
-        cmat[a] = (int32_t)c;
-        return;
-    } else if (dside < 0 && a < mst + nS) {
-        int64_t i = a - mst;
-        int32_t u = S[i];
-        c = cost_make(X[u], Y[u], dc);
-        tail[a - mst] = (int32_t)i;
-        head[a - mst] = (int32_t)D;
-    } else if (dside > 0 && a < mst + nT) {
-        int64_t j = a - mst;
-        int32_t v = T[j];
-        c = cost_make(X[v], Y[v], dc);
-        tail[a - mst] = (int32_t)D;
-        head[a - mst] = (int32_t)(nS + j);
+        const int64_t i = a / ld, j = a - i * ld;
+        if (j < nT) {
+            const int32_t u = S[i], v = T[j];
+            const int64_t d = cost_l2(X[u], Y[u], X[v], Y[v]);
+            const int64_t g = cost_make(X[u], Y[u], dc) + cost_make(X[v], Y[v], dc);
+            c = d < g ? d : g;
+            cmat[a] = (int32_t)c;
+        } else {
+            cmat[a] = NS_PAD_COST;
+        }
+    } else if (a < mst + ((mx + 3) & ~(int64_t)3)) {
+        const int64_t x = a - mst;
+        int64_t t = 0, h = 0;
+        if (x < mx) {
+            const int32_t u = dside < 0 ? S[x] : T[x];
+            c = cost_make(X[u], Y[u], dc);
+            t = dside < 0 ? x : D;
+            h = dside < 0 ? D : nS + x;
+            tail[x] = (int32_t)t;
+            head[x] = (int32_t)h;
+        }
+        cost[x] = x < mx ? (int32_t)c : NS_PAD_COST;
+        if (th) th[x] = (uint32_t)t << 16 | (uint32_t)h;
+    }
+    const bool bad = c >= (int64_t(1) << 31);
+    if (__any_sync(0xffffffffu, bad)) {
+        if (bad) atomicAdd(&stat[0], 1ull);
     } else {
+        const uint32_t mx32 = __reduce_max_sync(0xffffffffu, (uint32_t)c);
+        if ((threadIdx.x & 31) == 0 && mx32 > *(volatile unsigned long long*)&stat[1])
+            atomicMax(&stat[1], (unsigned long long)mx32);
+    }
+}
+
+// One warp per row of the CSR network.
+__global__ void k_arc_pack(const int64_t* __restrict__ rp, const int32_t* __restrict__ hd,
+                           const int64_t* __restrict__ cost, int64_t n, int64_t m, uint32_t* __restrict__ th,
+                           int32_t* __restrict__ c32, unsigned long long* __restrict__ bad,
+                           unsigned long long* __restrict__ cmax) {
+    const int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (u > n) return;  // whole warps leave together
+    if (u == n) {       // the padding
+        if (lane < 3 && m + lane < ((m + 3) & ~(int64_t)3)) {
+            th[m + lane] = 0;
+            c32[m + lane] = NS_PAD_COST;
+        }
         return;
     }
-    if (c >= (int64_t(1) << 31)) atomicAdd(bad, 1ull);
-    cost[a - mst] = (int32_t)c;
+    uint32_t big = 0, wrong = 0;
+    const int64_t a1 = min(rp[u + 1], m);  // in bounds whatever the rows say: they may not be checked yet
+    for (int64_t a = max(rp[u], (int64_t)0) + lane; a < a1; a += 32) {
+        const int64_t c = cost[a];
+        const bool b = c < 0 || c >= (int64_t(1) << 31);
+        wrong += b;
+        big = max(big, b ? 0u : (uint32_t)c);
+        th[a] = (uint32_t)u << 16 | (uint32_t)hd[a];
+        c32[a] = (int32_t)c;
+    }
+    big = __reduce_max_sync(0xffffffffu, big);
+    wrong = __reduce_add_sync(0xffffffffu, wrong);
+    if (lane == 0) {
+        if (wrong) atomicAdd(bad, (unsigned long long)wrong);
+        if (big > *(volatile unsigned long long*)cmax) atomicMax(cmax, (unsigned long long)big);
+    }
 }
 
 // Total flow over the arcs of a solved arc-list network (rounding slack).
@@ -1149,12 +1282,16 @@ __global__ void k_tree_flow(const NSInst* __restrict__ I, unsigned long long* __
 pd_status ns_solve_network(Ctx* c, const pd_network& net, const pd_opts& o, SolveStats* out, cudaStream_t st) {
     int64_t n = net.n_nodes, m = net.n_arcs;
     if (n >= (int64_t(1) << 31) - 2) return fail(c, PD_ECAPACITY, "too many nodes");
-    int32_t* tail = bufT<int32_t>(c, B_S_TAIL, m);
-    int32_t* c32 = bufT<int32_t>(c, B_NS_COST, m);
+    const bool packed = n + 1 < 65535;  // 16-bit node ids, as simplex32.cu takes them
+    int32_t* tail = bufT<int32_t>(c, B_S_TAIL, m + 3);
+    int32_t* c32 = bufT<int32_t>(c, B_NS_COST, m + 3);
     unsigned long long* sm = bufT<unsigned long long>(c, B_SMALL, 64);
     if (!tail || !c32 || !sm) return PD_ENOMEM;
     PD_TRY_CUDA(c, cudaMemsetAsync(sm, 0, 8 * sizeof(unsigned long long), st));
-    if (m > 0) {
+    if (m > 0 && packed) {
+        k_arc_pack<<<grid_for(32 * (n + 1), 256), 256, 0, st>>>(net.row_ptr, net.head, net.cost, n, m, (uint32_t*)tail,
+                                                                c32, sm, sm + 1); pd::count_launch();
+    } else if (m > 0) {
         k_arc_tails<<<grid_for(m, 256), 256, 0, st>>>(net.row_ptr, n, m, tail); pd::count_launch();
         k_i64_to_i32_cost<<<grid_for(m, 256), 256, 0, st>>>(net.cost, m, c32, sm); pd::count_launch();
         k_max_cost<<<grid_for(m, 256), 256, 0, st>>>(net.cost, m, sm + 1); pd::count_launch();
@@ -1165,7 +1302,13 @@ pd_status ns_solve_network(Ctx* c, const pd_network& net, const pd_opts& o, Solv
     if (c->h_small[0]) return fail(c, PD_EOVERFLOW, "arc cost outside [0, 2^31)");
     int64_t cmax = c->h_small[1];
     NSInst r;
-    PD_TRY(ns_solve_arcs(c, (int32_t)n, m, 0, 0, 1, nullptr, tail, net.head, c32, net.supply, cmax, o, &r, st));
+    NSArcs arcs;
+    arcs.m = m;
+    arcs.th = packed ? (const uint32_t*)tail : nullptr;
+    arcs.tail = tail;
+    arcs.head = net.head;
+    arcs.cost = c32;
+    PD_TRY(ns_solve_arcs(c, (int32_t)n, arcs, net.supply, cmax, o, &r, st));
     PD_TRY_CUDA(c, cudaMemsetAsync(sm, 0, sizeof(unsigned long long), st));
     k_tree_flow<<<grid_for(n, 256), 256, 0, st>>>(bufT<NSInst>(c, B_NS_INST, 1), sm); pd::count_launch();
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -1210,31 +1353,50 @@ pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t d
     int32_t* S = bufT<int32_t>(c, B_TR_S, nS);
     int32_t* T = bufT<int32_t>(c, B_TR_T, nT);
     int64_t* sup = bufT<int64_t>(c, B_TR_SUP, nt);
-    int64_t mx = mt - mst;
+    const int64_t mx = mt - mst;
+    // rows padded to whole steps of simplex32.cu, unless the padding alone would take the arc ids past 2^31
+    int64_t ld = (nT + 7) & ~(int64_t)7;
+    if (nS * ld + mx >= (int64_t(1) << 31) - 1 - 8 * NS_THREADS) ld = nT;
+    mst = nS * ld;
+    mt = mst + mx;
+    const bool packed = nt + 1 < 65535;
     int32_t* cmat = bufT<int32_t>(c, B_NS_COST, mst);
     int32_t* tail = bufT<int32_t>(c, B_S_TAIL, mx);
     int32_t* head = bufT<int32_t>(c, B_S_HEAD, mx);
-    int32_t* cost = bufT<int32_t>(c, B_TR_XCOST, mx);
-    if (!S || !T || !sup || !tail || !head || !cost || !cmat) return PD_ENOMEM;
+    int32_t* cost = bufT<int32_t>(c, B_TR_XCOST, mx + 3);
+    uint32_t* th = packed ? bufT<uint32_t>(c, B_TR_XTH, mx + 3) : nullptr;
+    if (!S || !T || !sup || !tail || !head || !cost || !cmat || (packed && !th)) return PD_ENOMEM;
     k_side_lists<<<grid_for(N, 256), 256, 0, st>>>(nodes.cntA, nodes.cntB, N, fs, ft, S, T, sup, nS); pd::count_launch();
     c->h_small[20] = dsup;
     PD_TRY_CUDA(c, cudaMemcpyAsync(sup + nS + nT, c->h_small + 20, sizeof(int64_t), cudaMemcpyHostToDevice, st));
     PD_TRY_CUDA(c, cudaMemsetAsync(sm, 0, 8 * sizeof(unsigned long long), st));
-    if (mt > 0)
-        k_transport_arcs<<<grid_for(mt, 256), 256, 0, st>>>(S, T, nS, nT, dsup < 0 ? -1 : (dsup > 0 ? 1 : 0),
-                                                              nodes.X, nodes.Y, cmat, tail, head, cost, sm, diag_cost(o)); pd::count_launch();
+    if (mt > 0) {
+        k_transport_arcs<<<grid_for(mt + 3, 256), 256, 0, st>>>(S, T, nS, nT, ld, dsup < 0 ? -1 : (dsup > 0 ? 1 : 0),
+                                                                  nodes.X, nodes.Y, cmat, tail, head, cost, th, sm,
+                                                                  diag_cost(o)); pd::count_launch();
+    }
     PD_TRY_CUDA(c, cudaGetLastError());
-    if (mst > 0) k_max_cost32<<<grid_for(mst, 256), 256, 0, st>>>(cmat, mst, sm + 1); pd::count_launch();
-    if (mx > 0) k_max_cost32<<<grid_for(mx, 256), 256, 0, st>>>(cost, mx, sm + 1); pd::count_launch();
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
     if (c->h_small[0] != 0) return PD_OK;  // a cost does not fit in int32: solve the sparse network
-    PD_TRY(ns_prepare_arcs(c, (int32_t)nt, mt, mst, nS, nT, cmat, tail, head, cost, sup, c->h_small[1], o, &w->ns,
-                           st));
+    NSArcs arcs;
+    arcs.m = mt;
+    arcs.mst = mst;
+    arcs.nS = nS;
+    arcs.nT = nT;
+    arcs.ld = ld;
+    arcs.cmat = cmat;
+    arcs.th = th;
+    arcs.tail = tail;
+    arcs.head = head;
+    arcs.cost = cost;
+    arcs.complete = true;
+    PD_TRY(ns_prepare_arcs(c, (int32_t)nt, arcs, sup, c->h_small[1], o, &w->ns, st));
     w->S = S;
     w->T = T;
     w->nS = nS;
     w->nT = nT;
+    w->ld = ld;
     w->nt = nt;
     w->dc = diag_cost(o);
     return PD_OK;
@@ -1248,7 +1410,7 @@ pd_status ns_finish_w1(Ctx* c, const WsTree& tr, int64_t s, const pd_network* me
         unsigned long long* sm = bufT<unsigned long long>(c, B_SMALL, 64);
         if (!sm) return PD_ENOMEM;
         PD_TRY_CUDA(c, cudaMemsetAsync(sm, 0, 4 * sizeof(unsigned long long), st));
-        k_certify_tree<<<grid_for(w.nt, 256), 256, 0, st>>>(d_res, w.S, w.T, w.nS, w.nT, tr, s, w.dc, sm); pd::count_launch();
+        k_certify_tree<<<grid_for(w.nt, 256), 256, 0, st>>>(d_res, w.S, w.T, w.nS, w.ld, tr, s, w.dc, sm); pd::count_launch();
         PD_TRY_CUDA(c, cudaGetLastError());
         PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
         PD_TRY_CUDA(c, cudaStreamSynchronize(st));

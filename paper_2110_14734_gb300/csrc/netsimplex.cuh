@@ -12,12 +12,17 @@ constexpr int NS_THREADS = 1024;
 struct NSInst {
     int32_t n;         // real nodes (root = n)
     int64_t m;         // real arcs
-    // arcs a < mst are implicit: tail a / nT, head nS + a % nT, cost cmat[a];
-    // arcs mst <= a < m are explicit: tail/head/cost[a - mst]
+    // arcs a < mst = nS * ld are implicit: tail a / ld, head nS + a % ld, cost
+    // cmat[a]; columns nT <= j < ld pad a row to a multiple of eight (cost
+    // NS_PAD_COST, never chosen).  Arcs mst <= a < m are explicit: ends from
+    // th (tail << 16 | head) when given, else tail/head, cost[a - mst]; th and
+    // cost are readable up to a multiple of four arcs
     int64_t mst;
     int64_t nT;
     int64_t nS;
+    int64_t ld;
     const int32_t* cmat;
+    const uint32_t* th;
     const int32_t* tail;
     const int32_t* head;
     const int32_t* cost;
@@ -35,7 +40,10 @@ struct NSInst {
     int32_t* path;     // 2 (n + 1) scratch: the two half-cycles past the shared-memory part
     int32_t* seg;      // 3 * (2n + 3) scratch: segment start, length, output offset
     int64_t block;     // pricing block (arcs)
-    int64_t big;       // cost of the artificial arcs (more than any path cost)
+    int64_t big;       // cost of the artificial arcs
+    int64_t big64;     // ... that the 64-bit kernel takes when it solves the instance again: more than any path cost
+    int32_t lay32;     // k_simplex32's layout (1 .. 3); 0: the instance belongs to k_netsimplex
+    int32_t big_safe;  // 1: `big` proves infeasibility when artificial flow remains
     int32_t smem_nodes; // node arrays: 1 all in shared memory, 2 all but pred / flow, 3 the 16-bit ones, 0 global
     int32_t walk;      // shared-memory layout: longest half-cycle side followed by the two-lane walk (longer: the scan)
     int32_t init_tree;  // 1: pi, pred, parent, flow, up, ord, pos, size hold a strongly feasible start
@@ -47,9 +55,31 @@ struct NSInst {
     int64_t opt;
     int64_t pivots;
     int64_t degenerate;
-    int32_t status;    // 0 ok, 1 infeasible, 2 pivot cap / time, 3 unbounded, 4 path too long
+    int32_t status;    // 0 ok, 1 infeasible, 2 pivot cap / time, 3 unbounded, 4 path too long, S32_REDO
     int32_t pad;
 };
+
+constexpr int32_t NS_PAD_COST = 1 << 30;  // cost of a matrix row's padding columns
+constexpr int64_t S32_MAX_COST = int64_t(1) << 25;  // k_simplex32: largest arc cost ...
+constexpr int64_t S32_MAX_BIG = int64_t(1) << 26;   // ... and artificial cost
+constexpr int32_t S32_REDO = 5;  // status: k_netsimplex has to solve the instance
+
+// The simplex on 32-bit potentials (simplex32.cu), for records with lay32 > 0:
+// a kernel per class (layout and arc form), persistent like k_netsimplex, one
+// CTA per SM.
+constexpr int S32_CLASSES = 6;
+int s32_class(const NSInst& h);  // -1: not a 32-bit instance
+int s32_layout(int64_t N1);      // the smallest layout that holds N1 nodes (0: none)
+void s32_launch(int cls, int grid, NSInst* insts, const int32_t* order, int32_t count, int32_t* next,
+                cudaStream_t st);
+cudaError_t s32_kernel_setup();  // as ns_kernel_setup
+// Ends of CSR arcs packed as tail << 16 | head and their costs in 32 bits, both
+// padded to a multiple of four arcs; bad += costs outside [0, 2^31), *cmax =
+// the largest.  n < 65535.
+__global__ void k_arc_pack(const int64_t* __restrict__ rp, const int32_t* __restrict__ hd,
+                           const int64_t* __restrict__ cost, int64_t n, int64_t m, uint32_t* __restrict__ th,
+                           int32_t* __restrict__ c32, unsigned long long* __restrict__ bad,
+                           unsigned long long* __restrict__ cmax);
 
 // Persistent over `count` instance records taken in `order` (next = a zeroed
 // device counter); results are written back into the records.
@@ -74,7 +104,6 @@ __global__ void k_check_network(const int64_t* __restrict__ rp, const int32_t* _
 // An instance ready to launch (buffers of the context that prepared it).
 struct NSPrep {
     NSInst h{};
-    size_t smem = 0;     // dynamic shared memory it needs
     bool ready = false;  // false: nothing to solve
 };
 
@@ -84,16 +113,27 @@ struct W1Prep {
     DiagCost dc{1, 0, 0};  // creation / destruction costs of the diagonal node's routes
     const int32_t* S = nullptr;
     const int32_t* T = nullptr;
-    int64_t nS = 0, nT = 0, nt = 0;
+    int64_t nS = 0, nT = 0, ld = 0, nt = 0;
 };
 
-pd_status ns_prepare_arcs(Ctx* c, int32_t n, int64_t m, int64_t mst, int64_t nS, int64_t nT, const int32_t* cmat,
-                          const int32_t* tail, const int32_t* head, const int32_t* cost, const int64_t* supply,
-                          int64_t cmax, const pd_opts& o, NSPrep* p, cudaStream_t st);
-// Runs `count` prepared instances in one launch (one CTA each): h -> device
-// records d -> results r (host), synchronising the stream; smem = the largest
-// dynamic shared memory of the instances.
-pd_status ns_run(Ctx* c, const NSInst* h, int count, size_t smem, NSInst* d, NSInst* r, cudaStream_t st);
+// The arcs of an instance (see NSInst).
+struct NSArcs {
+    int64_t m = 0, mst = 0, nS = 0, nT = 1, ld = 1;
+    const int32_t* cmat = nullptr;
+    const uint32_t* th = nullptr;
+    const int32_t* tail = nullptr;
+    const int32_t* head = nullptr;
+    const int32_t* cost = nullptr;
+    bool complete = false;  // every supply node has an arc to every demand node
+};
+pd_status ns_prepare_arcs(Ctx* c, int32_t n, const NSArcs& a, const int64_t* supply, int64_t cmax, const pd_opts& o,
+                          NSPrep* p, cudaStream_t st);
+// Runs `count` prepared instances (one CTA each): h -> device records d ->
+// results r (host), synchronising the stream.
+pd_status ns_run(Ctx* c, const NSInst* h, int count, NSInst* d, NSInst* r, cudaStream_t st);
+// The kernel an instance goes to, its layout and its artificial costs.
+int64_t ns_default_block(const NSInst& h);
+void ns_choose_kernel(NSInst* h, int64_t cmax, bool complete, bool smem, int max_optin);
 pd_status ns_status(Ctx* c, const NSInst& r);
 pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t dsup, const pd_opts& o, W1Prep* w,
                         cudaStream_t st);
@@ -104,7 +144,7 @@ pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t d
 pd_status ns_finish_w1(Ctx* c, const WsTree& tr, int64_t s, const pd_network* merged, const pd_opts& o,
                        const W1Prep& w, const NSInst* d_res, const NSInst& r, SolveStats* out, cudaStream_t st);
 __global__ void k_certify_tree(const NSInst* __restrict__ I, const int32_t* __restrict__ S,
-                               const int32_t* __restrict__ T, int64_t nS, int64_t nT, WsTree tr, int64_t s,
+                               const int32_t* __restrict__ T, int64_t nS, int64_t ld, WsTree tr, int64_t s,
                                DiagCost dc, unsigned long long* __restrict__ out);
 
 // One pair's certificate in a batched launch: its solved record, its
@@ -114,7 +154,7 @@ struct CertJob {
     int64_t rec;         // index of the pair's record in the wave
     const int32_t* S;
     const int32_t* T;
-    int64_t nS, nT, s;
+    int64_t nS, ld, s;
     WsTree tree;
     DiagCost dc;
 };
@@ -124,7 +164,7 @@ __global__ void k_certify_batch(const CertJob* __restrict__ jobs, unsigned long 
 // One wave of a batch as a CUDA graph: upload of the records, the persistent
 // simplex over all of them, every pair's certificate, download of records and
 // certificate counts.  Captured once per configuration, replayed per wave.
-pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, size_t smem, const CertJob* jobs, NSInst* r,
+pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, const CertJob* jobs, NSInst* r,
                       unsigned long long* cert, cudaStream_t st);
 
 }  // namespace pd

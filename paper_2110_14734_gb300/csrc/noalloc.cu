@@ -22,8 +22,8 @@ constexpr int64_t NA_ARCS = PD_NOALLOC_MAX_ARCS;
 
 constexpr size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t OFF_TAIL = 0;
-constexpr size_t OFF_COST = OFF_TAIL + al(4 * NA_ARCS);
-constexpr size_t OFF_PI = OFF_COST + al(4 * NA_ARCS);
+constexpr size_t OFF_COST = OFF_TAIL + al(4 * (NA_ARCS + 3));
+constexpr size_t OFF_PI = OFF_COST + al(4 * (NA_ARCS + 3));
 constexpr size_t OFF_PRED = OFF_PI + al(8 * NA_NODES);
 constexpr size_t OFF_PARENT = OFF_PRED + al(4 * NA_NODES);
 constexpr size_t OFF_FLOW = OFF_PARENT + al(4 * NA_NODES);
@@ -91,7 +91,7 @@ extern "C" pd_status pd_mcf_solve_noalloc(const pd_network* net, int64_t* opt_ou
         return PD_ECUDA;
     }
     unsigned char* base = (unsigned char*)basev;
-    int32_t* tail = (int32_t*)(base + OFF_TAIL);
+    uint32_t* th = (uint32_t*)(base + OFF_TAIL);
     int32_t* c32 = (int32_t*)(base + OFF_COST);
     unsigned long long* flags = (unsigned long long*)(base + OFF_FLAGS);
     NSInst* dinst = (NSInst*)(base + OFF_INST);
@@ -108,9 +108,8 @@ extern "C" pd_status pd_mcf_solve_noalloc(const pd_network* net, int64_t* opt_ou
     NA_TRY(cudaMemsetAsync(flags, 0, 64, st));
     k_check_network<<<grid_for(n, 256), 256, 0, st>>>(net->row_ptr, net->head, n, m, flags); pd::count_launch();
     if (m > 0) {
-        k_arc_tails<<<grid_for(m, 256), 256, 0, st>>>(net->row_ptr, n, m, tail); pd::count_launch();
-        k_i64_to_i32_cost<<<grid_for(m, 256), 256, 0, st>>>(net->cost, m, c32, flags + 1); pd::count_launch();
-        k_max_cost<<<grid_for(m, 256), 256, 0, st>>>(net->cost, m, flags + 2); pd::count_launch();
+        k_arc_pack<<<grid_for(32 * (n + 1), 256), 256, 0, st>>>(net->row_ptr, net->head, net->cost, n, m, th, c32,
+                                                                flags + 1, flags + 2); pd::count_launch();
     }
     k_abs_sum<<<grid_for(n, 256), 256, 0, st>>>(net->supply, n, flags + 3); pd::count_launch();
     NA_TRY(cudaGetLastError());
@@ -130,12 +129,10 @@ extern "C" pd_status pd_mcf_solve_noalloc(const pd_network* net, int64_t* opt_ou
     h.mst = 0;
     h.nS = 0;
     h.nT = 1;
-    h.cmat = nullptr;
-    h.tail = tail;
-    h.head = net->head;
+    h.ld = 1;
+    h.th = th;
     h.cost = c32;
     h.supply = net->supply;
-    h.big = N1 * (cmax + 1) + 1;
     h.pi = (int64_t*)(base + OFF_PI);
     h.pred = (int32_t*)(base + OFF_PRED);
     h.parent = (int32_t*)(base + OFF_PARENT);
@@ -147,25 +144,33 @@ extern "C" pd_status pd_mcf_solve_noalloc(const pd_network* net, int64_t* opt_ou
     h.tmp = (int32_t*)(base + OFF_TMP);
     h.path = (int32_t*)(base + OFF_PATH);
     h.seg = (int32_t*)(base + OFF_SEG);
-    int64_t M = m + n;
-    int64_t blk = (int64_t)sqrt((double)M);
-    if (blk < 8 * NS_THREADS) blk = 8 * NS_THREADS;
-    h.block = (blk + 7) & ~(int64_t)7;
     h.max_pivots = int64_t(1) << 40;
     h.time_limit_ns = 60000ull * 1000000ull;
     int dev = 0, max_optin = 0;
     NA_TRY(cudaGetDevice(&dev));
     NA_TRY(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    h.smem_nodes = ns_smem_layout(N1, max_optin);
-    const size_t smem = h.smem_nodes ? ns_smem_bytes(N1, h.smem_nodes) : 0;
+    ns_choose_kernel(&h, cmax, false, true, max_optin);
+    h.block = ns_default_block(h);
     NA_TRY(ns_kernel_setup());
+    NA_TRY(s32_kernel_setup());
     NA_TRY(cudaMemcpyAsync(dinst, &h, sizeof(NSInst), cudaMemcpyHostToDevice, st));
-    int32_t* order = (int32_t*)(flags + 4);  // zeroed with the flags: order = {0}, next = 0
-    k_netsimplex<<<1, NS_THREADS, smem, st>>>(dinst, order, 1, order + 1); pd::count_launch();
-    NA_TRY(cudaGetLastError());
+    int32_t* order = (int32_t*)(flags + 4);  // zeroed with the flags: order = {0}, then both kernels' counters
     NSInst r;
-    NA_TRY(cudaMemcpyAsync(&r, dinst, sizeof(NSInst), cudaMemcpyDeviceToHost, st));
-    NA_TRY(cudaStreamSynchronize(st));
+    r.status = S32_REDO;
+    if (h.lay32) {
+        s32_launch(s32_class(h), 1, dinst, order, 1, order + 1, st);
+        pd::count_launch();
+        NA_TRY(cudaGetLastError());
+        NA_TRY(cudaMemcpyAsync(&r, dinst, sizeof(NSInst), cudaMemcpyDeviceToHost, st));
+        NA_TRY(cudaStreamSynchronize(st));
+    }
+    if (r.status == S32_REDO) {
+        const size_t smem = h.smem_nodes ? ns_smem_bytes(N1, h.smem_nodes) : 0;
+        k_netsimplex<<<1, NS_THREADS, smem, st>>>(dinst, order, 1, order + 2); pd::count_launch();
+        NA_TRY(cudaGetLastError());
+        NA_TRY(cudaMemcpyAsync(&r, dinst, sizeof(NSInst), cudaMemcpyDeviceToHost, st));
+        NA_TRY(cudaStreamSynchronize(st));
+    }
 #undef NA_TRY
     if (r.status == 2) return PD_ETIMEOUT;
     if (r.status == 1 || r.status == 3) return PD_EINFEASIBLE;

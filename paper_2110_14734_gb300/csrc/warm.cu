@@ -28,7 +28,7 @@ constexpr int WS_K = 8;  // candidate arcs per source and per sink
 
 // Top WS_K reduced costs of each listed source row rs[a] over the listed sink
 // columns rt[0..nrt) (one warp per row).  outj: column indices into rt.
-__global__ void k_topk_rows(const int32_t* __restrict__ cmat, int64_t nS, int64_t nT, const float* __restrict__ p,
+__global__ void k_topk_rows(const int32_t* __restrict__ cmat, int64_t nS, int64_t ld, const float* __restrict__ p,
                             const int32_t* __restrict__ rs, int64_t nrs, const int32_t* __restrict__ rt, int64_t nrt,
                             int32_t* __restrict__ outj) {
     const int64_t a = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -45,7 +45,7 @@ __global__ void k_topk_rows(const int32_t* __restrict__ cmat, int64_t nS, int64_
     const float pi = p[row];
     for (int64_t b = lane; b < nrt; b += 32) {
         const int32_t j = rt[b];
-        float r = (float)cmat[row * nT + j] - pi + p[nS + j];
+        float r = (float)cmat[row * ld + j] - pi + p[nS + j];
         if (r < bv[WS_K - 1]) {
             int q = WS_K - 1;
             while (q > 0 && bv[q - 1] > r) {
@@ -86,7 +86,7 @@ __global__ void k_topk_rows(const int32_t* __restrict__ cmat, int64_t nS, int64_
 // Top WS_K reduced costs of each listed sink column rt[b] over the listed
 // source rows (one thread per column; the listed columns ascend, so a warp's
 // loads of one row are close together).  outi: row indices into rs.
-__global__ void k_topk_cols(const int32_t* __restrict__ cmat, int64_t nS, int64_t nT, const float* __restrict__ p,
+__global__ void k_topk_cols(const int32_t* __restrict__ cmat, int64_t nS, int64_t ld, const float* __restrict__ p,
                             const int32_t* __restrict__ rs, int64_t nrs, const int32_t* __restrict__ rt, int64_t nrt,
                             int32_t* __restrict__ outi) {
     const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -102,7 +102,7 @@ __global__ void k_topk_cols(const int32_t* __restrict__ cmat, int64_t nS, int64_
     const float pj = p[nS + j];
     for (int64_t a = 0; a < nrs; a++) {
         const int32_t i = rs[a];
-        float r = (float)cmat[(int64_t)i * nT + j] - p[i] + pj;
+        float r = (float)cmat[(int64_t)i * ld + j] - p[i] + pj;
         if (r < bv[WS_K - 1]) {
             int q = WS_K - 1;
             while (q > 0 && bv[q - 1] > r) {
@@ -119,13 +119,13 @@ __global__ void k_topk_cols(const int32_t* __restrict__ cmat, int64_t nS, int64_
 }
 
 // Reduced costs of the arcs between residual sources rs and residual sinks rt.
-__global__ void k_residual_costs(const int32_t* __restrict__ cmat, int64_t nS, int64_t nT,
+__global__ void k_residual_costs(const int32_t* __restrict__ cmat, int64_t nS, int64_t ld,
                                  const int32_t* __restrict__ rs, int64_t ns, const int32_t* __restrict__ rt, int64_t nt,
                                  int32_t* __restrict__ out) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= ns * nt) return;
     const int64_t a = t / nt, b = t - a * nt;
-    out[t] = cmat[(int64_t)rs[a] * nT + rt[b]];
+    out[t] = cmat[(int64_t)rs[a] * ld + rt[b]];
 }
 
 // Costs of given implicit arcs.
@@ -149,8 +149,8 @@ pd_status ns_warm_tree(Ctx* c, NSPrep* prep, const double* p, int64_t max_residu
     *used = false;
     NSInst& h = prep->h;
     if (!prep->ready) return PD_OK;
-    const int64_t nS = h.nS, nT = h.nT, mst = h.mst, m = h.m, nt = h.n, N1 = nt + 1;
-    if (mst != nS * nT || nt != nS + nT + 1) return PD_OK;  // not a transportation instance
+    const int64_t nS = h.nS, nT = h.nT, ld = h.ld, mst = h.mst, m = h.m, nt = h.n, N1 = nt + 1;
+    if (mst != nS * ld || nt != nS + nT + 1) return PD_OK;  // not a transportation instance
     const int64_t mx = m - mst;
     // supplies and the diagonal node's arcs
     std::vector<int64_t> sup((size_t)nt);
@@ -214,19 +214,19 @@ pd_status ns_warm_tree(Ctx* c, NSPrep* prep, const double* p, int64_t max_residu
         if (full) {
             int32_t* dcost = bufT<int32_t>(c, B_WS_RC, nrs * nrt);
             if (!dcost) return PD_ENOMEM;
-            k_residual_costs<<<grid_for(nrs * nrt, 256), 256, 0, st>>>(h.cmat, nS, nT, drs, nrs, drt, nrt, dcost); pd::count_launch();
+            k_residual_costs<<<grid_for(nrs * nrt, 256), 256, 0, st>>>(h.cmat, nS, ld, drs, nrs, drt, nrt, dcost); pd::count_launch();
             PD_TRY_CUDA(c, cudaGetLastError());
             cc.resize((size_t)(nrs * nrt));
             PD_TRY_CUDA(c, cudaMemcpyAsync(cc.data(), dcost, sizeof(int32_t) * nrs * nrt, cudaMemcpyDeviceToHost, st));
             PD_TRY_CUDA(c, cudaStreamSynchronize(st));
             for (int64_t a = 0; a < nrs; a++)
-                for (int64_t b = 0; b < nrt; b++) cand.push_back((int64_t)rs[(size_t)a] * nT + rt[(size_t)b]);
+                for (int64_t b = 0; b < nrt; b++) cand.push_back((int64_t)rs[(size_t)a] * ld + rt[(size_t)b]);
         } else {
             int32_t* rj = bufT<int32_t>(c, B_WS_ROWK, nrs * WS_K);
             int32_t* ci = bufT<int32_t>(c, B_WS_COLK, nrt * WS_K);
             if (!rj || !ci) return PD_ENOMEM;
-            k_topk_rows<<<grid_for(nrs * 32, 256), 256, 0, st>>>(h.cmat, nS, nT, dp, drs, nrs, drt, nrt, rj); pd::count_launch();
-            k_topk_cols<<<grid_for(nrt, 128), 128, 0, st>>>(h.cmat, nS, nT, dp, drs, nrs, drt, nrt, ci); pd::count_launch();
+            k_topk_rows<<<grid_for(nrs * 32, 256), 256, 0, st>>>(h.cmat, nS, ld, dp, drs, nrs, drt, nrt, rj); pd::count_launch();
+            k_topk_cols<<<grid_for(nrt, 128), 128, 0, st>>>(h.cmat, nS, ld, dp, drs, nrs, drt, nrt, ci); pd::count_launch();
             PD_TRY_CUDA(c, cudaGetLastError());
             hr.resize((size_t)(nrs * WS_K));
             hc.resize((size_t)(nrt * WS_K));
@@ -236,12 +236,12 @@ pd_status ns_warm_tree(Ctx* c, NSPrep* prep, const double* p, int64_t max_residu
             for (int64_t a = 0; a < nrs; a++)
                 for (int q = 0; q < WS_K; q++) {
                     const int32_t b = hr[(size_t)(a * WS_K + q)];
-                    if (b >= 0) cand.push_back((int64_t)rs[(size_t)a] * nT + rt[(size_t)b]);
+                    if (b >= 0) cand.push_back((int64_t)rs[(size_t)a] * ld + rt[(size_t)b]);
                 }
             for (int64_t b = 0; b < nrt; b++)
                 for (int q = 0; q < WS_K; q++) {
                     const int32_t a = hc[(size_t)(b * WS_K + q)];
-                    if (a >= 0) cand.push_back((int64_t)rs[(size_t)a] * nT + rt[(size_t)b]);
+                    if (a >= 0) cand.push_back((int64_t)rs[(size_t)a] * ld + rt[(size_t)b]);
                 }
             std::sort(cand.begin(), cand.end());
             cand.erase(std::unique(cand.begin(), cand.end()), cand.end());
@@ -260,14 +260,14 @@ pd_status ns_warm_tree(Ctx* c, NSPrep* prep, const double* p, int64_t max_residu
         order.resize(cand.size());
         for (size_t q = 0; q < cand.size(); q++) {
             const int64_t a = cand[q];
-            const int32_t t = (int32_t)(a / nT), hh = (int32_t)(nS + a % nT);
+            const int32_t t = (int32_t)(a / ld), hh = (int32_t)(nS + a % ld);
             order[q] = {(double)cc[q] - p[t] + p[hh], (int64_t)q};
         }
         std::sort(order.begin(), order.end());
         bool moved = false;
         for (auto& o : order) {
             const int64_t a = cand[(size_t)o.second];
-            moved |= take(a, (int32_t)(a / nT), (int32_t)(nS + a % nT), cc[(size_t)o.second]);
+            moved |= take(a, (int32_t)(a / ld), (int32_t)(nS + a % ld), cc[(size_t)o.second]);
         }
         if (full || !moved) break;
     }
@@ -281,7 +281,7 @@ pd_status ns_warm_tree(Ctx* c, NSPrep* prep, const double* p, int64_t max_residu
         while (a < rs.size() && b < rt.size()) {
             const int32_t i = rs[a], j = rt[b];
             const int64_t f = std::min(sim[(size_t)i], sim[(size_t)(nS + j)]);
-            cand.push_back((int64_t)i * nT + j);
+            cand.push_back((int64_t)i * ld + j);
             sim[(size_t)i] -= f;
             sim[(size_t)(nS + j)] -= f;
             if (sim[(size_t)i] == 0) a++;
@@ -298,7 +298,7 @@ pd_status ns_warm_tree(Ctx* c, NSPrep* prep, const double* p, int64_t max_residu
         PD_TRY_CUDA(c, cudaMemcpyAsync(cc.data(), dc, sizeof(int32_t) * nc, cudaMemcpyDeviceToHost, st));
         PD_TRY_CUDA(c, cudaStreamSynchronize(st));
         for (int64_t q = 0; q < nc; q++)
-            take(cand[(size_t)q], (int32_t)(cand[(size_t)q] / nT), (int32_t)(nS + cand[(size_t)q] % nT), cc[(size_t)q]);
+            take(cand[(size_t)q], (int32_t)(cand[(size_t)q] / ld), (int32_t)(nS + cand[(size_t)q] % ld), cc[(size_t)q]);
     }
     // the diagonal node's arcs, in ascending reduced cost, for what is left
     std::vector<std::pair<double, int64_t>> dorder((size_t)mx);

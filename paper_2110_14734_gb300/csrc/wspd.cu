@@ -195,18 +195,18 @@ PD_D bool ws_arc_exists(int32_t a, int32_t b, int64_t N, const int32_t* __restri
 // always exist.  out[0] = pairs missing, out[1] = total flow over the arcs of
 // the sparse network that the flow uses (rounding slack).
 __global__ void k_certify_tree(const NSInst* __restrict__ I, const int32_t* __restrict__ S,
-                               const int32_t* __restrict__ T, int64_t nS, int64_t nT, WsTree tr, int64_t s,
+                               const int32_t* __restrict__ T, int64_t nS, int64_t ld, WsTree tr, int64_t s,
                                DiagCost dc, unsigned long long* __restrict__ out) {
     int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= I->n) return;
     int64_t a = I->pred[v], f = I->flow[v];
     if (a >= I->m || f <= 0) return;
-    int64_t mst = nS * nT;
+    int64_t mst = nS * ld;
     if (a >= mst) {  // arc of the diagonal node: one arc of the sparse network
         atomicAdd(&out[1], (unsigned long long)f);
         return;
     }
-    int64_t i = a / nT, j = a - i * nT;
+    int64_t i = a / ld, j = a - i * ld;
     int32_t u = S[i], w = T[j];
     int64_t d = cost_l2(tr.X[u], tr.Y[u], tr.X[w], tr.Y[w]);
     int64_t g = cost_make(tr.X[u], tr.Y[u], dc) + cost_make(tr.X[w], tr.Y[w], dc);
@@ -223,7 +223,7 @@ __global__ void k_certify_batch(const CertJob* __restrict__ jobs, unsigned long 
     const CertJob J = jobs[blockIdx.y];
     const NSInst* I = J.inst;
     unsigned long long* o = out + 2 * (int64_t)blockIdx.y;
-    const int64_t mst = J.nS * J.nT;
+    const int64_t mst = J.nS * J.ld;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < I->n; v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t a = I->pred[v], f = I->flow[v];
         if (a >= I->m || f <= 0) continue;
@@ -231,7 +231,7 @@ __global__ void k_certify_batch(const CertJob* __restrict__ jobs, unsigned long 
             atomicAdd(&o[1], (unsigned long long)f);
             continue;
         }
-        const int64_t i = a / J.nT, j = a - i * J.nT;
+        const int64_t i = a / J.ld, j = a - i * J.ld;
         const int32_t u = J.S[i], w = J.T[j];
         const WsTree& tr = J.tree;
         const int64_t d = cost_l2(tr.X[u], tr.Y[u], tr.X[w], tr.Y[w]);
