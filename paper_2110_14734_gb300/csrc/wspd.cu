@@ -5,6 +5,8 @@
 #include "netsimplex.cuh"
 #include "prims.cuh"
 
+#include <algorithm>
+
 namespace pd {
 
 // ---------------------------------------------------------------------------
@@ -246,213 +248,210 @@ __global__ void k_certify_batch(const CertJob* __restrict__ jobs, unsigned long 
     }
 }
 
-__global__ void k_frontier_init(int64_t N, const int32_t* __restrict__ left, const int32_t* __restrict__ right,
-                                int2* __restrict__ F) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N - 1) F[i] = make_int2(left[i], right[i]);
-}
+// ---------------------------------------------------------------------------
+// enumeration: warps walk the pair tree depth first
+// ---------------------------------------------------------------------------
+//
+// The recursion visits as many pairs as the decomposition has, twice over (at
+// 2 M nodes and s = 167: 21 G separated pairs and as many split ones), and a pair
+// needs only its two nodes.  So what bounds it is the gather of node records
+// and the instructions of a test, as long as the pairs waiting to be visited
+// never leave the SM: every warp keeps them in a stack in shared memory and
+// visits the 32 topmost at a time.  These descend from one pair a few levels
+// up, so the 32 lanes touch about a dozen different nodes.
+//
+// The records.  An internal node's 32 bytes: doubled centre, separation
+// threshold (s + 2)^2 diagonal^2, larger side, children, representative.  A
+// leaf needs its coordinates only, and a pair of leaves nothing: it is always
+// separated, and is counted where it would be pushed.
+//
+// Balance.  Initial pairs (one per internal node) differ by many orders of
+// magnitude in the pairs below them, so a warp that has walked `budget` steps
+// on its chunk hands what is left on its stack to the next launch, where other
+// warps take it up.
+//
+// Measured (pd_w1_sparsify_count's WSPD stage, mixture points, s = 167): 1,000,000
+// + 1,000,000 points 493 -> 165 ms, 100,000 + 100,000 23 -> 7.4 ms, against
+// level-by-level frontiers in global memory (689 GB of DRAM traffic a call, and
+// 128-bit products per test).  Now 70 % of the issue slots and of the L1's
+// throughput are used.
 
-__global__ void k_ws_classify(const int2* __restrict__ F, int64_t nf, const int32_t* __restrict__ X,
-                              const int32_t* __restrict__ Y, const int4* __restrict__ bb,
-                              const int32_t* __restrict__ rep, const int32_t* __restrict__ left,
-                              const int32_t* __restrict__ right, int64_t s, int64_t* __restrict__ flag,
-                              int64_t* __restrict__ off) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nf) return;
-    int2 p = F[i];
-    TNode u = load_tnode(p.x, X, Y, bb, rep, left, right);
-    TNode v = load_tnode(p.y, X, Y, bb, rep, left, right);
-    int64_t w = well_separated(u, v, s) ? 1 : 0;
-    flag[i] = w;
-    off[i] = w;
-}
+struct __align__(32) WsRec {
+    int32_t cx, cy;  // doubled centre
+    uint64_t thr;    // least doubled squared distance that separates (saturated)
+    uint32_t side;   // larger box side
+    int32_t l, r;    // children
+    int32_t rep;
+};
 
-// Well-separated pair -> two directed arcs between the representatives;
-// otherwise split the node with the larger box side (ties split v) into two
-// pairs of the next frontier.
-__global__ void k_ws_expand(const int2* __restrict__ F, int64_t nf, const int64_t* __restrict__ flag,
-                            const int64_t* __restrict__ off, const int32_t* __restrict__ X,
-                            const int32_t* __restrict__ Y, const int4* __restrict__ bb,
-                            const int32_t* __restrict__ rep, const int32_t* __restrict__ left,
-                            const int32_t* __restrict__ right, int hb, uint64_t* __restrict__ arcs,
-                            int2* __restrict__ Fn) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nf) return;
-    int2 p = F[i];
-    TNode u = load_tnode(p.x, X, Y, bb, rep, left, right);
-    TNode v = load_tnode(p.y, X, Y, bb, rep, left, right);
-    int64_t o = off[i];
-    if (flag[i]) {
-        if (arcs) {  // null: only the frontier is built (the arcs are counted by the caller)
-            arcs[2 * o] = ((uint64_t)u.rep << hb) | (uint64_t)v.rep;
-            arcs[2 * o + 1] = ((uint64_t)v.rep << hb) | (uint64_t)u.rep;
-        }
-    } else {
-        int64_t j = i - o;
-        if (max_side(u) > max_side(v)) {
-            Fn[2 * j] = make_int2(u.l, p.y);
-            Fn[2 * j + 1] = make_int2(u.r, p.y);
-        } else {
-            Fn[2 * j] = make_int2(p.x, v.l);
-            Fn[2 * j + 1] = make_int2(p.x, v.r);
-        }
-    }
-}
-
-// Count-only level of the frontier: well-separated pairs are counted, the
-// others split (same rule as k_ws_expand) into the next frontier at slots
-// taken with block-aggregated atomics -- the next frontier's order may differ
-// from run to run, the counts do not.  lv[0] += well-separated pairs, lv[1] = size
-// of the next frontier (capacity 2 nf).
-__global__ void k_ws_count_split(const int2* __restrict__ F, int64_t nf, const int32_t* __restrict__ X,
-                                 const int32_t* __restrict__ Y, const int4* __restrict__ bb,
-                                 const int32_t* __restrict__ rep, const int32_t* __restrict__ left,
-                                 const int32_t* __restrict__ right, int64_t s, int2* __restrict__ Fn,
-                                 unsigned long long* __restrict__ lv) {
+__global__ void k_ws_records(int64_t M, const int4* __restrict__ bb, const int32_t* __restrict__ rep,
+                             const int32_t* __restrict__ left, const int32_t* __restrict__ right, int64_t s,
+                             WsRec* __restrict__ rec, int2* __restrict__ F) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool act = i < nf;
-    bool ws = false;
-    int2 p = make_int2(0, 0);
-    TNode u{}, v{};
-    if (act) {
-        p = F[i];
-        u = load_tnode(p.x, X, Y, bb, rep, left, right);
-        v = load_tnode(p.y, X, Y, bb, rep, left, right);
-        ws = well_separated(u, v, s);
-    }
-    // block-aggregated: one pair of atomics per block (same-address atomics
-    // from every warp of a level of millions of pairs would serialise)
-    __shared__ unsigned s_ws[32], s_sp[32];
-    __shared__ unsigned long long s_base;
-    const unsigned mws = __ballot_sync(0xffffffffu, act && ws), msp = __ballot_sync(0xffffffffu, act && !ws);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    if (lane == 0) {
-        s_ws[wid] = __popc(mws);
-        s_sp[wid] = __popc(msp);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned tw = 0, ts = 0;
-        for (int w = 0; w < nw; w++) {
-            tw += s_ws[w];
-            const unsigned c = s_sp[w];
-            s_sp[w] = ts;  // exclusive prefix of the splits
-            ts += c;
-        }
-        if (tw) atomicAdd(&lv[0], (unsigned long long)tw);
-        s_base = ts ? atomicAdd(&lv[1], 2ull * (unsigned long long)ts) : 0ull;
-    }
-    __syncthreads();
-    if (act && !ws) {
-        const unsigned long long slot =
-            s_base + 2ull * (unsigned long long)(s_sp[wid] + __popc(msp & ((1u << lane) - 1u)));
-        if (max_side(u) > max_side(v)) {
-            Fn[slot] = make_int2(u.l, p.y);
-            Fn[slot + 1] = make_int2(u.r, p.y);
-        } else {
-            Fn[slot] = make_int2(p.x, v.l);
-            Fn[slot + 1] = make_int2(p.x, v.r);
-        }
-    }
+    if (i >= M) return;
+    const int4 b = bb[i];
+    const uint64_t wx = (uint64_t)((int64_t)b.y - b.x), wy = (uint64_t)((int64_t)b.w - b.z);
+    const uint64_t k = (uint64_t)(s + 2) * (uint64_t)(s + 2);
+    const unsigned __int128 t = (unsigned __int128)k * (wx * wx + wy * wy);
+    WsRec q;
+    q.cx = b.x + b.y;  // |coordinate| < 2^30: no overflow
+    q.cy = b.z + b.w;
+    q.thr = (t >> 64) != 0 ? ~0ull : (uint64_t)t;
+    q.side = (uint32_t)(wx > wy ? wx : wy);
+    q.l = left[i];
+    q.r = right[i];
+    q.rep = rep[i];
+    rec[i] = q;
+    F[i] = make_int2(q.l, q.r);  // the first pairs: every internal node's children
 }
 
-// Count-only, three levels per launch: the pair F[i] is tested, its two
-// children, then their up to four children, all in registers (the same test
-// and split rule as k_ws_count_split); separated pairs are counted and the up
-// to eight great-grandchildren go to the next frontier at slots taken with
-// block-aggregated atomics.  Equivalent to three launches of
-// k_ws_count_split, with a third of the launches, host syncs and frontier
-// traffic.  Slots at or above `cap` are not written and lv[2] records it (with
-// cap = 8 nf it cannot happen).
-// lv[0] += separated pairs, lv[1] = size of the next frontier.
-PD_D void ws_split(const TNode& u, const TNode& v, int2 p, int2* c0, int2* c1) {
-    if (max_side(u) > max_side(v)) {
-        *c0 = make_int2(u.l, p.y);
-        *c1 = make_int2(u.r, p.y);
+PD_D WsRec ws_load(int32_t ref, const WsRec* __restrict__ rec, const int32_t* __restrict__ X,
+                   const int32_t* __restrict__ Y) {
+    WsRec q;
+    if (ref < 0) {
+        const int32_t p = ~ref;
+        q.cx = 2 * X[p];
+        q.cy = 2 * Y[p];
+        q.thr = 0;
+        q.side = 0;
+        q.l = q.r = 0;
+        q.rep = p;
     } else {
-        *c0 = make_int2(p.x, v.l);
-        *c1 = make_int2(p.x, v.r);
+        uint32_t w0, w1, w2, w3, w4, w5, w6, w7;
+        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3), "=r"(w4), "=r"(w5), "=r"(w6), "=r"(w7)
+            : "l"(rec + ref));
+        q.cx = (int32_t)w0;
+        q.cy = (int32_t)w1;
+        q.thr = (uint64_t)w3 << 32 | w2;
+        q.side = w4;
+        q.l = (int32_t)w5;
+        q.r = (int32_t)w6;
+        q.rep = (int32_t)w7;
     }
+    return q;
 }
 
-__global__ void __launch_bounds__(256) k_ws_count_split3(const int2* __restrict__ F, int64_t nf,
-                                                         const int32_t* __restrict__ X,
-                                                         const int32_t* __restrict__ Y, const int4* __restrict__ bb,
-                                                         const int32_t* __restrict__ rep,
-                                                         const int32_t* __restrict__ left,
-                                                         const int32_t* __restrict__ right, int64_t s,
-                                                         int2* __restrict__ Fn, unsigned long long cap,
-                                                         unsigned long long* __restrict__ lv) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned cnt = 0;
-    int2 L1[2], L2[4], L3[8];
-    unsigned m1 = 0, m2 = 0, m3 = 0;  // which entries of each level are live
-    if (i < nf) {
-        const int2 p = F[i];
-        const TNode u = load_tnode(p.x, X, Y, bb, rep, left, right);
-        const TNode v = load_tnode(p.y, X, Y, bb, rep, left, right);
-        if (well_separated(u, v, s)) cnt++;
-        else {
-            ws_split(u, v, p, &L1[0], &L1[1]);
-            m1 = 3u;
+// well_separated on records: doubled squared distance >= both thresholds.  The
+// distance's 64 bits overflow only for coordinates near the limit; then the
+// 128-bit test decides.
+PD_D bool ws_far(const WsRec& a, const WsRec& b, int32_t ra, int32_t rb, int64_t s, const WsTree& tr) {
+    const uint32_t dx = a.cx > b.cx ? (uint32_t)a.cx - (uint32_t)b.cx : (uint32_t)b.cx - (uint32_t)a.cx;
+    const uint32_t dy = a.cy > b.cy ? (uint32_t)a.cy - (uint32_t)b.cy : (uint32_t)b.cy - (uint32_t)a.cy;
+    const uint64_t x2 = (uint64_t)dx * dx, d2 = x2 + (uint64_t)dy * dy;
+    if (d2 < x2)
+        return well_separated(load_tnode(ra, tr.X, tr.Y, tr.bb, tr.rep, tr.left, tr.right),
+                              load_tnode(rb, tr.X, tr.Y, tr.bb, tr.rep, tr.left, tr.right), s);
+    return d2 >= a.thr && d2 >= b.thr;
+}
+
+constexpr int WS_WARPS = 8;      // per block
+constexpr int WS_STACK = 736;    // pairs a warp's stack holds
+constexpr int WS_MARGIN = 200;   // above WS_STACK - WS_MARGIN pairs it visits one at a time: a path is
+                                 // at most 2 * 65 splits long (78 + 78 on the split tree), each net +1
+
+// lv[0] += separated pairs, lv[1] = pairs offered to the next launch (the first
+// cap of them are in Fn), lv[2] = initial pairs taken.  STORE: both arcs of every separated
+// pair to arcs, at slots from lv[0] (which counts pairs).
+template <bool STORE>
+__global__ void __launch_bounds__(32 * WS_WARPS) k_ws_walk(const int2* __restrict__ F, int64_t nf, int chunk,
+                                                           const WsRec* __restrict__ rec, WsTree tr, int64_t s,
+                                                           int64_t budget, int2* __restrict__ Fn,
+                                                           unsigned long long cap, int hb, uint64_t* __restrict__ arcs,
+                                                           unsigned long long* __restrict__ lv) {
+    __shared__ int2 stack_[WS_WARPS][WS_STACK];
+    const int lane = threadIdx.x & 31;
+    int2* const st = stack_[threadIdx.x >> 5];
+    const unsigned below = (1u << lane) - 1u;
+    unsigned long long count = 0;
+    // up to three separated pairs of a lane, by their representatives
+    auto emit = [&](bool on0, int2 a0, bool on1, int2 a1, bool on2, int2 a2) {
+        if constexpr (STORE) {
+            const unsigned m0 = __ballot_sync(0xffffffffu, on0), m1 = __ballot_sync(0xffffffffu, on1),
+                           m2 = __ballot_sync(0xffffffffu, on2);
+            if ((m0 | m1 | m2) == 0) return;
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(&lv[0], (unsigned long long)(__popc(m0) + __popc(m1) + __popc(m2)));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            auto put = [&](bool on, unsigned m, int2 a) {
+                if (on) {
+                    ulonglong2 w;
+                    w.x = (uint64_t)a.x << hb | (uint64_t)a.y;
+                    w.y = (uint64_t)a.y << hb | (uint64_t)a.x;
+                    *(ulonglong2*)(arcs + 2 * (at + __popc(m & below))) = w;
+                }
+                at += __popc(m);
+            };
+            put(on0, m0, a0);
+            put(on1, m1, a1);
+            put(on2, m2, a2);
+        } else {
+            count += (unsigned)on0 + (unsigned)on1 + (unsigned)on2;
         }
-    }
-#pragma unroll
-    for (int q = 0; q < 2; q++)
-        if (m1 >> q & 1u) {
-            const TNode u = load_tnode(L1[q].x, X, Y, bb, rep, left, right);
-            const TNode v = load_tnode(L1[q].y, X, Y, bb, rep, left, right);
-            if (well_separated(u, v, s)) cnt++;
-            else {
-                ws_split(u, v, L1[q], &L2[2 * q], &L2[2 * q + 1]);
-                m2 |= 3u << (2 * q);
+    };
+    int h = 0;  // height of the stack
+    int64_t steps = 0;
+    for (;;) {
+        int2 p = make_int2(0, 0);
+        bool on;
+        if (h == 0) {
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(&lv[2], (unsigned long long)chunk);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (at >= (unsigned long long)nf) break;
+            on = lane < chunk && at + lane < (unsigned long long)nf;
+            if (on) p = F[at + lane];
+            const bool leaves = on && p.x < 0 && p.y < 0;
+            emit(leaves, make_int2(~p.x, ~p.y), false, p, false, p);
+            on = on && !leaves;
+            steps = 0;
+        } else {
+            const int take = h > WS_STACK - WS_MARGIN ? 1 : min(h, 32);
+            h -= take;
+            on = lane < take;
+            if (on) p = st[h + lane];
+            __syncwarp();
+        }
+        int2 c0 = make_int2(-1, -1), c1 = make_int2(-1, -1);
+        bool far = false;
+        WsRec u{}, v{};
+        if (on) {
+            u = ws_load(p.x, rec, tr.X, tr.Y);
+            v = ws_load(p.y, rec, tr.X, tr.Y);
+            far = ws_far(u, v, p.x, p.y, s, tr);
+            if (!far) {
+                // split the node with the larger box side, ties split the second
+                const bool su = u.side > v.side;
+                c0 = su ? make_int2(u.l, p.y) : make_int2(p.x, v.l);
+                c1 = su ? make_int2(u.r, p.y) : make_int2(p.x, v.r);
             }
         }
-#pragma unroll
-    for (int q = 0; q < 4; q++)
-        if (m2 >> q & 1u) {
-            const TNode u = load_tnode(L2[q].x, X, Y, bb, rep, left, right);
-            const TNode v = load_tnode(L2[q].y, X, Y, bb, rep, left, right);
-            if (well_separated(u, v, s)) cnt++;
-            else {
-                ws_split(u, v, L2[q], &L3[2 * q], &L3[2 * q + 1]);
-                m3 |= 3u << (2 * q);
-            }
+        const bool open = on && !far;
+        const bool l0 = open && (c0.x & c0.y) < 0, l1 = open && (c1.x & c1.y) < 0;  // two leaves
+        emit(far, make_int2(u.rep, v.rep), l0, make_int2(~c0.x, ~c0.y), l1, make_int2(~c1.x, ~c1.y));
+        const bool p0 = open && !l0, p1 = open && !l1;
+        const unsigned m0 = __ballot_sync(0xffffffffu, p0), m1 = __ballot_sync(0xffffffffu, p1);
+        const int at = h + __popc(m0 & below) + __popc(m1 & below);
+        if (p0) st[at] = c0;
+        if (p1) st[at + p0] = c1;
+        h += __popc(m0) + __popc(m1);
+        __syncwarp();
+        if (++steps > budget && h > 0) {
+            // to the next launch, as far as it still has room
+            unsigned long long at2 = cap;
+            if (lane == 0 && *(volatile unsigned long long*)&lv[1] < cap) at2 = atomicAdd(&lv[1], (unsigned long long)h);
+            at2 = __shfl_sync(0xffffffffu, at2, 0);
+            const int give = at2 >= cap ? 0 : (int)min((unsigned long long)h, cap - at2);
+            for (int q = lane; q < give; q += 32) Fn[at2 + q] = st[h - give + q];
+            h -= give;
+            steps = 0;
+            __syncwarp();
         }
-    // counts and slots: warp sums and prefixes, then one atomic per block
-    __shared__ unsigned s_ws[32], s_sp[32];
-    __shared__ unsigned long long s_base;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    const unsigned k = __popc(m3);
-    unsigned incl = k, wc = cnt;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
     }
-    for (int o = 16; o > 0; o >>= 1) wc += __shfl_xor_sync(0xffffffffu, wc, o);
-    if (lane == 31) s_sp[wid] = incl;
-    if (lane == 0) s_ws[wid] = wc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long tw = 0, ts = 0;
-        for (int w = 0; w < nw; w++) {
-            tw += s_ws[w];
-            const unsigned c = s_sp[w];
-            s_sp[w] = (unsigned)ts;  // exclusive prefix of the warps' outputs
-            ts += c;
-        }
-        if (tw) atomicAdd(&lv[0], tw);
-        s_base = ts ? atomicAdd(&lv[1], ts) : 0ull;
-        if (ts && s_base + ts > cap) atomicOr(&lv[2], 1ull);
+    if constexpr (!STORE) {
+        for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
+        if (lane == 0 && count) atomicAdd(&lv[0], count);
     }
-    __syncthreads();
-    unsigned long long slot = s_base + s_sp[wid] + (incl - k);
-#pragma unroll
-    for (int q = 0; q < 8; q++)
-        if (m3 >> q & 1u) {
-            if (slot < cap) Fn[slot] = L3[q];
-            slot++;
-        }
 }
 
 // Diagonal arcs: u -> ā if u holds A mass, b̄ -> u if u holds B mass, and
@@ -587,6 +586,54 @@ pd_status merge_diagonal(Ctx* c, const pd_network& net, int64_t N, pd_network* o
     return PD_OK;
 }
 
+// All launches of the walk over the tree's pairs (see k_ws_walk): *pairs =
+// separated pairs; arcs (may be null): where their arcs go.
+static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, int64_t s, int hb, uint64_t* arcs, int64_t* pairs,
+                         cudaStream_t st) {
+    unsigned long long* lv = bufT<unsigned long long>(c, B_SMALL, 64) + 12;
+    const int blocks = 4 * std::max(c->sm_count, 1);  // the stacks of four blocks fit an SM
+    const int64_t warps = (int64_t)blocks * WS_WARPS;
+    // room for handed-on pairs: the more, the better the balance; less will do
+    int64_t cap = std::min<int64_t>(int64_t(1) << 27, std::max<int64_t>(int64_t(1) << 16, 64 * (tr.N - 1)));
+    int2* out[2];
+    for (;; cap /= 4) {
+        out[0] = bufT<int2>(c, B_F1, cap);
+        out[1] = out[0] ? bufT<int2>(c, B_WSOFF, cap) : nullptr;
+        if (out[0] && out[1]) break;
+        if (cap <= (int64_t(1) << 16)) return PD_ENOMEM;
+        c->err.clear();
+    }
+    const int2* F = (const int2*)c->ptr[B_F0];
+    int64_t nf = tr.N - 1, total = 0;
+    // short first launches spread the few large pairs, later ones finish
+    // Steps a warp spends on a chunk.  Many chunks: longer, so that the handed-on
+    // pairs fit (2 M nodes: 165 ms with 512, 166 with 128, the room used up and
+    // 3,700 ms with 48).  Few: shorter (8,271 lattice nodes: 0.55 ms with 48, 0.66
+    // with 128, 0.90 with 512).
+    const int64_t budget = tr.N > (int64_t(1) << 20) ? 512 : 64;
+    for (int64_t round = 0; nf > 0; round++) {
+        const int chunk = (int)std::min<int64_t>(32, std::max<int64_t>(1, nf / warps));
+        PD_TRY_CUDA(c, cudaMemsetAsync(lv + (arcs && round > 0 ? 1 : 0), 0,
+                                       (arcs && round > 0 ? 2 : 3) * sizeof(unsigned long long), st));
+        const unsigned grid = (unsigned)std::min<int64_t>(blocks, ((nf + chunk - 1) / chunk + WS_WARPS - 1) / WS_WARPS);
+        if (arcs) {
+            k_ws_walk<true><<<grid, 32 * WS_WARPS, 0, st>>>(F, nf, chunk, rec, tr, s, budget, out[round & 1],
+                                                            (unsigned long long)cap, hb, arcs, lv); pd::count_launch();
+        } else {
+            k_ws_walk<false><<<grid, 32 * WS_WARPS, 0, st>>>(F, nf, chunk, rec, tr, s, budget, out[round & 1],
+                                                             (unsigned long long)cap, hb, nullptr, lv); pd::count_launch();
+        }
+        PD_TRY_CUDA(c, cudaGetLastError());
+        PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, lv, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        PD_TRY_CUDA(c, cudaStreamSynchronize(st));
+        total = arcs ? c->h_small[0] : total + c->h_small[0];  // with arcs, lv[0] runs on as their slot counter
+        nf = std::min<int64_t>(c->h_small[1], cap);
+        F = out[round & 1];
+    }
+    *pairs = total;
+    return PD_OK;
+}
+
 pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* out, float* ms_tree,
                         float* ms_wspd, float* ms_csr, cudaStream_t st, bool count_only, WsTree* tree,
                         const WsTree* given, DiagCost dc) {
@@ -634,80 +681,27 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
     int hb = bits_for((uint64_t)(N + 2));
     int kb = 2 * hb;
     uint64_t sent = (kb >= 64) ? ~0ull : ((1ull << kb) - 1);
-    // WSPD frontier, one level at a time
-    int64_t nf = N >= 2 ? N - 1 : 0;
-    int64_t fcap = nf > 0 ? nf : 1;
-    int2* F = bufT<int2>(c, B_F0, fcap);
-    if (!F) return PD_ENOMEM;
-    if (nf > 0) k_frontier_init<<<grid_for(nf, 256), 256, 0, st>>>(N, left, right, F); pd::count_launch();
+    // the pairs of the WSPD: counted, then (unless only the count is wanted) stored
+    const WsTree tr{N, nodes.X, nodes.Y, left, right, bb, rep};
     int64_t narcs = 0;
-    int64_t acap = 0;
     uint64_t* arcs = nullptr;
-    int fb = 0;
     int64_t* h = c->h_small;
-    // count only: three levels per launch into a next frontier of 8 nf pairs
-    // (at most 2^32, and only if that much memory can be had), else one level
-    // into 2 nf
-    while (count_only && nf > 0) {
-        unsigned long long* lv = cnts + 12;
-        const Buf nid = fb ? B_F0 : B_F1;
-        int2* Fn = nullptr;
-        if (8 * nf <= (int64_t(1) << 32)) {
-            Fn = bufT<int2>(c, nid, 8 * nf);
-            if (!Fn) c->err.clear();
-        }
-        PD_TRY_CUDA(c, cudaMemsetAsync(lv, 0, 3 * sizeof(unsigned long long), st));
-        if (Fn) {
-            k_ws_count_split3<<<grid_for(nf, 256), 256, 0, st>>>(F, nf, nodes.X, nodes.Y, bb, rep, left, right, s, Fn,
-                                                                 (unsigned long long)(8 * nf), lv); pd::count_launch();
-        } else {
-            Fn = bufT<int2>(c, nid, 2 * nf);
-            if (!Fn) return PD_ENOMEM;
-            k_ws_count_split<<<grid_for(nf, 256), 256, 0, st>>>(F, nf, nodes.X, nodes.Y, bb, rep, left, right, s, Fn,
-                                                                lv); pd::count_launch();
-        }
+    if (N >= 2) {
+        WsRec* rec = bufT<WsRec>(c, B_WSFLAG, N - 1);
+        int2* F = bufT<int2>(c, B_F0, N - 1);
+        if (!rec || !F) return PD_ENOMEM;
+        k_ws_records<<<grid_for(N - 1, 256), 256, 0, st>>>(N - 1, bb, rep, left, right, s, rec, F); pd::count_launch();
         PD_TRY_CUDA(c, cudaGetLastError());
-        PD_TRY_CUDA(c, cudaMemcpyAsync(h, lv, 3 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        PD_TRY_CUDA(c, cudaStreamSynchronize(st));
-        if (h[2]) return fail(c, PD_ECUDA, "WSPD count: frontier slots overflowed");  // cannot happen: 8 per pair
-        narcs += 2 * h[0];
-        nf = h[1];
-        F = Fn;
-        fb ^= 1;
-    }
-    while (nf > 0) {
-        int64_t* flag = bufT<int64_t>(c, B_WSFLAG, nf);
-        int64_t* off = bufT<int64_t>(c, B_WSOFF, nf);
-        if (!flag || !off) return PD_ENOMEM;
-        k_ws_classify<<<grid_for(nf, 256), 256, 0, st>>>(F, nf, nodes.X, nodes.Y, bb, rep, left, right, s, flag, off); pd::count_launch();
-        PD_TRY(scan_i64(c, off, off, nf, (int64_t*)cnts + 8, st));
-        PD_TRY_CUDA(c, cudaMemcpyAsync(h, (int64_t*)cnts + 8, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        PD_TRY_CUDA(c, cudaStreamSynchronize(st));
-        int64_t nws = h[0];
-        int64_t need = narcs + 2 * nws + 2 * N + 1;
-        if (!count_only && need > acap) {
-            // grow the arc buffer, keeping what is there
-            int64_t ncap = need + need / 2 + 1024;
-            uint64_t* tmp = bufT<uint64_t>(c, B_ARCKEY2, ncap);
-            if (!tmp) return PD_ENOMEM;
-            if (narcs) PD_TRY_CUDA(c, cudaMemcpyAsync(tmp, arcs, sizeof(uint64_t) * narcs, cudaMemcpyDeviceToDevice, st));
-            uint64_t* na = bufT<uint64_t>(c, B_ARCKEY, ncap);
-            if (!na) return PD_ENOMEM;
-            if (narcs) PD_TRY_CUDA(c, cudaMemcpyAsync(na, tmp, sizeof(uint64_t) * narcs, cudaMemcpyDeviceToDevice, st));
-            arcs = na;
-            acap = ncap;
+        int64_t pairs = 0;
+        PD_TRY(ws_walk(c, tr, rec, s, hb, nullptr, &pairs, st));
+        narcs = 2 * pairs;
+        if (!count_only) {
+            arcs = bufT<uint64_t>(c, B_ARCKEY, narcs + 2 * N + 1);
+            if (!arcs) return PD_ENOMEM;
+            int64_t again = 0;
+            PD_TRY(ws_walk(c, tr, rec, s, hb, arcs, &again, st));
+            if (again != pairs) return fail(c, PD_ECUDA, "the WSPD's pairs changed between counting and storing");
         }
-        int64_t nn = 2 * (nf - nws);
-        int2* Fn = bufT<int2>(c, fb ? B_F0 : B_F1, nn > 0 ? nn : 1);
-        if (!Fn) return PD_ENOMEM;
-        // F may have moved if its buffer grew: it did not (only Fn's buffer is resized here)
-        k_ws_expand<<<grid_for(nf, 256), 256, 0, st>>>(F, nf, flag, off, nodes.X, nodes.Y, bb, rep, left, right, hb,
-                                                        count_only ? nullptr : arcs + narcs, Fn); pd::count_launch();
-        PD_TRY_CUDA(c, cudaGetLastError());
-        narcs += 2 * nws;
-        nf = nn;
-        F = Fn;
-        fb ^= 1;
     }
     PD_TRY_CUDA(c, cudaEventRecord(ev[2], st));
     if (count_only) {
@@ -727,8 +721,7 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
         return PD_OK;
     }
     if (!arcs) {
-        acap = 2 * N + 1;
-        arcs = bufT<uint64_t>(c, B_ARCKEY, acap);
+        arcs = bufT<uint64_t>(c, B_ARCKEY, 2 * N + 1);
         if (!arcs) return PD_ENOMEM;
     }
     // diagonal arcs + masses
