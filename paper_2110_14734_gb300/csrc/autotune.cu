@@ -127,7 +127,7 @@ extern "C" pd_status pd_autotune(pd_ctx* cx, const pd_diagram* A, const pd_diagr
         Front f;
         PD_TRY(front_half(c, A[i], B[i], eps, o, &f, st, true));
         W1Prep w;
-        PD_TRY(ns_prepare_w1(c, f.nodes, f.net.n_arcs, f.h.FB - f.h.FA, o, &w, st));
+        PD_TRY(ns_prepare_w1(c, f.nodes, f.net.n_arcs, f.h.FA, f.h.FB, o, &w, st));
         if (!w.ns.ready) continue;
         const int64_t M = w.ns.h.m + w.ns.h.n;
         const int cls = tune_class(M);

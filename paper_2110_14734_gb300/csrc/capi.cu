@@ -90,20 +90,6 @@ void* buf(Ctx* c, Buf id, size_t bytes) {
     return p;
 }
 
-pd_status sort_u64(Ctx* c, uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, uint32_t* vals_alt, int64_t n,
-                   int bits, cudaStream_t st) {
-    if (n <= 1 || bits <= 0) return PD_OK;
-    RadixScratch<uint64_t> s;
-    s.k_alt = keys_alt;
-    s.v_alt = vals_alt;
-    int64_t nc = (int64_t)radix_counts_elems<uint64_t>(n);
-    s.counts = bufT<int64_t>(c, B_RS_COUNTS, nc);
-    s.part = bufT<int64_t>(c, B_RS_PART, scan_tiles(nc) + 1);
-    if (!s.counts || !s.part) return PD_ENOMEM;
-    PD_TRY_CUDA(c, radix_sort<uint64_t>(keys, vals, n, bits, s, st));
-    return PD_OK;
-}
-
 pd_status scan_i64(Ctx* c, const int64_t* in, int64_t* out, int64_t n, int64_t* total_dev, cudaStream_t st) {
     int64_t* part = bufT<int64_t>(c, B_SCAN_PART, scan_tiles(n) + 1);
     if (!part) return PD_ENOMEM;
@@ -199,6 +185,7 @@ static bool ctx_init(Ctx* c, int device, size_t cap) {
         cudaGetLastError();
         return false;
     }
+    memset(c->h_small, 0, 64 * sizeof(int64_t));
     return true;
 }
 
@@ -665,7 +652,7 @@ extern "C" pd_status pd_w1_approx(pd_ctx* c, pd_diagram A, pd_diagram B, double 
         PD_TRY(stage_solve(c, f.mnet, o, &ss, st));
     } else {
         W1Prep w;
-        if (transport) PD_TRY(ns_prepare_w1(c, f.nodes, f.net.n_arcs, f.h.FB - f.h.FA, o, &w, st));
+        if (transport) PD_TRY(ns_prepare_w1(c, f.nodes, f.net.n_arcs, f.h.FA, f.h.FB, o, &w, st));
         if (w.ns.ready) {
             bool used = false;
             PD_TRY(warm_start(c, c, f, &w, o, &used, &wst, st));
@@ -795,7 +782,7 @@ static pd_status batch_prepare(Ctx* work, Ctx* slot, const pd_diagram& A, const 
     const bool transport = o.ns_transport != 0;
     PD_TRY(front_half(work, A, B, eps, o, &bp->f, st, transport));
     if (transport)
-        PD_TRY(ns_prepare_w1(slot, bp->f.nodes, bp->f.net.n_arcs, bp->f.h.FB - bp->f.h.FA, o, &bp->w, st));
+        PD_TRY(ns_prepare_w1(slot, bp->f.nodes, bp->f.net.n_arcs, bp->f.h.FA, bp->f.h.FB, o, &bp->w, st));
     if (bp->w.ns.ready) {
         if (o.warm_start != 0 && o.warm_start != 1 && o.warm_start != 4 && o.warm_start != -1)
             return fail(work, PD_EINVAL, "the batched solve takes warm_start -1, 0, 1 or 4");
@@ -1038,7 +1025,7 @@ extern "C" pd_status pd_ws_train(pd_ctx* c, const pd_diagram* A, const pd_diagra
         Front f;
         PD_TRY(front_half(c, A[i], B[i], eps, o, &f, st, true));
         W1Prep w;
-        PD_TRY(ns_prepare_w1(c, f.nodes, f.net.n_arcs, f.h.FB - f.h.FA, o, &w, st));
+        PD_TRY(ns_prepare_w1(c, f.nodes, f.net.n_arcs, f.h.FA, f.h.FB, o, &w, st));
         if (!w.ns.ready) continue;
         NSInst* d = bufT<NSInst>(c, B_NS_INST, 1);
         if (!d) return PD_ENOMEM;

@@ -136,7 +136,7 @@ pd_status ws_coarse_potentials(Ctx* c, const Front& f, const W1Prep& w, const pd
     oc.warm_start = 0;
     oc.ns_block = 0;
     W1Prep wc;
-    if (e == PD_OK) e = ns_prepare_w1(cc, cn, int64_t(1) << 40, f.h.FB - f.h.FA, oc, &wc, st);
+    if (e == PD_OK) e = ns_prepare_w1(cc, cn, int64_t(1) << 40, f.h.FA, f.h.FB, oc, &wc, st);
     if (e != PD_OK) return fail(c, e, "coarse solve: " + cc->err);
     if (!wc.ns.ready) return PD_OK;  // nothing to solve at the coarse level: start cold
     NSInst* d = bufT<NSInst>(cc, B_NS_INST, 1);

@@ -24,8 +24,32 @@ __global__ void k_init_small(int64_t* s) {
     }
 }
 
-// a1: X = rint(b 2^k), Y = rint(d 2^k); keep unless X == Y; flag non-finite
-// or |X|,|Y| >= 2^29; track min/max and the masses of A and B.
+// a1: X = rint(b 2^k), Y = rint(d 2^k) of one point; false (X = Y = 0) when
+// non-finite or |X|, |Y| >= 2^29.
+PD_D bool quantize_point(const void* __restrict__ p, int64_t j, int dt, int k, int32_t* X, int32_t* Y) {
+    int64_t qx = 0, qy = 0;
+    bool ok = true;
+    if (dt == PD_F32) {
+        const float2 v = ((const float2*)p)[j];
+        const double s = ldexp(1.0, k), rb = rint((double)v.x * s), rd = rint((double)v.y * s);
+        ok = fabs(rb) < (double)COORD_LIMIT && fabs(rd) < (double)COORD_LIMIT;  // false for a NaN
+        if (ok) {
+            qx = (int64_t)rb;
+            qy = (int64_t)rd;
+        }
+    } else {
+        const uchar2 v = ((const uchar2*)p)[j];
+        qx = (int64_t)v.x << k;
+        qy = (int64_t)v.y << k;
+        ok = qx < COORD_LIMIT && qy < COORD_LIMIT;
+    }
+    *X = (int32_t)qx;
+    *Y = (int32_t)qy;
+    return ok;
+}
+
+// Quantises all points: keep unless X == Y; track min/max and the masses of A
+// and B; count the rejected ones.
 __global__ void k_quantize(const void* __restrict__ a, int64_t na, int dta, const void* __restrict__ b, int64_t nb,
                            int dtb, int k, int32_t* __restrict__ X, int32_t* __restrict__ Y,
                            uint8_t* __restrict__ keep, int64_t* __restrict__ sm) {
@@ -35,36 +59,11 @@ __global__ void k_quantize(const void* __restrict__ a, int64_t na, int dta, cons
     int isB = 0, kp = 0, bad = 0;
     if (i < n) {
         isB = i >= na;
-        int64_t j = isB ? i - na : i;
-        const void* p = isB ? b : a;
-        int dt = isB ? dtb : dta;
-        int64_t qx, qy;
-        if (dt == PD_F32) {
-            float2 v = ((const float2*)p)[j];
-            double fb = v.x, fd = v.y;
-            double s = ldexp(1.0, k);
-            if (!isfinite(fb) || !isfinite(fd)) {
-                bad = 1;
-                qx = qy = 0;
-            } else {
-                double rb = rint(fb * s), rd = rint(fd * s);
-                if (fabs(rb) >= (double)COORD_LIMIT || fabs(rd) >= (double)COORD_LIMIT) {
-                    bad = 1;
-                    qx = qy = 0;
-                } else {
-                    qx = (int64_t)rb;
-                    qy = (int64_t)rd;
-                }
-            }
-        } else {
-            uchar2 v = ((const uchar2*)p)[j];
-            qx = (int64_t)v.x << k;
-            qy = (int64_t)v.y << k;
-            if (qx >= COORD_LIMIT || qy >= COORD_LIMIT) bad = 1;
-        }
+        int32_t qx, qy;
+        bad = !quantize_point(isB ? b : a, isB ? i - na : i, isB ? dtb : dta, k, &qx, &qy);
         kp = !bad && qx != qy;
-        X[i] = (int32_t)qx;
-        Y[i] = (int32_t)qy;
+        X[i] = qx;
+        Y[i] = qy;
         keep[i] = (uint8_t)kp;
         if (kp) {
             mnx = mxx = qx;
@@ -141,17 +140,161 @@ __global__ void k_hat_counts(const int64_t* __restrict__ start, int64_t M, int64
     cnt[j] = e - start[j];
 }
 
+// ---- short inputs: a whole stage in one block, one launch -----------------
+//
+// At a few thousand points a stage is all launches (18 for the 0-condensation,
+// 35 for the delta-condensation, of 2 to 3 microseconds each, and a host round
+// trip in the middle for the key's width).  One block of 1,024 threads holds up
+// to CS_MAX points in registers, sorts them in shared memory and writes the
+// results; widths stay on the device.  out (host memory): the stage's scalars.
+// Measured for two diagrams of 2,000 points: pd_rwmd_lower_bound 250 -> (see
+// k_rwmd_small), the two condensations together 0.53 -> 0.08 ms.
+
+struct CtaStage {
+    CtaSort sort;
+    int32_t ext[4][CS_WARPS];
+    uint32_t count[4];
+};
+
+// Extremes of the block's x and y (min x, max x, min y, max y) in every thread;
+// values beyond the items are passed as the neutral ones.
+PD_D void cta_box(CtaStage& s, int32_t (&b)[4]) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        b[q] = q & 1 ? __reduce_max_sync(0xffffffffu, b[q]) : __reduce_min_sync(0xffffffffu, b[q]);
+        if (lane == 0) s.ext[q][w] = b[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; q++)
+        b[q] = q & 1 ? __reduce_max_sync(0xffffffffu, s.ext[q][lane]) : __reduce_min_sync(0xffffffffu, s.ext[q][lane]);
+    __syncthreads();
+}
+
+PD_D int dev_bits_for(uint32_t v) { return 32 - __clz((int)v); }  // 0 for 0
+
+__global__ void __launch_bounds__(CS_THREADS) k_condense0_small(const void* __restrict__ a, int na, int dta,
+                                                                const void* __restrict__ b, int nb, int dtb, int k,
+                                                                int32_t* __restrict__ HX, int32_t* __restrict__ HY,
+                                                                int64_t* __restrict__ cnt, int64_t* __restrict__ sm,
+                                                                int64_t* out) {
+    extern __shared__ __align__(16) unsigned char cond_dyn[];
+    CtaStage& s = *(CtaStage*)cond_dyn;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, n = na + nb;
+    const int base = w * 32 * CS_ITEMS + lane;
+    if (tid < 4) s.count[tid] = 0;
+    if (tid < S_COUNT) sm[tid] = 0;  // what the next stages add to
+    int32_t box[4] = {INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN}, x[CS_ITEMS], y[CS_ITEMS];
+    uint32_t keep = 0, fa = 0, fb = 0, bad = 0;
+#pragma unroll
+    for (int q = 0; q < CS_ITEMS; q++) {
+        const int i = base + 32 * q;
+        x[q] = y[q] = 0;
+        if (i < n) {
+            const bool isB = i >= na;
+            if (!quantize_point(isB ? b : a, isB ? i - na : i, isB ? dtb : dta, k, &x[q], &y[q])) {
+                bad++;
+            } else if (x[q] != y[q]) {
+                keep |= 1u << q;
+                fa += !isB;
+                fb += isB;
+                box[0] = min(box[0], x[q]);
+                box[1] = max(box[1], x[q]);
+                box[2] = min(box[2], y[q]);
+                box[3] = max(box[3], y[q]);
+            }
+        }
+    }
+    cta_box(s, box);
+    fa = __reduce_add_sync(0xffffffffu, fa);
+    fb = __reduce_add_sync(0xffffffffu, fb);
+    bad = __reduce_add_sync(0xffffffffu, bad);
+    if (lane == 0) {
+        atomicAdd(&s.count[0], fa);
+        atomicAdd(&s.count[1], fb);
+        atomicAdd(&s.count[2], bad);
+    }
+    __syncthreads();
+    const int nv = (int)(s.count[0] + s.count[1]);
+    if (s.count[2] || nv == 0) {
+        if (tid == 0) {
+            out[S_ERR] = s.count[2];
+            out[S_FA] = out[S_FB] = out[S_M] = out[S_NA] = 0;
+        }
+        return;
+    }
+    // diagram bit, then X, then Y; dropped points keep the all-ones key
+    const int bx = dev_bits_for((uint32_t)(box[1] - box[0])), by = dev_bits_for((uint32_t)(box[3] - box[2]));
+    uint64_t key[CS_ITEMS];
+    uint32_t none[CS_ITEMS];
+#pragma unroll
+    for (int q = 0; q < CS_ITEMS; q++) {
+        const uint64_t isB = base + 32 * q >= na;
+        key[q] = keep >> q & 1u ? isB << (bx + by) | (uint64_t)(uint32_t)(x[q] - box[0]) << by | (uint32_t)(y[q] - box[2])
+                                : ~0ull;
+        none[q] = 0;
+    }
+    cta_sort(s.sort, key, none, bx + by + 2);
+    // runs: a thread's items are CS_ITEMS consecutive positions now
+    uint32_t heads = 0;
+    const int p0 = tid * CS_ITEMS;
+#pragma unroll
+    for (int q = 0; q < CS_ITEMS; q++) {
+        const int i = p0 + q;
+        if (i < nv && (i == 0 || s.sort.key[i - 1] != s.sort.key[i])) heads |= 1u << q;
+    }
+    uint32_t M;
+    uint32_t j = block_excl_scan<uint32_t>(__popc(heads), &M);
+    uint32_t* start = s.sort.val;  // first position of every node
+    uint32_t inA = 0;
+    for (uint32_t h = heads; h; h &= h - 1, j++) {
+        const int i = p0 + __ffs(h) - 1;
+        const uint64_t kk = s.sort.key[i];
+        HX[j] = (int32_t)((kk >> by) & ((1ull << bx) - 1)) + box[0];
+        HY[j] = (int32_t)(kk & ((1ull << by) - 1)) + box[2];
+        start[j] = (uint32_t)i;
+        inA += (kk >> (bx + by) & 1ull) == 0;
+    }
+    inA = __reduce_add_sync(0xffffffffu, inA);
+    if (lane == 0) atomicAdd(&s.count[3], inA);
+    __syncthreads();
+    for (uint32_t q = tid; q < M; q += CS_THREADS) cnt[q] = (int64_t)((q + 1 < M ? start[q + 1] : (uint32_t)nv) - start[q]);
+    if (tid == 0) {
+        out[S_ERR] = 0;
+        out[S_FA] = s.count[0];
+        out[S_FB] = s.count[1];
+        out[S_M] = M;
+        out[S_NA] = s.count[3];
+    }
+}
+
 pd_status stage_condense0(Ctx* c, const DevDiag& A, const DevDiag& B, int k, Hats* out, cudaStream_t st) {
     int64_t n = A.n + B.n;
     int64_t* sm = bufT<int64_t>(c, B_SMALL, 64);
     if (!sm) return PD_ENOMEM;
-    k_init_small<<<1, 64, 0, st>>>(sm); pd::count_launch();
     out->nA = out->nB = out->FA = out->FB = 0;
     out->X = bufT<int32_t>(c, B_HAT_X, n);
     out->Y = bufT<int32_t>(c, B_HAT_Y, n);
     out->cnt = bufT<int64_t>(c, B_HAT_C, n);
     if (!out->X || !out->Y || !out->cnt) return PD_ENOMEM;
     if (n == 0) return PD_OK;
+    if (n <= CS_MAX) {
+        int64_t* h = c->h_small;
+        PD_TRY_CUDA(c, cudaFuncSetAttribute(k_condense0_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)sizeof(CtaStage)));
+        k_condense0_small<<<1, CS_THREADS, sizeof(CtaStage), st>>>(A.bd, (int)A.n, A.dtype, B.bd, (int)B.n, B.dtype, k,
+                                                                   out->X, out->Y, out->cnt, sm, h); pd::count_launch();
+        PD_TRY_CUDA(c, cudaGetLastError());
+        PD_TRY_CUDA(c, cudaStreamSynchronize(st));
+        if (h[S_ERR]) return fail(c, PD_EINVAL, "diagram has a non-finite coordinate or |coordinate| * 2^k >= 2^29");
+        out->FA = h[S_FA];
+        out->FB = h[S_FB];
+        out->nA = h[S_NA];
+        out->nB = h[S_M] - h[S_NA];
+        return PD_OK;
+    }
+    k_init_small<<<1, 64, 0, st>>>(sm); pd::count_launch();
     int32_t* X = bufT<int32_t>(c, B_QX, n);
     int32_t* Y = bufT<int32_t>(c, B_QY, n);
     uint8_t* keep = bufT<uint8_t>(c, B_FLAG, n);
@@ -174,7 +317,8 @@ pd_status stage_condense0(Ctx* c, const DevDiag& A, const DevDiag& B, int k, Hat
     int kb = bx + by + 2;
     uint64_t sent = (kb >= 64) ? ~0ull : ((1ull << kb) - 1);
     k_point_keys<<<grid_for(n, 256), 256, 0, st>>>(X, Y, keep, A.n, n, sm, bx, by, key); pd::count_launch();
-    PD_TRY(sort_u64(c, key, key2, nullptr, nullptr, n, kb, st));
+    uint32_t *none = nullptr, *none2 = nullptr;
+    PD_TRY(sort_u64(c, key, key2, none, none2, n, kb, st));
     k_run_flags<<<grid_for(n, 256), 256, 0, st>>>(key, n, sent, flag); pd::count_launch();
     PD_TRY(scan_i64(c, flag, flag, n, sm + S_M, st));
     k_hat_compact<<<grid_for(n, 256), 256, 0, st>>>(key, n, sent, flag, sm, bx, by, out->X, out->Y, start,
@@ -182,6 +326,7 @@ pd_status stage_condense0(Ctx* c, const DevDiag& A, const DevDiag& B, int k, Hat
     PD_TRY_CUDA(c, cudaGetLastError());
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, sizeof(int64_t) * S_COUNT, cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
+    PD_TRY(sort_done(c));
     int64_t M = h[S_M];
     out->nA = h[S_NA];
     out->nB = M - out->nA;
@@ -257,6 +402,53 @@ __global__ void k_rwmd_sum(const int32_t* __restrict__ X, const int32_t* __restr
         if (vb) atomicAdd((unsigned long long*)&L[1], vb);
     }
 }
+
+// ---- short sides: minima and sums in one launch -----------------------------
+// A block takes 32 nodes (a lane each); its eight warps scan an eighth of the
+// other side each, every node of it read by a whole warp at once.
+__global__ void __launch_bounds__(RW_THREADS) k_rwmd_small(const int32_t* __restrict__ X, const int32_t* __restrict__ Y,
+                                                           const int64_t* __restrict__ cnt, int nA, int nB, int blocksA,
+                                                           DiagCost dc, int64_t* __restrict__ L) {
+    __shared__ unsigned long long m[RW_THREADS / 32][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const bool a = (int)blockIdx.x < blocksA;
+    const int first = 32 * ((int)blockIdx.x - (a ? 0 : blocksA)) + lane, np = a ? nA : nB, nq = a ? nB : nA;
+    const int u = (a ? 0 : nA) + first;
+    const int32_t *qx = X + (a ? nA : 0), *qy = Y + (a ? nA : 0);
+    int32_t ux = 0, uy = 0;
+    if (first < np) {
+        ux = X[u];
+        uy = Y[u];
+    }
+    unsigned long long best = ~0ull;
+    const int per = (nq + RW_THREADS / 32 - 1) / (RW_THREADS / 32), q1 = min(nq, (w + 1) * per);
+#pragma unroll 4
+    for (int q = w * per; q < q1; q++) {
+        const long long dx = (long long)(ux - qx[q]), dy = (long long)(uy - qy[q]);
+        const unsigned long long d2 = (unsigned long long)(dx * dx) + (unsigned long long)(dy * dy);
+        best = d2 < best ? d2 : best;
+    }
+    m[w][lane] = best;
+    __syncthreads();
+    if (w != 0) return;
+    unsigned long long v = 0;
+    if (first < np) {
+#pragma unroll
+        for (int q = 1; q < RW_THREADS / 32; q++) best = m[q][lane] < best ? m[q][lane] : best;
+        int64_t c = cost_make(ux, uy, dc);
+        if (best != ~0ull) {
+            const int64_t cn = (int64_t)ceil_sqrt_u64(best);
+            c = cn < c ? cn : c;
+        }
+        v = (unsigned long long)(c * cnt[u]);
+    }
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0 && v) atomicAdd((unsigned long long*)&L[a ? 0 : 1], v);
+}
+
+// One launch instead of three up to here: the scan of a side by one warp's share
+// (nq / 8 nodes) is then no longer than the launches saved.
+constexpr int64_t RW_SMALL = 8192;
 
 // ---- the same minima through a uniform grid over each side ----------------
 // Large sides make the all-pairs scan quadratic (about 10^12 distance
@@ -519,7 +711,11 @@ pd_status stage_rwmd(Ctx* c, const Hats& h, int64_t L[3], DiagCost dc, cudaStrea
     unsigned long long* mind2 = bufT<unsigned long long>(c, B_QKEY2, n);
     if (!sm || !mind2) return PD_ENOMEM;
     PD_TRY_CUDA(c, cudaMemsetAsync(sm + S_L0, 0, 2 * sizeof(int64_t), st));
-    if (n > 0) {
+    if (n > 0 && n <= RW_SMALL) {
+        const int ba = (int)((h.nA + 31) / 32), bb = (int)((h.nB + 31) / 32);
+        k_rwmd_small<<<ba + bb, RW_THREADS, 0, st>>>(h.X, h.Y, h.cnt, (int)h.nA, (int)h.nB, ba, dc, sm + S_L0); pd::count_launch();
+        PD_TRY_CUDA(c, cudaGetLastError());
+    } else if (n > 0) {
         k_fill_u64<<<grid_for(n, 256), 256, 0, st>>>(mind2, n, ~0ull); pd::count_launch();
         int64_t npmax = h.nA > h.nB ? h.nA : h.nB;
         int64_t gx = (npmax + RW_THREADS - 1) / RW_THREADS;
@@ -634,7 +830,7 @@ __global__ void k_cell_accum(const uint64_t* __restrict__ key, const uint32_t* _
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int64_t j = idx[i] + ((i == 0 || key[i - 1] != key[i]) ? 1 : 0) - 1;
-    uint32_t v = val[i];
+    const uint32_t v = min(val[i], (uint32_t)(n - 1));  // in bounds even after a sort that gave up
     atomicAdd((unsigned long long*)((int64_t)v < nA ? &CA[j] : &CB[j]), (unsigned long long)cnt[v]);
 }
 
@@ -653,7 +849,7 @@ __global__ void k_node_gather(const uint64_t* __restrict__ key, const uint32_t* 
                               uint64_t* __restrict__ OC) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    uint32_t v = val[i];
+    const uint32_t v = min(val[i], (uint32_t)(N - 1));  // in bounds even after a sort that gave up
     OX[i] = NX[v];
     OY[i] = NY[v];
     OA[i] = CA[v];
@@ -661,8 +857,118 @@ __global__ void k_node_gather(const uint64_t* __restrict__ key, const uint32_t* 
     OC[i] = key[i];
 }
 
-pd_status stage_condense_delta(Ctx* c, const Hats& h, int64_t G, int64_t P, uint64_t seed, pd_nodes* out,
+// The whole stage for at most CS_MAX 0-condensed nodes (see k_condense0_small).
+__global__ void __launch_bounds__(CS_THREADS) k_condense_delta_small(
+    const int32_t* __restrict__ HX, const int32_t* __restrict__ HY, const int64_t* __restrict__ cnt, int nA, int n,
+    int64_t G, int64_t P, uint64_t seed, int32_t* __restrict__ NX, int32_t* __restrict__ NY, int64_t* __restrict__ CA,
+    int64_t* __restrict__ CB, int32_t* __restrict__ OX, int32_t* __restrict__ OY, int64_t* __restrict__ OA,
+    int64_t* __restrict__ OB, uint64_t* __restrict__ OC, int64_t* out) {
+    extern __shared__ __align__(16) unsigned char cond_dyn[];
+    CtaStage& s = *(CtaStage*)cond_dyn;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int base = w * 32 * CS_ITEMS + lane, p0 = tid * CS_ITEMS;
+    if (tid == 0) s.count[0] = 0;
+    int32_t box[4] = {INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN};
+    uint64_t key[CS_ITEMS];
+    uint32_t val[CS_ITEMS];
+    int32_t cx[CS_ITEMS], cy[CS_ITEMS];  // |cell| <= 2^29: 32 bits
+#pragma unroll
+    for (int q = 0; q < CS_ITEMS; q++) {
+        const int i = base + 32 * q;
+        cx[q] = cy[q] = 0;
+        if (i < n) {
+            cx[q] = (int32_t)floor_div(2 * (int64_t)HX[i] + G, 2 * G);  // nearest lattice point, ties up
+            cy[q] = (int32_t)floor_div(2 * (int64_t)HY[i] + G, 2 * G);
+            box[0] = min(box[0], cx[q]);
+            box[1] = max(box[1], cx[q]);
+            box[2] = min(box[2], cy[q]);
+            box[3] = max(box[3], cy[q]);
+        }
+    }
+    cta_box(s, box);
+    const int bcx = dev_bits_for((uint32_t)(box[1] - box[0])), bcy = dev_bits_for((uint32_t)(box[3] - box[2]));
+#pragma unroll
+    for (int q = 0; q < CS_ITEMS; q++) {
+        const int i = base + 32 * q;
+        key[q] = i < n ? (uint64_t)(uint32_t)(cx[q] - box[0]) << bcy | (uint32_t)(cy[q] - box[2]) : ~0ull;
+        val[q] = (uint32_t)i;
+    }
+    cta_sort(s.sort, key, val, bcx + bcy);
+    // one node per distinct cell, at G * cell + shift(seed, cell)
+    uint32_t heads = 0;
+#pragma unroll
+    for (int q = 0; q < CS_ITEMS; q++) {
+        const int i = p0 + q;
+        if (i < n && (i == 0 || s.sort.key[i - 1] != s.sort.key[i])) heads |= 1u << q;
+    }
+    uint32_t N;
+    const uint32_t j0 = block_excl_scan<uint32_t>(__popc(heads), &N);
+    int32_t nb[4] = {INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN};
+    uint32_t bad = 0, j = j0;
+    for (uint32_t h = heads; h; h &= h - 1, j++) {
+        const uint64_t kk = s.sort.key[p0 + __ffs(h) - 1];
+        const int64_t ccx = (int64_t)(kk >> bcy) + box[0], ccy = (int64_t)(kk & ((1ull << bcy) - 1)) + box[2];
+        int64_t dx, dy;
+        cell_shift(seed, ccx, ccy, P, &dx, &dy);
+        const int64_t X = G * ccx + dx, Y = G * ccy + dy, lim = int64_t(1) << 30;
+        bad |= X <= -lim || X >= lim || Y <= -lim || Y >= lim;
+        NX[j] = (int32_t)X;
+        NY[j] = (int32_t)Y;
+        CA[j] = CB[j] = 0;
+        nb[0] = min(nb[0], (int32_t)X);
+        nb[1] = max(nb[1], (int32_t)X);
+        nb[2] = min(nb[2], (int32_t)Y);
+        nb[3] = max(nb[3], (int32_t)Y);
+    }
+    if (__any_sync(0xffffffffu, bad) && lane == 0) s.count[0] = 1;
+    cta_box(s, nb);  // (and every CA, CB is zero)
+    if (s.count[0]) {
+        if (tid == 0) out[S_ERR] = 1;
+        return;
+    }
+    // multiplicities of the nodes snapped into each cell
+    j = j0;
+#pragma unroll
+    for (int q = 0; q < CS_ITEMS; q++) {
+        const int i = p0 + q;
+        if (i < n) {
+            j += heads >> q & 1u;
+            const uint32_t v = s.sort.val[i];
+            atomicAdd((unsigned long long*)((int)v < nA ? &CA[j - 1] : &CB[j - 1]), (unsigned long long)cnt[v]);
+        }
+    }
+    __syncthreads();
+    // Morton order
+#pragma unroll
+    for (int q = 0; q < CS_ITEMS; q++) {
+        const int i = base + 32 * q;
+        key[q] = i < (int)N ? morton2((uint32_t)NX[i] - (uint32_t)nb[0], (uint32_t)NY[i] - (uint32_t)nb[2]) : ~0ull;
+        val[q] = (uint32_t)i;
+    }
+    const int bm = dev_bits_for(max((uint32_t)nb[1] - (uint32_t)nb[0], (uint32_t)nb[3] - (uint32_t)nb[2]));
+    __syncthreads();
+    cta_sort(s.sort, key, val, 2 * bm);
+#pragma unroll
+    for (int q = 0; q < CS_ITEMS; q++) {
+        const int i = base + 32 * q;
+        if (i < (int)N) {
+            const uint32_t v = val[q];
+            OX[i] = NX[v];
+            OY[i] = NY[v];
+            OA[i] = __ldcg(&CA[v]);  // summed by atomics: not through L1
+            OB[i] = __ldcg(&CB[v]);
+            OC[i] = key[q];
+        }
+    }
+    if (tid == 0) {
+        out[S_ERR] = 0;
+        out[S_N] = N;
+    }
+}
+
+pd_status stage_condense_delta(Ctx* c, const Hats& hats, int64_t G, int64_t P, uint64_t seed, pd_nodes* out,
                                cudaStream_t st) {
+    const Hats& h = hats;
     int64_t n = h.nA + h.nB;
     out->n_nodes = 0;
     out->X = bufT<int32_t>(c, B_NX, n);
@@ -673,6 +979,24 @@ pd_status stage_condense_delta(Ctx* c, const Hats& h, int64_t G, int64_t P, uint
     int64_t* sm = bufT<int64_t>(c, B_SMALL, 64);
     if (!out->X || !out->Y || !out->cntA || !out->cntB || !out->morton || !sm) return PD_ENOMEM;
     if (n == 0) return PD_OK;
+    if (n <= CS_MAX) {
+        int32_t* NX = bufT<int32_t>(c, B_QX, n);
+        int32_t* NY = bufT<int32_t>(c, B_QY, n);
+        int64_t* CA = bufT<int64_t>(c, B_CA, n);
+        int64_t* CB = bufT<int64_t>(c, B_CB, n);
+        if (!NX || !NY || !CA || !CB) return PD_ENOMEM;
+        int64_t* hs = c->h_small;
+        PD_TRY_CUDA(c, cudaFuncSetAttribute(k_condense_delta_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)sizeof(CtaStage)));
+        k_condense_delta_small<<<1, CS_THREADS, sizeof(CtaStage), st>>>(hats.X, hats.Y, hats.cnt, (int)hats.nA, (int)n, G, P,
+                                                                        seed, NX, NY, CA, CB, out->X, out->Y, out->cntA,
+                                                                        out->cntB, out->morton, hs); pd::count_launch();
+        PD_TRY_CUDA(c, cudaGetLastError());
+        PD_TRY_CUDA(c, cudaStreamSynchronize(st));
+        if (hs[S_ERR]) return fail(c, PD_EINVAL, "condensed node coordinate outside (-2^30, 2^30)");
+        out->n_nodes = hs[S_N];
+        return PD_OK;
+    }
     int64_t* CX = bufT<int64_t>(c, B_CX, n);
     int64_t* CY = bufT<int64_t>(c, B_CY, n);
     uint64_t* key = bufT<uint64_t>(c, B_CKEY, n);
@@ -703,6 +1027,7 @@ pd_status stage_condense_delta(Ctx* c, const Hats& h, int64_t G, int64_t P, uint
     PD_TRY_CUDA(c, cudaGetLastError());
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, sizeof(int64_t) * S_COUNT, cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
+    PD_TRY(sort_done(c));
     if (hs[S_ERR]) return fail(c, PD_EINVAL, "condensed node coordinate outside (-2^30, 2^30)");
     int64_t N = hs[S_N];
     int bm = bits_for((uint64_t)(hs[S_NMXX] - hs[S_NMNX]));

@@ -26,7 +26,7 @@ enum Buf : int {
     B_S_ROWPTR, B_S_HEAD, B_S_CW, B_S_TWIN, B_S_X, B_S_PAIR, B_S_XKEY, B_S_XKEY2, B_S_XVAL,
     B_S_XVAL2, B_S_XPTR, B_S_XPOS, B_S_TAIL,
     B_S_E, B_S_P, B_S_D, B_S_CUR, B_S_RELAB, B_S_CTL, B_S_Q,
-    B_RS_COUNTS, B_RS_PART, B_SCAN_PART,
+    B_RS_COUNTS, B_SCAN_PART,
     B_M_ROWPTR, B_M_SUPPLY,
     B_NS_PI, B_NS_PARENT, B_NS_PRED, B_NS_FLOW, B_NS_UP, B_NS_ORD, B_NS_POS, B_NS_SIZE, B_NS_TMP,
     B_NS_PATH, B_NS_SEG, B_NS_INST, B_NS_ORDER, B_NS_COST, B_NS_ART, B_TR_S, B_TR_T, B_TR_SUP, B_TR_XCOST, B_TR_XTH,
@@ -232,9 +232,14 @@ int tune_class(int64_t M);
 int64_t tuned_block(const Ctx* c, int64_t M);
 int32_t tuned_walk(const Ctx* c, int64_t M);  // the walk limit (16 when none was tuned)
 
-// radix sort / scan with context scratch
-pd_status sort_u64(Ctx* c, uint64_t* keys, uint64_t* keys_alt, uint32_t* vals, uint32_t* vals_alt, int64_t n,
+// Stable radix sort of keys (and vals, may be null) by the low `bits` bits with
+// context scratch; the result is in keys / vals, which may have changed places
+// with the alternates.  Needs n < 2^32 when there are values.
+pd_status sort_u64(Ctx* c, uint64_t*& keys, uint64_t*& keys_alt, uint32_t*& vals, uint32_t*& vals_alt, int64_t n,
                    int bits, cudaStream_t st);
+// After the stream has been synchronised: whether every sort since then ended.
+pd_status sort_done(Ctx* c);
+constexpr int H_SORT_LATE = 63;  // its word of h_small
 pd_status scan_i64(Ctx* c, const int64_t* in, int64_t* out, int64_t n, int64_t* total_dev, cudaStream_t st);
 
 }  // namespace pd

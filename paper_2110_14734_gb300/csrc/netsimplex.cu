@@ -889,7 +889,7 @@ pd_status ns_prepare_arcs(Ctx* c, int32_t n, const NSArcs& a, const int64_t* sup
     h.max_pivots = o.max_rounds > 0 ? o.max_rounds : (int64_t(1) << 40);
     h.time_limit_ns = (o.time_limit_ms > 0 ? (uint64_t)o.time_limit_ms : 60000ull) * 1000000ull;
     // flows are int32: the total supply must stay below 2^31
-    {
+    if (a.supply_bound < 0 || a.supply_bound >= (int64_t(1) << 31)) {
         unsigned long long* sm = bufT<unsigned long long>(c, B_SMALL, 64);
         if (!sm) return PD_ENOMEM;
         PD_TRY_CUDA(c, cudaMemsetAsync(sm + 16, 0, sizeof(unsigned long long), st));
@@ -1191,6 +1191,50 @@ __global__ void k_side_lists(const int64_t* __restrict__ cntA, const int64_t* __
     }
 }
 
+// The lists of sources and sinks of at most SIDES_MAX nodes in node order, with
+// their supplies, by one block (k_side_flags, two scans and k_side_lists in one
+// launch): a count of the sources, then both lists behind running offsets.  The
+// diagonal node's supply dsup follows.  out (host memory) = sources, sinks.
+constexpr int64_t SIDES_MAX = int64_t(1) << 16;
+__global__ void __launch_bounds__(1024) k_sides_small(const int64_t* __restrict__ cntA,
+                                                      const int64_t* __restrict__ cntB, int N, int64_t dsup,
+                                                      int32_t* __restrict__ S, int32_t* __restrict__ T,
+                                                      int64_t* __restrict__ sup, int64_t* out) {
+    __shared__ uint32_t s_n;
+    const int tid = threadIdx.x;
+    if (tid == 0) s_n = 0;
+    __syncthreads();
+    uint32_t c = 0;
+    for (int u = tid; u < N; u += 1024) c += cntA[u] > cntB[u];
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((tid & 31) == 0 && c) atomicAdd(&s_n, c);
+    __syncthreads();
+    const uint32_t nS = s_n;
+    uint32_t ns = 0, nt = 0;
+    for (int b = 0; b < N; b += 1024) {
+        const int u = b + tid;
+        const int64_t s = u < N ? cntA[u] - cntB[u] : 0;
+        uint32_t tot;  // sources in the low half, sinks in the high one
+        const uint32_t ex = block_excl_scan<uint32_t>((uint32_t)(s > 0) | (uint32_t)(s < 0) << 16, &tot);
+        if (s > 0) {
+            const uint32_t i = ns + (ex & 0xffffu);
+            S[i] = u;
+            sup[i] = s;
+        } else if (s < 0) {
+            const uint32_t j = nt + (ex >> 16);
+            T[j] = u;
+            sup[nS + j] = s;
+        }
+        ns += tot & 0xffffu;
+        nt += tot >> 16;
+    }
+    if (tid == 0) {
+        sup[nS + nt] = dsup;
+        out[0] = nS;
+        out[1] = nt;
+    }
+}
+
 // Arc i*ld + j: source i -> sink j at min(l2, diag(i) + diag(j)) (the route
 // through the diagonal node has unbounded capacity), rows padded to ld columns;
 // then the arcs of the diagonal node if its supply |B| - |A| is not 0 (th, when
@@ -1327,20 +1371,35 @@ pd_status ns_solve_network(Ctx* c, const pd_network& net, const pd_opts& o, Solv
 // much larger than the sparse network (prepared here, launched by the caller,
 // checked by ns_finish_w1); otherwise, or if its certificate fails, the
 // simplex runs on the sparse network itself.  n_arcs = arcs of the sparse
-// network, dsup = |B| - |A| (supply of the merged diagonal node).
-pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t dsup, const pd_opts& o, W1Prep* w,
-                        cudaStream_t st) {
+// network, massA = |A|, massB = |B| (their difference is the supply of the
+// merged diagonal node).
+pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t massA, int64_t massB, const pd_opts& o,
+                        W1Prep* w, cudaStream_t st) {
     *w = W1Prep{};
+    const int64_t dsup = massB - massA;
+    const int64_t supply_bound = 2 * (massA + massB);  // of all |supplies|: the nodes' and the diagonal's
     int64_t N = nodes.n_nodes;
     if (N == 0 || o.ns_transport == 0) return PD_OK;
-    int64_t* fs = bufT<int64_t>(c, B_WSFLAG, N);
-    int64_t* ft = bufT<int64_t>(c, B_WSOFF, N);
     unsigned long long* sm = bufT<unsigned long long>(c, B_SMALL, 64);
-    if (!fs || !ft || !sm) return PD_ENOMEM;
-    k_side_flags<<<grid_for(N, 256), 256, 0, st>>>(nodes.cntA, nodes.cntB, N, fs, ft); pd::count_launch();
-    PD_TRY(scan_i64(c, fs, fs, N, (int64_t*)sm + 2, st));
-    PD_TRY(scan_i64(c, ft, ft, N, (int64_t*)sm + 3, st));
-    PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, 4 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    if (!sm) return PD_ENOMEM;
+    const bool small = N <= SIDES_MAX;
+    int64_t *fs = nullptr, *ft = nullptr;
+    if (small) {
+        int32_t* S = bufT<int32_t>(c, B_TR_S, N);
+        int32_t* T = bufT<int32_t>(c, B_TR_T, N);
+        int64_t* sup = bufT<int64_t>(c, B_TR_SUP, N + 1);
+        if (!S || !T || !sup) return PD_ENOMEM;
+        k_sides_small<<<1, 1024, 0, st>>>(nodes.cntA, nodes.cntB, (int)N, dsup, S, T, sup, c->h_small + 2); pd::count_launch();
+        PD_TRY_CUDA(c, cudaGetLastError());
+    } else {
+        fs = bufT<int64_t>(c, B_WSFLAG, N);
+        ft = bufT<int64_t>(c, B_WSOFF, N);
+        if (!fs || !ft) return PD_ENOMEM;
+        k_side_flags<<<grid_for(N, 256), 256, 0, st>>>(nodes.cntA, nodes.cntB, N, fs, ft); pd::count_launch();
+        PD_TRY(scan_i64(c, fs, fs, N, (int64_t*)sm + 2, st));
+        PD_TRY(scan_i64(c, ft, ft, N, (int64_t*)sm + 3, st));
+        PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, 4 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    }
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
     int64_t nS = c->h_small[2], nT = c->h_small[3];
     int64_t mst = nS * nT;
@@ -1350,9 +1409,9 @@ pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t d
     if (!((o.ns_transport == 2 || mt <= 2 * n_arcs + 4096) && mt < (int64_t(1) << 31) - 1 - 8 * NS_THREADS))
         return PD_OK;
     int64_t nt = nS + nT + 1;
-    int32_t* S = bufT<int32_t>(c, B_TR_S, nS);
-    int32_t* T = bufT<int32_t>(c, B_TR_T, nT);
-    int64_t* sup = bufT<int64_t>(c, B_TR_SUP, nt);
+    int32_t* S = bufT<int32_t>(c, B_TR_S, small ? N : nS);
+    int32_t* T = bufT<int32_t>(c, B_TR_T, small ? N : nT);
+    int64_t* sup = bufT<int64_t>(c, B_TR_SUP, small ? N + 1 : nt);
     const int64_t mx = mt - mst;
     // rows padded to whole steps of simplex32.cu, unless the padding alone would take the arc ids past 2^31
     int64_t ld = (nT + 7) & ~(int64_t)7;
@@ -1366,9 +1425,11 @@ pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t d
     int32_t* cost = bufT<int32_t>(c, B_TR_XCOST, mx + 3);
     uint32_t* th = packed ? bufT<uint32_t>(c, B_TR_XTH, mx + 3) : nullptr;
     if (!S || !T || !sup || !tail || !head || !cost || !cmat || (packed && !th)) return PD_ENOMEM;
-    k_side_lists<<<grid_for(N, 256), 256, 0, st>>>(nodes.cntA, nodes.cntB, N, fs, ft, S, T, sup, nS); pd::count_launch();
-    c->h_small[20] = dsup;
-    PD_TRY_CUDA(c, cudaMemcpyAsync(sup + nS + nT, c->h_small + 20, sizeof(int64_t), cudaMemcpyHostToDevice, st));
+    if (!small) {
+        k_side_lists<<<grid_for(N, 256), 256, 0, st>>>(nodes.cntA, nodes.cntB, N, fs, ft, S, T, sup, nS); pd::count_launch();
+        c->h_small[20] = dsup;
+        PD_TRY_CUDA(c, cudaMemcpyAsync(sup + nS + nT, c->h_small + 20, sizeof(int64_t), cudaMemcpyHostToDevice, st));
+    }
     PD_TRY_CUDA(c, cudaMemsetAsync(sm, 0, 8 * sizeof(unsigned long long), st));
     if (mt > 0) {
         k_transport_arcs<<<grid_for(mt + 3, 256), 256, 0, st>>>(S, T, nS, nT, ld, dsup < 0 ? -1 : (dsup > 0 ? 1 : 0),
@@ -1391,6 +1452,7 @@ pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t d
     arcs.head = head;
     arcs.cost = cost;
     arcs.complete = true;
+    arcs.supply_bound = supply_bound;
     PD_TRY(ns_prepare_arcs(c, (int32_t)nt, arcs, sup, c->h_small[1], o, &w->ns, st));
     w->S = S;
     w->T = T;

@@ -125,6 +125,7 @@ struct NSArcs {
     const int32_t* head = nullptr;
     const int32_t* cost = nullptr;
     bool complete = false;  // every supply node has an arc to every demand node
+    int64_t supply_bound = -1;  // of the sum of |supplies| (-1: not known, it is summed)
 };
 pd_status ns_prepare_arcs(Ctx* c, int32_t n, const NSArcs& a, const int64_t* supply, int64_t cmax, const pd_opts& o,
                           NSPrep* p, cudaStream_t st);
@@ -135,8 +136,8 @@ pd_status ns_run(Ctx* c, const NSInst* h, int count, NSInst* d, NSInst* r, cudaS
 int64_t ns_default_block(const NSInst& h);
 void ns_choose_kernel(NSInst* h, int64_t cmax, bool complete, bool smem, int max_optin);
 pd_status ns_status(Ctx* c, const NSInst& r);
-pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t dsup, const pd_opts& o, W1Prep* w,
-                        cudaStream_t st);
+pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t massA, int64_t massB, const pd_opts& o,
+                        W1Prep* w, cudaStream_t st);
 // Certificate (on the WSPD tree of s) and fallback after the launch; d_res =
 // the device record of the solved instance, r = its host copy.  merged ==
 // nullptr: no fallback here -- out->method = -1 tells the caller to solve the

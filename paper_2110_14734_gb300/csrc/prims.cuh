@@ -1,7 +1,5 @@
-// Device-wide primitives written for this library: exclusive scan (reduce,
-// scan of tile sums, scan of tiles) and a stable LSD radix sort (8-bit
-// digits; per-tile digit histograms, a scan over the digit-major histogram,
-// and a stable in-tile scatter that ranks equal digits with warp match).
+// Primitives written for this library: exclusive scan (reduce, scan of tile
+// sums, scan of tiles) and a stable LSD radix sort.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -172,117 +170,141 @@ cudaError_t exclusive_scan(const T* in, T* out, int64_t n, T* part, T* total_dev
 }
 
 // ---------------------------------------------------------------------------
-// LSD radix sort
+// LSD radix sort, 8-bit digits
 // ---------------------------------------------------------------------------
+//
+// Long arrays: one read for the digit counts of every pass, then one launch per
+// pass.  A tile ranks its keys in registers, takes each digit's offset from the
+// tiles before it by decoupled look-back (Merrill & Garland: a tile first
+// publishes its own counts, then their running sum; tile numbers are tickets, so
+// the tiles looked back at have started), orders the keys in shared memory and
+// writes them in runs.  A pass moves each key once in and once out; what bounds it
+// is the ranking and the look-back's latency.
+//
+// Short arrays (at most CS_MAX): one block sorts in shared memory, one launch for
+// all passes.
 
 constexpr int RS_THREADS = 256;
 constexpr int RS_ITEMS = 16;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
+constexpr int RS_WARPS = RS_THREADS / 32;
+constexpr int RS_MAXPASS = 8;
+constexpr uint64_t RS_VALUE = (1ull << 62) - 1;  // of a state word: flag << 62 | value
+constexpr int RS_POLLS = 1 << 22;                // bound of a look-back wait (it is microseconds)
 
 inline int64_t radix_tiles(int64_t n) { return (n + RS_TILE - 1) / RS_TILE; }
-
-template <typename K>
-__global__ void k_radix_hist(const K* __restrict__ keys, int64_t n, int shift, int64_t nb,
-                             int64_t* __restrict__ counts) {
-    __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * RS_TILE;
-#pragma unroll 4
-    for (int j = 0; j < RS_ITEMS; j++) {
-        int64_t i = base + (int64_t)j * RS_THREADS + threadIdx.x;
-        if (i < n) atomicAdd(&h[(uint32_t)(keys[i] >> shift) & 0xFFu], 1u);
-    }
-    __syncthreads();
-    counts[(int64_t)threadIdx.x * nb + blockIdx.x] = h[threadIdx.x];
+inline int radix_passes(int bits) { return (bits + 7) / 8; }
+// Words of scratch: counts of every pass, tickets, states.
+inline int64_t radix_words(int64_t n, int bits) {
+    return 256 * RS_MAXPASS + RS_MAXPASS + 256 * (int64_t)radix_passes(bits) * radix_tiles(n);
 }
 
-template <typename K>
-__global__ void k_radix_scatter(const K* __restrict__ kin, const uint32_t* __restrict__ vin, K* __restrict__ kout,
-                                uint32_t* __restrict__ vout, int64_t n, int shift, int64_t nb,
-                                const int64_t* __restrict__ offs) {
-    __shared__ uint32_t digit_base[256];
-    __shared__ uint32_t wcnt[RS_THREADS / 32][256];
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    digit_base[tid] = 0;
-    const int64_t my_off = offs[(int64_t)tid * nb + blockIdx.x];
-    __shared__ int64_t doff[256];
-    doff[tid] = my_off;
-    int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    const uint32_t lt = (1u << lane) - 1u;
-    for (int c = 0; c < RS_ITEMS; c++) {
-        int64_t i = base + (int64_t)c * RS_THREADS + tid;
-        bool valid = i < n;
-        K k = valid ? kin[i] : K(0);
-        uint32_t v = (valid && vin) ? vin[i] : 0u;
-        uint32_t d = valid ? ((uint32_t)(k >> shift) & 0xFFu) : 256u;
-#pragma unroll
-        for (int q = 0; q < RS_THREADS / 32; q++) wcnt[q][tid] = 0;
-        __syncthreads();
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
-        uint32_t rank = __popc(peers & lt);
-        if (valid && rank == 0) wcnt[w][d] = __popc(peers);
-        __syncthreads();
-        if (valid) {
-            uint32_t pre = digit_base[d];
-            for (int q = 0; q < w; q++) pre += wcnt[q][d];
-            int64_t pos = doff[d] + pre + rank;
-            kout[pos] = k;
-            if (vin) vout[pos] = v;
-        }
-        __syncthreads();
-        uint32_t add = 0;
-#pragma unroll
-        for (int q = 0; q < RS_THREADS / 32; q++) add += wcnt[q][tid];
-        digit_base[tid] += add;
-        __syncthreads();
-    }
-}
+// Digit counts of all passes.
+__global__ void __launch_bounds__(RS_THREADS) k_radix_counts(const uint64_t* __restrict__ keys, int64_t n, int passes,
+                                                             unsigned long long* __restrict__ hist);
+// One pass; vin / vout may be null.  *late (host memory) is set when a wait gave up.
+__global__ void __launch_bounds__(RS_THREADS) k_radix_pass(const uint64_t* __restrict__ kin,
+                                                           const uint32_t* __restrict__ vin,
+                                                           uint64_t* __restrict__ kout, uint32_t* __restrict__ vout,
+                                                           int64_t n, int shift,
+                                                           const unsigned long long* __restrict__ hist,
+                                                           unsigned long long* ticket, volatile unsigned long long* state,
+                                                           int64_t* late);
 
-template <typename K>
-struct RadixScratch {
-    K* k_alt;          // n keys
-    uint32_t* v_alt;   // n values (if values are sorted)
-    int64_t* counts;   // 256 * radix_tiles(n)
-    int64_t* part;     // scan_tiles(256 * radix_tiles(n)) + 1
+// ---- sort of one block of CS_THREADS threads
+
+constexpr int CS_THREADS = 1024;
+constexpr int CS_ITEMS = 8;
+constexpr int CS_MAX = CS_THREADS * CS_ITEMS;
+constexpr int CS_WARPS = CS_THREADS / 32;
+
+struct CtaSort {
+    uint64_t key[CS_MAX];
+    uint32_t val[CS_MAX];
+    uint32_t cnt[CS_WARPS][256];
+    uint32_t part[4][256];
+    uint32_t wsum[8];
 };
 
-template <typename K>
-inline size_t radix_counts_elems(int64_t n) {
-    return (size_t)256 * (size_t)radix_tiles(n);
-}
-
-// Stable sort of (keys, vals) by the low `bits` bits of the keys.  vals may be
-// NULL.  The result is left in keys / vals.
-template <typename K>
-cudaError_t radix_sort(K* keys, uint32_t* vals, int64_t n, int bits, RadixScratch<K> s, cudaStream_t st) {
-    if (n <= 1 || bits <= 0) return cudaSuccess;
-    int64_t nb = radix_tiles(n);
-    K* ka = keys;
-    K* kb = s.k_alt;
-    uint32_t* va = vals;
-    uint32_t* vb = vals ? s.v_alt : nullptr;
-    int passes = (bits + 7) / 8;
-    for (int p = 0; p < passes; p++) {
-        int shift = 8 * p;
-        k_radix_hist<K><<<(unsigned)nb, RS_THREADS, 0, st>>>(ka, n, shift, nb, s.counts); pd::count_launch();
-        cudaError_t e = exclusive_scan<int64_t>(s.counts, s.counts, 256 * nb, s.part, nullptr, st);
-        if (e != cudaSuccess) return e;
-        k_radix_scatter<K><<<(unsigned)nb, RS_THREADS, 0, st>>>(ka, va, kb, vb, n, shift, nb, s.counts); pd::count_launch();
-        K* t = ka;
-        ka = kb;
-        kb = t;
-        uint32_t* tv = va;
-        va = vb;
-        vb = tv;
+// Stable sort of the block's items by the low `bits` bits of their keys.  Thread
+// t of warp w holds items w * 32 * CS_ITEMS + 32 q + lane; past the end the
+// keys are all ones.  The result is in k / v and in s.key / s.val.
+PD_D void cta_sort(CtaSort& s, uint64_t (&k)[CS_ITEMS], uint32_t (&v)[CS_ITEMS], int bits) {
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const uint32_t below = (1u << lane) - 1u;
+    const int base = w * 32 * CS_ITEMS + lane;
+    for (int shift = 0; shift < bits; shift += 8) {
+        for (int q = tid; q < CS_WARPS * 256; q += CS_THREADS) (&s.cnt[0][0])[q] = 0;
+        __syncthreads();
+        uint32_t rank[CS_ITEMS];
+#pragma unroll
+        for (int q = 0; q < CS_ITEMS; q++) {
+            const uint32_t d = (uint32_t)(k[q] >> shift) & 0xffu;
+            const uint32_t peers = __match_any_sync(0xffffffffu, d);
+            const uint32_t seen = s.cnt[w][d];
+            __syncwarp();
+            if ((peers & below) == 0) s.cnt[w][d] = seen + __popc(peers);
+            __syncwarp();
+            rank[q] = seen + __popc(peers & below);
+        }
+        __syncthreads();
+        // per digit: an exclusive sum over the warps (four threads, eight warps each), then over the digits
+        {
+            const int d = tid & 255, g = tid >> 8;
+            uint32_t c[8], t = 0;
+#pragma unroll
+            for (int q = 0; q < 8; q++) c[q] = s.cnt[8 * g + q][d];
+#pragma unroll
+            for (int q = 0; q < 8; q++) t += c[q];
+            s.part[g][d] = t;
+            __syncthreads();
+            uint32_t at = 0, tot = 0;
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                at += q < g ? s.part[q][d] : 0u;
+                tot += s.part[q][d];
+            }
+            uint32_t inc = tot;
+            if (g == 0) {
+                inc = warp_incl_scan(tot);
+                if (lane == 31) s.wsum[w] = inc;
+            }
+            __syncthreads();
+            if (g == 0) {
+                uint32_t o = inc - tot;
+                for (int q = 0; q < w; q++) o += s.wsum[q];
+                s.part[0][d] = o;  // (the four sums have been read)
+            }
+            __syncthreads();
+            at += s.part[0][d];
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                s.cnt[8 * g + q][d] = at;
+                at += c[q];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < CS_ITEMS; q++) {
+            const uint32_t at = s.cnt[w][(uint32_t)(k[q] >> shift) & 0xffu] + rank[q];
+            s.key[at] = k[q];
+            s.val[at] = v[q];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < CS_ITEMS; q++) {
+            k[q] = s.key[base + 32 * q];
+            v[q] = s.val[base + 32 * q];
+        }
     }
-    if (ka != keys) {
-        cudaError_t e = cudaMemcpyAsync(keys, ka, sizeof(K) * n, cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
-        if (vals) e = cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
+    if (bits <= 0) {
+#pragma unroll
+        for (int q = 0; q < CS_ITEMS; q++) {
+            s.key[base + 32 * q] = k[q];
+            s.val[base + 32 * q] = v[q];
+        }
+        __syncthreads();
     }
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

@@ -22,9 +22,11 @@ PD_D int code_delta(const uint64_t* __restrict__ code, int64_t N, int64_t i, int
 // index below the highest bit where the range's codes differ.  Children:
 // c >= 0 internal c, c < 0 leaf ~c.
 __global__ void k_karras(const uint64_t* __restrict__ code, int64_t N, int32_t* __restrict__ left,
-                         int32_t* __restrict__ right, int32_t* __restrict__ par_int, int32_t* __restrict__ par_leaf) {
+                         int32_t* __restrict__ right, int32_t* __restrict__ par_int, int32_t* __restrict__ par_leaf,
+                         int32_t* __restrict__ visit) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N - 1) return;
+    visit[i] = 0;
     int d = (code_delta(code, N, i, i + 1) - code_delta(code, N, i, i - 1)) > 0 ? 1 : -1;
     int dmin = code_delta(code, N, i, i - d);
     int64_t lmax = 2;
@@ -461,14 +463,12 @@ __global__ void k_diag_arcs(int64_t N, const int64_t* __restrict__ cntA, const i
     int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (u > N) return;
     if (u == N) {
-        if (arcs) arcs[2 * N] = ((uint64_t)(N + 1) << hb) | (uint64_t)N;
+        arcs[2 * N] = ((uint64_t)(N + 1) << hb) | (uint64_t)N;
         return;
     }
     bool a = cntA[u] > 0, b = cntB[u] > 0;
-    if (arcs) {  // null: count only
-        arcs[2 * u] = a ? (((uint64_t)u << hb) | (uint64_t)N) : sent;
-        arcs[2 * u + 1] = b ? (((uint64_t)(N + 1) << hb) | (uint64_t)u) : sent;
-    }
+    arcs[2 * u] = a ? (((uint64_t)u << hb) | (uint64_t)N) : sent;
+    arcs[2 * u + 1] = b ? (((uint64_t)(N + 1) << hb) | (uint64_t)u) : sent;
     unsigned ma = __ballot_sync(__activemask(), a), mb = __ballot_sync(__activemask(), b);
     if ((threadIdx.x & 31) == (__ffs(__activemask()) - 1)) {
         atomicAdd(&counts[0], (unsigned long long)__popc(ma));
@@ -512,6 +512,25 @@ __global__ void k_supply(int64_t N, const int64_t* __restrict__ cntA, const int6
     if (u < N) sup[u] = cntA[u] - cntB[u];
     if (u == N) sup[N] = -FA;
     if (u == N + 1) sup[N + 1] = FB;
+}
+
+// Nodes that hold A mass, B mass, and both masses (out[0 .. 3]), in one pass.
+__global__ void k_diag_counts(int64_t N, const int64_t* __restrict__ cntA, const int64_t* __restrict__ cntB,
+                              unsigned long long* __restrict__ out) {
+    const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned long long a = u < N ? (unsigned long long)cntA[u] : 0ull, b = u < N ? (unsigned long long)cntB[u] : 0ull;
+    const unsigned ma = __ballot_sync(0xffffffffu, a > 0), mb = __ballot_sync(0xffffffffu, b > 0);
+    const unsigned long long sa = warp_sum(a), sb = warp_sum(b);
+    if ((threadIdx.x & 31) == 0) {
+        if (ma) {
+            atomicAdd(&out[0], (unsigned long long)__popc(ma));
+            atomicAdd(&out[2], sa);
+        }
+        if (mb) {
+            atomicAdd(&out[1], (unsigned long long)__popc(mb));
+            atomicAdd(&out[3], sb);
+        }
+    }
 }
 
 __global__ void k_mass(int64_t N, const int64_t* __restrict__ cntA, const int64_t* __restrict__ cntB,
@@ -669,8 +688,7 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
         bb = b;
         rep = rp;
         if (N >= 2) {
-            k_karras<<<grid_for(N - 1, 256), 256, 0, st>>>(nodes.morton, N, l, r, par_int, par_leaf); pd::count_launch();
-            PD_TRY_CUDA(c, cudaMemsetAsync(visit, 0, sizeof(int32_t) * M, st));
+            k_karras<<<grid_for(N - 1, 256), 256, 0, st>>>(nodes.morton, N, l, r, par_int, par_leaf, visit); pd::count_launch();
             k_bbox<<<grid_for(N, 256), 256, 0, st>>>(N, nodes.X, nodes.Y, l, r, par_int, par_leaf, b, rp, visit); pd::count_launch();
             PD_TRY_CUDA(c, cudaGetLastError());
         }
@@ -707,8 +725,7 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
     if (count_only) {
         // only the counts: arcs of the WSPD, diagonal arcs and the masses
         PD_TRY_CUDA(c, cudaMemsetAsync(cnts, 0, 8 * sizeof(unsigned long long), st));
-        k_diag_arcs<<<grid_for(N + 1, 256), 256, 0, st>>>(N, nodes.cntA, nodes.cntB, hb, sent, nullptr, cnts); pd::count_launch();
-        k_mass<<<grid_for(N, 256), 256, 0, st>>>(N, nodes.cntA, nodes.cntB, cnts); pd::count_launch();
+        k_diag_counts<<<grid_for(N, 256), 256, 0, st>>>(N, nodes.cntA, nodes.cntB, cnts); pd::count_launch();
         PD_TRY_CUDA(c, cudaGetLastError());
         PD_TRY_CUDA(c, cudaMemcpyAsync(h, cnts, 4 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
         PD_TRY_CUDA(c, cudaEventRecord(ev[3], st));
@@ -733,8 +750,10 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
     int64_t ntot = narcs + 2 * N + 1;
     uint64_t* alt = bufT<uint64_t>(c, B_ARCKEY2, ntot);
     if (!alt) return PD_ENOMEM;
-    PD_TRY(sort_u64(c, arcs, alt, nullptr, nullptr, ntot, kb, st));
+    uint32_t *none = nullptr, *none2 = nullptr;
+    PD_TRY(sort_u64(c, arcs, alt, none, none2, ntot, kb, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
+    PD_TRY(sort_done(c));
     int64_t na = h[0], nb = h[1], FA = h[2], FB = h[3];
     int64_t m = narcs + na + nb + 1;
     int64_t nrows = N + 2;
