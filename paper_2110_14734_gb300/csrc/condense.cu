@@ -24,6 +24,39 @@ __global__ void k_init_small(int64_t* s) {
     }
 }
 
+// Sums and extremes over all blocks end in atomics on a handful of words.  One set
+// of them per warp serialises (2,000,000 points: 201 microseconds for k_quantize,
+// 160 for k_cells), so the kernels that need them run few blocks that stride over
+// the data, and each block adds one set.
+constexpr int BOX_THREADS = 256;
+static unsigned box_grid(const Ctx* c, int64_t n) {
+    return (unsigned)std::min<int64_t>(grid_for(n, BOX_THREADS), 4 * std::max(c->sm_count, 1));
+}
+
+// Block extremes b = (min x, max x, min y, max y) into at[0 .. 3] (min, max, min, max).
+PD_D void box_to(int32_t (&b)[4], int64_t* at) {
+    __shared__ int32_t s[4][BOX_THREADS / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        b[q] = q & 1 ? __reduce_max_sync(0xffffffffu, b[q]) : __reduce_min_sync(0xffffffffu, b[q]);
+        if (lane == 0) s[q][w] = b[q];
+    }
+    __syncthreads();
+    if (w != 0) return;
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const int32_t v = s[q][lane & (BOX_THREADS / 32 - 1)];
+        b[q] = q & 1 ? __reduce_max_sync(0xffffffffu, v) : __reduce_min_sync(0xffffffffu, v);
+    }
+    if (lane == 0 && b[0] <= b[1]) {
+        atomicMin((long long*)&at[0], (long long)b[0]);
+        atomicMax((long long*)&at[1], (long long)b[1]);
+        atomicMin((long long*)&at[2], (long long)b[2]);
+        atomicMax((long long*)&at[3], (long long)b[3]);
+    }
+}
+
 // a1: X = rint(b 2^k), Y = rint(d 2^k) of one point; false (X = Y = 0) when
 // non-finite or |X|, |Y| >= 2^29.
 PD_D bool quantize_point(const void* __restrict__ p, int64_t j, int dt, int k, int32_t* X, int32_t* Y) {
@@ -50,46 +83,45 @@ PD_D bool quantize_point(const void* __restrict__ p, int64_t j, int dt, int k, i
 
 // Quantises all points: keep unless X == Y; track min/max and the masses of A
 // and B; count the rejected ones.
-__global__ void k_quantize(const void* __restrict__ a, int64_t na, int dta, const void* __restrict__ b, int64_t nb,
-                           int dtb, int k, int32_t* __restrict__ X, int32_t* __restrict__ Y,
-                           uint8_t* __restrict__ keep, int64_t* __restrict__ sm) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t n = na + nb;
-    int64_t mnx = INT64_MAX, mxx = INT64_MIN, mny = INT64_MAX, mxy = INT64_MIN;
-    int isB = 0, kp = 0, bad = 0;
-    if (i < n) {
-        isB = i >= na;
+__global__ void __launch_bounds__(BOX_THREADS) k_quantize(const void* __restrict__ a, int64_t na, int dta,
+                                                          const void* __restrict__ b, int64_t nb, int dtb, int k,
+                                                          int32_t* __restrict__ X, int32_t* __restrict__ Y,
+                                                          uint8_t* __restrict__ keep, int64_t* __restrict__ sm) {
+    const int64_t n = na + nb, step = (int64_t)gridDim.x * BOX_THREADS;
+    int32_t box[4] = {INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN};
+    uint32_t c[3] = {0, 0, 0};  // kept of A, of B, rejected
+    for (int64_t i = (int64_t)blockIdx.x * BOX_THREADS + threadIdx.x; i < n; i += step) {
+        const bool isB = i >= na;
         int32_t qx, qy;
-        bad = !quantize_point(isB ? b : a, isB ? i - na : i, isB ? dtb : dta, k, &qx, &qy);
-        kp = !bad && qx != qy;
+        const bool bad = !quantize_point(isB ? b : a, isB ? i - na : i, isB ? dtb : dta, k, &qx, &qy);
+        const bool kp = !bad && qx != qy;
         X[i] = qx;
         Y[i] = qy;
         keep[i] = (uint8_t)kp;
         if (kp) {
-            mnx = mxx = qx;
-            mny = mxy = qy;
+            box[0] = min(box[0], qx);
+            box[1] = max(box[1], qx);
+            box[2] = min(box[2], qy);
+            box[3] = max(box[3], qy);
         }
+        c[0] += kp && !isB;
+        c[1] += kp && isB;
+        c[2] += bad;
     }
-    // warp-reduce then one atomic per warp
-    for (int o = 16; o > 0; o >>= 1) {
-        mnx = min(mnx, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)mnx, o));
-        mxx = max(mxx, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)mxx, o));
-        mny = min(mny, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)mny, o));
-        mxy = max(mxy, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)mxy, o));
+    __shared__ uint32_t s_c[3];
+    if (threadIdx.x < 3) s_c[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        c[q] = __reduce_add_sync(0xffffffffu, c[q]);
+        if ((threadIdx.x & 31) == 0 && c[q]) atomicAdd(&s_c[q], c[q]);
     }
-    unsigned ka = __ballot_sync(0xffffffffu, kp && !isB), kb = __ballot_sync(0xffffffffu, kp && isB);
-    unsigned bd = __ballot_sync(0xffffffffu, bad);
-    if ((threadIdx.x & 31) == 0) {
-        if (ka | kb) {
-            atomicMin((long long*)&sm[S_MNX], (long long)mnx);
-            atomicMax((long long*)&sm[S_MXX], (long long)mxx);
-            atomicMin((long long*)&sm[S_MNY], (long long)mny);
-            atomicMax((long long*)&sm[S_MXY], (long long)mxy);
-        }
-        if (ka) atomicAdd((unsigned long long*)&sm[S_FA], (unsigned long long)__popc(ka));
-        if (kb) atomicAdd((unsigned long long*)&sm[S_FB], (unsigned long long)__popc(kb));
-        if (bd) atomicAdd((unsigned long long*)&sm[S_ERR], 1ull);
+    __syncthreads();
+    if (threadIdx.x < 3 && s_c[threadIdx.x]) {
+        const int slot[3] = {S_FA, S_FB, S_ERR};
+        atomicAdd((unsigned long long*)&sm[slot[threadIdx.x]], (unsigned long long)s_c[threadIdx.x]);
     }
+    box_to(box, &sm[S_MNX]);
 }
 
 // Sort key: diagram bit, then X, then Y (lexicographic); dropped points get
@@ -130,7 +162,8 @@ __global__ void k_hat_compact(const uint64_t* __restrict__ key, int64_t n, uint6
     HX[j] = (int32_t)((int64_t)((k >> by) & xmask) + sm[S_MNX]);
     HY[j] = (int32_t)((int64_t)(k & ymask) + sm[S_MNY]);
     start[j] = i;
-    if (!((k >> (bx + by)) & 1ull)) atomicAdd((unsigned long long*)nA, 1ull);
+    // A's nodes come first: B's first node says how many there are
+    if ((k >> (bx + by)) & 1ull && (i == 0 || !((key[i - 1] >> (bx + by)) & 1ull))) *nA = j;
 }
 
 __global__ void k_hat_counts(const int64_t* __restrict__ start, int64_t M, int64_t nvalid, int64_t* __restrict__ cnt) {
@@ -303,7 +336,7 @@ pd_status stage_condense0(Ctx* c, const DevDiag& A, const DevDiag& B, int k, Hat
     int64_t* flag = bufT<int64_t>(c, B_IDX, n);
     int64_t* start = bufT<int64_t>(c, B_QVAL, n);
     if (!X || !Y || !keep || !key || !key2 || !flag || !start) return PD_ENOMEM;
-    k_quantize<<<grid_for(n, 256), 256, 0, st>>>(A.bd, A.n, A.dtype, B.bd, B.n, B.dtype, k, X, Y, keep, sm); pd::count_launch();
+    k_quantize<<<box_grid(c, n), BOX_THREADS, 0, st>>>(A.bd, A.n, A.dtype, B.bd, B.n, B.dtype, k, X, Y, keep, sm); pd::count_launch();
     PD_TRY_CUDA(c, cudaGetLastError());
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, sizeof(int64_t) * S_COUNT, cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
@@ -328,7 +361,7 @@ pd_status stage_condense0(Ctx* c, const DevDiag& A, const DevDiag& B, int k, Hat
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
     PD_TRY(sort_done(c));
     int64_t M = h[S_M];
-    out->nA = h[S_NA];
+    out->nA = out->FB > 0 ? h[S_NA] : M;
     out->nB = M - out->nA;
     k_hat_counts<<<grid_for(M, 256), 256, 0, st>>>(start, M, nvalid, out->cnt); pd::count_launch();
     PD_TRY_CUDA(c, cudaGetLastError());
@@ -375,31 +408,32 @@ __global__ void __launch_bounds__(RW_THREADS) k_rwmd_min(const int32_t* __restri
     if (u < np) atomicMin(&mind2[pbase + u], best);
 }
 
-__global__ void k_rwmd_sum(const int32_t* __restrict__ X, const int32_t* __restrict__ Y,
-                           const int64_t* __restrict__ cnt, int64_t nA, int64_t n,
-                           const unsigned long long* __restrict__ mind2, DiagCost dc, int64_t* __restrict__ L) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(BOX_THREADS) k_rwmd_sum(const int32_t* __restrict__ X, const int32_t* __restrict__ Y,
+                                                          const int64_t* __restrict__ cnt, int64_t nA, int64_t n,
+                                                          const unsigned long long* __restrict__ mind2, DiagCost dc,
+                                                          int64_t* __restrict__ L) {
+    __shared__ unsigned long long s[2][BOX_THREADS / 32];
     unsigned long long va = 0, vb = 0;
-    if (i < n) {
+    for (int64_t i = (int64_t)blockIdx.x * BOX_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * BOX_THREADS) {
         int64_t c = cost_make(X[i], Y[i], dc);
-        unsigned long long m = mind2[i];
+        const unsigned long long m = mind2[i];
         if (m != ~0ull) {
-            int64_t cn = (int64_t)ceil_sqrt_u64(m);
+            const int64_t cn = (int64_t)ceil_sqrt_u64(m);
             c = cn < c ? cn : c;
         }
-        unsigned long long v = (unsigned long long)(c * cnt[i]);
-        if (i < nA)
-            va = v;
-        else
-            vb = v;
+        (i < nA ? va : vb) += (unsigned long long)(c * cnt[i]);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        va += __shfl_xor_sync(0xffffffffu, va, o);
-        vb += __shfl_xor_sync(0xffffffffu, vb, o);
-    }
+    va = warp_sum(va);
+    vb = warp_sum(vb);
     if ((threadIdx.x & 31) == 0) {
-        if (va) atomicAdd((unsigned long long*)&L[0], va);
-        if (vb) atomicAdd((unsigned long long*)&L[1], vb);
+        s[0][threadIdx.x >> 5] = va;
+        s[1][threadIdx.x >> 5] = vb;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        unsigned long long v = 0;
+        for (int q = 0; q < BOX_THREADS / 32; q++) v += s[threadIdx.x][q];
+        if (v) atomicAdd((unsigned long long*)&L[threadIdx.x], v);
     }
 }
 
@@ -452,20 +486,28 @@ constexpr int64_t RW_SMALL = 8192;
 
 // ---- the same minima through a uniform grid over each side ----------------
 // Large sides make the all-pairs scan quadratic (about 10^12 distance
-// evaluations at a million nodes a side).  Each side's nodes are bucketed
-// into a grid of about two nodes a cell (a counting sort by cell), and every
-// node of the other side searches square rings of cells around its own cell.
-// After ring K every node not yet seen lies beyond one of the square's sides
-// that are not the grid's border, so its distance is at least LB, the
-// distance from the query to the nearest such side.  The search stops when
-// LB^2 >= the best squared distance found (the minimum is exact), or when
-// LB >= the query's diagonal cost c_make: every unseen node then costs at
-// least c_make, the relaxed flow takes min(c(u, nearest), c_make) either way,
-// and the stored value min(best, c_make^2) gives the same term.  A query that
-// has not stopped after RW_KMAX rings (a far outlier) keeps its best as an
-// upper bound and is finished by the all-pairs scan over the other side.
+// evaluations at a million nodes a side).  Each side's nodes are bucketed into a
+// grid (a counting sort by cell), and every node of the other side searches square
+// rings of cells around its own cell.  After ring K every node not yet seen lies
+// beyond one of the square's sides that are not the grid's border, so its distance
+// is at least LB, the distance from the query to the nearest such side.  The
+// search stops when LB^2 >= the best squared distance found (the minimum is
+// exact), or when LB >= the query's diagonal cost c_make: every unseen node then
+// costs at least c_make, the relaxed flow takes min(c(u, nearest), c_make) either
+// way, and the stored value min(best, c_make^2) gives the same term.  A query that
+// has not stopped after RW_KMAX rings (a far outlier) keeps its best as an upper
+// bound and is finished by the all-pairs scan over the other side.
+//
+// Bound by the distances evaluated and by the gathers of cells.  Diagrams crowd
+// near the diagonal, so cells of two nodes on average hold dozens where most
+// nodes are: the grid has RW_CELLS cells a node instead.  Queries run in the
+// order of their own side's cells, so the lanes of a warp search the same cells,
+// and a row of a ring is one stretch of nodes between two cell starts.  1,000,000
+// nodes a side (mixture): 2.31 ms with half a cell a node and queries by
+// coordinate.
 
 constexpr int RW_KMAX = 24;
+constexpr int64_t RW_CELLS = 8;
 constexpr int64_t RW_GRID_MIN = int64_t(1) << 28;  // nA * nB from which the grid is used
 
 struct RwGrid {
@@ -474,35 +516,21 @@ struct RwGrid {
     int64_t base;       // first cell of this grid in the shared cell arrays
 };
 
-__global__ void k_rw_box_init(int* box) {
-    if (threadIdx.x < 8) box[threadIdx.x] = (threadIdx.x & 1) ? INT32_MIN : INT32_MAX;
+// box[4 s ..] = min x, max x, min y, max y of side s (blockIdx.y).
+__global__ void k_rw_box_init(int64_t* box) {
+    if (threadIdx.x < 8) box[threadIdx.x] = (threadIdx.x & 1) ? INT64_MIN : INT64_MAX;
 }
-
-// Bounding box of each side: box[4 s ..] = xmin, xmax, ymin, ymax of side s.
-__global__ void k_rw_box(const int32_t* __restrict__ X, const int32_t* __restrict__ Y, int64_t nA, int64_t n,
-                         int* __restrict__ box) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int v[8];  // per side: -xmin, xmax, -ymin, ymax (maxima of all four)
-#pragma unroll
-    for (int k = 0; k < 8; k++) v[k] = INT32_MIN;
-    if (i < n) {
-        const int s = i < nA ? 0 : 4;
-        v[s + 0] = -X[i];  // coordinates are above -2^30: negation is exact
-        v[s + 1] = X[i];
-        v[s + 2] = -Y[i];
-        v[s + 3] = Y[i];
+__global__ void __launch_bounds__(BOX_THREADS) k_rw_box(const int32_t* __restrict__ X, const int32_t* __restrict__ Y,
+                                                        int64_t nA, int64_t n, int64_t* __restrict__ box) {
+    const int64_t i0 = blockIdx.y ? nA : 0, i1 = blockIdx.y ? n : nA;
+    int32_t b[4] = {INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN};
+    for (int64_t i = i0 + (int64_t)blockIdx.x * BOX_THREADS + threadIdx.x; i < i1; i += (int64_t)gridDim.x * BOX_THREADS) {
+        b[0] = min(b[0], X[i]);
+        b[1] = max(b[1], X[i]);
+        b[2] = min(b[2], Y[i]);
+        b[3] = max(b[3], Y[i]);
     }
-#pragma unroll
-    for (int k = 0; k < 8; k++)
-        for (int o = 16; o > 0; o >>= 1) v[k] = max(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
-    if ((threadIdx.x & 31) == 0)
-        for (int s = 0; s < 8; s += 4)
-            if (v[s + 1] != INT32_MIN) {
-                atomicMin(&box[s + 0], -v[s + 0]);
-                atomicMax(&box[s + 1], v[s + 1]);
-                atomicMin(&box[s + 2], -v[s + 2]);
-                atomicMax(&box[s + 3], v[s + 3]);
-            }
+    box_to(b, box + 4 * blockIdx.y);
 }
 
 PD_D int32_t rw_cell_axis(int64_t v, int64_t o, int64_t h, int32_t g) {
@@ -511,69 +539,72 @@ PD_D int32_t rw_cell_axis(int64_t v, int64_t o, int64_t h, int32_t g) {
     return c >= g ? g - 1 : (int32_t)c;
 }
 
+PD_D uint32_t rw_cell(const RwGrid& g, int32_t x, int32_t y) {
+    return (uint32_t)(g.base + (int64_t)rw_cell_axis(y, g.y0, g.h, g.gh) * g.gw + rw_cell_axis(x, g.x0, g.h, g.gw));
+}
+
 // Node i of side s goes into grid s (its cell's count).
 __global__ void k_rw_hist(const int32_t* __restrict__ X, const int32_t* __restrict__ Y, int64_t nA, int64_t n,
-                          RwGrid g0, RwGrid g1, unsigned long long* __restrict__ cnt) {
+                          RwGrid g0, RwGrid g1, uint32_t* __restrict__ cnt) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const RwGrid& g = i < nA ? g0 : g1;
-    const int64_t c = g.base + (int64_t)rw_cell_axis(Y[i], g.y0, g.h, g.gh) * g.gw + rw_cell_axis(X[i], g.x0, g.h, g.gw);
-    atomicAdd(&cnt[c], 1ull);
+    if (i < n) atomicAdd(&cnt[rw_cell(i < nA ? g0 : g1, X[i], Y[i])], 1u);
 }
 
-// Nodes placed by cell (order inside a cell is arbitrary: only minima are read).
+// Nodes placed by cell (order inside a cell is arbitrary: only minima are read),
+// with their index.  cur: the cells' starts, moved to their ends.
 __global__ void k_rw_scatter(const int32_t* __restrict__ X, const int32_t* __restrict__ Y, int64_t nA, int64_t n,
-                             RwGrid g0, RwGrid g1, unsigned long long* __restrict__ cur, int2* __restrict__ pts) {
+                             RwGrid g0, RwGrid g1, uint32_t* __restrict__ cur, int2* __restrict__ pts,
+                             uint32_t* __restrict__ id) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const RwGrid& g = i < nA ? g0 : g1;
-    const int64_t c = g.base + (int64_t)rw_cell_axis(Y[i], g.y0, g.h, g.gh) * g.gw + rw_cell_axis(X[i], g.x0, g.h, g.gw);
-    const unsigned long long k = atomicAdd(&cur[c], 1ull);
-    pts[k] = make_int2(X[i], Y[i]);
+    const int2 p = make_int2(X[i], Y[i]);
+    const uint32_t k = atomicAdd(&cur[rw_cell(i < nA ? g0 : g1, p.x, p.y)], 1u);
+    pts[k] = p;
+    id[k] = (uint32_t)i;
 }
 
-// Ring search of node i (side s) in the other side's grid; see above.
-// Unfinished queries are listed: side A's from list[0], side B's from
-// list[nA], their counts in nl[0], nl[1].
-__global__ void k_rw_query(const int32_t* __restrict__ X, const int32_t* __restrict__ Y, int64_t nA, int64_t n,
-                           RwGrid g0, RwGrid g1, const unsigned long long* __restrict__ start,
-                           const int2* __restrict__ pts, DiagCost dc, unsigned long long* __restrict__ mind2,
-                           int32_t* __restrict__ list, int* __restrict__ nl) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const bool sa = i < nA;
-    const RwGrid& g = sa ? g1 : g0;  // the other side's grid
-    const int64_t ux = X[i], uy = Y[i];
-    const int64_t cm = cost_make((int32_t)ux, (int32_t)uy, dc);
-    const int32_t cx = rw_cell_axis(ux, g.x0, g.h, g.gw), cy = rw_cell_axis(uy, g.y0, g.h, g.gh);
+// Ring search of the q-th placed node in the other side's grid; see above.  end:
+// the cells' ends (a cell starts where the one before it ends).  Unfinished queries
+// are listed: side A's from list[0], side B's from list[nA], their counts in nl[0],
+// nl[1].
+__global__ void k_rw_query(int64_t nA, int64_t n, RwGrid g0, RwGrid g1, const uint32_t* __restrict__ end,
+                           const int2* __restrict__ pts, const uint32_t* __restrict__ id, DiagCost dc,
+                           unsigned long long* __restrict__ mind2, int32_t* __restrict__ list, int* __restrict__ nl) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= n) return;
+    const bool sa = q < nA;  // A's grid comes first, and its nodes
+    const RwGrid& g = sa ? g1 : g0;
+    const int2 u = pts[q];
+    const int64_t cm = cost_make(u.x, u.y, dc);
+    const int32_t cx = rw_cell_axis(u.x, g.x0, g.h, g.gw), cy = rw_cell_axis(u.y, g.y0, g.h, g.gh);
     unsigned long long best = ~0ull;
-    auto visit = [&](int32_t x, int32_t y) {
-        const int64_t c = g.base + (int64_t)y * g.gw + x;
-        const unsigned long long k1 = start[c + 1];
-        for (unsigned long long k = start[c]; k < k1; k++) {
+    // cells x0 .. x1 of row y hold one stretch of nodes
+    auto row = [&](int32_t y, int32_t x0, int32_t x1) {
+        const int64_t c = g.base + (int64_t)y * g.gw;
+        const uint32_t k1 = end[c + x1];
+        for (uint32_t k = c + x0 > 0 ? end[c + x0 - 1] : 0u; k < k1; k++) {
             const int2 v = pts[k];
-            const long long dx = ux - v.x, dy = uy - v.y;
+            const long long dx = (long long)u.x - v.x, dy = (long long)u.y - v.y;
             const unsigned long long d2 = (unsigned long long)(dx * dx) + (unsigned long long)(dy * dy);
             best = d2 < best ? d2 : best;
         }
     };
     int state = 0;  // 0 searching, 1 exact, 2 stopped by the diagonal cost
-    for (int32_t K = 0; K <= RW_KMAX && state == 0; K++) {
-        if (K == 0) {
-            visit(cx, cy);
+    for (int32_t K = 1; K <= RW_KMAX && state == 0; K++) {
+        const int32_t xlo = max(cx - K, 0), xhi = min(cx + K, g.gw - 1);
+        if (K == 1) {  // the first nine cells at once
+            for (int32_t y = max(cy - 1, 0); y <= min(cy + 1, g.gh - 1); y++) row(y, xlo, xhi);
         } else {
-            const int32_t xlo = max(cx - K, 0), xhi = min(cx + K, g.gw - 1);
-            if (cy - K >= 0)
-                for (int32_t x = xlo; x <= xhi; x++) visit(x, cy - K);
-            if (cy + K < g.gh)
-                for (int32_t x = xlo; x <= xhi; x++) visit(x, cy + K);
+            if (cy - K >= 0) row(cy - K, xlo, xhi);
+            if (cy + K < g.gh) row(cy + K, xlo, xhi);
             const int32_t ylo = max(cy - K + 1, 0), yhi = min(cy + K - 1, g.gh - 1);
             if (cx - K >= 0)
-                for (int32_t y = ylo; y <= yhi; y++) visit(cx - K, y);
+                for (int32_t y = ylo; y <= yhi; y++) row(y, cx - K, cx - K);
             if (cx + K < g.gw)
-                for (int32_t y = ylo; y <= yhi; y++) visit(cx + K, y);
+                for (int32_t y = ylo; y <= yhi; y++) row(y, cx + K, cx + K);
         }
         // distance to the nearest side of the searched square beyond which nodes may remain
+        const int64_t ux = u.x, uy = u.y;
         int64_t lb = INT64_MAX;
         if (cx - K > 0) lb = min(lb, ux - (g.x0 + (int64_t)(cx - K) * g.h));
         if (cx + K < g.gw - 1) lb = min(lb, g.x0 + (int64_t)(cx + K + 1) * g.h - ux);
@@ -591,6 +622,7 @@ __global__ void k_rw_query(const int32_t* __restrict__ X, const int32_t* __restr
         const unsigned long long c2 = (unsigned long long)cm * (unsigned long long)cm;
         best = c2 < best ? c2 : best;
     }
+    const uint32_t i = id[q];
     mind2[i] = best;
     if (state == 0) {
         const int k = atomicAdd(&nl[sa ? 0 : 1], 1);
@@ -640,16 +672,17 @@ __global__ void k_fill_u64(unsigned long long* p, int64_t n, unsigned long long 
 }
 
 // Grid geometry of one side with box b (xmin, xmax, ymin, ymax) and n nodes:
-// about two nodes a cell, at most 4 n + 64 cells.
-static RwGrid rw_grid(const int* b, int64_t n, int64_t base) {
+// about RW_CELLS cells a node, at most twice as many and 64.
+static RwGrid rw_grid(const int64_t* b, int64_t n, int64_t base) {
     RwGrid g{};
-    const int64_t W = (int64_t)b[1] - b[0], H = (int64_t)b[3] - b[2];
-    const double cells = (double)std::max<int64_t>(1, n / 2);
+    const int64_t W = b[1] - b[0], H = b[3] - b[2];
+    const int64_t want = std::min<int64_t>(RW_CELLS * n, int64_t(1) << 29);  // both grids below 2^32 cells
+    const double cells = (double)want;
     int64_t hs = (int64_t)ceil(sqrt((double)(W + 1) * (double)(H + 1) / cells));
     hs = std::max<int64_t>(hs, 1);
     for (;;) {
         const int64_t gw = W / hs + 1, gh = H / hs + 1;
-        if (gw * gh <= 4 * n + 64) {
+        if (gw * gh <= 2 * want + 64) {
             g.gw = (int32_t)gw;
             g.gh = (int32_t)gh;
             break;
@@ -668,30 +701,29 @@ static RwGrid rw_grid(const int* b, int64_t n, int64_t base) {
 static pd_status rwmd_grid(Ctx* c, const Hats& h, DiagCost dc, unsigned long long* mind2, int64_t chunk, int64_t gy,
                            cudaStream_t st) {
     const int64_t n = h.nA + h.nB;
-    int* box = bufT<int>(c, B_RW_BOX, 8);
+    int64_t* box = bufT<int64_t>(c, B_RW_BOX, 8);
     int* nl = bufT<int>(c, B_RW_NL, 2);
     if (!box || !nl) return PD_ENOMEM;
     k_rw_box_init<<<1, 32, 0, st>>>(box); pd::count_launch();
-    k_rw_box<<<grid_for(n, 256), 256, 0, st>>>(h.X, h.Y, h.nA, n, box); pd::count_launch();
-    int hb[8];
+    k_rw_box<<<dim3(box_grid(c, std::max(h.nA, h.nB)), 2), BOX_THREADS, 0, st>>>(h.X, h.Y, h.nA, n, box); pd::count_launch();
+    int64_t hb[8];
     PD_TRY_CUDA(c, cudaMemcpyAsync(hb, box, sizeof(hb), cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
     const RwGrid g0 = rw_grid(hb, h.nA, 0);
     const RwGrid g1 = rw_grid(hb + 4, h.nB, (int64_t)g0.gw * g0.gh);
     const int64_t cells = g1.base + (int64_t)g1.gw * g1.gh;
-    unsigned long long* start = bufT<unsigned long long>(c, B_RW_START, cells + 1);
-    unsigned long long* cur = bufT<unsigned long long>(c, B_RW_CUR, cells + 1);
-    unsigned long long* part = bufT<unsigned long long>(c, B_SCAN_PART, scan_tiles(cells + 1) + 1);
+    uint32_t* cell = bufT<uint32_t>(c, B_RW_START, cells);
+    uint32_t* part = bufT<uint32_t>(c, B_SCAN_PART, scan_tiles(cells) + 1);
     int2* pts = bufT<int2>(c, B_RW_PTS, n);
+    uint32_t* id = bufT<uint32_t>(c, B_RW_CUR, n);
     int32_t* list = bufT<int32_t>(c, B_RW_LIST, n);
-    if (!start || !cur || !part || !pts || !list) return PD_ENOMEM;
-    PD_TRY_CUDA(c, cudaMemsetAsync(start, 0, sizeof(unsigned long long) * (cells + 1), st));
+    if (!cell || !part || !pts || !id || !list) return PD_ENOMEM;
+    PD_TRY_CUDA(c, cudaMemsetAsync(cell, 0, sizeof(uint32_t) * cells, st));
     PD_TRY_CUDA(c, cudaMemsetAsync(nl, 0, 2 * sizeof(int), st));
-    k_rw_hist<<<grid_for(n, 256), 256, 0, st>>>(h.X, h.Y, h.nA, n, g0, g1, start); pd::count_launch();
-    PD_TRY_CUDA(c, exclusive_scan<unsigned long long>(start, start, cells + 1, part, nullptr, st));
-    PD_TRY_CUDA(c, cudaMemcpyAsync(cur, start, sizeof(unsigned long long) * (cells + 1), cudaMemcpyDeviceToDevice, st));
-    k_rw_scatter<<<grid_for(n, 256), 256, 0, st>>>(h.X, h.Y, h.nA, n, g0, g1, cur, pts); pd::count_launch();
-    k_rw_query<<<grid_for(n, 128), 128, 0, st>>>(h.X, h.Y, h.nA, n, g0, g1, start, pts, dc, mind2, list, nl); pd::count_launch();
+    k_rw_hist<<<grid_for(n, 256), 256, 0, st>>>(h.X, h.Y, h.nA, n, g0, g1, cell); pd::count_launch();
+    PD_TRY_CUDA(c, exclusive_scan<uint32_t>(cell, cell, cells, part, nullptr, st));
+    k_rw_scatter<<<grid_for(n, 256), 256, 0, st>>>(h.X, h.Y, h.nA, n, g0, g1, cell, pts, id); pd::count_launch();
+    k_rw_query<<<grid_for(n, 128), 128, 0, st>>>(h.nA, n, g0, g1, cell, pts, id, dc, mind2, list, nl); pd::count_launch();
     PD_TRY_CUDA(c, cudaGetLastError());
     int hn[2];
     PD_TRY_CUDA(c, cudaMemcpyAsync(hn, nl, sizeof(hn), cudaMemcpyDeviceToHost, st));
@@ -731,7 +763,7 @@ pd_status stage_rwmd(Ctx* c, const Hats& h, int64_t L[3], DiagCost dc, cudaStrea
         } else if (gx > 0 && h.nA > 0 && h.nB > 0) {
             k_rwmd_min<<<dim3((unsigned)gx, (unsigned)gy, 2), RW_THREADS, 0, st>>>(h.X, h.Y, h.nA, h.nB, chunk, mind2); pd::count_launch();
         }
-        k_rwmd_sum<<<grid_for(n, 256), 256, 0, st>>>(h.X, h.Y, h.cnt, h.nA, n, mind2, dc, sm + S_L0); pd::count_launch();
+        k_rwmd_sum<<<box_grid(c, n), BOX_THREADS, 0, st>>>(h.X, h.Y, h.cnt, h.nA, n, mind2, dc, sm + S_L0); pd::count_launch();
         PD_TRY_CUDA(c, cudaGetLastError());
     }
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, sizeof(int64_t) * S_COUNT, cudaMemcpyDeviceToHost, st));
@@ -746,33 +778,24 @@ pd_status stage_rwmd(Ctx* c, const Hats& h, int64_t L[3], DiagCost dc, cudaStrea
 // delta-condensation (Algorithm 2) and Morton order
 // ---------------------------------------------------------------------------
 
-__global__ void k_cells(const int32_t* __restrict__ X, const int32_t* __restrict__ Y, int64_t n, int64_t G,
-                        int64_t* __restrict__ CX, int64_t* __restrict__ CY, int64_t* __restrict__ sm) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t cx = INT64_MAX, cy = INT64_MAX, xx = INT64_MIN, xy = INT64_MIN;
-    if (i < n) {
-        cx = floor_div(2 * (int64_t)X[i] + G, 2 * G);  // nearest lattice point, ties up
-        cy = floor_div(2 * (int64_t)Y[i] + G, 2 * G);
+__global__ void __launch_bounds__(BOX_THREADS) k_cells(const int32_t* __restrict__ X, const int32_t* __restrict__ Y,
+                                                       int64_t n, int64_t G, int32_t* __restrict__ CX,
+                                                       int32_t* __restrict__ CY, int64_t* __restrict__ sm) {
+    int32_t box[4] = {INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN};
+    for (int64_t i = (int64_t)blockIdx.x * BOX_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * BOX_THREADS) {
+        const int32_t cx = (int32_t)floor_div(2 * (int64_t)X[i] + G, 2 * G);  // nearest lattice point, ties up
+        const int32_t cy = (int32_t)floor_div(2 * (int64_t)Y[i] + G, 2 * G);  // |cell| <= 2^29
         CX[i] = cx;
         CY[i] = cy;
-        xx = cx;
-        xy = cy;
+        box[0] = min(box[0], cx);
+        box[1] = max(box[1], cx);
+        box[2] = min(box[2], cy);
+        box[3] = max(box[3], cy);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        cx = min(cx, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)cx, o));
-        cy = min(cy, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)cy, o));
-        xx = max(xx, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)xx, o));
-        xy = max(xy, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)xy, o));
-    }
-    if ((threadIdx.x & 31) == 0 && xx != INT64_MIN) {
-        atomicMin((long long*)&sm[S_CMNX], (long long)cx);
-        atomicMin((long long*)&sm[S_CMNY], (long long)cy);
-        atomicMax((long long*)&sm[S_CMXX], (long long)xx);
-        atomicMax((long long*)&sm[S_CMXY], (long long)xy);
-    }
+    box_to(box, &sm[S_CMNX]);
 }
 
-__global__ void k_cell_keys(const int64_t* __restrict__ CX, const int64_t* __restrict__ CY, int64_t n,
+__global__ void k_cell_keys(const int32_t* __restrict__ CX, const int32_t* __restrict__ CY, int64_t n,
                             const int64_t* __restrict__ sm, int bcy, uint64_t* __restrict__ key,
                             uint32_t* __restrict__ val) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -782,45 +805,35 @@ __global__ void k_cell_keys(const int64_t* __restrict__ CX, const int64_t* __res
 }
 
 // One node per distinct cell: place it at G * cell + shift(seed, cell).
-__global__ void k_cell_place(const uint64_t* __restrict__ key, int64_t n, const int64_t* __restrict__ idx,
-                             const int64_t* __restrict__ sm, int bcy, int64_t G, int64_t P, uint64_t seed,
-                             int32_t* __restrict__ NX, int32_t* __restrict__ NY, int64_t* __restrict__ smw) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t x = INT64_MAX, y = INT64_MAX, xx = INT64_MIN, xy = INT64_MIN;
+__global__ void __launch_bounds__(BOX_THREADS) k_cell_place(const uint64_t* __restrict__ key, int64_t n,
+                                                            const int64_t* __restrict__ idx,
+                                                            const int64_t* __restrict__ sm, int bcy, int64_t G,
+                                                            int64_t P, uint64_t seed, int32_t* __restrict__ NX,
+                                                            int32_t* __restrict__ NY, int64_t* __restrict__ CA,
+                                                            int64_t* __restrict__ CB, int64_t* __restrict__ smw) {
+    int32_t box[4] = {INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN};
     bool bad = false;
-    if (i < n && (i == 0 || key[i - 1] != key[i])) {
-        uint64_t k = key[i];
-        uint64_t ymask = bcy >= 64 ? ~0ull : ((1ull << bcy) - 1);
-        int64_t cx = (int64_t)(k >> bcy) + sm[S_CMNX];
-        int64_t cy = (int64_t)(k & ymask) + sm[S_CMNY];
+    const uint64_t ymask = bcy >= 64 ? ~0ull : ((1ull << bcy) - 1);
+    const int64_t mnx = sm[S_CMNX], mny = sm[S_CMNY];
+    for (int64_t i = (int64_t)blockIdx.x * BOX_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * BOX_THREADS) {
+        const uint64_t k = key[i];
+        if (i > 0 && key[i - 1] == k) continue;
+        const int64_t cx = (int64_t)(k >> bcy) + mnx, cy = (int64_t)(k & ymask) + mny;
         int64_t dx, dy;
         cell_shift(seed, cx, cy, P, &dx, &dy);
-        x = G * cx + dx;
-        y = G * cy + dy;
-        const int64_t lim = int64_t(1) << 30;
-        bad = x <= -lim || x >= lim || y <= -lim || y >= lim;
-        int64_t j = idx[i];
+        const int64_t x = G * cx + dx, y = G * cy + dy, lim = int64_t(1) << 30;
+        bad |= x <= -lim || x >= lim || y <= -lim || y >= lim;
+        const int64_t j = idx[i];
         NX[j] = (int32_t)x;
         NY[j] = (int32_t)y;
-        xx = x;
-        xy = y;
+        CA[j] = CB[j] = 0;
+        box[0] = min(box[0], (int32_t)x);
+        box[1] = max(box[1], (int32_t)x);
+        box[2] = min(box[2], (int32_t)y);
+        box[3] = max(box[3], (int32_t)y);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        x = min(x, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)x, o));
-        y = min(y, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)y, o));
-        xx = max(xx, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)xx, o));
-        xy = max(xy, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)xy, o));
-    }
-    unsigned b = __ballot_sync(0xffffffffu, bad);
-    if ((threadIdx.x & 31) == 0) {
-        if (xx != INT64_MIN) {
-            atomicMin((long long*)&smw[S_NMNX], (long long)x);
-            atomicMin((long long*)&smw[S_NMNY], (long long)y);
-            atomicMax((long long*)&smw[S_NMXX], (long long)xx);
-            atomicMax((long long*)&smw[S_NMXY], (long long)xy);
-        }
-        if (b) atomicAdd((unsigned long long*)&smw[S_ERR], 1ull);
-    }
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicAdd((unsigned long long*)&smw[S_ERR], 1ull);
+    box_to(box, &smw[S_NMNX]);
 }
 
 // Aggregate the multiplicities of the nodes snapped into each cell.
@@ -997,8 +1010,8 @@ pd_status stage_condense_delta(Ctx* c, const Hats& hats, int64_t G, int64_t P, u
         out->n_nodes = hs[S_N];
         return PD_OK;
     }
-    int64_t* CX = bufT<int64_t>(c, B_CX, n);
-    int64_t* CY = bufT<int64_t>(c, B_CY, n);
+    int32_t* CX = bufT<int32_t>(c, B_CX, n);
+    int32_t* CY = bufT<int32_t>(c, B_CY, n);
     uint64_t* key = bufT<uint64_t>(c, B_CKEY, n);
     uint64_t* key2 = bufT<uint64_t>(c, B_CKEY2, n);
     uint32_t* val = bufT<uint32_t>(c, B_CVAL, n);
@@ -1010,7 +1023,7 @@ pd_status stage_condense_delta(Ctx* c, const Hats& hats, int64_t G, int64_t P, u
     int64_t* CB = bufT<int64_t>(c, B_CB, n);
     if (!CX || !CY || !key || !key2 || !val || !val2 || !idx || !NX || !NY || !CA || !CB) return PD_ENOMEM;
     k_init_small<<<1, 64, 0, st>>>(sm); pd::count_launch();
-    k_cells<<<grid_for(n, 256), 256, 0, st>>>(h.X, h.Y, n, G, CX, CY, sm); pd::count_launch();
+    k_cells<<<box_grid(c, n), BOX_THREADS, 0, st>>>(h.X, h.Y, n, G, CX, CY, sm); pd::count_launch();
     PD_TRY_CUDA(c, cudaGetLastError());
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, sizeof(int64_t) * S_COUNT, cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
@@ -1020,9 +1033,7 @@ pd_status stage_condense_delta(Ctx* c, const Hats& hats, int64_t G, int64_t P, u
     PD_TRY(sort_u64(c, key, key2, val, val2, n, bcx + bcy, st));
     k_run_flags<<<grid_for(n, 256), 256, 0, st>>>(key, n, ~0ull, idx); pd::count_launch();
     PD_TRY(scan_i64(c, idx, idx, n, sm + S_N, st));
-    k_cell_place<<<grid_for(n, 256), 256, 0, st>>>(key, n, idx, sm, bcy, G, P, seed, NX, NY, sm); pd::count_launch();
-    PD_TRY_CUDA(c, cudaMemsetAsync(CA, 0, sizeof(int64_t) * n, st));
-    PD_TRY_CUDA(c, cudaMemsetAsync(CB, 0, sizeof(int64_t) * n, st));
+    k_cell_place<<<box_grid(c, n), BOX_THREADS, 0, st>>>(key, n, idx, sm, bcy, G, P, seed, NX, NY, CA, CB, sm); pd::count_launch();
     k_cell_accum<<<grid_for(n, 256), 256, 0, st>>>(key, val, n, idx, h.cnt, h.nA, CA, CB); pd::count_launch();
     PD_TRY_CUDA(c, cudaGetLastError());
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, sizeof(int64_t) * S_COUNT, cudaMemcpyDeviceToHost, st));

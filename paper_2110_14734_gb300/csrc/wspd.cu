@@ -348,45 +348,57 @@ PD_D bool ws_far(const WsRec& a, const WsRec& b, int32_t ra, int32_t rb, int64_t
 }
 
 constexpr int WS_WARPS = 8;      // per block
+constexpr int WS_OUT = 256;      // separated pairs a warp gathers before it stores them
 constexpr int WS_STACK = 736;    // pairs a warp's stack holds
 constexpr int WS_MARGIN = 200;   // above WS_STACK - WS_MARGIN pairs it visits one at a time: a path is
                                  // at most 2 * 65 splits long (78 + 78 on the split tree), each net +1
 
 // lv[0] += separated pairs, lv[1] = pairs offered to the next launch (the first
 // cap of them are in Fn), lv[2] = initial pairs taken.  STORE: both arcs of every separated
-// pair to arcs, at slots from lv[0] (which counts pairs).
+// pair to arcs (room for `room` pairs), at slots from lv[0], which counts all
+// pairs.
 template <bool STORE>
 __global__ void __launch_bounds__(32 * WS_WARPS) k_ws_walk(const int2* __restrict__ F, int64_t nf, int chunk,
                                                            const WsRec* __restrict__ rec, WsTree tr, int64_t s,
                                                            int64_t budget, int2* __restrict__ Fn,
                                                            unsigned long long cap, int hb, uint64_t* __restrict__ arcs,
+                                                           unsigned long long room,
                                                            unsigned long long* __restrict__ lv) {
     __shared__ int2 stack_[WS_WARPS][WS_STACK];
+    extern __shared__ int2 out_[];  // STORE: separated pairs on their way out, WS_OUT a warp
+    int2* const ow = out_ + (threadIdx.x >> 5) * WS_OUT;
+    int on_out = 0;
     const int lane = threadIdx.x & 31;
     int2* const st = stack_[threadIdx.x >> 5];
     const unsigned below = (1u << lane) - 1u;
     unsigned long long count = 0;
+    // the buffered pairs' arcs, at slots taken with one atomic; past `room` they are only counted
+    auto flush = [&]() {
+        __syncwarp();
+        unsigned long long at = 0;
+        if (lane == 0) at = atomicAdd(&lv[0], (unsigned long long)on_out);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        for (int q = lane; q < on_out && at + q < room; q += 32) {
+            const int2 a = ow[q];
+            ulonglong2 w;
+            w.x = (uint64_t)a.x << hb | (uint64_t)a.y;
+            w.y = (uint64_t)a.y << hb | (uint64_t)a.x;
+            *(ulonglong2*)(arcs + 2 * (at + q)) = w;
+        }
+        on_out = 0;
+        __syncwarp();
+    };
     // up to three separated pairs of a lane, by their representatives
     auto emit = [&](bool on0, int2 a0, bool on1, int2 a1, bool on2, int2 a2) {
         if constexpr (STORE) {
             const unsigned m0 = __ballot_sync(0xffffffffu, on0), m1 = __ballot_sync(0xffffffffu, on1),
                            m2 = __ballot_sync(0xffffffffu, on2);
-            if ((m0 | m1 | m2) == 0) return;
-            unsigned long long at = 0;
-            if (lane == 0) at = atomicAdd(&lv[0], (unsigned long long)(__popc(m0) + __popc(m1) + __popc(m2)));
-            at = __shfl_sync(0xffffffffu, at, 0);
-            auto put = [&](bool on, unsigned m, int2 a) {
-                if (on) {
-                    ulonglong2 w;
-                    w.x = (uint64_t)a.x << hb | (uint64_t)a.y;
-                    w.y = (uint64_t)a.y << hb | (uint64_t)a.x;
-                    *(ulonglong2*)(arcs + 2 * (at + __popc(m & below))) = w;
-                }
-                at += __popc(m);
-            };
-            put(on0, m0, a0);
-            put(on1, m1, a1);
-            put(on2, m2, a2);
+            const int c0 = __popc(m0), c1 = __popc(m1), c2 = __popc(m2);
+            if (on0) ow[on_out + __popc(m0 & below)] = a0;
+            if (on1) ow[on_out + c0 + __popc(m1 & below)] = a1;
+            if (on2) ow[on_out + c0 + c1 + __popc(m2 & below)] = a2;
+            on_out += c0 + c1 + c2;
+            if (on_out > WS_OUT - 96) flush();
         } else {
             count += (unsigned)on0 + (unsigned)on1 + (unsigned)on2;
         }
@@ -450,7 +462,9 @@ __global__ void __launch_bounds__(32 * WS_WARPS) k_ws_walk(const int2* __restric
             __syncwarp();
         }
     }
-    if constexpr (!STORE) {
+    if constexpr (STORE) {
+        if (on_out > 0) flush();
+    } else {
         for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
         if (lane == 0 && count) atomicAdd(&lv[0], count);
     }
@@ -607,14 +621,16 @@ pd_status merge_diagonal(Ctx* c, const pd_network& net, int64_t N, pd_network* o
 
 // All launches of the walk over the tree's pairs (see k_ws_walk): *pairs =
 // separated pairs; arcs (may be null): where their arcs go.
-static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, int64_t s, int hb, uint64_t* arcs, int64_t* pairs,
-                         cudaStream_t st) {
+static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, int64_t s, int hb, uint64_t* arcs, int64_t room,
+                         int64_t* pairs, cudaStream_t st) {
     unsigned long long* lv = bufT<unsigned long long>(c, B_SMALL, 64) + 12;
     const int blocks = 4 * std::max(c->sm_count, 1);  // the stacks of four blocks fit an SM
     const int64_t warps = (int64_t)blocks * WS_WARPS;
     // room for handed-on pairs: the more, the better the balance; less will do
     int64_t cap = std::min<int64_t>(int64_t(1) << 27, std::max<int64_t>(int64_t(1) << 16, 64 * (tr.N - 1)));
     int2* out[2];
+    if (arcs) PD_TRY_CUDA(c, cudaFuncSetAttribute(k_ws_walk<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)(sizeof(int2) * WS_WARPS * WS_OUT)));
     for (;; cap /= 4) {
         out[0] = bufT<int2>(c, B_F1, cap);
         out[1] = out[0] ? bufT<int2>(c, B_WSOFF, cap) : nullptr;
@@ -636,11 +652,12 @@ static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, int64_t s, 
                                        (arcs && round > 0 ? 2 : 3) * sizeof(unsigned long long), st));
         const unsigned grid = (unsigned)std::min<int64_t>(blocks, ((nf + chunk - 1) / chunk + WS_WARPS - 1) / WS_WARPS);
         if (arcs) {
-            k_ws_walk<true><<<grid, 32 * WS_WARPS, 0, st>>>(F, nf, chunk, rec, tr, s, budget, out[round & 1],
-                                                            (unsigned long long)cap, hb, arcs, lv); pd::count_launch();
+            k_ws_walk<true><<<grid, 32 * WS_WARPS, sizeof(int2) * WS_WARPS * WS_OUT, st>>>(
+                F, nf, chunk, rec, tr, s, budget, out[round & 1], (unsigned long long)cap, hb, arcs,
+                (unsigned long long)room, lv); pd::count_launch();
         } else {
             k_ws_walk<false><<<grid, 32 * WS_WARPS, 0, st>>>(F, nf, chunk, rec, tr, s, budget, out[round & 1],
-                                                             (unsigned long long)cap, hb, nullptr, lv); pd::count_launch();
+                                                             (unsigned long long)cap, hb, nullptr, 0, lv); pd::count_launch();
         }
         PD_TRY_CUDA(c, cudaGetLastError());
         PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, lv, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -711,15 +728,22 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
         k_ws_records<<<grid_for(N - 1, 256), 256, 0, st>>>(N - 1, bb, rep, left, right, s, rec, F); pd::count_launch();
         PD_TRY_CUDA(c, cudaGetLastError());
         int64_t pairs = 0;
-        PD_TRY(ws_walk(c, tr, rec, s, hb, nullptr, &pairs, st));
-        narcs = 2 * pairs;
-        if (!count_only) {
-            arcs = bufT<uint64_t>(c, B_ARCKEY, narcs + 2 * N + 1);
-            if (!arcs) return PD_ENOMEM;
-            int64_t again = 0;
-            PD_TRY(ws_walk(c, tr, rec, s, hb, arcs, &again, st));
-            if (again != pairs) return fail(c, PD_ECUDA, "the WSPD's pairs changed between counting and storing");
+        if (count_only) {
+            PD_TRY(ws_walk(c, tr, rec, s, hb, nullptr, 0, &pairs, st));
+        } else {
+            // stored into the buffer the context has (64 arcs a node the first time);
+            // if they are more, the walk has counted them and the second one stores them
+            int64_t room = 0;
+            for (int pass = 0; pass < 2; pass++) {
+                arcs = bufT<uint64_t>(c, B_ARCKEY, 2 * (pass ? pairs : 32 * N) + 2 * N + 1);
+                if (!arcs) return PD_ENOMEM;
+                room = ((int64_t)(c->bytes[B_ARCKEY] / sizeof(uint64_t)) - (2 * N + 1)) / 2;
+                PD_TRY(ws_walk(c, tr, rec, s, hb, arcs, room, &pairs, st));
+                if (pairs <= room) break;
+            }
+            if (pairs > room) return fail(c, PD_ECUDA, "the WSPD's pairs changed between two walks");
         }
+        narcs = 2 * pairs;
     }
     PD_TRY_CUDA(c, cudaEventRecord(ev[2], st));
     if (count_only) {
