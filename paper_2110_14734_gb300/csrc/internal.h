@@ -38,7 +38,7 @@ enum Buf : int {
     B_SP_ORD, B_SP_ORD2, B_SP_SEG, B_SP_SEG2, B_SP_HI, B_SP_HI2, B_SP_NUM, B_SP_NUM2,  // split tree
     B_SP_BB, B_SP_REPK, B_SP_REPN, B_SP_FLAG, B_SP_RANK, B_SP_X, B_SP_Y, B_SP_CA, B_SP_CB, B_SP_CODE, B_SP_POS,
     B_CO_BOX, B_CO_P, B_CO_P2, B_CO_GAP,  // coarse-solve warm start
-    B_MLP_BEST, B_WS_BF, B_WS_BT, B_WS_BM, B_WS_IDX,  // network training: best weights, shuffled batch
+    B_MLP_BEST, B_WS_RAW, B_WS_BF, B_WS_BT, B_WS_BM, B_WS_IDX,  // network training: best weights, shuffled batch
     B_NS_JOBS, B_NS_CERT,           // batched certificate
     B_RW_BOX, B_RW_START, B_RW_CUR, B_RW_PTS, B_RW_LIST, B_RW_NL,  // RWMD grid
     B_SMALL,                        // small device scalars

@@ -25,6 +25,8 @@
 #include <algorithm>
 #include <chrono>
 #include <cstring>
+#include <memory>
+#include <new>
 #include <vector>
 
 #include <cuda_bf16.h>
@@ -192,8 +194,19 @@ pd_status ws_diag_potentials(Ctx* c, const pd_nodes& nodes, const W1Prep& w, std
 }
 
 // ---------------------------------------------------------------------------
-// the network: tiles of WS_TILE nodes, thread j owns hidden unit j
+// the network: tiles of WS_TILE rows, one block of WS_THREADS threads each
 // ---------------------------------------------------------------------------
+//
+// 25,728 multiply-adds a row forward, twice that backward, in float32 (weights
+// bf16): the CUDA cores' work, so what matters is multiply-adds per shared-memory
+// load and enough blocks.  Activations lie transposed, [unit][row], so that one
+// 16-byte load gives a unit for four rows: a thread computes 4 rows x 2 units
+// of a layer (8 multiply-adds per two loads) and 8 x 8 of the 128 x 128 weight
+// gradients (256 per 16 loads), the latter in registers over all tiles of its
+// block.  16 rows a tile: the 2,048 rows of a training step fill 128 SMs.  With 32
+// rows, one unit a thread, gradients summed in shared memory and the features
+// rounded on the host, pd_ws_grad took 335 microseconds on 2,048 rows and
+// pd_ws_forward 207; now 115 and 59, copies included.
 
 struct MlpW {
     const __nv_bfloat16* W1;  // [WS_IN][WS_H]
@@ -204,163 +217,219 @@ struct MlpW {
     const float* b3;          // [1]
 };
 
-// Forward of one tile: x (smem, [WS_TILE][WS_IN] float) -> h1, h2 (smem) and
-// the outputs (smem, [WS_TILE]).
-PD_D void tile_forward(const MlpW& w, const float* x, float* h1, float* h2, float* out, int nrow) {
-    const int j = threadIdx.x;
-    float acc[WS_TILE];
-#pragma unroll
-    for (int r = 0; r < WS_TILE; r++) acc[r] = 0.f;
-    for (int k = 0; k < WS_IN; k++) {
-        const float wk = __bfloat162float(w.W1[k * WS_H + j]);
-#pragma unroll
-        for (int r = 0; r < WS_TILE; r++) acc[r] = fmaf(x[r * WS_IN + k], wk, acc[r]);
-    }
-    const float bj = w.b1[j];
-#pragma unroll
-    for (int r = 0; r < WS_TILE; r++) h1[r * WS_H + j] = fmaxf(acc[r] + bj, 0.f);
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < WS_TILE; r++) acc[r] = 0.f;
-    for (int k = 0; k < WS_H; k++) {
-        const float wk = __bfloat162float(w.W2[k * WS_H + j]);
-#pragma unroll
-        for (int r = 0; r < WS_TILE; r++) acc[r] = fmaf(h1[r * WS_H + k], wk, acc[r]);
-    }
-    const float b2j = w.b2[j];
-#pragma unroll
-    for (int r = 0; r < WS_TILE; r++) h2[r * WS_H + j] = fmaxf(acc[r] + b2j, 0.f);
-    __syncthreads();
-    // out[r] = sum_j h2[r][j] w3[j] + b3: warp r % 4 .. sums rows
-    const int lane = j & 31, wid = j >> 5;
-    for (int r = wid; r < nrow; r += WS_H / 32) {
-        float s = 0.f;
-        for (int k = lane; k < WS_H; k += 32) s = fmaf(h2[r * WS_H + k], __bfloat162float(w.w3[k]), s);
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) out[r] = s + w.b3[0];
-    }
-    __syncthreads();
-}
+constexpr int WS_THREADS = 256;
+constexpr int WS_LD = WS_TILE + 4;  // floats between units: 16-byte loads, two-way conflicts at most
 
-PD_D void load_tile(const __nv_bfloat16* __restrict__ F, int64_t r0, int nrow, float* x) {
-    for (int t = threadIdx.x; t < WS_TILE * WS_IN; t += WS_H) {
-        const int r = t / WS_IN;
-        x[t] = r < nrow ? __bfloat162float(F[(r0 + r) * WS_IN + (t - r * WS_IN)]) : 0.f;
+// Thread t: rows 4 (t / 64) .. + 3, units 2 (t % 64) and the next.
+struct MlpTile {
+    float x[WS_IN][WS_LD];
+    float h1[WS_H][WS_LD];    // then delta1
+    float h2[WS_H][WS_LD];    // delta2
+    float out[2][WS_TILE];    // the output's two half sums, then delta3 in out[0]
+    float sums[4][3][WS_H];   // per group of rows: gradients of b1, b2, w3
+    float loss[3];            // gradient of b3, loss, mask
+};
+
+PD_D void tile_load(MlpTile& s, const __nv_bfloat16* __restrict__ F, int64_t r0, int nrow) {
+    for (int t = threadIdx.x; t < WS_TILE * WS_IN; t += WS_THREADS) {
+        const int r = t / WS_IN, k = t - r * WS_IN;
+        s.x[k][r] = r < nrow ? __bfloat162float(F[(r0 + r) * WS_IN + k]) : 0.f;
     }
 }
 
-__global__ void __launch_bounds__(WS_H) k_mlp_forward(MlpW w, const __nv_bfloat16* __restrict__ F, int64_t n,
-                                                      float* __restrict__ y) {
-    __shared__ float x[WS_TILE * WS_IN];
-    __shared__ float h1[WS_TILE * WS_H];
-    __shared__ float h2[WS_TILE * WS_H];
-    __shared__ float out[WS_TILE];
+// acc[row][unit] += sum over K of in[k][rows] w[k][units] (w: rows of WS_H bf16)
+template <int K>
+PD_D void tile_product(const float (*in)[WS_LD], const __nv_bfloat16* __restrict__ w, int row, int unit,
+                       float (&acc)[4][2]) {
+#pragma unroll 8
+    for (int k = 0; k < K; k++) {
+        const float4 v = *(const float4*)&in[k][row];
+        const float2 f = __bfloat1622float2(*(const __nv_bfloat162*)(w + k * WS_H + unit));
+        acc[0][0] = fmaf(v.x, f.x, acc[0][0]);
+        acc[0][1] = fmaf(v.x, f.y, acc[0][1]);
+        acc[1][0] = fmaf(v.y, f.x, acc[1][0]);
+        acc[1][1] = fmaf(v.y, f.y, acc[1][1]);
+        acc[2][0] = fmaf(v.z, f.x, acc[2][0]);
+        acc[2][1] = fmaf(v.z, f.y, acc[2][1]);
+        acc[3][0] = fmaf(v.w, f.x, acc[3][0]);
+        acc[3][1] = fmaf(v.w, f.y, acc[3][1]);
+    }
+}
+
+// x -> h1 (kept), h2 (registers), out[0] + out[1].  Ends with a barrier.
+PD_D void tile_forward(MlpTile& s, const MlpW& w, float (&h2)[4][2]) {
+    const int tid = threadIdx.x, unit = 2 * (tid & 63), row = 4 * (tid >> 6);
+    float a[4][2] = {};
+    tile_product<WS_IN>(s.x, w.W1, row, unit, a);
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        const float b = w.b1[unit + c];
+        *(float4*)&s.h1[unit + c][row] = make_float4(fmaxf(a[0][c] + b, 0.f), fmaxf(a[1][c] + b, 0.f),
+                                                     fmaxf(a[2][c] + b, 0.f), fmaxf(a[3][c] + b, 0.f));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; r++) h2[r][0] = h2[r][1] = 0.f;
+    tile_product<WS_H>(s.h1, w.W2, row, unit, h2);
+    float o[4];
+    const float2 w3 = __bfloat1622float2(*(const __nv_bfloat162*)(w.w3 + unit));
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        h2[r][0] = fmaxf(h2[r][0] + w.b2[unit], 0.f);
+        h2[r][1] = fmaxf(h2[r][1] + w.b2[unit + 1], 0.f);
+        o[r] = fmaf(h2[r][0], w3.x, h2[r][1] * w3.y);
+        for (int q = 16; q > 0; q >>= 1) o[r] += __shfl_xor_sync(0xffffffffu, o[r], q);
+    }
+    if ((tid & 31) == 0)
+#pragma unroll
+        for (int r = 0; r < 4; r++) s.out[(tid >> 5) & 1][row + r] = o[r];
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(WS_THREADS) k_mlp_forward(MlpW w, const __nv_bfloat16* __restrict__ F, int64_t n,
+                                                            float* __restrict__ y) {
+    __shared__ __align__(16) MlpTile s;
     for (int64_t r0 = (int64_t)blockIdx.x * WS_TILE; r0 < n; r0 += (int64_t)gridDim.x * WS_TILE) {
         const int nrow = (int)min((int64_t)WS_TILE, n - r0);
         __syncthreads();
-        load_tile(F, r0, nrow, x);
+        tile_load(s, F, r0, nrow);
         __syncthreads();
-        tile_forward(w, x, h1, h2, out, nrow);
-        if (threadIdx.x < nrow) y[r0 + threadIdx.x] = out[threadIdx.x];
+        float h2[4][2];
+        tile_forward(s, w, h2);
+        if (threadIdx.x < nrow) y[r0 + threadIdx.x] = s.out[0][threadIdx.x] + s.out[1][threadIdx.x] + w.b3[0];
     }
 }
 
 // Loss sum(mask * (y - t)^2) / sum(mask) and its gradients; every block sums
 // its tiles' gradients into its own row of `part` (WS_NPARAMS floats + 2:
 // loss sum, mask sum), reduced afterwards in a fixed order.
-__global__ void __launch_bounds__(WS_H) k_mlp_backward(MlpW w, const __nv_bfloat16* __restrict__ F,
-                                                       const float* __restrict__ tgt, const float* __restrict__ mask,
-                                                       int64_t n, float inv_norm, float* __restrict__ part) {
-    extern __shared__ float sm[];
-    float* x = sm;                            // WS_TILE * WS_IN
-    float* h1 = x + WS_TILE * WS_IN;          // WS_TILE * WS_H
-    float* h2 = h1 + WS_TILE * WS_H;          // WS_TILE * WS_H (becomes delta2)
-    float* out = h2 + WS_TILE * WS_H;         // WS_TILE (becomes delta3)
-    float* gW1 = out + WS_TILE;               // WS_IN * WS_H
-    float* gW2 = gW1 + WS_IN * WS_H;          // WS_H * WS_H
-    float* gsm = gW2 + WS_H * WS_H;           // b1, b2, w3 (3 * WS_H), b3, loss, mask
-    const int j = threadIdx.x;
-    for (int t = j; t < WS_IN * WS_H; t += WS_H) gW1[t] = 0.f;
-    for (int t = j; t < WS_H * WS_H; t += WS_H) gW2[t] = 0.f;
-    for (int t = j; t < 3 * WS_H + 3; t += WS_H) gsm[t] = 0.f;
-    float gb1 = 0.f, gb2 = 0.f, gw3 = 0.f;
+__global__ void __launch_bounds__(WS_THREADS) k_mlp_backward(MlpW w, const __nv_bfloat16* __restrict__ F,
+                                                             const float* __restrict__ tgt,
+                                                             const float* __restrict__ mask, int64_t n, float inv_norm,
+                                                             float* __restrict__ part) {
+    extern __shared__ __align__(16) unsigned char mlp_dyn[];
+    MlpTile& s = *(MlpTile*)mlp_dyn;
+    __nv_bfloat16* wt = (__nv_bfloat16*)(&s + 1);  // W2 transposed: [unit of layer 2][unit of layer 1]
+    const int tid = threadIdx.x, unit = 2 * (tid & 63), row = 4 * (tid >> 6);
+    const int k2 = 8 * (tid >> 4), j2 = 8 * (tid & 15);  // this thread's 8 x 8 of W2's gradient
+    const int k1 = 9 * (tid >> 5), j1 = 4 * (tid & 31);  // ... and 9 x 4 of W1's
+    for (int t = tid; t < WS_H * WS_H; t += WS_THREADS) wt[(t & (WS_H - 1)) * WS_H + (t >> 7)] = w.W2[t];
+    float g2[8][8] = {}, g1[9][4] = {}, gb1[2] = {}, gb2[2] = {}, gw3[2] = {}, gl[3] = {};
+    const float2 w3 = __bfloat1622float2(*(const __nv_bfloat162*)(w.w3 + unit));
     for (int64_t r0 = (int64_t)blockIdx.x * WS_TILE; r0 < n; r0 += (int64_t)gridDim.x * WS_TILE) {
         const int nrow = (int)min((int64_t)WS_TILE, n - r0);
         __syncthreads();
-        load_tile(F, r0, nrow, x);
+        tile_load(s, F, r0, nrow);
         __syncthreads();
-        tile_forward(w, x, h1, h2, out, nrow);
-        // delta3 = 2 mask (y - t) / norm
-        if (j < WS_TILE) {
-            float d = 0.f;
-            if (j < nrow) {
-                const float e = out[j] - tgt[r0 + j];
-                const float mk = mask[r0 + j];
-                d = 2.f * mk * e * inv_norm;
-                atomicAdd(&gsm[3 * WS_H + 1], mk * e * e);
-                atomicAdd(&gsm[3 * WS_H + 2], mk);
-                atomicAdd(&gsm[3 * WS_H], d);
+        float h2[4][2];
+        tile_forward(s, w, h2);
+        // delta3 = 2 mask (y - t) / norm; rows past the end have none
+        float d3 = 0.f;
+        if (tid < nrow) {
+            const float e = s.out[0][tid] + s.out[1][tid] + w.b3[0] - tgt[r0 + tid], mk = mask[r0 + tid];
+            d3 = 2.f * mk * e * inv_norm;
+            gl[0] += d3;
+            gl[1] += mk * e * e;
+            gl[2] += mk;
+        }
+        __syncthreads();
+        if (tid < WS_TILE) s.out[0][tid] = d3;
+        __syncthreads();
+        // delta2 = delta3 w3 relu'(h2)
+        {
+            const float4 d = *(const float4*)&s.out[0][row];
+            const float dr[4] = {d.x, d.y, d.z, d.w};
+            float d2[2][4];
+#pragma unroll
+            for (int r = 0; r < 4; r++) {
+                gw3[0] = fmaf(h2[r][0], dr[r], gw3[0]);
+                gw3[1] = fmaf(h2[r][1], dr[r], gw3[1]);
+                d2[0][r] = h2[r][0] > 0.f ? dr[r] * w3.x : 0.f;
+                d2[1][r] = h2[r][1] > 0.f ? dr[r] * w3.y : 0.f;
+                gb2[0] += d2[0][r];
+                gb2[1] += d2[1][r];
             }
-            out[j] = d;
+#pragma unroll
+            for (int c = 0; c < 2; c++)
+                *(float4*)&s.h2[unit + c][row] = make_float4(d2[c][0], d2[c][1], d2[c][2], d2[c][3]);
         }
         __syncthreads();
-        // w3, then delta2 = delta3 * w3 * relu'(h2) (in place of h2)
-        const float w3j = __bfloat162float(w.w3[j]);
-#pragma unroll 4
-        for (int r = 0; r < WS_TILE; r++) {
-            const float hv = h2[r * WS_H + j];
-            gw3 = fmaf(hv, out[r], gw3);
-            const float d2 = hv > 0.f ? out[r] * w3j : 0.f;
-            h2[r * WS_H + j] = d2;
-            gb2 += d2;
+        // delta1 = (delta2 W2^T) relu'(h1), and W2's gradient from the h1 it replaces
+        float d1[4][2] = {};
+        tile_product<WS_H>(s.h2, wt, row, unit, d1);
+#pragma unroll
+        for (int r = 0; r < WS_TILE; r += 4) {
+            float4 b[8];
+#pragma unroll
+            for (int q = 0; q < 8; q++) b[q] = *(const float4*)&s.h2[j2 + q][r];
+#pragma unroll
+            for (int p = 0; p < 8; p++) {
+                const float4 a = *(const float4*)&s.h1[k2 + p][r];
+#pragma unroll
+                for (int q = 0; q < 8; q++)
+                    g2[p][q] = fmaf(a.x, b[q].x, fmaf(a.y, b[q].y, fmaf(a.z, b[q].z, fmaf(a.w, b[q].w, g2[p][q]))));
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            const float4 h = *(const float4*)&s.h1[unit + c][row];
+            d1[0][c] = h.x > 0.f ? d1[0][c] : 0.f;
+            d1[1][c] = h.y > 0.f ? d1[1][c] : 0.f;
+            d1[2][c] = h.z > 0.f ? d1[2][c] : 0.f;
+            d1[3][c] = h.w > 0.f ? d1[3][c] : 0.f;
+            gb1[c] += (d1[0][c] + d1[1][c]) + (d1[2][c] + d1[3][c]);
         }
         __syncthreads();
-        // gW2[k][j] += sum_r h1[r][k] delta2[r][j]; delta1[r][j] = sum_t delta2[r][t] W2[j][t] relu'(h1[r][j])
-        for (int k = 0; k < WS_H; k++) {
-            float s = 0.f;
-#pragma unroll 4
-            for (int r = 0; r < WS_TILE; r++) s = fmaf(h1[r * WS_H + k], h2[r * WS_H + j], s);
-            gW2[k * WS_H + j] += s;
-        }
-        float d1[WS_TILE];
 #pragma unroll
-        for (int r = 0; r < WS_TILE; r++) d1[r] = 0.f;
-        for (int t = 0; t < WS_H; t++) {
-            const float wjt = __bfloat162float(w.W2[j * WS_H + t]);
-#pragma unroll
-            for (int r = 0; r < WS_TILE; r++) d1[r] = fmaf(h2[r * WS_H + t], wjt, d1[r]);
-        }
-        __syncthreads();  // h1 is overwritten by delta1 below
-#pragma unroll
-        for (int r = 0; r < WS_TILE; r++) {
-            const float v = h1[r * WS_H + j] > 0.f ? d1[r] : 0.f;
-            h1[r * WS_H + j] = v;
-            gb1 += v;
-        }
+        for (int c = 0; c < 2; c++)
+            *(float4*)&s.h1[unit + c][row] = make_float4(d1[0][c], d1[1][c], d1[2][c], d1[3][c]);
         __syncthreads();
-        // gW1[k][j] += sum_r x[r][k] delta1[r][j]
-        for (int k = 0; k < WS_IN; k++) {
-            float s = 0.f;
-#pragma unroll 4
-            for (int r = 0; r < WS_TILE; r++) s = fmaf(x[r * WS_IN + k], h1[r * WS_H + j], s);
-            gW1[k * WS_H + j] += s;
+#pragma unroll
+        for (int r = 0; r < WS_TILE; r += 4) {
+            float4 b[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) b[q] = *(const float4*)&s.h1[j1 + q][r];
+#pragma unroll
+            for (int p = 0; p < 9; p++) {
+                const float4 a = *(const float4*)&s.x[k1 + p][r];
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    g1[p][q] = fmaf(a.x, b[q].x, fmaf(a.y, b[q].y, fmaf(a.z, b[q].z, fmaf(a.w, b[q].w, g1[p][q]))));
+            }
         }
     }
-    gsm[j] = gb1;
-    gsm[WS_H + j] = gb2;
-    gsm[2 * WS_H + j] = gw3;
-    __syncthreads();
     // layout of a gradient row: W1, b1, W2, b2, w3, b3, then loss sum, mask sum
-    float* row = part + (int64_t)blockIdx.x * WS_PART;
-    for (int t = j; t < WS_IN * WS_H; t += WS_H) row[WS_OFF_W1 + t] = gW1[t];
-    for (int t = j; t < WS_H * WS_H; t += WS_H) row[WS_OFF_W2 + t] = gW2[t];
-    row[WS_OFF_B1 + j] = gsm[j];
-    row[WS_OFF_B2 + j] = gsm[WS_H + j];
-    row[WS_OFF_W3 + j] = gsm[2 * WS_H + j];
-    if (j == 0) {
-        row[WS_OFF_B3] = gsm[3 * WS_H];
-        row[WS_NPARAMS] = gsm[3 * WS_H + 1];
-        row[WS_NPARAMS + 1] = gsm[3 * WS_H + 2];
+    float* out = part + (int64_t)blockIdx.x * WS_PART;
+#pragma unroll
+    for (int p = 0; p < 9; p++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) out[WS_OFF_W1 + (k1 + p) * WS_H + j1 + q] = g1[p][q];
+#pragma unroll
+    for (int p = 0; p < 8; p++)
+#pragma unroll
+        for (int q = 0; q < 8; q++) out[WS_OFF_W2 + (k2 + p) * WS_H + j2 + q] = g2[p][q];
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        s.sums[tid >> 6][0][unit + c] = gb1[c];
+        s.sums[tid >> 6][1][unit + c] = gb2[c];
+        s.sums[tid >> 6][2][unit + c] = gw3[c];
+    }
+    if (tid < 32)
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+            for (int o = 16; o > 0; o >>= 1) gl[q] += __shfl_xor_sync(0xffffffffu, gl[q], o);
+            if (tid == 0) s.loss[q] = gl[q];
+        }
+    __syncthreads();
+    for (int t = tid; t < 3 * WS_H; t += WS_THREADS) {
+        const int q = t / WS_H, j = t - q * WS_H;
+        out[(q == 0 ? WS_OFF_B1 : q == 1 ? WS_OFF_B2 : WS_OFF_W3) + j] =
+            (s.sums[0][q][j] + s.sums[1][q][j]) + (s.sums[2][q][j] + s.sums[3][q][j]);
+    }
+    if (tid == 0) {
+        out[WS_OFF_B3] = s.loss[0];
+        out[WS_NPARAMS] = s.loss[1];
+        out[WS_NPARAMS + 1] = s.loss[2];
     }
 }
 
@@ -369,6 +438,7 @@ __global__ void k_reduce_parts(const float* __restrict__ part, int nb, float* __
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= WS_PART) return;
     float s = 0.f;
+#pragma unroll 16
     for (int b = 0; b < nb; b++) s += part[(int64_t)b * WS_PART + t];
     g[t] = s;
 }
@@ -432,9 +502,7 @@ static MlpW weights_of(Ctx* c) {
     return MlpW{wb + WS_OFF_W1, p + WS_OFF_B1, wb + WS_OFF_W2, p + WS_OFF_B2, wb + WS_OFF_W3, p + WS_OFF_B3};
 }
 
-static size_t backward_smem() {
-    return sizeof(float) * (WS_TILE * WS_IN + 2 * WS_TILE * WS_H + WS_TILE + WS_IN * WS_H + WS_H * WS_H + 3 * WS_H + 3);
-}
+static size_t backward_smem() { return sizeof(MlpTile) + sizeof(__nv_bfloat16) * WS_H * WS_H; }
 
 // Parameters: allocated and initialised once per context (hidden layers
 // He-uniform from a SplitMix64 stream of `seed`, output layer and biases 0).
@@ -494,7 +562,7 @@ pd_status mlp_forward(Ctx* c, const __nv_bfloat16* F, int64_t n, float* y, cudaS
     if (n <= 0) return PD_OK;
     const int64_t tiles = (n + WS_TILE - 1) / WS_TILE;
     const int grid = (int)std::min<int64_t>(tiles, 4 * std::max(c->sm_count, 1));
-    k_mlp_forward<<<grid, WS_H, 0, st>>>(weights_of(c), F, n, y); pd::count_launch();
+    k_mlp_forward<<<grid, WS_THREADS, 0, st>>>(weights_of(c), F, n, y); pd::count_launch();
     PD_TRY_CUDA(c, cudaGetLastError());
     return PD_OK;
 }
@@ -510,7 +578,7 @@ pd_status mlp_grad(Ctx* c, const __nv_bfloat16* F, const float* t, const float* 
     if (!part) return PD_ENOMEM;
     const size_t smem = backward_smem();
     PD_TRY_CUDA(c, cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_mlp_backward<<<nb, WS_H, smem, st>>>(weights_of(c), F, t, mask, n, inv_norm, part); pd::count_launch();
+    k_mlp_backward<<<nb, WS_THREADS, smem, st>>>(weights_of(c), F, t, mask, n, inv_norm, part); pd::count_launch();
     k_reduce_parts<<<grid_for(WS_PART, 256), 256, 0, st>>>(part, nb, g); pd::count_launch();
     PD_TRY_CUDA(c, cudaGetLastError());
     return PD_OK;
@@ -712,14 +780,26 @@ extern "C" pd_status pd_ws_set_params(pd_ctx* cx, const float* params) {
     return mlp_set(c, params, 0);
 }
 
-// Host feature rows -> bf16 device rows in B_WS_IN.
+__global__ void k_rows_to_bf16(const float4* __restrict__ x, int64_t n4, uint2* __restrict__ y) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n4) return;
+    const float4 v = x[i];
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    y[i] = make_uint2(*(const uint32_t*)&a, *(const uint32_t*)&b);
+}
+
+// Host feature rows -> bf16 device rows in B_WS_IN: copied as they are and
+// rounded on the device (2,048 rows: rounding on the host took longer than the
+// copy and the network together).
 static pd_status upload_rows(Ctx* c, const float* feats, int64_t n, __nv_bfloat16** out, cudaStream_t st) {
-    std::vector<__nv_bfloat16> hb((size_t)(n * WS_IN));
-    for (int64_t t = 0; t < n * WS_IN; t++) hb[(size_t)t] = __float2bfloat16(feats[t]);
+    static_assert(WS_IN % 4 == 0, "whole 16-byte steps");
+    float* raw = bufT<float>(c, B_WS_RAW, n * WS_IN);
     __nv_bfloat16* F = bufT<__nv_bfloat16>(c, B_WS_IN, std::max<int64_t>(n, 1) * WS_IN);
-    if (!F) return PD_ENOMEM;
-    PD_TRY_CUDA(c, cudaMemcpyAsync(F, hb.data(), sizeof(__nv_bfloat16) * n * WS_IN, cudaMemcpyHostToDevice, st));
-    PD_TRY_CUDA(c, cudaStreamSynchronize(st));  // hb is freed on return
+    if (!raw || !F) return PD_ENOMEM;
+    PD_TRY_CUDA(c, cudaMemcpyAsync(raw, feats, sizeof(float) * n * WS_IN, cudaMemcpyHostToDevice, st));
+    const int64_t n4 = n * WS_IN / 4;
+    k_rows_to_bf16<<<grid_for(n4, 256), 256, 0, st>>>((const float4*)raw, n4, (uint2*)F); pd::count_launch();
+    PD_TRY_CUDA(c, cudaGetLastError());
     *out = F;
     return PD_OK;
 }
@@ -762,10 +842,11 @@ extern "C" pd_status pd_ws_grad(pd_ctx* cx, const float* feats, const float* tar
     PD_TRY_CUDA(c, cudaMemcpyAsync(dt, target, sizeof(float) * n, cudaMemcpyHostToDevice, st));
     PD_TRY_CUDA(c, cudaMemcpyAsync(dm, mask, sizeof(float) * n, cudaMemcpyHostToDevice, st));
     PD_TRY(mlp_grad(c, F, dt, dm, n, 1.f / (float)n, g, st));
-    std::vector<float> hg(WS_PART);
-    PD_TRY_CUDA(c, cudaMemcpyAsync(hg.data(), g, sizeof(float) * WS_PART, cudaMemcpyDeviceToHost, st));
+    const std::unique_ptr<float[]> hg(new (std::nothrow) float[WS_PART]);
+    if (!hg) return fail(c, PD_ENOMEM, "no host memory for the gradient");
+    PD_TRY_CUDA(c, cudaMemcpyAsync(hg.get(), g, sizeof(float) * WS_PART, cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
-    std::memcpy(grad, hg.data(), sizeof(float) * WS_NPARAMS);
+    std::memcpy(grad, hg.get(), sizeof(float) * WS_NPARAMS);
     if (loss) *loss = hg[WS_NPARAMS] / (float)n;
     return PD_OK;
 }

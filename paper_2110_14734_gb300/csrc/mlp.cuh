@@ -14,7 +14,7 @@ namespace pd {
 
 constexpr int WS_IN = 72;    // features per node
 constexpr int WS_H = 128;    // hidden width (both layers)
-constexpr int WS_TILE = 32;  // nodes per block step
+constexpr int WS_TILE = 16;  // rows per block step
 constexpr int WS_GRID = 64;  // density grid per axis
 // parameter layout: W1 [WS_IN][WS_H], b1, W2 [WS_H][WS_H], b2, w3 [WS_H], b3
 constexpr int WS_OFF_W1 = 0;
