@@ -1285,16 +1285,18 @@ __global__ void k_transport_arcs(const int32_t* __restrict__ S, const int32_t* _
 
 // One warp per row of the CSR network.
 __global__ void k_arc_pack(const int64_t* __restrict__ rp, const int32_t* __restrict__ hd,
-                           const int64_t* __restrict__ cost, int64_t n, int64_t m, uint32_t* __restrict__ th,
-                           int32_t* __restrict__ c32, unsigned long long* __restrict__ bad,
+                           const int64_t* __restrict__ cost, int64_t n, int64_t m, int64_t stride,
+                           uint32_t* __restrict__ th, int32_t* __restrict__ c32, unsigned long long* __restrict__ bad,
                            unsigned long long* __restrict__ cmax) {
+    const int64_t chunks = ns_chunks(m);
+    auto place = [&](int64_t a) { return a / NS_CHUNK * stride % chunks * NS_CHUNK + a % NS_CHUNK; };
     const int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (u > n) return;  // whole warps leave together
     if (u == n) {       // the padding
-        if (lane < 3 && m + lane < ((m + 3) & ~(int64_t)3)) {
-            th[m + lane] = 0;
-            c32[m + lane] = NS_PAD_COST;
+        for (int64_t a = m + lane; a < chunks * NS_CHUNK; a += 32) {
+            th[place(a)] = 0;
+            c32[place(a)] = NS_PAD_COST;
         }
         return;
     }
@@ -1305,8 +1307,9 @@ __global__ void k_arc_pack(const int64_t* __restrict__ rp, const int32_t* __rest
         const bool b = c < 0 || c >= (int64_t(1) << 31);
         wrong += b;
         big = max(big, b ? 0u : (uint32_t)c);
-        th[a] = (uint32_t)u << 16 | (uint32_t)hd[a];
-        c32[a] = (int32_t)c;
+        const int64_t p = place(a);
+        th[p] = (uint32_t)u << 16 | (uint32_t)hd[a];
+        c32[p] = (int32_t)c;
     }
     big = __reduce_max_sync(0xffffffffu, big);
     wrong = __reduce_add_sync(0xffffffffu, wrong);
@@ -1326,15 +1329,17 @@ __global__ void k_tree_flow(const NSInst* __restrict__ I, unsigned long long* __
 pd_status ns_solve_network(Ctx* c, const pd_network& net, const pd_opts& o, SolveStats* out, cudaStream_t st) {
     int64_t n = net.n_nodes, m = net.n_arcs;
     if (n >= (int64_t(1) << 31) - 2) return fail(c, PD_ECAPACITY, "too many nodes");
-    const bool packed = n + 1 < 65535;  // 16-bit node ids, as simplex32.cu takes them
-    int32_t* tail = bufT<int32_t>(c, B_S_TAIL, m + 3);
-    int32_t* c32 = bufT<int32_t>(c, B_NS_COST, m + 3);
+    // 16-bit node ids, as simplex32.cu takes them
+    const bool packed = n + 1 < 65535 && m < (int64_t(1) << 31) - (int64_t(1) << 18);
+    int32_t* tail = bufT<int32_t>(c, B_S_TAIL, ns_chunks(m) * NS_CHUNK);
+    int32_t* c32 = bufT<int32_t>(c, B_NS_COST, ns_chunks(m) * NS_CHUNK);
     unsigned long long* sm = bufT<unsigned long long>(c, B_SMALL, 64);
     if (!tail || !c32 || !sm) return PD_ENOMEM;
     PD_TRY_CUDA(c, cudaMemsetAsync(sm, 0, 8 * sizeof(unsigned long long), st));
     if (m > 0 && packed) {
-        k_arc_pack<<<grid_for(32 * (n + 1), 256), 256, 0, st>>>(net.row_ptr, net.head, net.cost, n, m, (uint32_t*)tail,
-                                                                c32, sm, sm + 1); pd::count_launch();
+        k_arc_pack<<<grid_for(32 * (n + 1), 256), 256, 0, st>>>(net.row_ptr, net.head, net.cost, n, m,
+                                                                ns_chunk_stride(m), (uint32_t*)tail, c32, sm,
+                                                                sm + 1); pd::count_launch();
     } else if (m > 0) {
         k_arc_tails<<<grid_for(m, 256), 256, 0, st>>>(net.row_ptr, n, m, tail); pd::count_launch();
         k_i64_to_i32_cost<<<grid_for(m, 256), 256, 0, st>>>(net.cost, m, c32, sm); pd::count_launch();
@@ -1347,7 +1352,7 @@ pd_status ns_solve_network(Ctx* c, const pd_network& net, const pd_opts& o, Solv
     int64_t cmax = c->h_small[1];
     NSInst r;
     NSArcs arcs;
-    arcs.m = m;
+    arcs.m = packed ? ns_chunks(m) * NS_CHUNK : m;
     arcs.th = packed ? (const uint32_t*)tail : nullptr;
     arcs.tail = tail;
     arcs.head = net.head;

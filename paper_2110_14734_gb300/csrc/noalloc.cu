@@ -22,8 +22,9 @@ constexpr int64_t NA_ARCS = PD_NOALLOC_MAX_ARCS;
 
 constexpr size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t OFF_TAIL = 0;
-constexpr size_t OFF_COST = OFF_TAIL + al(4 * (NA_ARCS + 3));
-constexpr size_t OFF_PI = OFF_COST + al(4 * (NA_ARCS + 3));
+constexpr size_t OFF_COST = OFF_TAIL + al(4 * NA_ARCS);
+constexpr size_t OFF_PI = OFF_COST + al(4 * NA_ARCS);
+static_assert(NA_ARCS % NS_CHUNK == 0, "whole chunks of arcs");
 constexpr size_t OFF_PRED = OFF_PI + al(8 * NA_NODES);
 constexpr size_t OFF_PARENT = OFF_PRED + al(4 * NA_NODES);
 constexpr size_t OFF_FLOW = OFF_PARENT + al(4 * NA_NODES);
@@ -108,7 +109,8 @@ extern "C" pd_status pd_mcf_solve_noalloc(const pd_network* net, int64_t* opt_ou
     NA_TRY(cudaMemsetAsync(flags, 0, 64, st));
     k_check_network<<<grid_for(n, 256), 256, 0, st>>>(net->row_ptr, net->head, n, m, flags); pd::count_launch();
     if (m > 0) {
-        k_arc_pack<<<grid_for(32 * (n + 1), 256), 256, 0, st>>>(net->row_ptr, net->head, net->cost, n, m, th, c32,
+        k_arc_pack<<<grid_for(32 * (n + 1), 256), 256, 0, st>>>(net->row_ptr, net->head, net->cost, n, m,
+                                                                ns_chunk_stride(m), th, c32,
                                                                 flags + 1, flags + 2); pd::count_launch();
     }
     k_abs_sum<<<grid_for(n, 256), 256, 0, st>>>(net->supply, n, flags + 3); pd::count_launch();
@@ -125,7 +127,7 @@ extern "C" pd_status pd_mcf_solve_noalloc(const pd_network* net, int64_t* opt_ou
 
     NSInst h{};
     h.n = (int32_t)n;
-    h.m = m;
+    h.m = ns_chunks(m) * NS_CHUNK;
     h.mst = 0;
     h.nS = 0;
     h.nT = 1;
