@@ -961,16 +961,34 @@ static pd_status ns_plan(Ctx* c, const NSInst* h, int count, int32_t* order, NSL
     PD_TRY_CUDA(c, ns_kernel_setup());
     PD_TRY_CUDA(c, s32_kernel_setup());
     *L = NSLaunch{};
+    // Two CTAs of half the threads share an SM when more of the matrices that fit
+    // are there than SMs (276 pairs of 2,000 uniform points 57 -> 38 ms, 153 of them
+    // 44 -> 34, 304 of 600 points 17.2 -> 9.7), or when all are small: a short order
+    // keeps 512 threads idle (one pair of 369 nodes 2.70 -> 2.12 ms, 712 nodes 4.83
+    // -> 4.11, 1,177 nodes 8.19 -> 8.04).  A larger one alone is faster with 512
+    // (2,843 nodes: 25.7 ms, 27.9 with 256).
+    int matrices = 0, halves = 0, small = 0;
+    for (int q = 0; q < count; q++) {
+        if (s32_class(h[q]) != S32_MATRIX) continue;
+        matrices++;
+        halves += h[q].n < S32_HALF_NODES;
+        small += h[q].n < S32_SMALL_NODES;
+    }
+    const bool half = halves > c->sm_count || small == matrices;
+    auto cls = [&](const NSInst& x) {
+        const int k = s32_class(x);
+        return half && k == S32_MATRIX && x.n < S32_HALF_NODES ? S32_HALF : k;
+    };
     for (int q = 0; q < count; q++) {
         order[q] = q;
-        const int k = s32_class(h[q]);
+        const int k = cls(h[q]);
         if (k < 0) L->own64++;
         else L->num[k]++;
         if (h[q].smem_nodes) L->smem64 = std::max(L->smem64, ns_smem_bytes((int64_t)h[q].n + 1, h[q].smem_nodes));
     }
     for (int k = 1; k < S32_CLASSES; k++) L->first[k] = L->first[k - 1] + L->num[k - 1];
     std::stable_sort(order, order + count, [&](int32_t x, int32_t y) {
-        const unsigned cx = (unsigned)s32_class(h[x]), cy = (unsigned)s32_class(h[y]);  // -1 sorts last
+        const unsigned cx = (unsigned)cls(h[x]), cy = (unsigned)cls(h[y]);  // -1 sorts last
         if (cx != cy) return cx < cy;
         return h[x].n != h[y].n ? h[x].n > h[y].n : h[x].m > h[y].m;
     });
@@ -1003,7 +1021,7 @@ pd_status ns_run(Ctx* c, const NSInst* h, int count, NSInst* d, NSInst* r, cudaS
         if (pass == 0) {
             for (int k = 0; k < S32_CLASSES; k++)
                 if (L.num[k] > 0) {
-                    s32_launch(k, std::min(L.num[k], std::max(c->sm_count, 1)), d, dord + L.first[k], L.num[k],
+                    s32_launch(k, s32_grid(k, L.num[k], c->sm_count), d, dord + L.first[k], L.num[k],
                                dord + count + k, st);
                     pd::count_launch();
                 }
@@ -1104,8 +1122,8 @@ pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, const CertJob* jobs, N
         cudaMemsetAsync(dcert, 0, 2 * sizeof(unsigned long long) * count, gs);
         for (int k = 0; k < S32_CLASSES; k++)
             if (NL.num[k] > 0)
-                s32_launch(k, std::min(NL.num[k], std::max(c->sm_count, 1)), d, dord + NL.first[k], NL.num[k],
-                           dord + count + k, gs);
+                s32_launch(k, s32_grid(k, NL.num[k], c->sm_count), d, dord + NL.first[k], NL.num[k], dord + count + k,
+                           gs);
         k_netsimplex<<<NL.grid64, NS_THREADS, NL.smem64, gs>>>(d, dord, count, dord + count + S32_CLASSES);
         k_certify_batch<<<dim3(WAVE_CERT_BLOCKS, count), 256, 0, gs>>>(djobs, dcert);
         cudaMemcpyAsync(p_out, d, sizeof(NSInst) * count, cudaMemcpyDeviceToHost, gs);

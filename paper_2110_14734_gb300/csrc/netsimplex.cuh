@@ -66,10 +66,18 @@ constexpr int32_t S32_REDO = 5;  // status: k_netsimplex has to solve the instan
 
 // The simplex on 32-bit potentials (simplex32.cu), for records with lay32 > 0:
 // a kernel per class (layout and arc form), persistent like k_netsimplex, one
-// CTA per SM.
-constexpr int S32_CLASSES = 6;
+// CTA per SM, two of S32_HALF (which ns_plan puts matrices of layout 1 into).
+constexpr int S32_CLASSES = 7;
+constexpr int S32_MATRIX = 1;             // matrices of layout 1
+constexpr int S32_HALF = 6;               // matrices on half an SM
+constexpr int32_t S32_HALF_NODES = 3712;  // nodes with the root that half an SM holds
+constexpr int32_t S32_SMALL_NODES = 1280; // ... up to which half the threads are the better choice anyway
 int s32_class(const NSInst& h);  // -1: not a 32-bit instance
 int s32_layout(int64_t N1);      // the smallest layout that holds N1 nodes (0: none)
+inline int s32_grid(int cls, int count, int sm_count) {
+    const int most = (cls == S32_HALF ? 2 : 1) * (sm_count > 1 ? sm_count : 1);
+    return count < most ? count : most;
+}
 void s32_launch(int cls, int grid, NSInst* insts, const int32_t* order, int32_t count, int32_t* next,
                 cudaStream_t st);
 cudaError_t s32_kernel_setup();  // as ns_kernel_setup

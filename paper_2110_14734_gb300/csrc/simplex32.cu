@@ -53,8 +53,7 @@ namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int S32_THREADS = 512;
-constexpr int S32_WARPS = S32_THREADS / 32;
-constexpr int S32_PRICERS = S32_THREADS - 32; // warps 1 .. price, warp 0 pivots
+constexpr int S32_HALF_THREADS = 256;         // layout 4
 constexpr int S32_HITS = 1024;                // path nodes listed in shared memory
 constexpr int S32_PATH = 1024;                // cut nodes listed in shared memory
 constexpr int S32_MOVE = 16;                  // moved positions held in registers, per thread
@@ -82,20 +81,28 @@ PD_D Shared& shared() { return *(Shared*)s32_dyn; }  // at the start of the dyna
 
 // Dynamic shared memory of a layout: 1 holds every node array (20 B a node), 2
 // all but flow and pred (12 B), 3 only the preorder, positions and parents (8 B).
+// 4 is 1 for half an SM: a smaller stage and half the threads, so that two
+// instances share an SM and one's instructions fill the other's waits (a lone
+// CTA issues in 31 % of the cycles).
 // The arrays lie at fixed offsets for the layout's capacity, so that no
 // register holds them.
 // Beside them lies the pricing block's stage.
-PD_HD constexpr int32_t s32_capacity(int layout) { return layout == 1 ? 7824 : layout == 2 ? 13040 : 23664; }
+PD_HD constexpr int32_t s32_capacity(int layout) {
+    return layout == 1 ? 7824 : layout == 2 ? 13040 : layout == 3 ? 23664 : S32_HALF_NODES;
+}
 template <int LAY>
 struct Layout {
     static constexpr uint32_t N = s32_capacity(LAY), W2 = 2 * N, W4 = 4 * N;
-    static constexpr uint32_t STAGE = LAY == 3 ? 32768 : 65536;  // bytes of a pricing block
+    static constexpr bool FLOWS = LAY != 2 && LAY != 3, PIS = LAY != 3;  // what shared memory holds
+    static constexpr int THREADS = LAY == 4 ? S32_HALF_THREADS : S32_THREADS, WARPS = THREADS / 32;
+    static constexpr int PRICERS = THREADS - 32;  // warps 1 .. price, warp 0 pivots
+    static constexpr uint32_t STAGE = LAY >= 3 ? 32768 : 65536;  // bytes of a pricing block
     static constexpr uint32_t stage = (sizeof(Shared) + 15) & ~15u, ord = stage + STAGE, pos = ord + W4, par = pos + W2;
-    static constexpr uint32_t fu = par + W2, pred = fu + (LAY == 1 ? W4 : 0);
+    static constexpr uint32_t fu = par + W2, pred = fu + (FLOWS ? W4 : 0);
     // the sinks' potentials pi[nS ..] start on a 16-byte boundary (up to three
     // words of shift), and padding columns are read past the last node
-    static constexpr uint32_t pi = pred + (LAY == 1 ? W4 : 0), total = pi + (LAY <= 2 ? W4 + 64 : 0);
-    static_assert(N % 16 == 0 && total + 16 <= 227 * 1024, "the layout does not fit an SM");
+    static constexpr uint32_t pi = pred + (FLOWS ? W4 : 0), total = pi + (PIS ? W4 + 64 : 0);
+    static_assert(N % 16 == 0 && total + 16 <= (LAY == 4 ? 113 : 227) * 1024, "the layout does not fit an SM");
 };
 
 template <int LAY>
@@ -106,25 +113,25 @@ struct Nodes {
     uint32_t* gfu;
     int32_t* gpred;
     PD_D int32_t& pi(int32_t v) const {
-        if constexpr (LAY <= 2) return *(int32_t*)(s32_dyn + L::pi + shift + 4 * v);
+        if constexpr (L::PIS) return *(int32_t*)(s32_dyn + L::pi + shift + 4 * v);
         else return gpi[v];
     }
     // the same by byte offset: pi(v) is at pi0() + 4 v
-    PD_D uint32_t pi0() const { return LAY <= 2 ? L::pi + shift : 0u; }
+    PD_D uint32_t pi0() const { return L::PIS ? L::pi + shift : 0u; }
     PD_D int32_t pi_at(uint32_t off) const {
-        if constexpr (LAY <= 2) return *(const int32_t*)(s32_dyn + off);
+        if constexpr (L::PIS) return *(const int32_t*)(s32_dyn + off);
         else return *(const int32_t*)((const char*)gpi + off);
     }
     PD_D int4 pi4_at(uint32_t off) const {
-        if constexpr (LAY <= 2) return *(const int4*)(s32_dyn + off);
+        if constexpr (L::PIS) return *(const int4*)(s32_dyn + off);
         else return *(const int4*)((const char*)gpi + off);
     }
     PD_D uint32_t& fu(int32_t v) const {
-        if constexpr (LAY == 1) return *(uint32_t*)(s32_dyn + L::fu + 4 * v);
+        if constexpr (L::FLOWS) return *(uint32_t*)(s32_dyn + L::fu + 4 * v);
         else return gfu[v];
     }
     PD_D int32_t& pred(int32_t v) const {
-        if constexpr (LAY == 1) return *(int32_t*)(s32_dyn + L::pred + 4 * v);
+        if constexpr (L::FLOWS) return *(int32_t*)(s32_dyn + L::pred + 4 * v);
         else return gpred[v];
     }
     // position x: node | end of its subtree << 16
@@ -204,13 +211,13 @@ PD_D void shift_and_insert(const Nodes<LAY>& T, int32_t a0, int32_t len, int32_t
     uint32_t w[NR], wm = 0;
 #pragma unroll
     for (int q = 0; q < NR; q++)
-        if (tid + q * S32_THREADS < len) w[q] = T.ord(a0 + tid + q * S32_THREADS + shift) + turn;
+        if (tid + q * Layout<LAY>::THREADS < len) w[q] = T.ord(a0 + tid + q * Layout<LAY>::THREADS + shift) + turn;
     if (tid < S) wm = moved<LAY>(T, shared().cut, k, S, ins, tid, dpi);
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < NR; q++)
-        if (tid + q * S32_THREADS < len) {
-            const int32_t x = a0 + tid + q * S32_THREADS;
+        if (tid + q * Layout<LAY>::THREADS < len) {
+            const int32_t x = a0 + tid + q * Layout<LAY>::THREADS;
             T.ord(x) = w[q];
             T.pos((int32_t)(w[q] & 0xffffu)) = (uint16_t)x;
         }
@@ -223,8 +230,9 @@ PD_D void shift_and_insert(const Nodes<LAY>& T, int32_t a0, int32_t len, int32_t
 // A wide move (more of the cut subtree than a position per thread) is gathered
 // into the stage, or global scratch where that is too small, before it is
 // written back.
+template <int LAY>
 PD_D bool wide_move(const Shared& s) {
-    return s.S > S32_THREADS || s.hi - s.lo - s.S > S32_MOVE * S32_THREADS || s.k >= S32_PATH;
+    return s.S > Layout<LAY>::THREADS || s.hi - s.lo - s.S > S32_MOVE * Layout<LAY>::THREADS || s.k >= S32_PATH;
 }
 
 // Moves the cut subtree (parameters in shared memory); ends without a barrier
@@ -237,17 +245,17 @@ PD_D void rehang(const Nodes<LAY>& T, bool wide, const uint32_t* gcut, uint32_t*
     // the shifted nodes fill [a0, a0 + len), beside the re-rooted segment
     const int32_t a0 = shift < 0 ? ins + S : lo, len = hi - lo - S;
     if (!wide) {
-        if (len <= 2 * S32_THREADS) shift_and_insert<LAY, 2>(T, a0, len, shift, k, S, ins, dpi);
-        else if (len <= 5 * S32_THREADS) shift_and_insert<LAY, 5>(T, a0, len, shift, k, S, ins, dpi);
+        if (len <= 2 * Layout<LAY>::THREADS) shift_and_insert<LAY, 2>(T, a0, len, shift, k, S, ins, dpi);
+        else if (len <= 5 * Layout<LAY>::THREADS) shift_and_insert<LAY, 5>(T, a0, len, shift, k, S, ins, dpi);
         else shift_and_insert<LAY, S32_MOVE>(T, a0, len, shift, k, S, ins, dpi);
     } else {
         const uint32_t turn = (uint32_t)-shift << 16;
         if (hi - lo <= (int32_t)(Layout<LAY>::STAGE / 4)) tmp = (uint32_t*)(s32_dyn + Layout<LAY>::stage) - lo;
-        for (int32_t x = a0 + tid; x < a0 + len; x += S32_THREADS) tmp[x] = T.ord(x + shift) + turn;
-        for (int32_t o = tid; o < S; o += S32_THREADS)
+        for (int32_t x = a0 + tid; x < a0 + len; x += Layout<LAY>::THREADS) tmp[x] = T.ord(x + shift) + turn;
+        for (int32_t o = tid; o < S; o += Layout<LAY>::THREADS)
             tmp[ins + o] = moved<LAY>(T, k < S32_PATH ? s.cut : gcut, k, S, ins, o, dpi);
         __syncthreads();
-        for (int32_t x = lo + tid; x < hi; x += S32_THREADS) {
+        for (int32_t x = lo + tid; x < hi; x += Layout<LAY>::THREADS) {
             const uint32_t w = tmp[x];
             T.ord(x) = w;
             T.pos((int32_t)(w & 0xffffu)) = (uint16_t)x;
@@ -471,7 +479,7 @@ PD_D void s32_body(NSInst& G) {
     T.gfu = (uint32_t*)I.flow;
     T.gpred = I.pred;
     constexpr int STEP = IMPL ? 8 : 4;     // arcs of a thread's step
-    constexpr int MAXIT = (s32_capacity(LAY) + 2047) / 2048;  // scan rounds of 2048 positions
+    constexpr int MAXIT = (s32_capacity(LAY) - 1) / (128 * Layout<LAY>::WARPS) + 1;  // scan rounds
     static_assert(4 * MAXIT <= 64, "a thread's scan mask");
     constexpr int32_t STAGED = (int32_t)(Layout<LAY>::STAGE / 32);  // steps a stage holds (8 costs, or 4 with their ends)
 
@@ -488,13 +496,13 @@ PD_D void s32_body(NSInst& G) {
     }
     if (I.init_tree) {
         // the 64-bit potentials share the memory of the 32-bit ones of layout 3: all are read first
-        for (int32_t v = tid; v < N1; v += S32_THREADS) {
+        for (int32_t v = tid; v < N1; v += Layout<LAY>::THREADS) {
             const int64_t p = G.pi[v];
             worst = max(worst, p > S32_LIMIT || p < -S32_LIMIT ? S32_LIMIT + 1 : (int32_t)(p < 0 ? -p : p));
             I.tmp[v] = (int32_t)p;
         }
         __syncthreads();
-        for (int32_t v = tid; v < N1; v += S32_THREADS) {
+        for (int32_t v = tid; v < N1; v += Layout<LAY>::THREADS) {
             const uint32_t f = (uint32_t)G.flow[v] | (G.up[v] ? 0x80000000u : 0u);
             const int32_t x = G.pos[v];
             T.pi(v) = I.tmp[v];
@@ -505,7 +513,7 @@ PD_D void s32_body(NSInst& G) {
             T.ord(x) = (uint32_t)v | (uint32_t)(x + G.size[v]) << 16;
         }
     } else {
-        for (int32_t v = tid; v < n; v += S32_THREADS) {
+        for (int32_t v = tid; v < n; v += Layout<LAY>::THREADS) {
             const int64_t b = I.supply[v];
             const int32_t ca = I.art ? big + (int32_t)I.art[v] : big;
             T.pi(v) = b >= 0 ? ca : -ca;
@@ -541,13 +549,13 @@ PD_D void s32_body(NSInst& G) {
     // are blocks of their own, read in place.
     const int32_t QI = IMPL ? (int32_t)(I.mst / STEP) : (int32_t)((I.m + 3) >> 2);  // staged steps
     const int32_t Q = IMPL ? QI + (int32_t)((I.m - I.mst + 3) >> 2) : QI;
-    const int32_t B = S32_PRICERS * max(1, (int32_t)min((I.block + STEP * S32_PRICERS / 2) / (STEP * S32_PRICERS),
-                                                        (int64_t)(STAGED / S32_PRICERS)));
+    const int32_t B = Layout<LAY>::PRICERS * max(1, (int32_t)min((I.block + STEP * Layout<LAY>::PRICERS / 2) / (STEP * Layout<LAY>::PRICERS),
+                                                        (int64_t)(STAGED / Layout<LAY>::PRICERS)));
     const int pt = tid - 32;  // this pricing thread
     const int32_t nS = (int32_t)I.nS, ldq = IMPL ? (int32_t)(I.ld / STEP) : 1;
     // row and sinks' potentials of a step, as byte offsets
     const uint32_t pb = T.pi0(), row_end = pb + 4u * (uint32_t)nS + 32u * (uint32_t)ldq;
-    const uint32_t step_i = 4u * (uint32_t)(S32_PRICERS / ldq), step_j = 32u * (uint32_t)(S32_PRICERS % ldq);
+    const uint32_t step_i = 4u * (uint32_t)(Layout<LAY>::PRICERS / ldq), step_j = 32u * (uint32_t)(Layout<LAY>::PRICERS % ldq);
     const uint32_t oi_0 = pb + 4u * (uint32_t)(max(pt, 0) / ldq);
     const uint32_t oj_0 = pb + 4u * (uint32_t)nS + 32u * (uint32_t)(max(pt, 0) % ldq);
     uint32_t oi = oi_0, oj = oj_0;  // of step next + pt
@@ -615,7 +623,7 @@ PD_D void s32_body(NSInst& G) {
                     const unsigned char* at = stage + 32 * pt + h;
                     const unsigned char* const end = stage + 32 * steps;
 #pragma unroll 1
-                    for (; at < end; at += 32 * S32_PRICERS) {
+                    for (; at < end; at += 32 * Layout<LAY>::PRICERS) {
                         const int4 c0 = *(const int4*)at, c1 = *(const int4*)(at + 16 - 2 * (int)h);
                         const int4 p0 = T.pi4_at(oj + h), p1 = T.pi4_at(oj + 16u - h);
                         const int32_t r0 = c0.x + p0.x, r1 = c0.y + p0.y, r2 = c0.z + p0.z, r3 = c0.w + p0.w,
@@ -637,12 +645,12 @@ PD_D void s32_body(NSInst& G) {
                     }
                 } else {
 #pragma unroll 1
-                    for (int32_t a = pt; a < steps; a += S32_PRICERS)
+                    for (int32_t a = pt; a < steps; a += Layout<LAY>::PRICERS)
                         four(qa + a, *(const int4*)(stage + 16 * a), *(const int4*)(stage + Layout<LAY>::STAGE / 2 + 16 * a));
                 }
             } else {  // (matrix instances)
 #pragma unroll 1
-                for (int32_t a = qa - QI + pt; a < qe - QI; a += S32_PRICERS)
+                for (int32_t a = qa - QI + pt; a < qe - QI; a += Layout<LAY>::PRICERS)
                     four(a, __ldcg((const int4*)I.cost + a), __ldcg((const int4*)I.th + a));
             }
             cost = best + T.pi_at(bi) - T.pi_at(bj);
@@ -674,8 +682,8 @@ PD_D void s32_body(NSInst& G) {
         if (!IMPL && wmin < 0 && cand == wends) s.arc[buf][wid] = arc;
         __syncthreads();
         if (tid == 0 && !stale && Q > 0) fetch();
-        const int32_t k2 = s.key[buf][lane & (S32_WARPS - 1)];
-        const uint32_t e2 = s.ends[buf][lane & (S32_WARPS - 1)];
+        const int32_t k2 = s.key[buf][lane & (Layout<LAY>::WARPS - 1)];
+        const uint32_t e2 = s.ends[buf][lane & (Layout<LAY>::WARPS - 1)];
         const int32_t rc = __reduce_min_sync(FULL, k2);
         if (rc >= 0) {
             buf ^= 1;
@@ -702,7 +710,7 @@ PD_D void s32_body(NSInst& G) {
             if (tid == 0) s.maxpi = 0;
             __syncthreads();
             int32_t w = 0;
-            for (int32_t v = tid; v < N1; v += S32_THREADS) w = max(w, abs(T.pi(v)));
+            for (int32_t v = tid; v < N1; v += Layout<LAY>::THREADS) w = max(w, abs(T.pi(v)));
             w = __reduce_max_sync(FULL, w);
             if (lane == 0) atomicMax(&s.maxpi, w);
             __syncthreads();
@@ -727,8 +735,8 @@ PD_D void s32_body(NSInst& G) {
             Mask m = 0;
             int32_t x = 128 * wid + lane;
 #pragma unroll
-            for (int it = 0; it < MAXIT; it++, x += 128 * S32_WARPS) {
-                const int32_t xb = 128 * wid + it * 128 * S32_WARPS;
+            for (int it = 0; it < MAXIT; it++, x += 128 * Layout<LAY>::WARPS) {
+                const int32_t xb = 128 * wid + it * 128 * Layout<LAY>::WARPS;
                 if (xb > ph) break;
                 uint32_t w[4];
 #pragma unroll
@@ -749,7 +757,7 @@ PD_D void s32_body(NSInst& G) {
                 int32_t at = atomicAdd(&s.hits, __popcll(m));
                 for (; m; m &= m - 1, at++) {
                     const int b = __ffsll((long long)m) - 1;
-                    const int32_t y = 128 * (wid + S32_WARPS * (b >> 2)) + 32 * (b & 3) + lane;
+                    const int32_t y = 128 * (wid + Layout<LAY>::WARPS * (b >> 2)) + 32 * (b & 3) + lane;
                     if (at < S32_HITS) s.list[at] = (uint16_t)y;
                     else I.path[at] = y;
                 }
@@ -779,7 +787,7 @@ PD_D void s32_body(NSInst& G) {
             if (p >= I.max_pivots || ((p & 127) == 0 && s32_now() - s.t0 > I.time_limit_ns)) s.late = 1;
         }
         __syncthreads();
-        const bool wide = wide_move(s);
+        const bool wide = wide_move<LAY>(s);
         if (tid == 0) {
             if (!wide) fetch();
             s.hits = 0;
@@ -810,10 +818,10 @@ PD_D void s32_body(NSInst& G) {
         s.obj = 0;
         s.art = 0;
     }
-    for (int32_t v = tid; v < N1; v += S32_THREADS) I.tmp[v] = T.pi(v);
+    for (int32_t v = tid; v < N1; v += Layout<LAY>::THREADS) I.tmp[v] = T.pi(v);
     __syncthreads();
     unsigned long long obj = 0, art = 0;
-    for (int32_t v = tid; v < N1; v += S32_THREADS) {
+    for (int32_t v = tid; v < N1; v += Layout<LAY>::THREADS) {
         const uint32_t w = T.fu(v);
         const int32_t a = T.pred(v), f = (int32_t)(w & 0x7fffffffu);
         if (v < n) {
@@ -844,7 +852,7 @@ PD_D void s32_body(NSInst& G) {
 // Persistent over `count` instances of one layout and arc form (a kernel of its
 // own per variant: several bodies in one kernel spill).
 template <int LAY, bool IMPL>
-__global__ void __launch_bounds__(S32_THREADS, 1) k_simplex32(NSInst* insts, const int32_t* __restrict__ order,
+__global__ void __launch_bounds__(Layout<LAY>::THREADS, LAY == 4 ? 2 : 1) k_simplex32(NSInst* insts, const int32_t* __restrict__ order,
                                                              int32_t count, int32_t* __restrict__ next) {
     __shared__ int32_t s_k;
     for (;;) {
@@ -861,12 +869,13 @@ __global__ void __launch_bounds__(S32_THREADS, 1) k_simplex32(NSInst* insts, con
 }
 
 size_t smem_bytes(int layout) {
-    return layout == 1 ? Layout<1>::total : layout == 2 ? Layout<2>::total : layout == 3 ? Layout<3>::total : 0;
+    return layout == 1 ? Layout<1>::total : layout == 2 ? Layout<2>::total : layout == 3 ? Layout<3>::total : Layout<4>::total;
 }
 
 using Kernel = void (*)(NSInst*, const int32_t*, int32_t, int32_t*);
 const Kernel kernels[S32_CLASSES] = {k_simplex32<1, false>, k_simplex32<1, true>, k_simplex32<2, false>,
-                                     k_simplex32<2, true>,  k_simplex32<3, false>, k_simplex32<3, true>};
+                                     k_simplex32<2, true>,  k_simplex32<3, false>, k_simplex32<3, true>,
+                                     k_simplex32<4, true>};
 
 }  // namespace
 
@@ -874,7 +883,7 @@ int s32_class(const NSInst& h) { return h.lay32 ? 2 * (h.lay32 - 1) + (h.mst > 0
 
 void s32_launch(int cls, int grid, NSInst* insts, const int32_t* order, int32_t count, int32_t* next,
                 cudaStream_t st) {
-    kernels[cls]<<<grid, S32_THREADS, smem_bytes(cls / 2 + 1), st>>>(insts, order, count, next);
+    kernels[cls]<<<grid, cls == S32_HALF ? S32_HALF_THREADS : S32_THREADS, smem_bytes(cls / 2 + 1), st>>>(insts, order, count, next);
 }
 
 int s32_layout(int64_t N1) {

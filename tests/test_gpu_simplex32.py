@@ -132,3 +132,40 @@ def test_pivot_cap(pd, ctx):
         pd.pd_w1_approx(ctx, A, B, 0.5, pd.opts(max_rounds=3))
     assert e.value.status == pd.PD_ETIMEOUT
     assert pd.pd_w1_approx(ctx, A, B, 0.5)["opt_quanta"] == full
+
+
+def _grid_pair(nodes, seed):
+    """Two disjoint diagrams of `nodes` points in all on a lattice of 4,096 places."""
+    rng = np.random.default_rng(seed)
+    at = rng.permutation(4096)[:nodes]
+    pts = np.stack([at // 64, at // 64 + 1 + at % 64], 1).astype(np.float32) / 64
+    k = nodes // 2 + int(rng.integers(-40, 41))
+    return tuple(torch.from_numpy(np.ascontiguousarray(p)).cuda() for p in (pts[:k], pts[k:]))
+
+
+# around the sizes up to which an instance takes half an SM by itself, and up
+# to which half an SM holds it (more such pairs than SMs)
+@pytest.mark.parametrize("nodes", [1277, 1278, 1279, 1280, 1281])
+def test_small_instances_on_half_an_sm(pd, ctx, nodes):
+    A, B = _grid_pair(nodes, nodes)
+    got = pd.pd_w1_approx(ctx, A, B, 0.01, pd.opts(warm_start=0))
+    assert got["opt_quanta"] == pd.pd_w1_approx(ctx, A, B, 0.01, pd.opts(ns_smem=0))["opt_quanta"]
+
+
+def test_two_instances_per_sm(pd, ctx):
+    pairs = [_grid_pair(n, n) for n in (3708, 3709, 3710, 3711, 3712, 3713, 700)]
+    exp = [pd.pd_w1_approx(ctx, a, b, 0.01, pd.opts(ns_smem=0))["opt_quanta"] for a, b in pairs]
+    many = [i for i in range(4) for _ in range(40)] + list(range(4, len(pairs)))  # 160 that surely fit, then the edge
+    got = pd.pd_w1_approx_batch(ctx, [pairs[i][0] for i in many], [pairs[i][1] for i in many], 0.01)
+    assert [r["opt_quanta"] for r in got] == [exp[i] for i in many]
+
+
+# arc lists around the size from which their chunks are spread over the pricing
+# blocks, with and without a part chunk: assignment problems
+@pytest.mark.parametrize("k", [2047, 2048, 2050])
+def test_spread_arc_lists(pd, ctx, k):
+    from scipy.optimize import linear_sum_assignment
+    cost = np.random.default_rng(k).integers(0, 1 << 20, (k, k))
+    u, v = np.divmod(np.arange(k * k), k)
+    net = _net(2 * k, u, v + k, cost.reshape(-1), np.r_[np.ones(k, np.int64), -np.ones(k, np.int64)])
+    assert pd.pd_mcf_solve(ctx, net)[0] == cost[linear_sum_assignment(cost)].sum()
