@@ -199,10 +199,27 @@ Ctx* ctx_new(int device, size_t cap) {
     return c;
 }
 
+pd_status ctx_events(Ctx* c, int first, int n, cudaEvent_t** ev) {
+    *ev = c->ev + first;
+    for (int q = 0; q < n; q++)
+        if (!(*ev)[q]) PD_TRY_CUDA(c, cudaEventCreate(&(*ev)[q]));
+    return PD_OK;
+}
+
+pd_status smem_limit(Ctx* c, std::atomic<uint64_t>& done, const void* kernel, size_t bytes) {
+    const uint64_t bit = c->device < 64 ? uint64_t(1) << c->device : 0;
+    if (done.load() & bit) return PD_OK;
+    PD_TRY_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    done |= bit;
+    return PD_OK;
+}
+
 static void wave_free(Ctx* c) {
     if (c->wave_exec) cudaGraphExecDestroy(c->wave_exec);
     if (c->wave_stream) cudaStreamDestroy(c->wave_stream);
     for (cudaEvent_t& e : c->wave_ev)
+        if (e) cudaEventDestroy(e);
+    for (cudaEvent_t& e : c->ev)
         if (e) cudaEventDestroy(e);
     if (c->wave_pin) cudaFreeHost(c->wave_pin);
     c->wave_exec = nullptr;
@@ -470,14 +487,8 @@ namespace pd {
 
 pd_status front_half(Ctx* c, const pd_diagram& A, const pd_diagram& B, double eps, const pd_opts& o, Front* f,
                      cudaStream_t st, bool count_only) {
-    cudaEvent_t ev[4];
-    for (int q = 0; q < 4; q++) PD_TRY_CUDA(c, cudaEventCreate(&ev[q]));
-    struct Guard {
-        cudaEvent_t* e;
-        ~Guard() {
-            for (int q = 0; q < 4; q++) cudaEventDestroy(e[q]);
-        }
-    } guard{ev};
+    cudaEvent_t* ev;
+    PD_TRY(ctx_events(c, EV_FRONT, 4, &ev));
     PD_TRY(check_diag_cost(c, o));
     PD_TRY_CUDA(c, cudaEventRecord(ev[0], st));
     DevDiag a, b;
@@ -848,8 +859,8 @@ pd_status batch_solve(Ctx* c, const pd_diagram* A, const pd_diagram* B, int64_t 
     for (Ctx* wk : c->workers) wk->mlp_owner = c;  // predictions use this context's network
     if (o.warm_start == 1 && !c->mlp_ready) return fail(c, PD_EINVAL, "warm_start = 1 needs a trained network");
     // the workers start after everything already queued on the caller's stream
-    cudaEvent_t ready;
-    PD_TRY_CUDA(c, cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
+    cudaEvent_t* ready;
+    PD_TRY(ctx_events(c, EV_READY, 1, &ready));
     std::vector<BatchPair> bp((size_t)W);
     std::vector<NSInst> hin, hout;
     std::vector<CertJob> jobs;
@@ -859,7 +870,7 @@ pd_status batch_solve(Ctx* c, const pd_diagram* A, const pd_diagram* B, int64_t 
         const int64_t nw = std::min<int64_t>(W, count - base);
         for (int64_t j = 0; j < nw; j++) bp[(size_t)j] = BatchPair{};
         // ---- preprocessing: host threads, one worker context and stream each
-        cudaEventRecord(ready, st);
+        cudaEventRecord(*ready, st);
         std::atomic<int64_t> next{0};
         std::mutex mu;
         pd_status first = PD_OK;
@@ -867,7 +878,7 @@ pd_status batch_solve(Ctx* c, const pd_diagram* A, const pd_diagram* B, int64_t 
         auto run = [&](int t) {
             Ctx* wk = c->workers[(size_t)t];
             cudaSetDevice(c->device);
-            cudaStreamWaitEvent(wk->own_stream, ready, 0);
+            cudaStreamWaitEvent(wk->own_stream, *ready, 0);
             for (;;) {
                 const int64_t j = next.fetch_add(1);
                 if (j >= nw) break;
@@ -983,7 +994,6 @@ pd_status batch_solve(Ctx* c, const pd_diagram* A, const pd_diagram* B, int64_t 
             res.warm_pivots = p.wst.coarse_pivots;
         }
     }
-    cudaEventDestroy(ready);
     // the blocks the slots and workers outgrew: freed now that their work is done
     cudaStreamSynchronize(st);
     for (Ctx* sl : c->slots) ctx_release(sl);

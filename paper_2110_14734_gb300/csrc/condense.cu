@@ -314,8 +314,8 @@ pd_status stage_condense0(Ctx* c, const DevDiag& A, const DevDiag& B, int k, Hat
     if (n == 0) return PD_OK;
     if (n <= CS_MAX) {
         int64_t* h = c->h_small;
-        PD_TRY_CUDA(c, cudaFuncSetAttribute(k_condense0_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)sizeof(CtaStage)));
+        static std::atomic<uint64_t> done{0};
+        PD_TRY(smem_limit(c, done, (const void*)k_condense0_small, sizeof(CtaStage)));
         k_condense0_small<<<1, CS_THREADS, sizeof(CtaStage), st>>>(A.bd, (int)A.n, A.dtype, B.bd, (int)B.n, B.dtype, k,
                                                                    out->X, out->Y, out->cnt, sm, h); pd::count_launch();
         PD_TRY_CUDA(c, cudaGetLastError());
@@ -999,8 +999,8 @@ pd_status stage_condense_delta(Ctx* c, const Hats& hats, int64_t G, int64_t P, u
         int64_t* CB = bufT<int64_t>(c, B_CB, n);
         if (!NX || !NY || !CA || !CB) return PD_ENOMEM;
         int64_t* hs = c->h_small;
-        PD_TRY_CUDA(c, cudaFuncSetAttribute(k_condense_delta_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)sizeof(CtaStage)));
+        static std::atomic<uint64_t> done{0};
+        PD_TRY(smem_limit(c, done, (const void*)k_condense_delta_small, sizeof(CtaStage)));
         k_condense_delta_small<<<1, CS_THREADS, sizeof(CtaStage), st>>>(hats.X, hats.Y, hats.cnt, (int)hats.nA, (int)n, G, P,
                                                                         seed, NX, NY, CA, CB, out->X, out->Y, out->cntA,
                                                                         out->cntB, out->morton, hs); pd::count_launch();

@@ -1,5 +1,6 @@
 // Internal (C++) interface between the entry points and the stages.
 #pragma once
+#include <atomic>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -92,6 +93,9 @@ struct Ctx {
     cudaGraphExec_t wave_exec = nullptr;
     cudaStream_t wave_stream = nullptr;
     cudaEvent_t wave_ev[3] = {nullptr, nullptr, nullptr};
+    // the stages' timing events, made when first used: creating and destroying
+    // them costs about 10 us a pair of calls, under a lock that all threads share
+    cudaEvent_t ev[13] = {};
     uint64_t wave_key = 0;
     int64_t wave_launches = 0;        // graph launches (each replays the wave's kernels)
 };
@@ -110,6 +114,11 @@ T* bufT(Ctx* c, Buf id, int64_t n) {
 }
 
 pd_status fail(Ctx* c, pd_status st, const std::string& msg);
+// n events of the context from the first-th (a range per user: two stages may be under way at once).
+constexpr int EV_FRONT = 0, EV_NETWORK = 4, EV_SIMPLEX = 8, EV_BOUNDS = 10, EV_READY = 12;
+pd_status ctx_events(Ctx* c, int first, int n, cudaEvent_t** ev);
+// Raises a kernel's dynamic shared memory limit, once per device (`done`: the kernel's devices).
+pd_status smem_limit(Ctx* c, std::atomic<uint64_t>& done, const void* kernel, size_t bytes);
 pd_status cuda_fail(Ctx* c, cudaError_t e, const char* where);
 
 #define PD_TRY_CUDA(c, expr)                                    \

@@ -577,7 +577,8 @@ pd_status mlp_grad(Ctx* c, const __nv_bfloat16* F, const float* t, const float* 
     float* part = bufT<float>(c, B_MLP_PART, (int64_t)nb * WS_PART);
     if (!part) return PD_ENOMEM;
     const size_t smem = backward_smem();
-    PD_TRY_CUDA(c, cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static std::atomic<uint64_t> done{0};
+    PD_TRY(smem_limit(c, done, (const void*)k_mlp_backward, smem));
     k_mlp_backward<<<nb, WS_THREADS, smem, st>>>(weights_of(c), F, t, mask, n, inv_norm, part); pd::count_launch();
     k_reduce_parts<<<grid_for(WS_PART, 256), 256, 0, st>>>(part, nb, g); pd::count_launch();
     PD_TRY_CUDA(c, cudaGetLastError());

@@ -1010,14 +1010,13 @@ pd_status ns_run(Ctx* c, const NSInst* h, int count, NSInst* d, NSInst* r, cudaS
     if (!dord) return PD_ENOMEM;
     PD_TRY_CUDA(c, cudaMemcpyAsync(d, h, sizeof(NSInst) * count, cudaMemcpyHostToDevice, st));
     PD_TRY_CUDA(c, cudaMemcpyAsync(dord, order.data(), sizeof(int32_t) * order.size(), cudaMemcpyHostToDevice, st));
-    cudaEvent_t e0, e1;
-    PD_TRY_CUDA(c, cudaEventCreate(&e0));
-    PD_TRY_CUDA(c, cudaEventCreate(&e1));
+    cudaEvent_t* ev;
+    PD_TRY(ctx_events(c, EV_SIMPLEX, 2, &ev));
     // the 32-bit kernels, then the 64-bit one over its own instances and those handed back
     cudaError_t le = cudaSuccess;
     for (int pass = 0; pass < 2 && le == cudaSuccess; pass++) {
         if (pass == 0 ? L.own64 == count : !any64) continue;
-        le = cudaEventRecord(e0, st);
+        le = cudaEventRecord(ev[0], st);
         if (pass == 0) {
             for (int k = 0; k < S32_CLASSES; k++)
                 if (L.num[k] > 0) {
@@ -1030,17 +1029,15 @@ pd_status ns_run(Ctx* c, const NSInst* h, int count, NSInst* d, NSInst* r, cudaS
             pd::count_launch();
         }
         if (le == cudaSuccess) le = cudaGetLastError();
-        if (le == cudaSuccess) le = cudaEventRecord(e1, st);
+        if (le == cudaSuccess) le = cudaEventRecord(ev[1], st);
         if (le == cudaSuccess) le = cudaMemcpyAsync(r, d, sizeof(NSInst) * count, cudaMemcpyDeviceToHost, st);
         if (le == cudaSuccess) le = cudaStreamSynchronize(st);
         float nms = 0.f;
-        if (le == cudaSuccess) le = cudaEventElapsedTime(&nms, e0, e1);
+        if (le == cudaSuccess) le = cudaEventElapsedTime(&nms, ev[0], ev[1]);
         c->last_ns_ms += nms;
         if (pass == 0)
             for (int q = 0; q < count; q++) any64 |= r[q].lay32 != 0 && r[q].status == S32_REDO;
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     if (le != cudaSuccess) return cuda_fail(c, le, "network simplex");
     return PD_OK;
 }

@@ -324,10 +324,9 @@ extern "C" pd_status pd_nn_search(pd_ctx* cx, pd_diagram query, double eps, cons
     const int64_t s = o.s_override > 0 ? o.s_override : s_for_eps(eps);
     if (s < 1) return fail(c, PD_EINVAL, "no WSPD parameter s for this eps");
     // ---- lower bounds ----------------------------------------------------
-    cudaEvent_t e0, e1;
-    PD_TRY_CUDA(c, cudaEventCreate(&e0));
-    PD_TRY_CUDA(c, cudaEventCreate(&e1));
-    PD_TRY_CUDA(c, cudaEventRecord(e0, st));
+    cudaEvent_t* ev;
+    PD_TRY(ctx_events(c, EV_BOUNDS, 2, &ev));
+    PD_TRY_CUDA(c, cudaEventRecord(ev[0], st));
     const pd_diagram empty{nullptr, 0, query.dtype, 0};
     DevDiag a, b;
     PD_TRY(stage_inputs(c, query, empty, &a, &b, st));
@@ -385,13 +384,11 @@ extern "C" pd_status pd_nn_search(pd_ctx* cx, pd_diagram query, double eps, cons
         PD_TRY_CUDA(c, cudaMemsetAsync(LA, 0, sizeof(double) * n_db, st));
     }
     PD_TRY_CUDA(c, cudaGetLastError());
-    PD_TRY_CUDA(c, cudaEventRecord(e1, st));
+    PD_TRY_CUDA(c, cudaEventRecord(ev[1], st));
     std::vector<double> hl((size_t)(2 * n_db));
     PD_TRY_CUDA(c, cudaMemcpyAsync(hl.data(), LA, sizeof(double) * 2 * n_db, cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
-    cudaEventElapsedTime(&r.lb_ms, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
+    cudaEventElapsedTime(&r.lb_ms, ev[0], ev[1]);
     // OPT_int >= (1 - eps_c) max(RWMD, WCD / 2); the last factor covers double rounding
     const double ec = o.condense ? (s >= 12 ? 8.0 / (double)(s - 4) : 1.0) : 0.0;
     std::vector<int64_t> lb((size_t)n_db), lbw((size_t)n_db);

@@ -159,7 +159,8 @@ pd_status sort_u64(Ctx* c, uint64_t*& keys, uint64_t*& keys_alt, uint32_t*& vals
                    int bits, cudaStream_t st) {
     if (n <= 1 || bits <= 0) return PD_OK;
     if (n <= CS_MAX) {
-        PD_TRY_CUDA(c, cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CtaSort)));
+        static std::atomic<uint64_t> done{0};
+        PD_TRY(smem_limit(c, done, (const void*)k_sort_small, sizeof(CtaSort)));
         k_sort_small<<<1, CS_THREADS, sizeof(CtaSort), st>>>(keys, vals, (int)n, bits); pd::count_launch();
         PD_TRY_CUDA(c, cudaGetLastError());
         return PD_OK;

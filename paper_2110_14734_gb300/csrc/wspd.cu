@@ -629,8 +629,8 @@ static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, int64_t s, 
     // room for handed-on pairs: the more, the better the balance; less will do
     int64_t cap = std::min<int64_t>(int64_t(1) << 27, std::max<int64_t>(int64_t(1) << 16, 64 * (tr.N - 1)));
     int2* out[2];
-    if (arcs) PD_TRY_CUDA(c, cudaFuncSetAttribute(k_ws_walk<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)(sizeof(int2) * WS_WARPS * WS_OUT)));
+    static std::atomic<uint64_t> done{0};
+    if (arcs) PD_TRY(smem_limit(c, done, (const void*)k_ws_walk<true>, sizeof(int2) * WS_WARPS * WS_OUT));
     for (;; cap /= 4) {
         out[0] = bufT<int2>(c, B_F1, cap);
         out[1] = out[0] ? bufT<int2>(c, B_WSOFF, cap) : nullptr;
@@ -676,8 +676,8 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
     int64_t N = nodes.n_nodes;
     if (N >= (int64_t(1) << 31) - 4) return fail(c, PD_ECAPACITY, "more than 2^31 - 4 condensed nodes");
     if (s < 1) return fail(c, PD_EINVAL, "WSPD parameter s must be >= 1");
-    cudaEvent_t ev[4];
-    for (int q = 0; q < 4; q++) PD_TRY_CUDA(c, cudaEventCreate(&ev[q]));
+    cudaEvent_t* ev;
+    PD_TRY(ctx_events(c, EV_NETWORK, 4, &ev));
     PD_TRY_CUDA(c, cudaEventRecord(ev[0], st));
     int64_t M = N > 1 ? N - 1 : 1;
     unsigned long long* cnts = bufT<unsigned long long>(c, B_SMALL, 64);
@@ -758,7 +758,6 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
         if (ms_tree) cudaEventElapsedTime(ms_tree, ev[0], ev[1]);
         if (ms_wspd) cudaEventElapsedTime(ms_wspd, ev[1], ev[2]);
         if (ms_csr) cudaEventElapsedTime(ms_csr, ev[2], ev[3]);
-        for (int q = 0; q < 4; q++) cudaEventDestroy(ev[q]);
         return PD_OK;
     }
     if (!arcs) {
@@ -797,7 +796,6 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
     if (ms_tree) cudaEventElapsedTime(ms_tree, ev[0], ev[1]);
     if (ms_wspd) cudaEventElapsedTime(ms_wspd, ev[1], ev[2]);
     if (ms_csr) cudaEventElapsedTime(ms_csr, ev[2], ev[3]);
-    for (int q = 0; q < 4; q++) cudaEventDestroy(ev[q]);
     return PD_OK;
 }
 
