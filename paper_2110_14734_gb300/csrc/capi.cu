@@ -744,6 +744,22 @@ struct BatchPair {
     int inst = -1;      // index in the wave's launch
 };
 
+// One launch instead of six copies: of 10 to 100 KB each, they are all driver calls.
+__global__ void k_keep_tree(WsTree from, int32_t* __restrict__ X, int32_t* __restrict__ Y, int32_t* __restrict__ left,
+                            int32_t* __restrict__ right, int4* __restrict__ bb, int32_t* __restrict__ rep) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < from.N) {
+        X[i] = from.X[i];
+        Y[i] = from.Y[i];
+    }
+    if (i < from.N - 1) {
+        left[i] = from.left[i];
+        right[i] = from.right[i];
+        bb[i] = from.bb[i];
+        rep[i] = from.rep[i];
+    }
+}
+
 // What the certificate reads, copied from the worker into the pair's slot:
 // node coordinates and the WSPD tree (about 36 bytes per node).
 static pd_status persist_for_certificate(Ctx* slot, const Front& f, BatchPair* bp, cudaStream_t st) {
@@ -756,14 +772,8 @@ static pd_status persist_for_certificate(Ctx* slot, const Front& f, BatchPair* b
     int32_t* rep = bufT<int32_t>(slot, B_T_REP, M);
     if (!X || !Y || !l || !r || !bb || !rep) return PD_ENOMEM;
     if (N > 0) {
-        PD_TRY_CUDA(slot, cudaMemcpyAsync(X, f.nodes.X, sizeof(int32_t) * N, cudaMemcpyDeviceToDevice, st));
-        PD_TRY_CUDA(slot, cudaMemcpyAsync(Y, f.nodes.Y, sizeof(int32_t) * N, cudaMemcpyDeviceToDevice, st));
-    }
-    if (N > 1) {
-        PD_TRY_CUDA(slot, cudaMemcpyAsync(l, f.tree.left, sizeof(int32_t) * M, cudaMemcpyDeviceToDevice, st));
-        PD_TRY_CUDA(slot, cudaMemcpyAsync(r, f.tree.right, sizeof(int32_t) * M, cudaMemcpyDeviceToDevice, st));
-        PD_TRY_CUDA(slot, cudaMemcpyAsync(bb, f.tree.bb, sizeof(int4) * M, cudaMemcpyDeviceToDevice, st));
-        PD_TRY_CUDA(slot, cudaMemcpyAsync(rep, f.tree.rep, sizeof(int32_t) * M, cudaMemcpyDeviceToDevice, st));
+        k_keep_tree<<<grid_for(N, 256), 256, 0, st>>>(f.tree, X, Y, l, r, bb, rep); pd::count_launch();
+        PD_TRY_CUDA(slot, cudaGetLastError());
     }
     bp->tree = WsTree{N, X, Y, l, r, bb, rep};
     return PD_OK;

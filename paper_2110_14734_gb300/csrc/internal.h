@@ -20,7 +20,7 @@ enum Buf : int {
     B_HAT_X, B_HAT_Y, B_HAT_C,      // 0-condensed nodes of A then B
     B_CKEY, B_CKEY2, B_CVAL, B_CVAL2, B_CIDX, B_CX, B_CY, B_CA, B_CB,
     B_NX, B_NY, B_NCA, B_NCB, B_NCODE,  // output nodes
-    B_T_LEFT, B_T_RIGHT, B_T_BB, B_T_REP, B_T_PARENT, B_T_LPARENT, B_T_VISIT,
+    B_T_LEFT, B_T_RIGHT, B_T_BB, B_T_REP, B_T_PARENT, B_T_LPARENT, B_T_VISIT, B_T_LEAVES, B_T_LEAFXY,
     B_F0, B_F1, B_WSFLAG, B_WSOFF,  // WSPD frontier
     B_ARCKEY, B_ARCKEY2,            // arc keys (tail << hb | head)
     B_ROWPTR, B_HEAD, B_COST, B_SUPPLY,

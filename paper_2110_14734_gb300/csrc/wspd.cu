@@ -61,11 +61,12 @@ __global__ void k_karras(const uint64_t* __restrict__ code, int64_t N, int32_t* 
 }
 
 // Each leaf climbs; the second child to arrive at a node computes the node's
-// tight box and leftmost member (min X, then min Y) from its two children.
+// tight box, leftmost member (min X, then min Y) and leaf count from its two
+// children.
 __global__ void k_bbox(int64_t N, const int32_t* __restrict__ X, const int32_t* __restrict__ Y,
                        const int32_t* __restrict__ left, const int32_t* __restrict__ right,
                        const int32_t* __restrict__ par_int, const int32_t* __restrict__ par_leaf, int4* bb,
-                       int32_t* rep, int32_t* visit) {
+                       int32_t* rep, int32_t* leaves, int32_t* visit) {
     int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= N) return;
     int32_t cur = par_leaf[l];
@@ -73,7 +74,7 @@ __global__ void k_bbox(int64_t N, const int32_t* __restrict__ X, const int32_t* 
         __threadfence();
         if (atomicAdd(&visit[cur], 1) == 0) return;
         int4 b[2];
-        int32_t r[2];
+        int32_t r[2], n[2];
         int32_t ch[2] = {left[cur], right[cur]};
         for (int q = 0; q < 2; q++) {
             int32_t c = ch[q];
@@ -81,7 +82,9 @@ __global__ void k_bbox(int64_t N, const int32_t* __restrict__ X, const int32_t* 
                 int32_t p = ~c;
                 b[q] = make_int4(X[p], X[p], Y[p], Y[p]);
                 r[q] = p;
+                n[q] = 1;
             } else {
+                n[q] = __ldcg(&leaves[c]);
                 b[q] = __ldcg(&bb[c]);
                 r[q] = __ldcg(&rep[c]);
             }
@@ -90,6 +93,7 @@ __global__ void k_bbox(int64_t N, const int32_t* __restrict__ X, const int32_t* 
         int32_t rr = (X[r[1]] < X[r[0]] || (X[r[1]] == X[r[0]] && Y[r[1]] < Y[r[0]])) ? r[1] : r[0];
         __stcg(&bb[cur], u);
         __stcg(&rep[cur], rr);
+        __stcg(&leaves[cur], n[0] + n[1]);
         cur = par_int[cur];
     }
 }
@@ -254,18 +258,26 @@ __global__ void k_certify_batch(const CertJob* __restrict__ jobs, unsigned long 
 // enumeration: warps walk the pair tree depth first
 // ---------------------------------------------------------------------------
 //
-// The recursion visits as many pairs as the decomposition has, twice over (at
+// The recursion tests as many pairs as the decomposition has, twice over (at
 // 2 M nodes and s = 167: 21 G separated pairs and as many split ones), and a pair
 // needs only its two nodes.  So what bounds it is the gather of node records
-// and the instructions of a test, as long as the pairs waiting to be visited
-// never leave the SM: every warp keeps them in a stack in shared memory and
-// visits the 32 topmost at a time.  These descend from one pair a few levels
-// up, so the 32 lanes touch about a dozen different nodes.
+// and the instructions of a test, as long as what waits to be visited never
+// leaves the SM: every warp keeps it in a stack in shared memory and visits the
+// 32 topmost pairs at a time.  These descend from one pair a few levels up, so
+// the 32 lanes touch about a dozen different nodes.
 //
 // The records.  An internal node's 32 bytes: doubled centre, separation
-// threshold (s + 2)^2 diagonal^2, larger side, children, representative.  A
+// threshold (s + 2)^2 diagonal^2, larger side, children, and the representative
+// (when pairs are stored) or the leaves below it (when they are counted).  A
 // leaf needs its coordinates only, and a pair of leaves nothing: it is always
 // separated, and is counted where it would be pushed.
+//
+// Lattices.  Nodes snapped to a grid have no small boxes.  Below a pair of
+// nodes whose farthest points are closer than the smallest box's threshold, only
+// pairs of leaves can be separated: as many as the product of the leaf counts.
+// Where that reaches over more than a sixteenth of the nodes' extent, counting
+// stops there (8,205 lattice nodes, s = 327: 0.58 -> 0.18 ms; mixture points take no
+// notice of the test).
 //
 // Balance.  Initial pairs (one per internal node) differ by many orders of
 // magnitude in the pairs below them, so a warp that has walked `budget` steps
@@ -273,51 +285,81 @@ __global__ void k_certify_batch(const CertJob* __restrict__ jobs, unsigned long 
 // warps take it up.
 //
 // Measured (pd_w1_sparsify_count's WSPD stage, mixture points, s = 167): 1,000,000
-// + 1,000,000 points 493 -> 165 ms, 100,000 + 100,000 23 -> 7.4 ms, against
+// + 1,000,000 points 493 -> 161 ms, 100,000 + 100,000 23 -> 7.2 ms, against
 // level-by-level frontiers in global memory (689 GB of DRAM traffic a call, and
-// 128-bit products per test).  Now 70 % of the issue slots and of the L1's
-// throughput are used.
+// 128-bit products per test).  Entries of two pairs, a node and its partner's
+// children, were slower (269 ms).
 
 struct __align__(32) WsRec {
     int32_t cx, cy;  // doubled centre
     uint64_t thr;    // least doubled squared distance that separates (saturated)
     uint32_t side;   // larger box side
     int32_t l, r;    // children
-    int32_t rep;
+    int32_t last;    // representative, or leaves (see above)
 };
 
-__global__ void k_ws_records(int64_t M, const int4* __restrict__ bb, const int32_t* __restrict__ rep,
-                             const int32_t* __restrict__ left, const int32_t* __restrict__ right, int64_t s,
-                             WsRec* __restrict__ rec, int2* __restrict__ F) {
+// Also the leaves' doubled coordinates, and over all internal nodes ext[0] = ~
+// the least threshold and ext[1] = the largest side (maxima; both start at 0).
+// last: the leaf counts or the representatives.
+__global__ void k_ws_records(int64_t M, const int4* __restrict__ bb, const int32_t* __restrict__ last,
+                             const int32_t* __restrict__ left, const int32_t* __restrict__ right,
+                             const int32_t* __restrict__ X, const int32_t* __restrict__ Y, int64_t s,
+                             WsRec* __restrict__ rec, int2* __restrict__ leaf, int2* __restrict__ F,
+                             unsigned long long* __restrict__ ext) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M) return;
-    const int4 b = bb[i];
-    const uint64_t wx = (uint64_t)((int64_t)b.y - b.x), wy = (uint64_t)((int64_t)b.w - b.z);
-    const uint64_t k = (uint64_t)(s + 2) * (uint64_t)(s + 2);
-    const unsigned __int128 t = (unsigned __int128)k * (wx * wx + wy * wy);
-    WsRec q;
-    q.cx = b.x + b.y;  // |coordinate| < 2^30: no overflow
-    q.cy = b.z + b.w;
-    q.thr = (t >> 64) != 0 ? ~0ull : (uint64_t)t;
-    q.side = (uint32_t)(wx > wy ? wx : wy);
-    q.l = left[i];
-    q.r = right[i];
-    q.rep = rep[i];
-    rec[i] = q;
-    F[i] = make_int2(q.l, q.r);  // the first pairs: every internal node's children
+    unsigned long long inv = 0, side = 0;
+    if (i <= M) leaf[i] = make_int2(2 * X[i], 2 * Y[i]);  // |coordinate| < 2^30: no overflow
+    if (i < M) {
+        const int4 b = bb[i];
+        const uint64_t wx = (uint64_t)((int64_t)b.y - b.x), wy = (uint64_t)((int64_t)b.w - b.z);
+        const uint64_t k = (uint64_t)(s + 2) * (uint64_t)(s + 2);
+        const unsigned __int128 t = (unsigned __int128)k * (wx * wx + wy * wy);
+        WsRec q;
+        q.cx = b.x + b.y;
+        q.cy = b.z + b.w;
+        q.thr = (t >> 64) != 0 ? ~0ull : (uint64_t)t;
+        q.side = (uint32_t)(wx > wy ? wx : wy);
+        q.l = left[i];
+        q.r = right[i];
+        q.last = last[i];
+        rec[i] = q;
+        F[i] = make_int2(q.l, q.r);  // the first pairs: every internal node's children
+        inv = ~q.thr;
+        side = q.side;
+    }
+    __shared__ unsigned long long part[2][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int pass = 0; pass < 2; pass++) {
+        for (int o = 16; o > 0; o >>= 1) {
+            inv = max(inv, __shfl_xor_sync(0xffffffffu, inv, o));
+            side = max(side, __shfl_xor_sync(0xffffffffu, side, o));
+        }
+        if (pass == 1) break;
+        if (lane == 0) {
+            part[0][wid] = inv;
+            part[1][wid] = side;
+        }
+        __syncthreads();
+        if (wid > 0) return;
+        inv = lane < (int)(blockDim.x >> 5) ? part[0][lane] : 0ull;
+        side = lane < (int)(blockDim.x >> 5) ? part[1][lane] : 0ull;
+    }
+    if (lane == 0) {
+        atomicMax(&ext[0], inv);
+        atomicMax(&ext[1], side);
+    }
 }
 
-PD_D WsRec ws_load(int32_t ref, const WsRec* __restrict__ rec, const int32_t* __restrict__ X,
-                   const int32_t* __restrict__ Y) {
+PD_D WsRec ws_load(int32_t ref, const WsRec* __restrict__ rec, const int2* __restrict__ leaf, bool counts) {
     WsRec q;
     if (ref < 0) {
-        const int32_t p = ~ref;
-        q.cx = 2 * X[p];
-        q.cy = 2 * Y[p];
+        const int2 p = __ldg(leaf + ~ref);
+        q.cx = p.x;
+        q.cy = p.y;
         q.thr = 0;
         q.side = 0;
         q.l = q.r = 0;
-        q.rep = p;
+        q.last = counts ? 1 : ~ref;
     } else {
         uint32_t w0, w1, w2, w3, w4, w5, w6, w7;
         asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -329,7 +371,7 @@ PD_D WsRec ws_load(int32_t ref, const WsRec* __restrict__ rec, const int32_t* __
         q.side = w4;
         q.l = (int32_t)w5;
         q.r = (int32_t)w6;
-        q.rep = (int32_t)w7;
+        q.last = (int32_t)w7;
     }
     return q;
 }
@@ -354,16 +396,18 @@ constexpr int WS_MARGIN = 200;   // above WS_STACK - WS_MARGIN pairs it visits o
                                  // at most 2 * 65 splits long (78 + 78 on the split tree), each net +1
 
 // lv[0] += separated pairs, lv[1] = pairs offered to the next launch (the first
-// cap of them are in Fn), lv[2] = initial pairs taken.  STORE: both arcs of every separated
-// pair to arcs (room for `room` pairs), at slots from lv[0], which counts all
-// pairs.
+// cap of them are in Fn), lv[2] = initial pairs taken; ext as in k_ws_records.
+// STORE: both arcs of every separated pair to arcs (room for `room` pairs), at
+// slots from lv[0], which counts all pairs.  counted: the records hold leaf counts.
 template <bool STORE>
 __global__ void __launch_bounds__(32 * WS_WARPS) k_ws_walk(const int2* __restrict__ F, int64_t nf, int chunk,
-                                                           const WsRec* __restrict__ rec, WsTree tr, int64_t s,
+                                                           const WsRec* __restrict__ rec,
+                                                           const int2* __restrict__ leaf, WsTree tr, int64_t s,
                                                            int64_t budget, int2* __restrict__ Fn,
                                                            unsigned long long cap, int hb, uint64_t* __restrict__ arcs,
                                                            unsigned long long room,
-                                                           unsigned long long* __restrict__ lv) {
+                                                           unsigned long long* __restrict__ lv,
+                                                           const unsigned long long* __restrict__ ext, int counted) {
     __shared__ int2 stack_[WS_WARPS][WS_STACK];
     extern __shared__ int2 out_[];  // STORE: separated pairs on their way out, WS_OUT a warp
     int2* const ow = out_ + (threadIdx.x >> 5) * WS_OUT;
@@ -372,6 +416,9 @@ __global__ void __launch_bounds__(32 * WS_WARPS) k_ws_walk(const int2* __restric
     int2* const st = stack_[threadIdx.x >> 5];
     const unsigned below = (1u << lane) - 1u;
     unsigned long long count = 0;
+    // lattices (sides below 2^28: nothing overflows)
+    const uint64_t least = ~ext[0], widest = ext[1];
+    const bool lattice = !STORE && counted && widest < (1u << 28) && least >= widest * widest / 64;
     // the buffered pairs' arcs, at slots taken with one atomic; past `room` they are only counted
     auto flush = [&]() {
         __syncwarp();
@@ -430,8 +477,8 @@ __global__ void __launch_bounds__(32 * WS_WARPS) k_ws_walk(const int2* __restric
         bool far = false;
         WsRec u{}, v{};
         if (on) {
-            u = ws_load(p.x, rec, tr.X, tr.Y);
-            v = ws_load(p.y, rec, tr.X, tr.Y);
+            u = ws_load(p.x, rec, leaf, !STORE);
+            v = ws_load(p.y, rec, leaf, !STORE);
             far = ws_far(u, v, p.x, p.y, s, tr);
             if (!far) {
                 // split the node with the larger box side, ties split the second
@@ -440,9 +487,19 @@ __global__ void __launch_bounds__(32 * WS_WARPS) k_ws_walk(const int2* __restric
                 c1 = su ? make_int2(u.r, p.y) : make_int2(p.x, v.r);
             }
         }
-        const bool open = on && !far;
+        bool open = on && !far;
+        if constexpr (!STORE) {
+            if (lattice && open) {  // only pairs of leaves separated below this one?
+                const uint64_t w = (uint64_t)u.side + v.side;
+                const uint64_t x = (uint64_t)abs(u.cx - v.cx) + w, y = (uint64_t)abs(u.cy - v.cy) + w;
+                if (x * x + y * y < least) {
+                    open = false;
+                    count += (unsigned long long)u.last * (unsigned long long)v.last;
+                }
+            }
+        }
         const bool l0 = open && (c0.x & c0.y) < 0, l1 = open && (c1.x & c1.y) < 0;  // two leaves
-        emit(far, make_int2(u.rep, v.rep), l0, make_int2(~c0.x, ~c0.y), l1, make_int2(~c1.x, ~c1.y));
+        emit(far, make_int2(u.last, v.last), l0, make_int2(~c0.x, ~c0.y), l1, make_int2(~c1.x, ~c1.y));
         const bool p0 = open && !l0, p1 = open && !l1;
         const unsigned m0 = __ballot_sync(0xffffffffu, p0), m1 = __ballot_sync(0xffffffffu, p1);
         const int at = h + __popc(m0 & below) + __popc(m1 & below);
@@ -619,19 +676,24 @@ pd_status merge_diagonal(Ctx* c, const pd_network& net, int64_t N, pd_network* o
     return PD_OK;
 }
 
+// The walk's device words: 0 .. 2 lv, 3 .. 4 ext, 5 .. 8 k_diag_counts (all cleared before k_ws_records).
+constexpr int WS_WORDS = 9;
+static unsigned long long* ws_words(Ctx* c) { return bufT<unsigned long long>(c, B_SMALL, 64) + 12; }
+
 // All launches of the walk over the tree's pairs (see k_ws_walk): *pairs =
-// separated pairs; arcs (may be null): where their arcs go.
-static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, int64_t s, int hb, uint64_t* arcs, int64_t room,
-                         int64_t* pairs, cudaStream_t st) {
-    unsigned long long* lv = bufT<unsigned long long>(c, B_SMALL, 64) + 12;
+// separated pairs; arcs (may be null): where their arcs go.  The walk's words end
+// up in h_small.
+static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, const int2* leaf, int64_t s, int hb, bool counted,
+                         uint64_t* arcs, int64_t room, int64_t* pairs, cudaStream_t st) {
+    unsigned long long* lv = ws_words(c);
     const int blocks = 4 * std::max(c->sm_count, 1);  // the stacks of four blocks fit an SM
     const int64_t warps = (int64_t)blocks * WS_WARPS;
     // room for handed-on pairs: the more, the better the balance; less will do
-    int64_t cap = std::min<int64_t>(int64_t(1) << 27, std::max<int64_t>(int64_t(1) << 16, 64 * (tr.N - 1)));
+    int64_t cap = std::min<int64_t>(int64_t(1) << 27, std::max<int64_t>(int64_t(1) << 16, 64 * (tr.N - 1)));  // even
     int2* out[2];
     static std::atomic<uint64_t> done{0};
     if (arcs) PD_TRY(smem_limit(c, done, (const void*)k_ws_walk<true>, sizeof(int2) * WS_WARPS * WS_OUT));
-    for (;; cap /= 4) {
+    for (;; cap = cap / 8 * 2) {
         out[0] = bufT<int2>(c, B_F1, cap);
         out[1] = out[0] ? bufT<int2>(c, B_WSOFF, cap) : nullptr;
         if (out[0] && out[1]) break;
@@ -648,19 +710,20 @@ static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, int64_t s, 
     const int64_t budget = tr.N > (int64_t(1) << 20) ? 512 : 64;
     for (int64_t round = 0; nf > 0; round++) {
         const int chunk = (int)std::min<int64_t>(32, std::max<int64_t>(1, nf / warps));
-        PD_TRY_CUDA(c, cudaMemsetAsync(lv + (arcs && round > 0 ? 1 : 0), 0,
-                                       (arcs && round > 0 ? 2 : 3) * sizeof(unsigned long long), st));
+        if (round > 0)
+            PD_TRY_CUDA(c, cudaMemsetAsync(lv + (arcs ? 1 : 0), 0, (arcs ? 2 : 3) * sizeof(unsigned long long), st));
         const unsigned grid = (unsigned)std::min<int64_t>(blocks, ((nf + chunk - 1) / chunk + WS_WARPS - 1) / WS_WARPS);
         if (arcs) {
             k_ws_walk<true><<<grid, 32 * WS_WARPS, sizeof(int2) * WS_WARPS * WS_OUT, st>>>(
-                F, nf, chunk, rec, tr, s, budget, out[round & 1], (unsigned long long)cap, hb, arcs,
-                (unsigned long long)room, lv); pd::count_launch();
+                F, nf, chunk, rec, leaf, tr, s, budget, out[round & 1], (unsigned long long)cap, hb, arcs,
+                (unsigned long long)room, lv, lv + 3, 0); pd::count_launch();
         } else {
-            k_ws_walk<false><<<grid, 32 * WS_WARPS, 0, st>>>(F, nf, chunk, rec, tr, s, budget, out[round & 1],
-                                                             (unsigned long long)cap, hb, nullptr, 0, lv); pd::count_launch();
+            k_ws_walk<false><<<grid, 32 * WS_WARPS, 0, st>>>(F, nf, chunk, rec, leaf, tr, s, budget, out[round & 1],
+                                                             (unsigned long long)cap, hb, nullptr, 0, lv, lv + 3,
+                                                             counted ? 1 : 0); pd::count_launch();
         }
         PD_TRY_CUDA(c, cudaGetLastError());
-        PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, lv, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, lv, WS_WORDS * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
         PD_TRY_CUDA(c, cudaStreamSynchronize(st));
         total = arcs ? c->h_small[0] : total + c->h_small[0];  // with arcs, lv[0] runs on as their slot counter
         nf = std::min<int64_t>(c->h_small[1], cap);
@@ -682,7 +745,7 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
     int64_t M = N > 1 ? N - 1 : 1;
     unsigned long long* cnts = bufT<unsigned long long>(c, B_SMALL, 64);
     if (!cnts) return PD_ENOMEM;
-    const int32_t *left, *right, *rep;
+    const int32_t *left, *right, *rep, *leaves = nullptr;  // (a given tree comes without its leaf counts)
     const int4* bb;
     if (given) {
         if (given->N != N || given->X != nodes.X || given->Y != nodes.Y)
@@ -699,14 +762,16 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
         int32_t* par_int = bufT<int32_t>(c, B_T_PARENT, M);
         int32_t* par_leaf = bufT<int32_t>(c, B_T_LPARENT, N);
         int32_t* visit = bufT<int32_t>(c, B_T_VISIT, M);
-        if (!l || !r || !b || !rp || !par_int || !par_leaf || !visit) return PD_ENOMEM;
+        int32_t* lc = bufT<int32_t>(c, B_T_LEAVES, M);
+        if (!l || !r || !b || !rp || !lc || !par_int || !par_leaf || !visit) return PD_ENOMEM;
         left = l;
         right = r;
         bb = b;
         rep = rp;
+        leaves = lc;
         if (N >= 2) {
             k_karras<<<grid_for(N - 1, 256), 256, 0, st>>>(nodes.morton, N, l, r, par_int, par_leaf, visit); pd::count_launch();
-            k_bbox<<<grid_for(N, 256), 256, 0, st>>>(N, nodes.X, nodes.Y, l, r, par_int, par_leaf, b, rp, visit); pd::count_launch();
+            k_bbox<<<grid_for(N, 256), 256, 0, st>>>(N, nodes.X, nodes.Y, l, r, par_int, par_leaf, b, rp, lc, visit); pd::count_launch();
             PD_TRY_CUDA(c, cudaGetLastError());
         }
     }
@@ -725,11 +790,17 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
         WsRec* rec = bufT<WsRec>(c, B_WSFLAG, N - 1);
         int2* F = bufT<int2>(c, B_F0, N - 1);
         if (!rec || !F) return PD_ENOMEM;
-        k_ws_records<<<grid_for(N - 1, 256), 256, 0, st>>>(N - 1, bb, rep, left, right, s, rec, F); pd::count_launch();
+        int2* leaf = bufT<int2>(c, B_T_LEAFXY, N);
+        if (!leaf) return PD_ENOMEM;
+        unsigned long long* words = ws_words(c);
+        PD_TRY_CUDA(c, cudaMemsetAsync(words, 0, WS_WORDS * sizeof(unsigned long long), st));
+        k_ws_records<<<grid_for(N, 256), 256, 0, st>>>(N - 1, bb, count_only && leaves ? leaves : rep, left, right, nodes.X,
+                                                       nodes.Y, s, rec, leaf, F, words + 3); pd::count_launch();
         PD_TRY_CUDA(c, cudaGetLastError());
         int64_t pairs = 0;
         if (count_only) {
-            PD_TRY(ws_walk(c, tr, rec, s, hb, nullptr, 0, &pairs, st));
+            k_diag_counts<<<grid_for(N, 256), 256, 0, st>>>(N, nodes.cntA, nodes.cntB, words + 5); pd::count_launch();
+            PD_TRY(ws_walk(c, tr, rec, leaf, s, hb, leaves != nullptr, nullptr, 0, &pairs, st));
         } else {
             // stored into the buffer the context has (64 arcs a node the first time);
             // if they are more, the walk has counted them and the second one stores them
@@ -738,7 +809,8 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
                 arcs = bufT<uint64_t>(c, B_ARCKEY, 2 * (pass ? pairs : 32 * N) + 2 * N + 1);
                 if (!arcs) return PD_ENOMEM;
                 room = ((int64_t)(c->bytes[B_ARCKEY] / sizeof(uint64_t)) - (2 * N + 1)) / 2;
-                PD_TRY(ws_walk(c, tr, rec, s, hb, arcs, room, &pairs, st));
+                if (pass) PD_TRY_CUDA(c, cudaMemsetAsync(words, 0, 3 * sizeof(unsigned long long), st));
+                PD_TRY(ws_walk(c, tr, rec, leaf, s, hb, false, arcs, room, &pairs, st));
                 if (pairs <= room) break;
             }
             if (pairs > room) return fail(c, PD_ECUDA, "the WSPD's pairs changed between two walks");
@@ -747,14 +819,16 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
     }
     PD_TRY_CUDA(c, cudaEventRecord(ev[2], st));
     if (count_only) {
-        // only the counts: arcs of the WSPD, diagonal arcs and the masses
-        PD_TRY_CUDA(c, cudaMemsetAsync(cnts, 0, 8 * sizeof(unsigned long long), st));
-        k_diag_counts<<<grid_for(N, 256), 256, 0, st>>>(N, nodes.cntA, nodes.cntB, cnts); pd::count_launch();
-        PD_TRY_CUDA(c, cudaGetLastError());
-        PD_TRY_CUDA(c, cudaMemcpyAsync(h, cnts, 4 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        // only the counts: arcs of the WSPD and (already here, unless there was nothing to walk) the diagonal's
+        if (N < 2) {
+            PD_TRY_CUDA(c, cudaMemsetAsync(cnts, 0, 4 * sizeof(unsigned long long), st));
+            k_diag_counts<<<grid_for(N, 256), 256, 0, st>>>(N, nodes.cntA, nodes.cntB, cnts); pd::count_launch();
+            PD_TRY_CUDA(c, cudaGetLastError());
+            PD_TRY_CUDA(c, cudaMemcpyAsync(h + 5, cnts, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        }
         PD_TRY_CUDA(c, cudaEventRecord(ev[3], st));
         PD_TRY_CUDA(c, cudaEventSynchronize(ev[3]));
-        *out = pd_network{N + 2, narcs + h[0] + h[1] + 1, nullptr, nullptr, nullptr, nullptr};
+        *out = pd_network{N + 2, narcs + h[5] + h[6] + 1, nullptr, nullptr, nullptr, nullptr};
         if (ms_tree) cudaEventElapsedTime(ms_tree, ev[0], ev[1]);
         if (ms_wspd) cudaEventElapsedTime(ms_wspd, ev[1], ev[2]);
         if (ms_csr) cudaEventElapsedTime(ms_csr, ev[2], ev[3]);

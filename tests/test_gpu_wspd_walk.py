@@ -69,3 +69,17 @@ def test_network_and_count_match_oracle(pd, ctx, name, nodes, s):
         np.testing.assert_array_equal(got[k].cpu().numpy(), exp[k])
     assert pd.pd_wspd_count(ctx, d, s, 0) == got["n_arcs"] == int(exp["row_ptr"][-1])
     assert pd.pd_wspd_count(ctx, d, s, 1) == pd.pd_wspd_sparsify_tree(ctx, d, s, 1)[0]["n_arcs"]
+
+
+# lattices with holes: counting stops at pairs of nodes below which only leaves
+# can be separated; spacings and s on both sides of where that is looked for
+@pytest.mark.parametrize("step,side,keep", [(1, 50, 0.6), (7, 40, 0.9), (1 << 20, 30, 0.8), (1 << 25, 20, 1.0)])
+@pytest.mark.parametrize("s", [1, 4, 9, 40, 327])
+def test_lattice_counts_match_oracle(pd, ctx, step, side, keep, s):
+    rng = np.random.default_rng(side)
+    X, Y = np.divmod(np.flatnonzero(rng.random(side * side) < keep), side)
+    nodes = _nodes(step * X, step * Y)
+    exp = oracle.build_network(nodes, *oracle.wspd(nodes, oracle.radix_tree(nodes), s))
+    d = {k: torch.from_numpy(np.ascontiguousarray(nodes[k])).cuda() for k in ("X", "Y", "cntA", "cntB")}
+    d["morton"] = torch.from_numpy(nodes["code"].view(np.int64)).cuda()
+    assert pd.pd_wspd_count(ctx, d, s, 0) == int(exp["row_ptr"][-1])
