@@ -52,12 +52,12 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_pass(const uint64_t* __res
     for (int q = 0; q < RS_ITEMS; q++) k[q] = i0 + 32 * q < m ? kin[t0 + i0 + 32 * q] : ~0ull;
 #pragma unroll
     for (int q = 0; q < RS_ITEMS; q++) {
-        // past the end: no digit, no count
-        const uint32_t d = i0 + 32 * q < m ? (uint32_t)(k[q] >> shift) & 0xffu : 256u;
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
-        const uint32_t seen = d < 256u ? cnt[w][d] : 0u;
+        const bool in = i0 + 32 * q < m;  // past the end: no count
+        const uint32_t d = (uint32_t)(k[q] >> shift) & 0xffu;
+        const uint32_t peers = same_digit(d) & __ballot_sync(0xffffffffu, in);
+        const uint32_t seen = cnt[w][d];
         __syncwarp();
-        if (d < 256u && (peers & below) == 0) cnt[w][d] = seen + __popc(peers);
+        if (in && (peers & below) == 0) cnt[w][d] = seen + __popc(peers);
         __syncwarp();
         at[q] = seen + __popc(peers & below);
     }
@@ -74,18 +74,23 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_pass(const uint64_t* __res
     const uint32_t ex = block_excl_scan<uint32_t>(c, &tot);
     unsigned long long all;
     const unsigned long long hx = block_excl_scan<unsigned long long>(hist[tid], &all);
+    // eight tiles back at a time: when all tiles run at once, most of them have
+    // only their own counts out yet (condensation of 2,000,000 points: 0.731 ms one
+    // by one, 0.714 so)
     unsigned long long before = 0;
-    for (int64_t t = tile - 1; t >= 0; t--) {
-        unsigned long long v = 0;
-        int polls = 0;
-        while ((v = state[256 * t + tid]) >> 62 == 0)
-            if (++polls > RS_POLLS) break;
-        if (v >> 62 == 0) {  // cannot happen while the tiles before this one run
-            s_late = 1;
-            break;
+    bool open = tile > 0;
+    for (int64_t t = tile - 1; open; t -= RS_BACK) {
+        unsigned long long v[RS_BACK];
+#pragma unroll
+        for (int j = 0; j < RS_BACK; j++) v[j] = t >= j ? state[256 * (t - j) + tid] : 2ull << 62;
+#pragma unroll
+        for (int j = 0; j < RS_BACK; j++) {
+            if (!open) continue;
+            for (int polls = 0; v[j] >> 62 == 0 && polls < RS_POLLS; polls++) v[j] = state[256 * (t - j) + tid];
+            before += v[j] & RS_VALUE;
+            open = v[j] >> 62 == 1;
+            if (v[j] >> 62 == 0) s_late = 1;  // cannot happen while the tiles before this one run
         }
-        before += v & RS_VALUE;
-        if (v >> 62 == 2) break;
     }
     if (tile > 0) state[256 * tile + tid] = 2ull << 62 | (before + c);
     first[tid] = ex;
