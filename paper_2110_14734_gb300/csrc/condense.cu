@@ -64,11 +64,22 @@ PD_D bool quantize_point(const void* __restrict__ p, int64_t j, int dt, int k, i
     bool ok = true;
     if (dt == PD_F32) {
         const float2 v = ((const float2*)p)[j];
-        const double s = ldexp(1.0, k), rb = rint((double)v.x * s), rd = rint((double)v.y * s);
-        ok = fabs(rb) < (double)COORD_LIMIT && fabs(rd) < (double)COORD_LIMIT;  // false for a NaN
-        if (ok) {
-            qx = (int64_t)rb;
-            qy = (int64_t)rd;
+        if (k <= 127) {
+            // a power of two scales a float exactly (2^k >= 1: nothing is lost below; above, infinity
+            // is rejected): single precision gives what double would, which has a 64th of its rate
+            const float s = __int_as_float((127 + k) << 23), rb = rintf(v.x * s), rd = rintf(v.y * s);
+            ok = fabsf(rb) < (float)COORD_LIMIT && fabsf(rd) < (float)COORD_LIMIT;  // false for a NaN
+            if (ok) {
+                qx = (int64_t)(int32_t)rb;
+                qy = (int64_t)(int32_t)rd;
+            }
+        } else {
+            const double s = ldexp(1.0, k), rb = rint((double)v.x * s), rd = rint((double)v.y * s);
+            ok = fabs(rb) < (double)COORD_LIMIT && fabs(rd) < (double)COORD_LIMIT;
+            if (ok) {
+                qx = (int64_t)rb;
+                qy = (int64_t)rd;
+            }
         }
     } else {
         const uchar2 v = ((const uchar2*)p)[j];

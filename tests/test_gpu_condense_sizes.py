@@ -76,3 +76,29 @@ def test_bad_and_empty_points(pd, ctx, n):
             pd.pd_condense(ctx, X, A)
         assert e.value.status == pd.PD_EINVAL
     assert pd.pd_condense(ctx, A, on)["n_nodes"] > 0  # the context stays usable
+
+
+# quantisation in single precision (a power of two scales a float exactly) up to
+# k = 127 and in double above: ties, denormals, both forms of the stage
+@pytest.mark.parametrize("k", [0, 1, 20, 100, 127, 128, 140])
+@pytest.mark.parametrize("n", [500, 9000])
+def test_quantised_coordinates_are_the_rounded_products(pd, ctx, k, n):
+    rng = np.random.default_rng(k)
+    q = rng.integers(-4000, 4000, (n, 2)) / 2.0  # whole numbers and ties
+    q[: n // 4] += rng.uniform(-0.5, 0.5, (n // 4, 2))
+    q[n // 4 : n // 3] *= 60000
+    with np.errstate(under="ignore"):
+        A = (q * 2.0 ** -k).astype(np.float32)
+    exp = np.rint(A.astype(np.float64) * 2.0 ** k).astype(np.int64)
+    exp = np.unique(exp[exp[:, 0] != exp[:, 1]], axis=0)
+    got = pd.pd_condense(ctx, torch.from_numpy(A).cuda(), torch.from_numpy(A[:0]).cuda(), 1, 0, pd.opts(coord_shift=k))
+    at = np.unique(np.stack([got["X"].cpu().numpy(), got["Y"].cpu().numpy()], 1), axis=0)
+    np.testing.assert_array_equal(at, exp)
+
+
+@pytest.mark.parametrize("v,k", [(np.inf, 20), (np.nan, 20), (3e38, 20), (1.0, 29), (1.0, 127), (2.0, 128)])
+def test_coordinates_past_the_limit_stay_rejected(pd, ctx, v, k):
+    A = torch.tensor([[0.0, v]], dtype=torch.float32).cuda()
+    with pytest.raises(pd.PDError) as e:
+        pd.pd_condense(ctx, A, A[:0], 1, 0, pd.opts(coord_shift=k))
+    assert e.value.status == pd.PD_EINVAL

@@ -54,6 +54,9 @@ def _cases():
     yield "doubling", _nodes(np.r_[g, -g, np.zeros(29, np.int64), 7 * g[:25]], np.r_[g, g, g, -3 * g[:25]])
     yield "grid", _nodes(np.repeat(np.arange(40), 40), np.tile(np.arange(40), 40))
     yield "cloud", _nodes(rng.integers(0, 1 << 20, 1500), rng.integers(0, 1 << 20, 1500))
+    # exact costs around squares, below and above where the float root alone is enough
+    d = np.array([0, 2896308, 2896309, (1 << 22) - 1, 1 << 22, (1 << 22) + 1, (1 << 26) + 3, (1 << 29) + 1, lim - 1, lim])
+    yield "squares", _nodes(np.r_[d, d], np.r_[0 * d, d % 2 + 1])
     yield "limits", _nodes(np.r_[rng.integers(-lim, lim, 120), -lim, lim], np.r_[rng.integers(-lim, lim, 120), -lim, lim])
 
 
