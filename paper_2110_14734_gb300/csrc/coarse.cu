@@ -47,19 +47,24 @@ __global__ void k_node_box(const int32_t* __restrict__ X, const int32_t* __restr
 // node's potential.  gap: half the distance between the envelopes (0 where
 // one of them is missing), a feature of the learned correction.  cpi: the
 // coarse instance's potentials (its sources, sinks, diagonal node); dsup:
-// supply of the diagonal node (|B| - |A|).
+// supply of the diagonal node (|B| - |A|).  A warp per fine node: its lanes share
+// the coarse nodes (a thread per node left the chip idle: 0.49 ms at 4,658 fine
+// and 1,200 coarse nodes, now 0.06).
 __global__ void k_ctransform_potential(const int32_t* __restrict__ S, const int32_t* __restrict__ T, int64_t nS,
                                        int64_t nT, const int32_t* __restrict__ X, const int32_t* __restrict__ Y,
                                        const int32_t* __restrict__ cS, const int32_t* __restrict__ cT, int64_t cnS,
                                        int64_t cnT, const int32_t* __restrict__ cX, const int32_t* __restrict__ cY,
                                        const int64_t* __restrict__ cpi, int64_t dsup, DiagCost dc,
                                        double* __restrict__ p, double* __restrict__ gap) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (v > nS + nT) return;
     const int64_t D = cnS + cnT;  // the coarse diagonal node
     if (v == nS + nT) {
-        p[v] = (double)cpi[D];
-        gap[v] = 0.0;
+        if (lane == 0) {
+            p[v] = (double)cpi[D];
+            gap[v] = 0.0;
+        }
         return;
     }
     const bool src = v < nS;
@@ -68,7 +73,7 @@ __global__ void k_ctransform_potential(const int32_t* __restrict__ S, const int3
     const int64_t du = cost_make(x, y, dc);
     // upper envelope over the coarse sinks, lower envelope over the coarse sources
     int64_t up = INT64_MAX, lo = INT64_MIN;
-    for (int64_t q = 0; q < cnS + cnT; q++) {
+    for (int64_t q = lane; q < cnS + cnT; q += 32) {
         const int32_t w = q < cnS ? cS[q] : cT[q - cnS];
         const int64_t l2 = cost_l2(x, y, cX[w], cY[w]);
         const int64_t g = du + cost_make(cX[w], cY[w], dc);
@@ -81,6 +86,11 @@ __global__ void k_ctransform_potential(const int32_t* __restrict__ S, const int3
             lo = t > lo ? t : lo;
         }
     }
+    for (int o = 16; o > 0; o >>= 1) {
+        up = min(up, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)up, o));
+        lo = max(lo, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)lo, o));
+    }
+    if (lane != 0) return;
     // the diagonal node's arcs: sources -> D when D demands (dsup < 0), D -> sinks when it supplies
     if (dsup < 0) up = min(up, cpi[D] + du);
     if (dsup > 0) lo = max(lo, cpi[D] - du);
@@ -149,7 +159,7 @@ pd_status ws_coarse_potentials(Ctx* c, const Front& f, const W1Prep& w, const pd
     double* dp = bufT<double>(c, B_CO_P, nt);
     double* dg = bufT<double>(c, B_CO_GAP, nt);
     if (!dp || !dg) return PD_ENOMEM;
-    k_ctransform_potential<<<grid_for(nt, 128), 128, 0, st>>>(w.S, w.T, w.nS, w.nT, f.nodes.X, f.nodes.Y, wc.S,
+    k_ctransform_potential<<<grid_for(32 * nt, 128), 128, 0, st>>>(w.S, w.T, w.nS, w.nT, f.nodes.X, f.nodes.Y, wc.S,
                                                                wc.T, wc.nS, wc.nT, cn.X, cn.Y, r.pi,
                                                                f.h.FB - f.h.FA, w.dc, dp, dg);
     pd::count_launch();

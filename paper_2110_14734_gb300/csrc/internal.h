@@ -35,7 +35,8 @@ enum Buf : int {
     B_DB_XY, B_DB_CNT, B_DB_ID, B_DB_OFF, B_DB_ROFF, B_Q_XY, B_Q_CNT, B_DB_LA, B_DB_BIG, B_DB_VAL, B_DB_PERS,
     B_MLP_P, B_MLP_M, B_MLP_V, B_MLP_WB, B_MLP_PART, B_MLP_G,  // warm-start network
     B_WS_GRID, B_WS_FEAT, B_WS_Y, B_WS_PS, B_WS_BOX, B_WS_DF, B_WS_DT, B_WS_DM, B_WS_IN, B_WS_TIN, B_WS_MIN,
-    B_WS_P, B_WS_ROWK, B_WS_COLK, B_WS_ARCS, B_WS_COST, B_WS_RS, B_WS_RT, B_WS_RC, B_WS_COMP, B_WS_CSIZE, B_WS_CSUM,
+    B_WS_P, B_WS_PD, B_WS_ROWK, B_WS_COLK, B_WS_ARCS, B_WS_KEY, B_WS_KEY2, B_WS_VAL, B_WS_VAL2, B_WS_OUT, B_WS_COST,
+    B_WS_RS, B_WS_RT, B_WS_COMP, B_WS_CSIZE, B_WS_CSUM,
     B_SP_ORD, B_SP_ORD2, B_SP_SEG, B_SP_SEG2, B_SP_HI, B_SP_HI2, B_SP_NUM, B_SP_NUM2,  // split tree
     B_SP_BB, B_SP_REPK, B_SP_REPN, B_SP_FLAG, B_SP_RANK, B_SP_X, B_SP_Y, B_SP_CA, B_SP_CB, B_SP_CODE, B_SP_POS,
     B_CO_BOX, B_CO_P, B_CO_P2, B_CO_GAP,  // coarse-solve warm start

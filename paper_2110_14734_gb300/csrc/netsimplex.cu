@@ -13,9 +13,9 @@
 // re-roots the cut path.  The spanning tree is kept as an explicit preorder
 // array (ord, pos, size), so re-hanging the cut subtree is a handful of
 // contiguous segment moves done by all threads plus one potential shift -- no
-// pointer chasing over the subtree.  Up to 9216 nodes the node arrays live in
-// shared memory with 16-bit indices (24 bytes per node); larger trees keep
-// 32-bit arrays in global memory.
+// pointer chasing over the subtree.  Up to about 9,175 nodes all node arrays live
+// in shared memory with 16-bit indices (24 bytes per node), up to about 27,500
+// some of them; larger trees keep 32-bit arrays in global memory.
 //
 // Big-M start: node i has an artificial arc to (supply >= 0) or from (< 0) an
 // extra root, of cost big (more than any path of real arcs) plus an optional
