@@ -683,11 +683,11 @@ __global__ void k_fill_u64(unsigned long long* p, int64_t n, unsigned long long 
 }
 
 // Grid geometry of one side with box b (xmin, xmax, ymin, ymax) and n nodes:
-// about RW_CELLS cells a node, at most twice as many and 64.
-static RwGrid rw_grid(const int64_t* b, int64_t n, int64_t base) {
+// about `pair` cells for two nodes, at most twice as many and 64.
+static RwGrid rw_grid(const int64_t* b, int64_t n, int64_t base, int64_t pair) {
     RwGrid g{};
     const int64_t W = b[1] - b[0], H = b[3] - b[2];
-    const int64_t want = std::min<int64_t>(RW_CELLS * n, int64_t(1) << 29);  // both grids below 2^32 cells
+    const int64_t want = std::min<int64_t>(std::max<int64_t>(pair * n / 2, 1), int64_t(1) << 29);  // both grids below 2^32 cells
     const double cells = (double)want;
     int64_t hs = (int64_t)ceil(sqrt((double)(W + 1) * (double)(H + 1) / cells));
     hs = std::max<int64_t>(hs, 1);
@@ -720,15 +720,24 @@ static pd_status rwmd_grid(Ctx* c, const Hats& h, DiagCost dc, unsigned long lon
     int64_t hb[8];
     PD_TRY_CUDA(c, cudaMemcpyAsync(hb, box, sizeof(hb), cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
-    const RwGrid g0 = rw_grid(hb, h.nA, 0);
-    const RwGrid g1 = rw_grid(hb + 4, h.nB, (int64_t)g0.gw * g0.gh);
-    const int64_t cells = g1.base + (int64_t)g1.gw * g1.gh;
-    uint32_t* cell = bufT<uint32_t>(c, B_RW_START, cells);
-    uint32_t* part = bufT<uint32_t>(c, B_SCAN_PART, scan_tiles(cells) + 1);
+    RwGrid g0, g1;
+    int64_t cells = 0;
+    uint32_t* cell = nullptr;
     int2* pts = bufT<int2>(c, B_RW_PTS, n);
     uint32_t* id = bufT<uint32_t>(c, B_RW_CUR, n);
     int32_t* list = bufT<int32_t>(c, B_RW_LIST, n);
-    if (!cell || !part || !pts || !id || !list) return PD_ENOMEM;
+    if (!pts || !id || !list) return PD_ENOMEM;
+    for (int64_t pair = 2 * RW_CELLS; pair > 0; pair /= 4) {  // fewer cells if memory is short
+        g0 = rw_grid(hb, h.nA, 0, pair);
+        g1 = rw_grid(hb + 4, h.nB, (int64_t)g0.gw * g0.gh, pair);
+        cells = g1.base + (int64_t)g1.gw * g1.gh;
+        if (pair > 1 && beyond_cap(c, 4 * cells)) continue;
+        cell = bufT<uint32_t>(c, B_RW_START, cells);
+        if (cell) break;
+        if (pair / 4 > 0) c->err.clear();
+    }
+    uint32_t* part = bufT<uint32_t>(c, B_SCAN_PART, scan_tiles(cells) + 1);
+    if (!cell || !part) return PD_ENOMEM;
     PD_TRY_CUDA(c, cudaMemsetAsync(cell, 0, sizeof(uint32_t) * cells, st));
     PD_TRY_CUDA(c, cudaMemsetAsync(nl, 0, 2 * sizeof(int), st));
     k_rw_hist<<<grid_for(n, 256), 256, 0, st>>>(h.X, h.Y, h.nA, n, g0, g1, cell); pd::count_launch();

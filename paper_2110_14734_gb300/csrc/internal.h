@@ -114,6 +114,9 @@ T* bufT(Ctx* c, Buf id, int64_t n) {
     return (T*)buf(c, id, sizeof(T) * (size_t)(n > 0 ? n : 1));
 }
 
+// Whether scratch of this size that only saves time is too much for the context's cap.
+inline bool beyond_cap(const Ctx* c, int64_t bytes) { return c->cap && (uint64_t)bytes > c->cap / 16; }
+
 pd_status fail(Ctx* c, pd_status st, const std::string& msg);
 // n events of the context from the first-th (a range per user: two stages may be under way at once).
 constexpr int EV_FRONT = 0, EV_NETWORK = 4, EV_SIMPLEX = 8, EV_BOUNDS = 10, EV_READY = 12;

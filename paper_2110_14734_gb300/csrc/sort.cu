@@ -171,16 +171,25 @@ pd_status sort_u64(Ctx* c, uint64_t*& keys, uint64_t*& keys_alt, uint32_t*& vals
         return PD_OK;
     }
     const int passes = radix_passes(bits);
-    const int64_t tiles = radix_tiles(n), words = radix_words(n, bits);
-    unsigned long long* w = bufT<unsigned long long>(c, B_RS_COUNTS, words);
+    const int64_t tiles = radix_tiles(n);
+    int64_t words = radix_words(n, bits);
+    unsigned long long* w = beyond_cap(c, 8 * words) ? nullptr : bufT<unsigned long long>(c, B_RS_COUNTS, words);
+    const bool shared = !w;  // short of memory: all passes use one set of tile states, cleared in between
+    if (shared) {
+        c->err.clear();
+        words -= 256 * (passes - 1) * tiles;
+        w = bufT<unsigned long long>(c, B_RS_COUNTS, words);
+    }
     if (!w) return PD_ENOMEM;
     unsigned long long *hist = w, *ticket = w + 256 * RS_MAXPASS, *state = ticket + RS_MAXPASS;
     PD_TRY_CUDA(c, cudaMemsetAsync(w, 0, sizeof(unsigned long long) * words, st));
     k_radix_counts<<<(unsigned)std::min<int64_t>(tiles, 4 * std::max(c->sm_count, 1)), RS_THREADS, 0, st>>>(keys, n, passes, hist);
     pd::count_launch();
     for (int p = 0; p < passes; p++) {
+        if (shared && p > 0) PD_TRY_CUDA(c, cudaMemsetAsync(state, 0, 256 * tiles * sizeof(unsigned long long), st));
         k_radix_pass<<<(unsigned)tiles, RS_THREADS, 0, st>>>(keys, vals, keys_alt, vals ? vals_alt : nullptr, n, 8 * p,
-                                                            hist + 256 * p, ticket + p, state + 256 * tiles * p,
+                                                            hist + 256 * p, ticket + p,
+                                                            state + (shared ? 0 : 256 * tiles * p),
                                                             c->h_small + H_SORT_LATE); pd::count_launch();
         std::swap(keys, keys_alt);
         std::swap(vals, vals_alt);

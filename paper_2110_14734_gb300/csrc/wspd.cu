@@ -690,6 +690,7 @@ static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, const int2*
     const int64_t warps = (int64_t)blocks * WS_WARPS;
     // room for handed-on pairs: the more, the better the balance; less will do
     int64_t cap = std::min<int64_t>(int64_t(1) << 27, std::max<int64_t>(int64_t(1) << 16, 64 * (tr.N - 1)));  // even
+    while (cap > (int64_t(1) << 16) && beyond_cap(c, 2 * sizeof(int2) * cap)) cap = cap / 8 * 2;
     int2* out[2];
     static std::atomic<uint64_t> done{0};
     if (arcs) PD_TRY(smem_limit(c, done, (const void*)k_ws_walk<true>, sizeof(int2) * WS_WARPS * WS_OUT));
@@ -806,7 +807,14 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
             // if they are more, the walk has counted them and the second one stores them
             int64_t room = 0;
             for (int pass = 0; pass < 2; pass++) {
-                arcs = bufT<uint64_t>(c, B_ARCKEY, 2 * (pass ? pairs : 32 * N) + 2 * N + 1);
+                const int64_t keys = 2 * (pass ? pairs : 32 * N) + 2 * N + 1;
+                const bool guess = pass == 0 && !beyond_cap(c, 8 * keys);
+                arcs = guess || pass ? bufT<uint64_t>(c, B_ARCKEY, keys) : nullptr;
+                if (!arcs && pass == 0) {  // no room for a guess: counted first
+                    c->err.clear();
+                    PD_TRY(ws_walk(c, tr, rec, leaf, s, hb, false, nullptr, 0, &pairs, st));
+                    continue;
+                }
                 if (!arcs) return PD_ENOMEM;
                 room = ((int64_t)(c->bytes[B_ARCKEY] / sizeof(uint64_t)) - (2 * N + 1)) / 2;
                 if (pass) PD_TRY_CUDA(c, cudaMemsetAsync(words, 0, 3 * sizeof(unsigned long long), st));
