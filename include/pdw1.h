@@ -85,11 +85,14 @@ typedef struct {
     int64_t update_every;   /* relabels between global price updates (0 = number of nodes, -1 = never) */
     int32_t seq_threshold;  /* cost scaling: at most this many active nodes, one block finishes them (-1 = 64) */
     int32_t solver;         /* 0 = network simplex (default), 1 = cost scaling with push/relabel */
-    int64_t ns_block;       /* network simplex pricing block in arcs (0 = max(8192, sqrt(arcs))) */
+    int64_t ns_block;       /* network simplex pricing block in arcs (0 = 16384 on a transportation
+                               form with 32-bit potentials, else max(8192, sqrt(arcs)); what shared
+                               memory holds of it is priced at a time) */
     int32_t ns_transport;   /* W1 only: 1 = try the transportation form with its certificate first when it
                                has at most twice the sparse network's arcs (default); 2 = whenever its
                                arcs fit the simplex (< 2^31); 0 = solve the sparse network itself */
-    int32_t ns_smem;        /* network simplex: 1 = hot node arrays in shared memory when they fit (default) */
+    int32_t ns_smem;        /* network simplex: 1 = hot node arrays in shared memory when they fit, and
+                               32-bit potentials when they hold them (default); 0 = neither */
     int32_t batch_slots;    /* pairs per simplex launch of pd_w1_approx_batch and pd_nn_search
                                (0 = twice the number of SMs) */
     int32_t batch_threads;  /* pd_w1_approx_batch: host threads preprocessing pairs (0 = 8) */
@@ -110,7 +113,7 @@ typedef struct {
                                condensed onto a coarser lattice (cell max(2 G, node box / warm_cells)),
                                mapped to the fine nodes by the coarse optimum's c-transforms
                                (the midpoint of the upper and lower envelope) */
-    int32_t ns_walk;        /* network simplex, trees in shared memory: the two half-cycles of a pivot are
+    int32_t ns_walk;        /* network simplex, 64-bit potentials, trees in shared memory: the two half-cycles of a pivot are
                                followed up the tree by two lanes when neither side is longer than this
                                many nodes, else found by a scan of the whole preorder by the CTA
                                (-1 = the autotuned value, else 0; 0 = always the scan; at most 512) */
@@ -299,8 +302,8 @@ pd_status pd_w1_sparsify_count(pd_ctx* ctx, pd_diagram A, pd_diagram B, double e
  * the number of SMs) pairs: host worker threads (opts->batch_threads) run the
  * preprocessing of the wave's pairs, each on its own stream after the work
  * already queued on `stream`; then the network simplex solves of the wave
- * share one persistent launch (one CTA per SM takes the pairs, largest
- * first); then each pair's certificate runs.
+ * share one persistent launch per form of the kernel (one CTA per SM, or two
+ * when more pairs than SMs fit half of one, takes the pairs, largest first); then each pair's certificate runs.
  * A and B: host arrays of `count` descriptors; out: host array of `count`
  * results (ns_kernel_ms and stage_ms[6] include the wave's shared launch).
  * Device memory: one buffer set per slot, grown on demand and kept by the

@@ -919,7 +919,7 @@ pd_status batch_solve(Ctx* c, const pd_diagram* A, const pd_diagram* B, int64_t 
             break;
         }
         // ---- the wave as one CUDA graph: records up, one persistent simplex
-        // launch (one CTA per SM takes the pairs, largest first), every pair's
+        // launch per form of the kernel (its CTAs take the pairs, largest first), every pair's
         // certificate in one launch, records and certificate counts down
         hin.clear();
         jobs.clear();
