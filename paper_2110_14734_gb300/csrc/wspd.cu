@@ -282,7 +282,10 @@ __global__ void k_certify_batch(const CertJob* __restrict__ jobs, unsigned long 
 // Balance.  Initial pairs (one per internal node) differ by many orders of
 // magnitude in the pairs below them, so a warp that has walked `budget` steps
 // on its chunk hands what is left on its stack to the next launch, where other
-// warps take it up.
+// warps take it up.  Once the room for these is half full, only every eighth
+// time: used up early, it would leave the largest stacks to single warps
+// (mixture points, counts: 50,000 + 50,000 at eps 0.01 167 -> 17 ms, 100,000 + 100,000
+// at 0.02 773 -> 30, 250,000 + 250,000 at 0.05 706 -> 51).
 //
 // Measured (pd_w1_sparsify_count's WSPD stage, mixture points, s = 167): 1,000,000
 // + 1,000,000 points 493 -> 161 ms, 100,000 + 100,000 23 -> 7.2 ms, against
@@ -452,6 +455,7 @@ __global__ void __launch_bounds__(32 * WS_WARPS) k_ws_walk(const int2* __restric
     };
     int h = 0;  // height of the stack
     int64_t steps = 0;
+    int tight = 0;  // budgets used up while the room was more than half full: every eighth hands on
     for (;;) {
         int2 p = make_int2(0, 0);
         bool on;
@@ -510,7 +514,10 @@ __global__ void __launch_bounds__(32 * WS_WARPS) k_ws_walk(const int2* __restric
         if (++steps > budget && h > 0) {
             // to the next launch, as far as it still has room
             unsigned long long at2 = cap;
-            if (lane == 0 && *(volatile unsigned long long*)&lv[1] < cap) at2 = atomicAdd(&lv[1], (unsigned long long)h);
+            if (lane == 0) {
+                const unsigned long long used = *(volatile unsigned long long*)&lv[1];
+                if (used < cap && (used < cap / 2 || (++tight & 7) == 0)) at2 = atomicAdd(&lv[1], (unsigned long long)h);
+            }
             at2 = __shfl_sync(0xffffffffu, at2, 0);
             const int give = at2 >= cap ? 0 : (int)min((unsigned long long)h, cap - at2);
             for (int q = lane; q < give; q += 32) Fn[at2 + q] = st[h - give + q];
