@@ -185,7 +185,6 @@ static bool ctx_init(Ctx* c, int device, size_t cap) {
         cudaGetLastError();
         return false;
     }
-    memset(c->h_small, 0, 64 * sizeof(int64_t));
     return true;
 }
 

@@ -370,7 +370,6 @@ pd_status stage_condense0(Ctx* c, const DevDiag& A, const DevDiag& B, int k, Hat
     PD_TRY_CUDA(c, cudaGetLastError());
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, sizeof(int64_t) * S_COUNT, cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
-    PD_TRY(sort_done(c));
     int64_t M = h[S_M];
     out->nA = out->FB > 0 ? h[S_NA] : M;
     out->nB = M - out->nA;
@@ -863,7 +862,7 @@ __global__ void k_cell_accum(const uint64_t* __restrict__ key, const uint32_t* _
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int64_t j = idx[i] + ((i == 0 || key[i - 1] != key[i]) ? 1 : 0) - 1;
-    const uint32_t v = min(val[i], (uint32_t)(n - 1));  // in bounds even after a sort that gave up
+    const uint32_t v = val[i];
     atomicAdd((unsigned long long*)((int64_t)v < nA ? &CA[j] : &CB[j]), (unsigned long long)cnt[v]);
 }
 
@@ -882,7 +881,7 @@ __global__ void k_node_gather(const uint64_t* __restrict__ key, const uint32_t* 
                               uint64_t* __restrict__ OC) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    const uint32_t v = min(val[i], (uint32_t)(N - 1));  // in bounds even after a sort that gave up
+    const uint32_t v = val[i];
     OX[i] = NX[v];
     OY[i] = NY[v];
     OA[i] = CA[v];
@@ -1058,7 +1057,6 @@ pd_status stage_condense_delta(Ctx* c, const Hats& hats, int64_t G, int64_t P, u
     PD_TRY_CUDA(c, cudaGetLastError());
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, sizeof(int64_t) * S_COUNT, cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
-    PD_TRY(sort_done(c));
     if (hs[S_ERR]) return fail(c, PD_EINVAL, "condensed node coordinate outside (-2^30, 2^30)");
     int64_t N = hs[S_N];
     int bm = bits_for((uint64_t)(hs[S_NMXX] - hs[S_NMNX]));

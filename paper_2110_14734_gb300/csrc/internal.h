@@ -247,12 +247,11 @@ int32_t tuned_walk(const Ctx* c, int64_t M);  // the walk limit (16 when none wa
 
 // Stable radix sort of keys (and vals, may be null) by the low `bits` bits with
 // context scratch; the result is in keys / vals, which may have changed places
-// with the alternates.  Needs n < 2^32 when there are values.
+// with the alternates.  Needs n < 2^32 when there are values.  polls: how often a
+// tile looks for another's counts (microseconds, as a rule) before it counts for itself.
+constexpr int SORT_POLLS = 1 << 12;
 pd_status sort_u64(Ctx* c, uint64_t*& keys, uint64_t*& keys_alt, uint32_t*& vals, uint32_t*& vals_alt, int64_t n,
-                   int bits, cudaStream_t st);
-// After the stream has been synchronised: whether every sort since then ended.
-pd_status sort_done(Ctx* c);
-constexpr int H_SORT_LATE = 63;  // its word of h_small
+                   int bits, cudaStream_t st, int polls = SORT_POLLS);
 pd_status scan_i64(Ctx* c, const int64_t* in, int64_t* out, int64_t n, int64_t* total_dev, cudaStream_t st);
 
 }  // namespace pd

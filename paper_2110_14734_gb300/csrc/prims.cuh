@@ -178,7 +178,9 @@ cudaError_t exclusive_scan(const T* in, T* out, int64_t n, T* part, T* total_dev
 // tiles before it by decoupled look-back (Merrill & Garland: a tile first
 // publishes its own counts, then their running sum; tile numbers are tickets, so
 // the tiles looked back at have started), orders the keys in shared memory and
-// writes them in runs.  A pass moves each key once in and once out; what bounds it
+// writes them in runs.  Should a tile looked back at not have published after the
+// bounded wait, its digits are counted from the keys, which this pass only
+// reads: the sort never waits without end and never ends unsorted.  A pass moves each key once in and once out; what bounds it
 // is the ranking and the look-back's latency: 2,000,000 64-bit keys 26 us a pass
 // (5 at the copy rate), two tiles an SM at a time.
 //
@@ -205,7 +207,6 @@ constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_MAXPASS = 8;
 constexpr uint64_t RS_VALUE = (1ull << 62) - 1;  // of a state word: flag << 62 | value
 constexpr int RS_BACK = 8;                                // tiles looked back at a time
-constexpr int RS_POLLS = 1 << 22;                // bound of a look-back wait (it is microseconds)
 
 inline int64_t radix_tiles(int64_t n) { return (n + RS_TILE - 1) / RS_TILE; }
 inline int radix_passes(int bits) { return (bits + 7) / 8; }
@@ -217,14 +218,14 @@ inline int64_t radix_words(int64_t n, int bits) {
 // Digit counts of all passes.
 __global__ void __launch_bounds__(RS_THREADS) k_radix_counts(const uint64_t* __restrict__ keys, int64_t n, int passes,
                                                              unsigned long long* __restrict__ hist);
-// One pass; vin / vout may be null.  *late (host memory) is set when a wait gave up.
+// One pass; vin / vout may be null.  polls: bound of a look-back wait.
 __global__ void __launch_bounds__(RS_THREADS) k_radix_pass(const uint64_t* __restrict__ kin,
                                                            const uint32_t* __restrict__ vin,
                                                            uint64_t* __restrict__ kout, uint32_t* __restrict__ vout,
                                                            int64_t n, int shift,
                                                            const unsigned long long* __restrict__ hist,
                                                            unsigned long long* ticket, volatile unsigned long long* state,
-                                                           int64_t* late);
+                                                           int polls);
 
 // ---- sort of one block of CS_THREADS threads
 

@@ -869,7 +869,6 @@ pd_status stage_solve(Ctx* c, const pd_network& net, const pd_opts& o, SolveStat
     PD_TRY(sort_u64(c, xkey, xkey2, xval, xval2, m, 2 * hb, st));
     PD_TRY_CUDA(c, cudaMemcpyAsync(c->h_small, sm, 3 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
-    PD_TRY(sort_done(c));
     if (c->h_small[0] & 0xffffffff) return fail(c, PD_EOVERFLOW, "arc cost outside [0, 2^31)");
     int64_t cmax = c->h_small[1];
     {

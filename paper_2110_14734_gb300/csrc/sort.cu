@@ -21,25 +21,28 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_counts(const uint64_t* __r
         if (h[p][threadIdx.x]) atomicAdd(&hist[256 * p + threadIdx.x], (unsigned long long)h[p][threadIdx.x]);
 }
 
+// Keys of the whole tile t with digit d.
+__device__ __noinline__ uint32_t tile_count(const uint64_t* __restrict__ keys, int64_t t, int shift, uint32_t d) {
+    uint32_t c = 0;
+    for (int i = 0; i < RS_TILE; i++) c += ((uint32_t)(keys[t * RS_TILE + i] >> shift) & 0xffu) == d;
+    return c;
+}
+
 __global__ void __launch_bounds__(RS_THREADS) k_radix_pass(const uint64_t* __restrict__ kin,
                                                            const uint32_t* __restrict__ vin,
                                                            uint64_t* __restrict__ kout, uint32_t* __restrict__ vout,
                                                            int64_t n, int shift,
                                                            const unsigned long long* __restrict__ hist,
                                                            unsigned long long* ticket, volatile unsigned long long* state,
-                                                           int64_t* late) {
+                                                           int polls) {
     __shared__ uint32_t cnt[RS_WARPS][256];
     __shared__ uint64_t skey[RS_TILE];
     __shared__ int64_t base[256];  // of a digit: output index less index in the tile's order
     __shared__ uint32_t first[256];
     __shared__ int64_t s_tile;
-    __shared__ int s_late;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t below = (1u << lane) - 1u;
-    if (tid == 0) {
-        s_tile = (int64_t)atomicAdd(ticket, 1ull);
-        s_late = 0;
-    }
+    if (tid == 0) s_tile = (int64_t)atomicAdd(ticket, 1ull);
 #pragma unroll
     for (int q = 0; q < RS_WARPS; q++) cnt[q][tid] = 0;
     __syncthreads();
@@ -86,20 +89,16 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_pass(const uint64_t* __res
 #pragma unroll
         for (int j = 0; j < RS_BACK; j++) {
             if (!open) continue;
-            for (int polls = 0; v[j] >> 62 == 0 && polls < RS_POLLS; polls++) v[j] = state[256 * (t - j) + tid];
+            for (int q = 0; v[j] >> 62 == 0 && q < polls; q++) v[j] = state[256 * (t - j) + tid];
+            if (v[j] >> 62 == 0) v[j] = 1ull << 62 | tile_count(kin, t - j, shift, tid);  // only the last tile is short
             before += v[j] & RS_VALUE;
             open = v[j] >> 62 == 1;
-            if (v[j] >> 62 == 0) s_late = 1;  // cannot happen while the tiles before this one run
         }
     }
     if (tile > 0) state[256 * tile + tid] = 2ull << 62 | (before + c);
     first[tid] = ex;
     base[tid] = (int64_t)(hx + before) - (int64_t)ex;
     __syncthreads();
-    if (s_late) {
-        if (tid == 0) *(volatile int64_t*)late = 1;
-        return;
-    }
 #pragma unroll
     for (int q = 0; q < RS_ITEMS; q++)
         if (i0 + 32 * q < m) {
@@ -161,7 +160,7 @@ __global__ void __launch_bounds__(CS_THREADS) k_sort_small(uint64_t* __restrict_
 // Above these sizes a block's sort (1,024 threads on one SM) takes longer than
 // the long sort's launches.
 pd_status sort_u64(Ctx* c, uint64_t*& keys, uint64_t*& keys_alt, uint32_t*& vals, uint32_t*& vals_alt, int64_t n,
-                   int bits, cudaStream_t st) {
+                   int bits, cudaStream_t st, int polls) {
     if (n <= 1 || bits <= 0) return PD_OK;
     if (n <= CS_MAX) {
         static std::atomic<uint64_t> done{0};
@@ -190,18 +189,12 @@ pd_status sort_u64(Ctx* c, uint64_t*& keys, uint64_t*& keys_alt, uint32_t*& vals
         k_radix_pass<<<(unsigned)tiles, RS_THREADS, 0, st>>>(keys, vals, keys_alt, vals ? vals_alt : nullptr, n, 8 * p,
                                                             hist + 256 * p, ticket + p,
                                                             state + (shared ? 0 : 256 * tiles * p),
-                                                            c->h_small + H_SORT_LATE); pd::count_launch();
+                                                            polls); pd::count_launch();
         std::swap(keys, keys_alt);
         std::swap(vals, vals_alt);
     }
     PD_TRY_CUDA(c, cudaGetLastError());
     return PD_OK;
-}
-
-pd_status sort_done(Ctx* c) {
-    if (c->h_small[H_SORT_LATE] == 0) return PD_OK;
-    c->h_small[H_SORT_LATE] = 0;
-    return fail(c, PD_ETIMEOUT, "radix sort: a wait ran out");
 }
 
 }  // namespace pd

@@ -333,7 +333,6 @@ pd_status ns_warm_tree(Ctx* c, NSPrep* prep, const double* p, int64_t max_residu
         order.resize((size_t)nc);
         PD_TRY_CUDA(c, cudaMemcpyAsync(order.data(), out, sizeof(int2) * nc, cudaMemcpyDeviceToHost, st));
         PD_TRY_CUDA(c, cudaStreamSynchronize(st));
-        PD_TRY(sort_done(c));
         bool moved = false;
         for (const int2& o : order) {
             if (o.x < 0) break;

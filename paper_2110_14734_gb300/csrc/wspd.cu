@@ -865,7 +865,6 @@ pd_status stage_network(Ctx* c, const pd_nodes& nodes, int64_t s, pd_network* ou
     uint32_t *none = nullptr, *none2 = nullptr;
     PD_TRY(sort_u64(c, arcs, alt, none, none2, ntot, kb, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
-    PD_TRY(sort_done(c));
     int64_t na = h[0], nb = h[1], FA = h[2], FB = h[3];
     int64_t m = narcs + na + nb + 1;
     int64_t nrows = N + 2;
