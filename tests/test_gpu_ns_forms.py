@@ -1,0 +1,61 @@
+"""The 64-bit simplex kernel's forms of an instance and the waves that mix them
+with the 32-bit kernel's.  Optima are integers: equality with the 32-bit kernel,
+closed forms or single solves."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2110_14734_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pd():
+    from paper_2110_14734_gb300 import build
+    build.build()
+    from paper_2110_14734_gb300 import pdw1
+    return pdw1
+
+
+@pytest.fixture(scope="module")
+def ctx(pd):
+    c = pd.pd_create(0)
+    yield c
+    c.close()
+
+
+def _circulant(n, k, cost, supply, seed=0):
+    """Network of n nodes with arcs to the same k distances from every node."""
+    d = np.random.default_rng(seed).choice(n - 1, k, replace=False) + 1
+    a = dict(row_ptr=k * np.arange(n + 1), head=np.sort((np.arange(n)[:, None] + d) % n, 1).reshape(-1).astype(np.int32),
+             cost=np.broadcast_to(np.asarray(cost, np.int64), (n * k,)).copy(), supply=np.asarray(supply, np.int64))
+    return {x: torch.from_numpy(v).cuda() for x, v in a.items()}
+
+
+# arc lists around whole chunks (64) and pricing blocks, which may end inside the
+# list, at its padding or among the artificial arcs
+@pytest.mark.parametrize("n,k", [(16, 3), (64, 1), (64, 63), (1024, 8), (1025, 8), (2049, 5)])
+@pytest.mark.parametrize("block", [0, 1, 8, 1000])
+def test_packed_lists(pd, ctx, n, k, block):
+    rng = np.random.default_rng(n * k)
+    sup = rng.integers(-5, 6, n)
+    sup[-1] -= sup.sum()
+    net = _circulant(n, k, rng.integers(0, 1000, n * k), sup, n * k)
+
+    def solve(**kw):
+        try:
+            return pd.pd_mcf_solve(ctx, net, pd.opts(**kw))[0]
+        except pd.PDError as e:
+            return e.status
+
+    assert solve(ns_smem=0, ns_block=block) == solve(ns_block=block) == solve()
+
+
+# One look at every arc (no supplies: the start is optimal).  0.60 ms; 1.46 with
+# the ends' form looked up arc by arc, 1.14 with tails and heads apart.
+def test_packed_lists_are_priced_at_their_rate(pd, ctx):
+    n, k = 9000, 222
+    net = _circulant(n, k, 1 << 26, np.zeros(n))
+    ms = [pd.pd_mcf_solve(ctx, net)[1]["ns_kernel_ms"] for _ in range(5)]
+    assert min(ms) < 1.1, ms
