@@ -1492,9 +1492,9 @@ pd_status ns_prepare_w1(Ctx* c, const pd_nodes& nodes, int64_t n_arcs, int64_t m
     int32_t* T = bufT<int32_t>(c, B_TR_T, small ? N : nT);
     int64_t* sup = bufT<int64_t>(c, B_TR_SUP, small ? N + 1 : nt);
     const int64_t mx = mt - mst;
-    // rows padded to whole steps of simplex32.cu, unless the padding alone would take the arc ids past 2^31
-    int64_t ld = (nT + 7) & ~(int64_t)7;
-    if (nS * ld + mx >= (int64_t(1) << 31) - 1 - 8 * NS_THREADS) ld = nT;
+    // rows padded to whole steps of simplex32.cu where that kernel can hold the nodes: for
+    // the other one padding is nothing but arcs to skip, and near 2^31 arcs too many
+    const int64_t ld = o.ns_smem != 0 && s32_layout(nt + 1) ? (nT + 7) & ~(int64_t)7 : nT;
     mst = nS * ld;
     mt = mst + mx;
     const bool packed = nt + 1 < 65535;

@@ -59,3 +59,18 @@ def test_packed_lists_are_priced_at_their_rate(pd, ctx):
     net = _circulant(n, k, 1 << 26, np.zeros(n))
     ms = [pd.pd_mcf_solve(ctx, net)[1]["ns_kernel_ms"] for _ in range(5)]
     assert min(ms) < 1.1, ms
+
+
+# 46,337 x 46,337 arcs and the nodes just fit 31-bit arc ids; rows padded to 46,344 would not
+def test_largest_matrix_is_taken(pd, ctx):
+    n = 46337
+    at = np.random.default_rng(3).permutation(1 << 17)[: 2 * n]
+    pts = np.stack([at // 512, at // 512 + 1 + at % 512], 1).astype(np.float32) / 64
+    A, B = (torch.from_numpy(np.ascontiguousarray(p)).cuda() for p in (pts[:n], pts[n:]))
+    c = pd.pd_create(0)
+    try:
+        with pytest.raises(pd.PDError) as e:  # one pivot is enough to see that it was taken
+            pd.pd_w1_approx(c, A, B, 0.5, pd.opts(condense=0, ns_transport=2, warm_start=0, max_rounds=1))
+    finally:
+        c.close()
+    assert e.value.status == pd.PD_ETIMEOUT
