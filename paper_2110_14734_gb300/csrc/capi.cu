@@ -218,6 +218,10 @@ static void wave_free(Ctx* c) {
     if (c->wave_stream) cudaStreamDestroy(c->wave_stream);
     for (cudaEvent_t& e : c->wave_ev)
         if (e) cudaEventDestroy(e);
+    for (cudaStream_t& s : c->wave_side)
+        if (s) cudaStreamDestroy(s);
+    for (cudaEvent_t& e : c->wave_join)
+        if (e) cudaEventDestroy(e);
     for (cudaEvent_t& e : c->ev)
         if (e) cudaEventDestroy(e);
     if (c->wave_pin) cudaFreeHost(c->wave_pin);

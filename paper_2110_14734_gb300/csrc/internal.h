@@ -94,6 +94,10 @@ struct Ctx {
     cudaGraphExec_t wave_exec = nullptr;
     cudaStream_t wave_stream = nullptr;
     cudaEvent_t wave_ev[3] = {nullptr, nullptr, nullptr};
+    // branches of the wave's graph (the last one is on wave_stream), their fork and joins
+    static constexpr int WAVE_SIDES = 7;
+    cudaStream_t wave_side[WAVE_SIDES] = {};
+    cudaEvent_t wave_join[WAVE_SIDES + 1] = {};
     // the stages' timing events, made when first used: creating and destroying
     // them costs about 10 us a pair of calls, under a lock that all threads share
     cudaEvent_t ev[13] = {};

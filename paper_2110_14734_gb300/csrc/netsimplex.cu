@@ -972,9 +972,10 @@ struct NSLaunch {
     int first[S32_CLASSES] = {}, num[S32_CLASSES] = {};  // stretches of the order
     int own64 = 0;                                       // instances of k_netsimplex
     size_t smem64 = 0;
-    int grid64 = 0;
+    int most64 = 0;  // its CTAs the device holds at a time
+    int grid64(int instances) const { return std::min(instances, most64); }
 };
-constexpr int NS_COUNTERS = S32_CLASSES + 1;  // instance counters behind the order
+constexpr int NS_COUNTERS = S32_CLASSES + 2;  // instance counters behind the order
 
 // Fills order (count indices, by class, largest instances first -- nodes, then
 // arcs, ties by index -- and the zeroed counters) and *L.
@@ -1017,7 +1018,7 @@ static pd_status ns_plan(Ctx* c, const NSInst* h, int count, int32_t* order, NSL
     int per_sm = 0;
     PD_TRY_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_netsimplex, NS_THREADS, L->smem64));
     if (per_sm < 1) return fail(c, PD_ECAPACITY, "network simplex kernel does not fit on an SM");
-    L->grid64 = std::min(count, per_sm * std::max(c->sm_count, 1));
+    L->most64 = per_sm * std::max(c->sm_count, 1);
     return PD_OK;
 }
 
@@ -1046,7 +1047,7 @@ pd_status ns_run(Ctx* c, const NSInst* h, int count, NSInst* d, NSInst* r, cudaS
                     pd::count_launch();
                 }
         } else {
-            k_netsimplex<<<L.grid64, NS_THREADS, L.smem64, st>>>(d, dord, count, dord + count + S32_CLASSES);
+            k_netsimplex<<<L.grid64(count), NS_THREADS, L.smem64, st>>>(d, dord, count, dord + count + S32_CLASSES);
             pd::count_launch();
         }
         if (le == cudaSuccess) le = cudaGetLastError();
@@ -1080,6 +1081,42 @@ struct WaveLayout {
 
 constexpr int WAVE_CERT_BLOCKS = 8;  // blocks per pair of the batched certificate (grid-stride)
 
+// Captures the wave's simplex launches: a branch per form of the kernel present, so
+// that a few large instances and many small ones share the device, then
+// k_netsimplex over what was handed back.  Branches start with the forms that take
+// longest; their streams' priorities keep the others' CTAs from filling every SM
+// first.  One launch after the other, 20 pairs of 3,500 uniform points beside 20 a
+// hundred times as far apart (k_netsimplex) took 238 ms, so 188, the latter alone
+// 187; 290 pairs of 1,500 points beside 8 of 100,000 lower-star points 337 ms of
+// simplex, so 311, the 8 alone 311.
+static cudaError_t ns_capture_wave(Ctx* c, const NSLaunch& L, int count, NSInst* d, int32_t* dord, cudaStream_t gs) {
+    static constexpr int order[] = {-1, 5, 4, 3, 2, 1, 0, S32_HALF};  // -1: k_netsimplex
+    static_assert(sizeof(order) / sizeof(order[0]) == S32_CLASSES + 1 && Ctx::WAVE_SIDES == S32_CLASSES, "every form once");
+    int form[S32_CLASSES + 1], n = 0;
+    for (int k : order)
+        if (k < 0 ? L.own64 > 0 : L.num[k] > 0) form[n++] = k;
+    cudaError_t e = n > 1 ? cudaEventRecord(c->wave_join[Ctx::WAVE_SIDES], gs) : cudaSuccess;
+    for (int b = 0; b < n - 1 && e == cudaSuccess; b++)
+        e = cudaStreamWaitEvent(c->wave_side[b], c->wave_join[Ctx::WAVE_SIDES], 0);
+    const int mine = count - L.own64;  // instances of k_simplex32: the order's first
+    for (int b = 0; b < n && e == cudaSuccess; b++) {
+        cudaStream_t st = b < n - 1 ? c->wave_side[b] : gs;
+        const int k = form[b];
+        if (k < 0)
+            k_netsimplex<<<L.grid64(L.own64), NS_THREADS, L.smem64, st>>>(d, dord + mine, L.own64, dord + count + S32_CLASSES);
+        else
+            s32_launch(k, s32_grid(k, L.num[k], c->sm_count), d, dord + L.first[k], L.num[k], dord + count + k, st);
+        e = cudaGetLastError();
+        if (e == cudaSuccess && b < n - 1) e = cudaEventRecord(c->wave_join[b], st);
+    }
+    for (int b = 0; b < n - 1 && e == cudaSuccess; b++) e = cudaStreamWaitEvent(gs, c->wave_join[b], 0);
+    if (e == cudaSuccess && mine > 0) {
+        k_netsimplex<<<L.grid64(mine), NS_THREADS, L.smem64, gs>>>(d, dord, mine, dord + count + S32_CLASSES + 1);
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
 pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, const CertJob* jobs, NSInst* r,
                       unsigned long long* cert, cudaStream_t st) {
     if (count <= 0) return PD_OK;
@@ -1096,6 +1133,16 @@ pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, const CertJob* jobs, N
     if (!c->wave_stream) PD_TRY_CUDA(c, cudaStreamCreateWithFlags(&c->wave_stream, cudaStreamNonBlocking));
     for (cudaEvent_t& e : c->wave_ev)
         if (!e) PD_TRY_CUDA(c, cudaEventCreate(&e));
+    for (cudaEvent_t& e : c->wave_join)
+        if (!e) PD_TRY_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    if (!c->wave_side[Ctx::WAVE_SIDES - 1]) {
+        int least = 0, greatest = 0;
+        PD_TRY_CUDA(c, cudaDeviceGetStreamPriorityRange(&least, &greatest));
+        for (int b = 0; b < Ctx::WAVE_SIDES; b++)
+            if (!c->wave_side[b])
+                PD_TRY_CUDA(c, cudaStreamCreateWithPriority(&c->wave_side[b], cudaStreamNonBlocking,
+                                                            std::min(greatest + b, least)));
+    }
     unsigned char* pin = (unsigned char*)c->wave_pin;
     NSInst* p_in = (NSInst*)(pin + L.in);
     NSInst* p_out = (NSInst*)(pin + L.out);
@@ -1122,7 +1169,7 @@ pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, const CertJob* jobs, N
     auto mix = [&](uint64_t v) { key = (key ^ v) * 1099511628211ull; };
     mix((uint64_t)count);
     for (int k = 0; k < S32_CLASSES; k++) mix((uint64_t)NL.num[k]);
-    mix((uint64_t)NL.grid64);
+    mix((uint64_t)NL.most64);
     mix((uint64_t)NL.smem64);
     mix((uint64_t)(uintptr_t)pin);
     mix((uint64_t)(uintptr_t)d);
@@ -1138,17 +1185,14 @@ pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, const CertJob* jobs, N
         cudaMemcpyAsync(dord, p_ord, sizeof(int32_t) * (count + NS_COUNTERS), cudaMemcpyHostToDevice, gs);
         cudaMemcpyAsync(djobs, p_jobs, sizeof(CertJob) * count, cudaMemcpyHostToDevice, gs);
         cudaMemsetAsync(dcert, 0, 2 * sizeof(unsigned long long) * count, gs);
-        for (int k = 0; k < S32_CLASSES; k++)
-            if (NL.num[k] > 0)
-                s32_launch(k, s32_grid(k, NL.num[k], c->sm_count), d, dord + NL.first[k], NL.num[k], dord + count + k,
-                           gs);
-        k_netsimplex<<<NL.grid64, NS_THREADS, NL.smem64, gs>>>(d, dord, count, dord + count + S32_CLASSES);
+        const cudaError_t le = ns_capture_wave(c, NL, count, d, dord, gs);
         k_certify_batch<<<dim3(WAVE_CERT_BLOCKS, count), 256, 0, gs>>>(djobs, dcert);
         cudaMemcpyAsync(p_out, d, sizeof(NSInst) * count, cudaMemcpyDeviceToHost, gs);
         cudaMemcpyAsync(p_cert, dcert, 2 * sizeof(unsigned long long) * count, cudaMemcpyDeviceToHost, gs);
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(gs, &g);
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&c->wave_exec, g, 0);
+        if (e == cudaSuccess) e = le;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&c->wave_exec, g, cudaGraphInstantiateFlagUseNodePriority);
         if (g) cudaGraphDestroy(g);
         if (e != cudaSuccess) {
             c->wave_exec = nullptr;
@@ -1165,7 +1209,8 @@ pd_status ns_run_wave(Ctx* c, const NSInst* h, int count, const CertJob* jobs, N
     PD_TRY_CUDA(c, cudaEventRecord(c->wave_ev[1], gs));
     for (int k = 0; k < S32_CLASSES; k++)
         if (NL.num[k] > 0) pd::count_launch();  // the persistent simplex on 32-bit potentials
-    pd::count_launch();                         // ... on 64-bit ones
+    if (NL.own64 > 0) pd::count_launch();       // ... on 64-bit ones
+    if (NL.own64 < count) pd::count_launch();   // ... on those handed back
     pd::count_launch();  // the batched certificate
     c->wave_launches++;
     PD_TRY_CUDA(c, cudaStreamSynchronize(gs));

@@ -74,3 +74,40 @@ def test_largest_matrix_is_taken(pd, ctx):
     finally:
         c.close()
     assert e.value.status == pd.PD_ETIMEOUT
+
+
+def _u(n, seed, scale=1.0):
+    return torch.from_numpy((synth.uniform_exp(n, seed) * scale).astype(np.float32)).cuda()
+
+
+# a wave of every form at once: matrices of the three layouts, of half an SM, for
+# the 64-bit kernel, and one-sided pairs (arc lists); twice, the second time from
+# the captured graph
+def test_a_wave_of_all_forms(pd, ctx):
+    def mixture(n, seed):
+        return torch.from_numpy(synth.mixture_f32(n, seed)).cuda()
+
+    none = _u(40, 1)[:0]
+    pairs = [(mixture(9000, 1), mixture(9000, 2)), (_u(200, 3), none), (mixture(6000, 1), mixture(6000, 2)),
+             (_u(400, 5, 100.0), _u(300, 6, 100.0)), (none, _u(90, 7)), (_u(2600, 8), _u(2500, 9))]
+    pairs += [(_u(300 + i, 20 + i), _u(280, 60 + i)) for i in range(4)] * 40
+    o = pd.opts(ns_transport=2, batch_slots=len(pairs))
+    exp = [pd.pd_w1_approx(ctx, a, b, 0.1, pd.opts(ns_transport=2, warm_start=0))["opt_quanta"] for a, b in pairs[:10]]
+    for _ in range(2):
+        got = pd.pd_w1_approx_batch(ctx, [a for a, _ in pairs], [b for _, b in pairs], 0.1, o)
+        assert [r["opt_quanta"] for r in got] == exp[:6] + exp[6:] * 40
+
+
+# Pairs for the two kernels take the device's time together, not one after the
+# other: 40 instances on 152 SMs, about 75 ms for each kernel alone.
+def test_a_mixed_wave_overlaps(pd, ctx):
+    far = [(_u(1500, i, 100.0), _u(1500, 50 + i, 100.0)) for i in range(4)] * 5
+    near = [(_u(6000, i), _u(6000, 50 + i)) for i in range(4)] * 5
+
+    def ms(pairs):
+        return min(max(r["ns_kernel_ms"] for r in pd.pd_w1_approx_batch(ctx, [a for a, _ in pairs], [b for _, b in pairs], 0.1))
+                   for _ in range(3))
+
+    apart = ms(far), ms(near)
+    assert min(apart) > 40
+    assert ms(far + near) < max(apart) + 0.5 * min(apart), apart
