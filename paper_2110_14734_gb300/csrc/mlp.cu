@@ -585,14 +585,25 @@ pd_status mlp_forward(Ctx* c, const __nv_bfloat16* F, int64_t n, float* y, cudaS
     return PD_OK;
 }
 
+// Rows of partial gradients, one per block of k_mlp_backward: fewer if memory is short.
+static float* mlp_parts(Ctx* c, int64_t n, int* nb) {
+    const int64_t tiles = std::max<int64_t>((n + WS_TILE - 1) / WS_TILE, 1);
+    *nb = (int)std::min<int64_t>(tiles, std::min(std::max(c->sm_count, 1), WS_BLOCKS));
+    if (beyond_cap(c, (int64_t)*nb * WS_PART * sizeof(float))) *nb = (*nb + 1) / 2;  // leaves room for what follows
+    for (;; *nb /= 2) {
+        float* part = bufT<float>(c, B_MLP_PART, (int64_t)*nb * WS_PART);
+        if (part || *nb == 1) return part;
+        c->err.clear();
+    }
+}
+
 // Loss and gradients of rows [0, n) into g (device, WS_PART floats: the
 // WS_NPARAMS gradients, loss sum, mask sum).
 pd_status mlp_grad(Ctx* c, const __nv_bfloat16* F, const float* t, const float* mask, int64_t n, float inv_norm,
                    float* g, cudaStream_t st) {
     if (!c->mlp_ready) return fail(c, PD_EINVAL, "the warm-start network has no parameters yet");
-    const int64_t tiles = std::max<int64_t>((n + WS_TILE - 1) / WS_TILE, 1);
-    const int nb = (int)std::min<int64_t>(tiles, std::min(std::max(c->sm_count, 1), WS_BLOCKS));
-    float* part = bufT<float>(c, B_MLP_PART, (int64_t)nb * WS_PART);
+    int nb;
+    float* part = mlp_parts(c, n, &nb);
     if (!part) return PD_ENOMEM;
     const size_t smem = backward_smem();
     static std::atomic<uint64_t> done{0};
@@ -809,17 +820,27 @@ __global__ void k_rows_to_bf16(const float4* __restrict__ x, int64_t n4, uint2* 
 
 // Host feature rows -> bf16 device rows in B_WS_IN: copied as they are and
 // rounded on the device (2,048 rows: rounding on the host took longer than the
-// copy and the network together).
+// copy and the network together), on the host where memory is short.  Called after
+// everything else that the call needs has its memory.
 static pd_status upload_rows(Ctx* c, const float* feats, int64_t n, __nv_bfloat16** out, cudaStream_t st) {
     static_assert(WS_IN % 4 == 0, "whole 16-byte steps");
-    float* raw = bufT<float>(c, B_WS_RAW, n * WS_IN);
-    __nv_bfloat16* F = bufT<__nv_bfloat16>(c, B_WS_IN, std::max<int64_t>(n, 1) * WS_IN);
-    if (!raw || !F) return PD_ENOMEM;
-    PD_TRY_CUDA(c, cudaMemcpyAsync(raw, feats, sizeof(float) * n * WS_IN, cudaMemcpyHostToDevice, st));
-    const int64_t n4 = n * WS_IN / 4;
-    k_rows_to_bf16<<<grid_for(n4, 256), 256, 0, st>>>((const float4*)raw, n4, (uint2*)F); pd::count_launch();
-    PD_TRY_CUDA(c, cudaGetLastError());
+    const int64_t m = n * WS_IN;
+    __nv_bfloat16* F = bufT<__nv_bfloat16>(c, B_WS_IN, std::max<int64_t>(m, 1));
+    if (!F) return PD_ENOMEM;
     *out = F;
+    float* raw = beyond_cap(c, sizeof(float) * m) ? nullptr : bufT<float>(c, B_WS_RAW, m);
+    if (!raw) {
+        c->err.clear();
+        const std::unique_ptr<__nv_bfloat16[]> hb(new (std::nothrow) __nv_bfloat16[m]);
+        if (!hb) return fail(c, PD_ENOMEM, "no host memory for the features");
+        for (int64_t t = 0; t < m; t++) hb[t] = __float2bfloat16(feats[t]);
+        PD_TRY_CUDA(c, cudaMemcpyAsync(F, hb.get(), sizeof(__nv_bfloat16) * m, cudaMemcpyHostToDevice, st));
+        PD_TRY_CUDA(c, cudaStreamSynchronize(st));  // hb is freed on return
+        return PD_OK;
+    }
+    PD_TRY_CUDA(c, cudaMemcpyAsync(raw, feats, sizeof(float) * m, cudaMemcpyHostToDevice, st));
+    k_rows_to_bf16<<<grid_for(m / 4, 256), 256, 0, st>>>((const float4*)raw, m / 4, (uint2*)F); pd::count_launch();
+    PD_TRY_CUDA(c, cudaGetLastError());
     return PD_OK;
 }
 
@@ -831,9 +852,9 @@ extern "C" pd_status pd_ws_forward(pd_ctx* cx, const float* feats, int64_t n, fl
     cudaStream_t st = (cudaStream_t)stream;
     if (n == 0) return PD_OK;
     __nv_bfloat16* F;
-    PD_TRY(upload_rows(c, feats, n, &F, st));
     float* dy = bufT<float>(c, B_WS_Y, n);
     if (!dy) return PD_ENOMEM;
+    PD_TRY(upload_rows(c, feats, n, &F, st));
     PD_TRY(mlp_forward(c, F, n, dy, st));
     PD_TRY_CUDA(c, cudaMemcpyAsync(y, dy, sizeof(float) * n, cudaMemcpyDeviceToHost, st));
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));
@@ -847,12 +868,13 @@ extern "C" pd_status pd_ws_grad(pd_ctx* cx, const float* feats, const float* tar
     c->err.clear();
     if (cudaSetDevice(c->device) != cudaSuccess) return cuda_fail(c, cudaGetLastError(), "cudaSetDevice");
     cudaStream_t st = (cudaStream_t)stream;
-    __nv_bfloat16* F;
-    PD_TRY(upload_rows(c, feats, n, &F, st));
+    __nv_bfloat16* F = bufT<__nv_bfloat16>(c, B_WS_IN, n * WS_IN);
     float* dt = bufT<float>(c, B_WS_TIN, n);
     float* dm = bufT<float>(c, B_WS_MIN, n);
     float* g = bufT<float>(c, B_MLP_G, WS_PART);
-    if (!dt || !dm || !g) return PD_ENOMEM;
+    int nb;
+    if (!F || !dt || !dm || !g || !mlp_parts(c, n, &nb)) return PD_ENOMEM;
+    PD_TRY(upload_rows(c, feats, n, &F, st));
     std::vector<float> ones;
     if (!mask) {
         ones.assign((size_t)n, 1.f);
