@@ -55,14 +55,14 @@ pd_status cuda_fail(Ctx* c, cudaError_t e, const char* where) {
 void* buf(Ctx* c, Buf id, size_t bytes) {
     if (bytes == 0) bytes = 1;
     if (c->bytes[id] >= bytes) return c->ptr[id];
-    // growth slack: an eighth, or a half where a grow would be deferred
+    // growth slack: an eighth, or a half where a grow would be deferred; none of the
+    // second half of a cap, which other buffers may need
     size_t want = bytes + (c->defer_free ? bytes / 2 : bytes / 8);
-    if (c->cap && c->held + c->retired_bytes - c->bytes[id] + want > c->cap) {
-        want = bytes;
-        if (c->held + c->retired_bytes - c->bytes[id] + want > c->cap) {
-            c->err = "device memory cap of the context reached";
-            return nullptr;
-        }
+    const size_t others = c->held + c->retired_bytes - c->bytes[id];
+    if (c->cap && others + want > c->cap / 2) want = bytes;
+    if (c->cap && others + want > c->cap) {
+        c->err = "device memory cap of the context reached";
+        return nullptr;
     }
     if (c->ptr[id]) {
         if (c->defer_free) {

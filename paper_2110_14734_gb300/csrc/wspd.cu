@@ -696,8 +696,9 @@ static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, const int2*
     const int blocks = 4 * std::max(c->sm_count, 1);  // the stacks of four blocks fit an SM
     const int64_t warps = (int64_t)blocks * WS_WARPS;
     // room for handed-on pairs: the more, the better the balance; less will do
+    constexpr int64_t least = 256;
     int64_t cap = std::min<int64_t>(int64_t(1) << 27, std::max<int64_t>(int64_t(1) << 16, 64 * (tr.N - 1)));  // even
-    while (cap > (int64_t(1) << 16) && beyond_cap(c, 2 * sizeof(int2) * cap)) cap = cap / 8 * 2;
+    while (cap > least && beyond_cap(c, 2 * sizeof(int2) * cap)) cap = cap / 8 * 2;
     int2* out[2];
     static std::atomic<uint64_t> done{0};
     if (arcs) PD_TRY(smem_limit(c, done, (const void*)k_ws_walk<true>, sizeof(int2) * WS_WARPS * WS_OUT));
@@ -705,7 +706,7 @@ static pd_status ws_walk(Ctx* c, const WsTree& tr, const WsRec* rec, const int2*
         out[0] = bufT<int2>(c, B_F1, cap);
         out[1] = out[0] ? bufT<int2>(c, B_WSOFF, cap) : nullptr;
         if (out[0] && out[1]) break;
-        if (cap <= (int64_t(1) << 16)) return PD_ENOMEM;
+        if (cap <= least) return PD_ENOMEM;
         c->err.clear();
     }
     const int2* F = (const int2*)c->ptr[B_F0];

@@ -51,3 +51,23 @@ def test_network_rows(pd, n, grad, forward):
     assert np.array_equal(a, b)
     (la, a), (lb, b) = _both(pd, grad, run(lambda c: pd.pd_ws_grad(c, x, t)))
     assert abs(la - lb) <= 1e-5 * la and np.linalg.norm(a - b) <= 1e-5 * np.linalg.norm(a)
+
+
+def _mixture(n):
+    return [torch.from_numpy(synth.mixture_f32(n, s)).cuda() for s in (1, 2)]
+
+
+# the WSPD walk's room for pairs handed on
+@pytest.mark.parametrize("n,s,cap", [(300, 1, 279551), (300, 8, 923644), (5000, 1, 6471655)])
+def test_network_of_nodes(pd, n, s, cap):
+    c = pd.pd_create(0)
+    nodes = pd.pd_condense(c, *_mixture(n), 1, 0)
+    c.close()
+    a, b = _both(pd, cap, lambda c: pd.pd_wspd_sparsify(c, nodes, s))
+    assert all(torch.equal(a[k], b[k]) for k in ("row_ptr", "head", "cost", "supply"))
+
+
+@pytest.mark.parametrize("tree,cap", [(0, 461822), (1, 449534)])
+def test_network_size(pd, tree, cap):
+    a, b = _both(pd, cap, lambda c: pd.pd_w1_sparsify_count(c, *_mixture(300), 0.5, pd.opts(tree=tree))["n_arcs"])
+    assert a == b
