@@ -210,14 +210,12 @@ constexpr int RS_BACK = 8;                                // tiles looked back a
 
 inline int64_t radix_tiles(int64_t n) { return (n + RS_TILE - 1) / RS_TILE; }
 inline int radix_passes(int bits) { return (bits + 7) / 8; }
-// Words of scratch: counts of every pass, tickets, states.
-inline int64_t radix_words(int64_t n, int bits) {
-    return 256 * RS_MAXPASS + RS_MAXPASS + 256 * (int64_t)radix_passes(bits) * radix_tiles(n);
-}
+// Words of scratch of `passes` passes: their counts, tickets and states.
+inline int64_t radix_words(int64_t n, int passes) { return passes * (256 + 1 + 256 * radix_tiles(n)); }
 
-// Digit counts of all passes.
-__global__ void __launch_bounds__(RS_THREADS) k_radix_counts(const uint64_t* __restrict__ keys, int64_t n, int passes,
-                                                             unsigned long long* __restrict__ hist);
+// Digit counts of the passes first .. first + passes - 1.
+__global__ void __launch_bounds__(RS_THREADS) k_radix_counts(const uint64_t* __restrict__ keys, int64_t n, int first,
+                                                             int passes, unsigned long long* __restrict__ hist);
 // One pass; vin / vout may be null.  polls: bound of a look-back wait.
 __global__ void __launch_bounds__(RS_THREADS) k_radix_pass(const uint64_t* __restrict__ kin,
                                                            const uint32_t* __restrict__ vin,

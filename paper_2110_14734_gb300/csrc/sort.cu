@@ -6,14 +6,14 @@
 
 namespace pd {
 
-__global__ void __launch_bounds__(RS_THREADS) k_radix_counts(const uint64_t* __restrict__ keys, int64_t n, int passes,
-                                                             unsigned long long* __restrict__ hist) {
+__global__ void __launch_bounds__(RS_THREADS) k_radix_counts(const uint64_t* __restrict__ keys, int64_t n, int first,
+                                                             int passes, unsigned long long* __restrict__ hist) {
     __shared__ uint32_t h[RS_MAXPASS][256];
     for (int p = 0; p < passes; p++) h[p][threadIdx.x] = 0;
     __syncthreads();
     const int64_t step = (int64_t)gridDim.x * RS_THREADS;
     for (int64_t i = (int64_t)blockIdx.x * RS_THREADS + threadIdx.x; i < n; i += step) {
-        const uint64_t k = keys[i];
+        const uint64_t k = keys[i] >> (8 * first);
         for (int p = 0; p < passes; p++) atomicAdd(&h[p][(uint32_t)(k >> (8 * p)) & 0xffu], 1u);
     }
     __syncthreads();
@@ -171,24 +171,26 @@ pd_status sort_u64(Ctx* c, uint64_t*& keys, uint64_t*& keys_alt, uint32_t*& vals
     }
     const int passes = radix_passes(bits);
     const int64_t tiles = radix_tiles(n);
-    int64_t words = radix_words(n, bits);
-    unsigned long long* w = beyond_cap(c, 8 * words) ? nullptr : bufT<unsigned long long>(c, B_RS_COUNTS, words);
-    const bool shared = !w;  // short of memory: all passes use one set of tile states, cleared in between
-    if (shared) {
+    // short of memory (a quarter of what other scratch may take: it stays beside the
+    // stages that follow): one pass's worth, counted and cleared before each
+    int sets = beyond_cap(c, 4 * 8 * radix_words(n, passes)) ? 1 : passes;
+    unsigned long long* w = bufT<unsigned long long>(c, B_RS_COUNTS, radix_words(n, sets));
+    if (!w && sets > 1) {
         c->err.clear();
-        words -= 256 * (passes - 1) * tiles;
-        w = bufT<unsigned long long>(c, B_RS_COUNTS, words);
+        sets = 1;
+        w = bufT<unsigned long long>(c, B_RS_COUNTS, radix_words(n, sets));
     }
     if (!w) return PD_ENOMEM;
-    unsigned long long *hist = w, *ticket = w + 256 * RS_MAXPASS, *state = ticket + RS_MAXPASS;
-    PD_TRY_CUDA(c, cudaMemsetAsync(w, 0, sizeof(unsigned long long) * words, st));
-    k_radix_counts<<<(unsigned)std::min<int64_t>(tiles, 4 * std::max(c->sm_count, 1)), RS_THREADS, 0, st>>>(keys, n, passes, hist);
-    pd::count_launch();
+    unsigned long long *hist = w, *ticket = w + 256 * sets, *state = ticket + sets;
+    const unsigned count_grid = (unsigned)std::min<int64_t>(tiles, 4 * std::max(c->sm_count, 1));
     for (int p = 0; p < passes; p++) {
-        if (shared && p > 0) PD_TRY_CUDA(c, cudaMemsetAsync(state, 0, 256 * tiles * sizeof(unsigned long long), st));
+        const int q = p % sets;
+        if (q == 0) {
+            PD_TRY_CUDA(c, cudaMemsetAsync(w, 0, sizeof(unsigned long long) * radix_words(n, sets), st));
+            k_radix_counts<<<count_grid, RS_THREADS, 0, st>>>(keys, n, p, sets, hist); pd::count_launch();
+        }
         k_radix_pass<<<(unsigned)tiles, RS_THREADS, 0, st>>>(keys, vals, keys_alt, vals ? vals_alt : nullptr, n, 8 * p,
-                                                            hist + 256 * p, ticket + p,
-                                                            state + (shared ? 0 : 256 * tiles * p),
+                                                            hist + 256 * q, ticket + q, state + 256 * tiles * q,
                                                             polls); pd::count_launch();
         std::swap(keys, keys_alt);
         std::swap(vals, vals_alt);

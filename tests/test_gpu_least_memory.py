@@ -71,3 +71,10 @@ def test_network_of_nodes(pd, n, s, cap):
 def test_network_size(pd, tree, cap):
     a, b = _both(pd, cap, lambda c: pd.pd_w1_sparsify_count(c, *_mixture(300), 0.5, pd.opts(tree=tree))["n_arcs"])
     assert a == b
+
+
+# the long sort's counts and tile states, kept while the next stage takes its own
+@pytest.mark.parametrize("n,cap", [(5000, 638973), (100000, 17366974)])
+def test_bounds(pd, n, cap):
+    a, b = _both(pd, cap, lambda c: tuple(pd.pd_rwmd_lower_bound(c, *_mixture(n))))
+    assert a == b
