@@ -371,30 +371,35 @@ pd_status pd_nn_search(pd_ctx* ctx, pd_diagram query, double eps, const pd_opts*
  * measures instead: it prepares the transportation instance of each sample
  * pair (A[i], B[i]) at eps/opts exactly as pd_w1_approx does, solves it once
  * per candidate (pricing block of 4096 ... 32768 arcs) x (walk limit 0, 8,
- * 32, see pd_opts.ns_walk), and once with the defaults, each launch timed by
- * CUDA events, and keeps the fastest pair of values of each size class
- * floor(log2(arcs + nodes)) in the context: later solves of that class whose
- * opts->ns_block is 0 (and ns_walk -1) use them (pd_w1_approx,
- * pd_w1_approx_batch, pd_nn_search, pd_mcf_solve).  Every candidate reaches
- * the same optimum (checked).  cache_path (may be NULL): a text file of lines
- * "gpu-name sms class block walk"; classes it already holds for this GPU are
- * loaded instead of timed, and newly timed classes are written back (other
- * GPUs' lines kept).  Must not run concurrently with other calls on the same
+ * 32, see pd_opts.ns_walk) that is not the same to its kernel as one before
+ * (32-bit potentials: no walk, and blocks are cut to what shared memory
+ * holds), and once with the defaults, each launch timed by CUDA events, and
+ * keeps the fastest pair of values of each size class floor(log2(arcs +
+ * nodes)) and form (kernel, its layout, cost matrix or arc list) in the
+ * context: later solves of that class and form whose opts->ns_block is 0 (and
+ * ns_walk -1) use them (pd_w1_approx, pd_w1_approx_batch, pd_nn_search,
+ * pd_mcf_solve).  Every candidate reaches the same optimum (checked).
+ * cache_path (may be NULL): a text file of lines "gpu-name sms f<form> class
+ * block walk"; what it already holds for this GPU is loaded instead of timed,
+ * and what was newly timed is written back (other GPUs' lines kept; lines of
+ * this GPU without a form were measured on another kernel and are dropped).
+ * Must not run concurrently with other calls on the same
  * context. */
 typedef struct {
     int64_t ns_block;   /* block chosen for the first sample pair's size class (0 if none) */
     int32_t ns_walk;    /* walk limit chosen for that class (pd_opts.ns_walk) */
     int32_t size_class; /* that class, floor(log2(arcs + nodes)); -1 if no pair had a transportation form */
-    int32_t candidates; /* candidate blocks */
+    int32_t candidates; /* candidate (block, walk) pairs, before those that are the same to the kernel */
     int32_t pairs;      /* pairs timed (not taken from the cache) */
     int32_t from_cache; /* 1: the first pair's class came from cache_path */
     float best_ms;      /* simplex device time of the timed pairs of that class with the chosen block */
-    float default_ms;   /* ... with the default block max(8192, sqrt(arcs + nodes)) and walk 0 */
+    float default_ms;   /* ... with the default block (pd_opts.ns_block) and walk 0 */
 } pd_tune_result;
 
 pd_status pd_autotune(pd_ctx* ctx, const pd_diagram* A, const pd_diagram* B, int64_t count, double eps,
                       const pd_opts* opts, const char* cache_path, pd_tune_result* out, void* stream);
-/* The block the context uses for an instance of arcs + nodes = M (0: none tuned, the default applies). */
+/* The block the context uses for an instance of arcs + nodes = M (0: none tuned, the default applies);
+ * of the forms tuned for M's class, cost matrices first, 32-bit potentials before 64-bit ones. */
 pd_status pd_tuned_block(const pd_ctx* ctx, int64_t arcs_and_nodes, int64_t* block_out);
 
 /* ---- learned warm start (no counterpart in the paper) ----------------------

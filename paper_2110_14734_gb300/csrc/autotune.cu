@@ -1,19 +1,21 @@
 // Autotuner of the network simplex's launch parameters (no counterpart in the
 // paper, whose block search uses a block of sqrt(arcs)): the pricing block,
 // which trades pricing work per pivot against the quality of the entering
-// arc, and the walk limit, below which the two half-cycles of a pivot are
-// followed by two lanes instead of scanned by the whole CTA.  The best values
-// depend on the instance's size and on the GPU, so they are measured: the
-// transportation instances of sample pairs are solved once per candidate
-// (block, walk), each launch timed by CUDA events, and the fastest is kept per
-// size class (floor(log2(arcs + nodes))) in the context -- every later solve
-// of that class whose pd_opts.ns_block is 0 (ns_walk -1) uses it -- and in an
-// optional cache file, one line per (GPU name, SM count, class):
-// "name sms class block walk".
+// arc, and, in the 64-bit kernel, the walk limit, below which the two half-cycles
+// of a pivot are followed by two lanes instead of scanned by the whole CTA.  The
+// best values depend on the instance's size, on the kernel that takes it and on the
+// GPU, so they are measured: the transportation instances of sample pairs are solved
+// once per candidate (block, walk) that makes a difference to their kernel, each
+// launch timed by CUDA events, and the fastest is kept per size class
+// (floor(log2(arcs + nodes))) and form (kernel, layout, matrix or list) in the
+// context -- every later solve of that class and form whose pd_opts.ns_block is 0
+// (ns_walk -1) uses it -- and in an optional cache file, one line per (GPU name, SM
+// count, form, class): "name sms f<form> class block walk".
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
 
+#include <fstream>
 #include <map>
 #include <string>
 #include <vector>
@@ -28,10 +30,7 @@ namespace {
 const int64_t kBlocks[] = {4096, 8192, 16384, 32768};
 const int32_t kWalks[] = {0, 8, 32};
 constexpr int kDefaultWalk = 0;
-struct Choice {
-    int64_t block;
-    int32_t walk;
-};
+using Choices = std::map<int, Ctx::Tuned>;  // by tune_key
 
 std::string device_key(int device, int sms) {
     cudaDeviceProp p;
@@ -43,40 +42,45 @@ std::string device_key(int device, int sms) {
     return name + " " + std::to_string(sms);
 }
 
-// Lines "name sms class block walk" of the cache file that match this GPU.
-std::map<int, Choice> read_cache(const char* path, const std::string& key) {
-    std::map<int, Choice> m;
-    FILE* f = path ? fopen(path, "r") : nullptr;
-    if (!f) return m;
-    char name[256];
-    int sms = 0, cls = 0, walk = 0;
-    long long blk = 0;
-    while (fscanf(f, "%255s %d %d %lld %d", name, &sms, &cls, &blk, &walk) == 5)
-        if (std::string(name) + " " + std::to_string(sms) == key && blk > 0 && walk >= 0)
-            m[cls] = Choice{(int64_t)blk, walk};
-    fclose(f);
-    return m;
+// The cache file's choices for this GPU, and the lines of other GPUs.  Lines of
+// this GPU that are not of the form above say nothing about the kernel they were
+// measured on and are left out.
+void read_cache(const char* path, const std::string& key, Choices* mine, std::vector<std::string>* others) {
+    if (!path) return;
+    std::ifstream f(path);
+    for (std::string line; std::getline(f, line);) {
+        char name[256];
+        int sms = 0, form = 0, cls = 0, walk = 0, end = 0;
+        long long blk = 0;
+        if (sscanf(line.c_str(), "%255s %d", name, &sms) != 2) continue;
+        if (std::string(name) + " " + std::to_string(sms) != key) {
+            others->push_back(line);
+        } else if (sscanf(line.c_str(), "%255s %d f%d %d %lld %d %n", name, &sms, &form, &cls, &blk, &walk, &end) == 6 &&
+                   line.c_str()[end] == 0 && form >= 0 && form < TUNE_FORMS && cls >= 0 && cls < 64 && blk > 0 && walk >= 0) {
+            (*mine)[tune_key(cls, form)] = Ctx::Tuned{(int64_t)blk, walk};
+        }
+    }
 }
 
-bool write_cache(const char* path, const std::string& key, const std::map<int, Choice>& mine) {
-    // keep other GPUs' lines, replace this GPU's
-    std::vector<std::string> keep;
-    if (FILE* f = fopen(path, "r")) {
-        char name[256];
-        int sms = 0, cls = 0, walk = 0;
-        long long blk = 0;
-        while (fscanf(f, "%255s %d %d %lld %d", name, &sms, &cls, &blk, &walk) == 5) {
-            const std::string k = std::string(name) + " " + std::to_string(sms);
-            if (k != key)
-                keep.push_back(k + " " + std::to_string(cls) + " " + std::to_string(blk) + " " + std::to_string(walk));
-        }
-        fclose(f);
-    }
+// Other GPUs' lines stay, this GPU's are replaced.
+bool write_cache(const char* path, const std::string& key, const Choices& mine, const std::vector<std::string>& others) {
     FILE* f = fopen(path, "w");
     if (!f) return false;
-    for (auto& l : keep) fprintf(f, "%s\n", l.c_str());
-    for (auto& e : mine) fprintf(f, "%s %d %lld %d\n", key.c_str(), e.first, (long long)e.second.block, e.second.walk);
+    for (auto& l : others) fprintf(f, "%s\n", l.c_str());
+    for (auto& e : mine)
+        fprintf(f, "%s f%d %d %lld %d\n", key.c_str(), e.first % TUNE_FORMS, e.first / TUNE_FORMS,
+                (long long)e.second.block, e.second.walk);
     return fclose(f) == 0;
+}
+
+// Whether candidate (b, w) is none of those before it to the kernel of h: only
+// k_netsimplex walks, and k_simplex32 cuts blocks to its stage.
+bool differs(const NSInst& h, int b, int w) {
+    if (!h.lay32) return true;
+    if (w > 0) return false;
+    const int cls = s32_class(h);
+    auto same = [&](int k) { return s32_block(k, kBlocks[b]) == s32_block(k, kBlocks[b - 1]); };
+    return b == 0 || !same(cls) || (cls == S32_MATRIX && h.n < S32_HALF_NODES && !same(S32_HALF));
 }
 
 }  // namespace
@@ -85,16 +89,10 @@ namespace pd {
 
 int tune_class(int64_t M) { return M > 0 ? (int)floor(log2((double)M)) : 0; }
 
-int64_t tuned_block(const Ctx* c, int64_t M) {
+const Ctx::Tuned* tuned(const Ctx* c, const NSInst& h) {
     const Ctx* o = c->parent ? c->parent : c;
-    auto it = o->tuned_block.find(tune_class(M));
-    return it == o->tuned_block.end() ? 0 : it->second;
-}
-
-int32_t tuned_walk(const Ctx* c, int64_t M) {
-    const Ctx* o = c->parent ? c->parent : c;
-    auto it = o->tuned_walk.find(tune_class(M));
-    return it == o->tuned_walk.end() ? kDefaultWalk : it->second;
+    auto it = o->tuned.find(tune_key(tune_class(h.m + h.n), tune_form(h)));
+    return it == o->tuned.end() ? nullptr : &it->second;
 }
 
 }  // namespace pd
@@ -116,13 +114,16 @@ extern "C" pd_status pd_autotune(pd_ctx* cx, const pd_diagram* A, const pd_diagr
     memset(&r, 0, sizeof(r));
     r.size_class = -1;
     const std::string key = device_key(c->device, c->sm_count);
-    const std::map<int, Choice> cached = read_cache(cache_path, key);
+    Choices cached;
+    std::vector<std::string> others;
+    read_cache(cache_path, key, &cached, &others);
     NSInst* d = bufT<NSInst>(c, B_NS_INST, 1);
     if (!d) return PD_ENOMEM;
     const int NB = (int)(sizeof(kBlocks) / sizeof(kBlocks[0])), NW = (int)(sizeof(kWalks) / sizeof(kWalks[0]));
-    // per size class: total device time of every candidate over the pairs timed
+    // per size class and form: total device time of every candidate over the pairs timed
     std::map<int, std::vector<double>> total;
     std::map<int, double> dflt;
+    int first = -1;  // the first pair's
     for (int64_t i = 0; i < count; i++) {
         Front f;
         PD_TRY(front_half(c, A[i], B[i], eps, o, &f, st, true));
@@ -130,14 +131,16 @@ extern "C" pd_status pd_autotune(pd_ctx* cx, const pd_diagram* A, const pd_diagr
         PD_TRY(ns_prepare_w1(c, f.nodes, f.net.n_arcs, f.h.FA, f.h.FB, o, &w, st));
         if (!w.ns.ready) continue;
         const int64_t M = w.ns.h.m + w.ns.h.n;
-        const int cls = tune_class(M);
-        if (r.size_class < 0) r.size_class = cls;
-        if (cached.count(cls)) {
-            c->tuned_block[cls] = cached.at(cls).block;
-            c->tuned_walk[cls] = cached.at(cls).walk;
+        const int what = tune_key(tune_class(M), tune_form(w.ns.h));
+        if (first < 0) {
+            first = what;
+            r.size_class = tune_class(M);
+        }
+        if (cached.count(what)) {
+            c->tuned[what] = cached.at(what);
             continue;
         }
-        std::vector<double>& t = total[cls];
+        std::vector<double>& t = total[what];
         t.resize((size_t)(NB * NW), 0.0);
         int64_t opt = -1;
         for (int q = 0; q <= NB * NW; q++) {  // the candidates, then the defaults
@@ -145,7 +148,7 @@ extern "C" pd_status pd_autotune(pd_ctx* cx, const pd_diagram* A, const pd_diagr
             if (q < NB * NW) {
                 h.block = kBlocks[q / NW];
                 h.walk = kWalks[q % NW];
-                if (h.block > 4 * M) continue;
+                if (h.block > 4 * M || !differs(h, q / NW, q % NW)) continue;
             } else {
                 h.block = ns_default_block(h);
                 h.walk = kDefaultWalk;
@@ -157,31 +160,28 @@ extern "C" pd_status pd_autotune(pd_ctx* cx, const pd_diagram* A, const pd_diagr
             if (opt >= 0 && res.opt != opt) return fail(c, PD_ECUDA, "tuner: the optimum changed with the parameters");
             opt = res.opt;
             if (q < NB * NW) t[(size_t)q] += c->last_ns_ms;
-            else dflt[cls] += c->last_ns_ms;
+            else dflt[what] += c->last_ns_ms;
         }
         r.pairs++;
     }
-    std::map<int, Choice> mine = cached;
+    Choices mine = cached;
     for (auto& e : total) {
         size_t best = 0;
         for (size_t q = 1; q < e.second.size(); q++)
             if (e.second[q] > 0.0 && (e.second[best] <= 0.0 || e.second[q] < e.second[best])) best = q;
-        const Choice ch{kBlocks[best / NW], kWalks[best % NW]};
-        c->tuned_block[e.first] = ch.block;
-        c->tuned_walk[e.first] = ch.walk;
-        mine[e.first] = ch;
-        if (e.first == r.size_class) {
+        c->tuned[e.first] = mine[e.first] = Ctx::Tuned{kBlocks[best / NW], kWalks[best % NW]};
+        if (e.first == first) {
             r.best_ms = (float)e.second[best];
             r.default_ms = (float)dflt[e.first];
         }
     }
     r.candidates = NB * NW;
-    r.from_cache = (r.size_class >= 0 && total.count(r.size_class) == 0) ? 1 : 0;
-    if (r.size_class >= 0 && c->tuned_block.count(r.size_class)) {
-        r.ns_block = c->tuned_block[r.size_class];
-        r.ns_walk = c->tuned_walk[r.size_class];
+    r.from_cache = (first >= 0 && total.count(first) == 0) ? 1 : 0;
+    if (first >= 0) {
+        r.ns_block = c->tuned[first].block;
+        r.ns_walk = c->tuned[first].walk;
     }
-    if (cache_path && !total.empty() && !write_cache(cache_path, key, mine))
+    if (cache_path && !total.empty() && !write_cache(cache_path, key, mine, others))
         return fail(c, PD_EINVAL, std::string("cannot write the tuning cache ") + cache_path);
     *out = r;
     return PD_OK;
@@ -189,6 +189,13 @@ extern "C" pd_status pd_autotune(pd_ctx* cx, const pd_diagram* A, const pd_diagr
 
 extern "C" pd_status pd_tuned_block(const pd_ctx* cx, int64_t arcs_and_nodes, int64_t* block_out) {
     if (!cx || !block_out) return PD_EINVAL;
-    *block_out = tuned_block(cx, arcs_and_nodes);
+    const Ctx* o = cx->parent ? cx->parent : cx;
+    *block_out = 0;
+    for (int form : {3, 5, 7, 1, 2, 4, 6, 0}) {  // matrices before lists, 32-bit kernel before 64-bit
+        auto it = o->tuned.find(tune_key(tune_class(arcs_and_nodes), form));
+        if (it == o->tuned.end()) continue;
+        *block_out = it->second.block;
+        break;
+    }
     return PD_OK;
 }

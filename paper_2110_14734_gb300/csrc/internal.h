@@ -79,10 +79,14 @@ struct Ctx {
     int64_t mlp_steps = 0;
     int64_t ws_rows = 0, ws_cap = 0;
     Ctx* mlp_owner = nullptr;
-    // pricing blocks chosen by pd_autotune, per size class (of the context that
-    // ran it: slots and workers of a batch look theirs up in `parent`)
-    std::map<int, int64_t> tuned_block;
-    std::map<int, int32_t> tuned_walk;
+    // pricing block and walk limit chosen by pd_autotune, per size class and form
+    // (tune_key; of the context that ran it: slots and workers of a batch look
+    // theirs up in `parent`)
+    struct Tuned {
+        int64_t block;
+        int32_t walk;
+    };
+    std::map<int, Tuned> tuned;
     Ctx* parent = nullptr;
     Ctx* coarse = nullptr;            // helper context of the coarse solve (warm_start 4)
     int64_t last_coarse_pivots = 0;   // pivots of the last coarse solve
@@ -242,12 +246,6 @@ pd_status stage_inputs(Ctx* c, const pd_diagram& A, const pd_diagram& B, DevDiag
 // pd_w1_approx_batch after argument checks (opts resolved)
 pd_status batch_solve(Ctx* c, const pd_diagram* A, const pd_diagram* B, int64_t count, double eps,
                       const pd_opts& o, pd_result* out, cudaStream_t st);
-
-// Size class of a simplex instance with M arcs + nodes, and the pricing block
-// pd_autotune chose for it (0 = none: the default block).
-int tune_class(int64_t M);
-int64_t tuned_block(const Ctx* c, int64_t M);
-int32_t tuned_walk(const Ctx* c, int64_t M);  // the walk limit (16 when none was tuned)
 
 // Stable radix sort of keys (and vals, may be null) by the low `bits` bits with
 // context scratch; the result is in keys / vals, which may have changed places

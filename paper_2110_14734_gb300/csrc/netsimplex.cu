@@ -906,7 +906,6 @@ pd_status ns_prepare_arcs(Ctx* c, int32_t n, const NSArcs& a, const int64_t* sup
     // arc ids, plus one pricing step past the last arc, stay below 2^31
     if (M >= (int64_t(1) << 31) - 1 - 8 * NS_THREADS)
         return fail(c, PD_ECAPACITY, "network simplex needs fewer than 2^31 - 8193 arcs");
-    h.walk = o.ns_walk >= 0 ? std::min<int32_t>(o.ns_walk, NS_LMAX) : tuned_walk(c, M);
     h.max_pivots = o.max_rounds > 0 ? o.max_rounds : (int64_t(1) << 40);
     h.time_limit_ns = (o.time_limit_ms > 0 ? (uint64_t)o.time_limit_ms : 60000ull) * 1000000ull;
     // flows are int32: the total supply must stay below 2^31
@@ -925,7 +924,9 @@ pd_status ns_prepare_arcs(Ctx* c, int32_t n, const NSArcs& a, const int64_t* sup
     int max_optin = 0;
     PD_TRY_CUDA(c, cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
     ns_choose_kernel(&h, cmax, a.complete, o.ns_smem != 0, max_optin);
-    const int64_t blk = o.ns_block > 0 ? o.ns_block : tuned_block(c, M);
+    const Ctx::Tuned* t = tuned(c, h);
+    h.walk = o.ns_walk >= 0 ? std::min<int32_t>(o.ns_walk, NS_LMAX) : t ? t->walk : 0;
+    const int64_t blk = o.ns_block > 0 ? o.ns_block : t ? t->block : 0;
     h.block = blk > 0 ? (blk + 7) & ~(int64_t)7 : ns_default_block(h);  // whole 32-byte steps
     p->ready = true;
     return PD_OK;

@@ -74,6 +74,7 @@ constexpr int32_t S32_HALF_NODES = 3712;  // nodes with the root that half an SM
 constexpr int32_t S32_SMALL_NODES = 1280; // ... up to which half the threads are the better choice anyway
 int s32_class(const NSInst& h);  // -1: not a 32-bit instance
 int s32_layout(int64_t N1);      // the smallest layout that holds N1 nodes (0: none)
+int64_t s32_block(int cls, int64_t block);  // arcs that a class prices at a time for a block of `block` arcs
 inline int s32_grid(int cls, int count, int sm_count) {
     const int most = (cls == S32_HALF ? 2 : 1) * (sm_count > 1 ? sm_count : 1);
     return count < most ? count : most;
@@ -168,6 +169,13 @@ pd_status ns_prepare_arcs(Ctx* c, int32_t n, const NSArcs& a, const int64_t* sup
 // Runs `count` prepared instances (one CTA each): h -> device records d ->
 // results r (host), synchronising the stream.
 pd_status ns_run(Ctx* c, const NSInst* h, int count, NSInst* d, NSInst* r, cudaStream_t st);
+// What pd_autotune tells apart: the size class floor(log2(arcs + nodes)) and the form,
+// which is the kernel with its layout and whether the arcs are a matrix.
+constexpr int TUNE_FORMS = 8;
+int tune_class(int64_t M);
+inline int tune_form(const NSInst& h) { return 2 * h.lay32 + (h.mst > 0 ? 1 : 0); }
+inline int tune_key(int cls, int form) { return cls * TUNE_FORMS + form; }
+const Ctx::Tuned* tuned(const Ctx* c, const NSInst& h);  // null: none, the defaults apply
 // The kernel an instance goes to, its layout and its artificial costs.
 int64_t ns_default_block(const NSInst& h);
 void ns_choose_kernel(NSInst* h, int64_t cmax, bool complete, bool smem, int max_optin);

@@ -105,6 +105,15 @@ struct Layout {
     static_assert(N % 16 == 0 && total + 16 <= (LAY == 4 ? 113 : 227) * 1024, "the layout does not fit an SM");
 };
 
+// Steps of a pricing block of `block` arcs (STEP: a step's arcs): a whole number of
+// the pricing threads, at most the stage.
+template <int LAY>
+PD_HD constexpr int32_t block_steps(int64_t block, int step) {
+    constexpr int P = Layout<LAY>::PRICERS, most = (int)(Layout<LAY>::STAGE / 32) / P;
+    const int64_t k = (block + step * P / 2) / (step * P);
+    return P * (int32_t)(k < 1 ? 1 : k < most ? k : most);
+}
+
 template <int LAY>
 struct Nodes {
     using L = Layout<LAY>;
@@ -481,7 +490,6 @@ PD_D void s32_body(NSInst& G) {
     constexpr int STEP = IMPL ? 8 : 4;     // arcs of a thread's step
     constexpr int MAXIT = (s32_capacity(LAY) - 1) / (128 * Layout<LAY>::WARPS) + 1;  // scan rounds
     static_assert(4 * MAXIT <= 64, "a thread's scan mask");
-    constexpr int32_t STAGED = (int32_t)(Layout<LAY>::STAGE / 32);  // steps a stage holds (8 costs, or 4 with their ends)
 
     // ---- initial tree ------------------------------------------------------
     const int32_t big = (int32_t)I.big;
@@ -544,13 +552,11 @@ PD_D void s32_body(NSInst& G) {
         return;
     }
 
-    // Arcs in steps; the matrix first.  A block is a whole number of steps of the
-    // pricing threads, at most the stage; the explicit arcs of a matrix instance
-    // are blocks of their own, read in place.
+    // Arcs in steps; the matrix first.  The explicit arcs of a matrix instance are
+    // blocks of their own, read in place.
     const int32_t QI = IMPL ? (int32_t)(I.mst / STEP) : (int32_t)((I.m + 3) >> 2);  // staged steps
     const int32_t Q = IMPL ? QI + (int32_t)((I.m - I.mst + 3) >> 2) : QI;
-    const int32_t B = Layout<LAY>::PRICERS * max(1, (int32_t)min((I.block + STEP * Layout<LAY>::PRICERS / 2) / (STEP * Layout<LAY>::PRICERS),
-                                                        (int64_t)(STAGED / Layout<LAY>::PRICERS)));
+    const int32_t B = block_steps<LAY>(I.block, STEP);
     const int pt = tid - 32;  // this pricing thread
     const int32_t nS = (int32_t)I.nS, ldq = IMPL ? (int32_t)(I.ld / STEP) : 1;
     // row and sinks' potentials of a step, as byte offsets
@@ -880,6 +886,15 @@ const Kernel kernels[S32_CLASSES] = {k_simplex32<1, false>, k_simplex32<1, true>
 }  // namespace
 
 int s32_class(const NSInst& h) { return h.lay32 ? 2 * (h.lay32 - 1) + (h.mst > 0 ? 1 : 0) : -1; }
+
+int64_t s32_block(int cls, int64_t block) {
+    const int step = cls == S32_HALF || (cls & 1) ? 8 : 4;
+    const int32_t steps = cls == S32_HALF ? block_steps<4>(block, step)
+                          : cls / 2 == 0  ? block_steps<1>(block, step)
+                          : cls / 2 == 1  ? block_steps<2>(block, step)
+                                          : block_steps<3>(block, step);
+    return (int64_t)steps * step;
+}
 
 void s32_launch(int cls, int grid, NSInst* insts, const int32_t* order, int32_t count, int32_t* next,
                 cudaStream_t st) {
