@@ -111,3 +111,22 @@ def test_a_mixed_wave_overlaps(pd, ctx):
     apart = ms(far), ms(near)
     assert min(apart) > 40
     assert ms(far + near) < max(apart) + 0.5 * min(apart), apart
+
+
+# cost matrices on the layouts with more nodes (N + 2 up to 13,040 and 23,664, then
+# the 64-bit kernel), rows from every alignment of the sinks' potentials, either
+# side the longer one, cold and from a start.  At s = 2,000 no two nodes of the
+# 128 x 256 lattice are separated before they are leaves: every arc of the matrix is
+# one of the network and the certificate holds.
+@pytest.mark.parametrize("na,nb", [(57, 12981), (58, 12981), (61, 13500), (64, 14001), (59, 23603), (60, 23603),
+                                   (13500, 62)])
+def test_large_matrices(pd, ctx, na, nb):
+    at = np.random.default_rng(na * nb).permutation(1 << 15)[: na + nb]
+    pts = np.stack([at // 256, at // 256 + 1 + at % 256], 1).astype(np.float32) / 64
+    A, B = (torch.from_numpy(np.ascontiguousarray(p)).cuda() for p in (pts[:na], pts[na:]))
+    kw = dict(condense=0, ns_transport=2, s_override=2000)
+    exp = pd.pd_w1_approx(ctx, A, B, 0.1, pd.opts(warm_start=0, ns_smem=0, **kw))
+    for start in (0, 3, 4):
+        got = pd.pd_w1_approx(ctx, A, B, 0.1, pd.opts(warm_start=start, **kw))
+        assert got["cert_failures"] == exp["cert_failures"] == 0
+        assert got["opt_quanta"] == exp["opt_quanta"]
