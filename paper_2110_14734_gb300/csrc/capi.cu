@@ -1058,8 +1058,7 @@ extern "C" pd_status pd_ws_train(pd_ctx* c, const pd_diagram* A, const pd_diagra
         NSInst rec{};
         PD_TRY(ns_run(c, &w.ns.h, 1, d, &rec, st));
         PD_TRY(ns_status(c, rec));
-        const int64_t cmax = (rec.big - 1) / (int64_t)(rec.n + 1) - 1;
-        PD_TRY(ws_collect(c, f.nodes, w, d, rec, cmax, base.empty() ? nullptr : &base, st));
+        PD_TRY(ws_collect(c, f.nodes, w, rec, base.empty() ? nullptr : &base, st));
         r.pairs++;
         r.cold_pivots += rec.pivots;
     }

@@ -218,7 +218,9 @@ struct MlpW {
 };
 
 constexpr int WS_THREADS = 256;
-constexpr int WS_LD = WS_TILE + 4;  // floats between units: 16-byte loads, two-way conflicts at most
+// Floats between units, for 16-byte loads: no conflicts in the products, two ways where
+// they are stored; the gradients' lanes lie 8 and 4 units apart, eight and four ways.
+constexpr int WS_LD = WS_TILE + 4;
 
 // Thread t: rows 4 (t / 64) .. + 3, units 2 (t % 64) and the next.
 struct MlpTile {
@@ -725,9 +727,9 @@ pd_status ws_predict(Ctx* c, const pd_nodes& nodes, const W1Prep& w, std::vector
 }
 
 // Training rows of one solved pair appended to the context's data set: the
-// instance's features and the targets from the solved record d_res.
-pd_status ws_collect(Ctx* c, const pd_nodes& nodes, const W1Prep& w, const NSInst* d_res, const NSInst& r,
-                     int64_t cmax, const std::vector<double>* base, cudaStream_t st) {
+// instance's features and the targets from the solved record r.
+pd_status ws_collect(Ctx* c, const pd_nodes& nodes, const W1Prep& w, const NSInst& r,
+                     const std::vector<double>* base, cudaStream_t st) {
     const int64_t n = w.nS + w.nT;
     if (n <= 0) return PD_OK;
     const int64_t have = c->ws_rows;
@@ -778,8 +780,6 @@ pd_status ws_collect(Ctx* c, const pd_nodes& nodes, const W1Prep& w, const NSIns
                                                 db ? c->last_coarse_cell : 0, T + have, M + have); pd::count_launch();
     PD_TRY_CUDA(c, cudaGetLastError());
     PD_TRY_CUDA(c, cudaStreamSynchronize(st));  // the base copy's host memory belongs to the caller
-    (void)d_res;
-    (void)cmax;
     c->ws_rows = have + n;
     return PD_OK;
 }

@@ -46,8 +46,8 @@ pd_status ws_features(Ctx* c, const pd_nodes& nodes, const W1Prep& w, __nv_bfloa
 pd_status ws_predict(Ctx* c, const pd_nodes& nodes, const W1Prep& w, std::vector<float>* p, cudaStream_t st);
 // Potentials +d(u) / -d(v) from the distance to the diagonal (host, nS + nT + 1).
 pd_status ws_diag_potentials(Ctx* c, const pd_nodes& nodes, const W1Prep& w, std::vector<float>* p, cudaStream_t st);
-pd_status ws_collect(Ctx* c, const pd_nodes& nodes, const W1Prep& w, const NSInst* d_res, const NSInst& r,
-                     int64_t cmax, const std::vector<double>* base, cudaStream_t st);
+pd_status ws_collect(Ctx* c, const pd_nodes& nodes, const W1Prep& w, const NSInst& r,
+                     const std::vector<double>* base, cudaStream_t st);
 
 // Strongly feasible start of a prepared transportation instance from
 // potentials p (host, one per transportation node, cost units); the greedy

@@ -42,7 +42,7 @@ struct NSInst {
     int64_t block;     // pricing block (arcs)
     int64_t big;       // cost of the artificial arcs
     int64_t big64;     // ... that the 64-bit kernel takes when it solves the instance again: more than any path cost
-    int32_t lay32;     // k_simplex32's layout (1 .. 3); 0: the instance belongs to k_netsimplex
+    int32_t lay32;     // k_simplex32's layout (1 .. 3; ns_plan may launch 1 as 4, on half an SM); 0: k_netsimplex's
     int32_t big_safe;  // 1: `big` proves infeasibility when artificial flow remains
     int32_t smem_nodes; // node arrays: 1 all in shared memory, 2 all but pred / flow, 3 the 16-bit ones, 0 global
     int32_t walk;      // shared-memory layout: longest half-cycle side followed by the two-lane walk (longer: the scan)

@@ -16,8 +16,8 @@
 //           so the entering arc's reduced cost is exact.
 //   scan    The preorder keeps, by position, node and end of its subtree in one
 //           word (end in the high half), so "the node at position x <= p has p
-//           in its subtree" is one unsigned comparison of that word, four
-//           positions per 16-byte load.  Nodes above exactly one end of the
+//           in its subtree" is one unsigned comparison of that word.  A warp
+//           reads 128 positions at a time, a lane every 32nd of them.  Nodes above exactly one end of the
 //           entering arc are the two half-cycles; they are collected unordered.
 //   pivot   One warp: ratio test (positions order a path, so neither the
 //           minimum nor its tie rule needs the path in order), flows and
@@ -145,7 +145,6 @@ struct Nodes {
     }
     // position x: node | end of its subtree << 16
     PD_D uint32_t& ord(int32_t x) const { return *(uint32_t*)(s32_dyn + L::ord + 4 * x); }
-    PD_D uint4 ord4(int32_t x) const { return *(const uint4*)(s32_dyn + L::ord + 4 * x); }
     PD_D uint16_t& pos(int32_t v) const { return *(uint16_t*)(s32_dyn + L::pos + 2 * v); }
     PD_D uint16_t& par(int32_t v) const { return *(uint16_t*)(s32_dyn + L::par + 2 * v); }
 };

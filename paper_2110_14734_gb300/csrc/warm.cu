@@ -397,8 +397,8 @@ pd_status ns_warm_tree(Ctx* c, NSPrep* prep, const double* p, int64_t max_residu
     std::vector<int32_t> comp_order;
     // Every component hangs from the root by the artificial arc of its root
     // node r0, whose cost big + art[r0] sets pi(r0): art[r0] = p(r0) - min p
-    // over the component roots keeps the predicted offsets between components
-    // (one common big would erase them).  The other supply nodes' artificial
+    // over the component roots keeps the predicted offsets between components, up
+    // to big - 1 (one common big would erase them).  The other supply nodes' artificial
     // arcs cost 2 big - 1, far above their potentials, so they never enter.
     // Every artificial cost is >= big: still a valid big-M start.
     std::vector<int64_t> art((size_t)nt, 0);
