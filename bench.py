@@ -575,7 +575,9 @@ def run_ours(args):
     algo_bytes = 4.0 * statistics.mean(priced)  # one int32 cost streamed per priced arc
     achieved = algo_bytes / (avg_ns_ms / 1000.0) / 1e9
     pk, pk_src = peaks()
-    roof = {"kernel": "k_simplex32", "bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
+    # (the kernel is bound by the latency of its pivots; the bandwidth is what it streams meanwhile, arcs
+    # priced in the shadow of a pivot and not used included)
+    roof = {"kernel": "k_simplex32", "bound": "latency", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
             "frac": achieved / pk["hbm_gbs"], "traffic": load_traffic("k_simplex32"), "peak_source": pk_src,
             "algorithmic_bytes_per_launch": algo_bytes, "avg_launch_ms": avg_ns_ms,
             "share_of_step": avg_ns_ms / statistics.mean(step_ms)}
@@ -590,7 +592,7 @@ def run_ours(args):
             "data": "synthetic (seeded lower-star uint8 diagrams of Gaussian-smoothed noise images)",
             "config": {"workload": WORKLOAD, "n_points": args.n, "eps": args.eps, "s": r0["s"],
                        "pairs_per_step": P, "diagrams": len(diags), "distinct_pairs": len(pairs_all),
-                       "form": "batched: one persistent simplex launch per step (one CTA per SM, pairs "
+                       "form": "batched: one persistent simplex launch per step and form of the kernel (pairs "
                                "largest first)",
                        "l2": "flushed between timed steps (256 MiB write); inputs of a step > L2",
                        "parallelism": "replicas" if ws > 1 else "single GPU",

@@ -248,10 +248,10 @@ pd_status pd_wspd_sparsify_tree(pd_ctx* ctx, const pd_nodes* nodes, int32_t s, i
 
 /*
  * Size of the sparse network of pd_wspd_sparsify_tree without building it:
- * the WSPD is enumerated level by level and its pairs counted, no arc is
- * stored.  *n_arcs_out (host) = WSPD biarcs + diagonal arcs + 1, exactly
- * pd_wspd_sparsify_tree's n_arcs.  Device memory: the pair frontier of one
- * level at a time (8 bytes per pair not yet separated).
+ * the WSPD's pairs are walked and counted, no arc is stored.  *n_arcs_out
+ * (host) = WSPD biarcs + diagonal arcs + 1, exactly pd_wspd_sparsify_tree's
+ * n_arcs.  Device memory: 48 bytes per node, and up to 1,024 for pairs handed
+ * from one launch to the next (less under a cap).
  */
 pd_status pd_wspd_count(pd_ctx* ctx, const pd_nodes* nodes, int32_t s, int32_t tree, int64_t* n_arcs_out,
                         void* stream);
@@ -303,7 +303,8 @@ pd_status pd_w1_sparsify_count(pd_ctx* ctx, pd_diagram A, pd_diagram B, double e
  * preprocessing of the wave's pairs, each on its own stream after the work
  * already queued on `stream`; then the network simplex solves of the wave
  * share one persistent launch per form of the kernel (one CTA per SM, or two
- * when more pairs than SMs fit half of one, takes the pairs, largest first); then each pair's certificate runs.
+ * when more pairs than SMs fit half of one, takes the pairs, largest first;
+ * the forms run side by side); then each pair's certificate runs.
  * A and B: host arrays of `count` descriptors; out: host array of `count`
  * results (ns_kernel_ms and stage_ms[6] include the wave's shared launch).
  * Device memory: one buffer set per slot, grown on demand and kept by the

@@ -21,7 +21,7 @@ enum Buf : int {
     B_CKEY, B_CKEY2, B_CVAL, B_CVAL2, B_CIDX, B_CX, B_CY, B_CA, B_CB,
     B_NX, B_NY, B_NCA, B_NCB, B_NCODE,  // output nodes
     B_T_LEFT, B_T_RIGHT, B_T_BB, B_T_REP, B_T_PARENT, B_T_LPARENT, B_T_VISIT, B_T_LEAVES, B_T_LEAFXY,
-    B_F0, B_F1, B_WSFLAG, B_WSOFF,  // WSPD frontier
+    B_F0, B_F1, B_WSFLAG, B_WSOFF,  // WSPD walk
     B_ARCKEY, B_ARCKEY2,            // arc keys (tail << hb | head)
     B_ROWPTR, B_HEAD, B_COST, B_SUPPLY,
     B_S_ROWPTR, B_S_HEAD, B_S_CW, B_S_TWIN, B_S_X, B_S_PAIR, B_S_XKEY, B_S_XKEY2, B_S_XVAL,

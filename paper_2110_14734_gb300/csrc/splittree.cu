@@ -17,7 +17,7 @@
 //
 // Node numbering is the radix tree's (root 0, a child covering [lo, split]
 // is numbered split, one covering [split + 1, hi] split + 1, leaves ~position),
-// and the nodes are renumbered by their leaf position, so the WSPD frontier,
+// and the nodes are renumbered by their leaf position, so the WSPD walk,
 // the network builder and the tree certificate run unchanged on this tree.
 #include "internal.h"
 #include "prims.cuh"

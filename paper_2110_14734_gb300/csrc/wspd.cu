@@ -1,5 +1,5 @@
 // Hierarchical tree (binary radix tree over Morton order), s-WSPD biarcs
-// (Algorithms 6-8 as a level-synchronous pair frontier), diagonal arcs
+// (Algorithms 6-8, pairs walked depth first), diagonal arcs
 // (Algorithm 9) and the CSR network.
 #include "internal.h"
 #include "netsimplex.cuh"
@@ -99,7 +99,7 @@ __global__ void k_bbox(int64_t N, const int32_t* __restrict__ X, const int32_t* 
 }
 
 // ---------------------------------------------------------------------------
-// s-WSPD as a pair frontier
+// separation test, and membership of one arc in the s-WSPD (certificate)
 // ---------------------------------------------------------------------------
 
 struct TNode {
@@ -153,7 +153,7 @@ PD_D int64_t max_side(const TNode& a) {
 // Is (a, b), a < b two leaves (Morton ranks), one of the biarcs of the
 // s-WSPD?  The pairs of the decomposition partition all leaf pairs, so (a, b)
 // lies in exactly one of them: start at the pair of children of the lowest
-// common ancestor and follow the same split rule as k_ws_expand (larger box
+// common ancestor and follow the same split rule as k_ws_walk (larger box
 // side, ties split the second node), always into the child holding a
 // (resp. b), until the pair is well separated.  (a, b) is an arc iff a and b
 // are the representatives of that pair.  A walk longer than any tree path
