@@ -179,9 +179,10 @@ cudaError_t exclusive_scan(const T* in, T* out, int64_t n, T* part, T* total_dev
 // publishes its own counts, then their running sum; tile numbers are tickets, so
 // the tiles looked back at have started), orders the keys in shared memory and
 // writes them in runs.  Should a tile looked back at not have published after the
-// bounded wait, its digits are counted from the keys, which this pass only
-// reads: the sort never waits without end and never ends unsorted.  A pass moves each key once in and once out; what bounds it
-// is the ranking and the look-back's latency: 2,000,000 64-bit keys 26 us a pass
+// bounded wait, its digits and all before it are counted from the keys, which this
+// pass only reads: the sort never waits without end and never ends unsorted.  A
+// pass moves each key once in and once out; what bounds it is the ranking and the
+// look-back's latency: 2,000,000 64-bit keys 26 us a pass
 // (5 at the copy rate), two tiles an SM at a time.
 //
 // Short arrays (at most CS_MAX): one block sorts in shared memory, one launch for
@@ -210,8 +211,9 @@ constexpr int RS_BACK = 8;                                // tiles looked back a
 
 inline int64_t radix_tiles(int64_t n) { return (n + RS_TILE - 1) / RS_TILE; }
 inline int radix_passes(int bits) { return (bits + 7) / 8; }
-// Words of scratch of `passes` passes: their counts, tickets and states.
-inline int64_t radix_words(int64_t n, int passes) { return passes * (256 + 1 + 256 * radix_tiles(n)); }
+// Words of scratch of `passes` passes: their counts, states (rows of 2 KB, aligned to
+// lines) and tickets.
+inline int64_t radix_words(int64_t n, int passes) { return passes * (256 + 256 * radix_tiles(n) + 1); }
 
 // Digit counts of the passes first .. first + passes - 1.
 __global__ void __launch_bounds__(RS_THREADS) k_radix_counts(const uint64_t* __restrict__ keys, int64_t n, int first,

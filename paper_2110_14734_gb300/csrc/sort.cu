@@ -21,10 +21,11 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_counts(const uint64_t* __r
         if (h[p][threadIdx.x]) atomicAdd(&hist[256 * p + threadIdx.x], (unsigned long long)h[p][threadIdx.x]);
 }
 
-// Keys of the whole tile t with digit d.
-__device__ __noinline__ uint32_t tile_count(const uint64_t* __restrict__ keys, int64_t t, int shift, uint32_t d) {
-    uint32_t c = 0;
-    for (int i = 0; i < RS_TILE; i++) c += ((uint32_t)(keys[t * RS_TILE + i] >> shift) & 0xffu) == d;
+// Keys with digit d among the first n.
+__device__ __noinline__ unsigned long long count_digit(const uint64_t* __restrict__ keys, int64_t n, int shift,
+                                                       uint32_t d) {
+    unsigned long long c = 0;
+    for (int64_t i = 0; i < n; i++) c += ((uint32_t)(keys[i] >> shift) & 0xffu) == d;
     return c;
 }
 
@@ -81,6 +82,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_pass(const uint64_t* __res
     // only their own counts out yet (condensation of 2,000,000 points: 0.731 ms one
     // by one, 0.714 so)
     unsigned long long before = 0;
+    int64_t rest = 0;  // keys before the tiles that answered, all of whose digits are to be counted
     bool open = tile > 0;
     for (int64_t t = tile - 1; open; t -= RS_BACK) {
         unsigned long long v[RS_BACK];
@@ -90,11 +92,12 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_pass(const uint64_t* __res
         for (int j = 0; j < RS_BACK; j++) {
             if (!open) continue;
             for (int q = 0; v[j] >> 62 == 0 && q < polls; q++) v[j] = state[256 * (t - j) + tid];
-            if (v[j] >> 62 == 0) v[j] = 1ull << 62 | tile_count(kin, t - j, shift, tid);  // only the last tile is short
+            if (v[j] >> 62 == 0) rest = (t - j + 1) * RS_TILE;  // and the search ends
             before += v[j] & RS_VALUE;
             open = v[j] >> 62 == 1;
         }
     }
+    if (rest > 0) before += count_digit(kin, rest, shift, tid);
     if (tile > 0) state[256 * tile + tid] = 2ull << 62 | (before + c);
     first[tid] = ex;
     base[tid] = (int64_t)(hx + before) - (int64_t)ex;
@@ -181,7 +184,7 @@ pd_status sort_u64(Ctx* c, uint64_t*& keys, uint64_t*& keys_alt, uint32_t*& vals
         w = bufT<unsigned long long>(c, B_RS_COUNTS, radix_words(n, sets));
     }
     if (!w) return PD_ENOMEM;
-    unsigned long long *hist = w, *ticket = w + 256 * sets, *state = ticket + sets;
+    unsigned long long *hist = w, *state = w + 256 * sets, *ticket = state + 256 * tiles * sets;
     const unsigned count_grid = (unsigned)std::min<int64_t>(tiles, 4 * std::max(c->sm_count, 1));
     for (int p = 0; p < passes; p++) {
         const int q = p % sets;
