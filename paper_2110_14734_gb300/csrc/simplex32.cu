@@ -107,11 +107,13 @@ struct Layout {
 
 // Steps of a pricing block of `block` arcs (STEP: a step's arcs): a whole number of
 // the pricing threads, at most the stage.
-template <int LAY>
-PD_HD constexpr int32_t block_steps(int64_t block, int step) {
-    constexpr int P = Layout<LAY>::PRICERS, most = (int)(Layout<LAY>::STAGE / 32) / P;
-    const int64_t k = (block + step * P / 2) / (step * P);
-    return P * (int32_t)(k < 1 ? 1 : k < most ? k : most);
+template <int LAY, int STEP>
+PD_HD constexpr int32_t block_steps(int64_t block) {
+    constexpr int P = Layout<LAY>::PRICERS;
+    constexpr int64_t most = (int32_t)(Layout<LAY>::STAGE / 32) / P;
+    const int64_t k = (block + STEP * P / 2) / (STEP * P);
+    const int32_t m = (int32_t)(k < most ? k : most);
+    return P * (m > 1 ? m : 1);
 }
 
 template <int LAY>
@@ -555,7 +557,7 @@ PD_D void s32_body(NSInst& G) {
     // blocks of their own, read in place.
     const int32_t QI = IMPL ? (int32_t)(I.mst / STEP) : (int32_t)((I.m + 3) >> 2);  // staged steps
     const int32_t Q = IMPL ? QI + (int32_t)((I.m - I.mst + 3) >> 2) : QI;
-    const int32_t B = block_steps<LAY>(I.block, STEP);
+    const int32_t B = block_steps<LAY, STEP>(I.block);
     const int pt = tid - 32;  // this pricing thread
     const int32_t nS = (int32_t)I.nS, ldq = IMPL ? (int32_t)(I.ld / STEP) : 1;
     // row and sinks' potentials of a step, as byte offsets
@@ -886,13 +888,15 @@ const Kernel kernels[S32_CLASSES] = {k_simplex32<1, false>, k_simplex32<1, true>
 
 int s32_class(const NSInst& h) { return h.lay32 ? 2 * (h.lay32 - 1) + (h.mst > 0 ? 1 : 0) : -1; }
 
+template <int LAY>
+static int64_t block_arcs(bool matrix, int64_t block) {
+    return matrix ? 8 * (int64_t)block_steps<LAY, 8>(block) : 4 * (int64_t)block_steps<LAY, 4>(block);
+}
+
 int64_t s32_block(int cls, int64_t block) {
-    const int step = cls == S32_HALF || (cls & 1) ? 8 : 4;
-    const int32_t steps = cls == S32_HALF ? block_steps<4>(block, step)
-                          : cls / 2 == 0  ? block_steps<1>(block, step)
-                          : cls / 2 == 1  ? block_steps<2>(block, step)
-                                          : block_steps<3>(block, step);
-    return (int64_t)steps * step;
+    if (cls == S32_HALF) return block_arcs<4>(true, block);
+    const bool matrix = cls & 1;
+    return cls / 2 == 0 ? block_arcs<1>(matrix, block) : cls / 2 == 1 ? block_arcs<2>(matrix, block) : block_arcs<3>(matrix, block);
 }
 
 void s32_launch(int cls, int grid, NSInst* insts, const int32_t* order, int32_t count, int32_t* next,
