@@ -26,7 +26,7 @@
 // An instance may instead carry its own strongly feasible start (warm start).
 //
 // Instances whose potentials fit 32 bits go to simplex32.cu; this kernel takes
-// the others (more than 65,533 nodes, arc costs above 2^25 quanta, ...) and the
+// the others (more than 23,662 nodes, arc costs above 2^25 quanta, ...) and the
 // few that simplex32.cu hands back.
 #include <algorithm>
 #include <mutex>
@@ -726,14 +726,45 @@ __device__ __forceinline__ void ns_body(NSInst& G, NSInst& I, Tree<IX>& T) {
     }
 }
 
+// The tree that k_simplex32 ended on, for artificial arcs that cost big: its arcs and
+// flows stay, and every part that hangs from the root by an artificial arc, a warp
+// each, moves with that arc's cost.  Costs up to 2^25 on a grid of 900 nodes: 4.9
+// ms from there, 12.3 from a cold start; 3,600 nodes: 30 and 71.
+__device__ __noinline__ void ns_raise(NSInst& G, int64_t big) {
+    const int32_t n = G.n;
+    const int lane = threadIdx.x & 31;
+    for (int32_t v = threadIdx.x; v <= n; v += NS_THREADS) G.ord[G.pos[v]] = v;
+    __syncthreads();
+    for (int32_t v = threadIdx.x >> 5; v < n; v += NS_THREADS / 32) {
+        if (G.parent[v] != n) continue;
+        const int64_t d = (G.up[v] ? big : -big) - G.pi[v];
+        __syncwarp();
+        const int32_t x0 = G.pos[v], x1 = x0 + G.size[v];
+        for (int32_t x = x0 + lane; x < x1; x += 32) G.pi[G.ord[x]] += d;
+    }
+    __syncthreads();
+}
+
 __device__ __forceinline__ void ns_instance(NSInst& G) {
+    __shared__ int64_t s_before[3];  // pivots, degenerate ones and arcs priced by k_simplex32 (thread 0's)
     NSInst I = G;
+    if (threadIdx.x < 3) s_before[threadIdx.x] = 0;
+    __syncthreads();
     if (I.lay32) {
-        // handed back by simplex32.cu: a cold start with costs that its 32 bits could not hold
+        // handed back by simplex32.cu: with artificial costs that its 32 bits could not hold
         if (I.status != S32_REDO) return;
         I.big = I.big64;
-        I.init_tree = 0;
         I.art = nullptr;
+        I.init_tree = I.pivots >= 0;
+        if (I.init_tree) {
+            if (threadIdx.x == 0) {
+                s_before[0] = I.pivots;
+                s_before[1] = I.degenerate;
+                s_before[2] = I.scanned;
+            }
+            I.max_pivots -= I.pivots;
+            ns_raise(G, I.big);
+        }
     }
     const int32_t N1 = I.n + 1;
     if (I.smem_nodes) {
@@ -778,6 +809,11 @@ __device__ __forceinline__ void ns_instance(NSInst& G) {
         T.ps = I.pos;
         T.od = I.ord;
         ns_body<int32_t>(G, I, T);
+    }
+    if (threadIdx.x == 0) {  // (the last writes of ns_body are this thread's)
+        G.pivots += s_before[0];
+        G.degenerate += s_before[1];
+        G.scanned += s_before[2];
     }
 }
 
@@ -958,6 +994,7 @@ void ns_choose_kernel(NSInst* h, int64_t cmax, bool complete, bool smem, int max
     if (!smem || cmax > S32_MAX_COST || (h->m > h->mst && !h->th) || (h->mst > 0 && h->ld % 8 != 0)) return;
     h->lay32 = s32_layout(N1);
     if (h->lay32 == 0) return;
+    h->pivots = -1;
     if (complete) {
         h->big = cmax + 1;
     } else if (h->big64 > S32_MAX_BIG) {

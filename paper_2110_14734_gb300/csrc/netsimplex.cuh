@@ -53,7 +53,7 @@ struct NSInst {
     uint64_t time_limit_ns;
     // results
     int64_t opt;
-    int64_t pivots;
+    int64_t pivots;    // (k_simplex32 leaves -1 when it has no tree to go on from)
     int64_t degenerate;
     int32_t status;    // 0 ok, 1 infeasible, 2 pivot cap / time, 3 unbounded, 4 path too long, S32_REDO
     int32_t pad;

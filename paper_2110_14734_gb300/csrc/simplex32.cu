@@ -38,8 +38,8 @@
 // subtree by |reduced cost|; the exact maximum is taken again when the bound is
 // reached), costs are at most 2^25, so no sum overflows.  An instance that
 // would leave the range, or that ends with flow on an artificial arc although
-// `big` was not above every path's cost, reports S32_REDO and is solved again
-// by the 64-bit kernel.  Artificial arcs leave the problem when they leave the
+// `big` was not above every path's cost, reports S32_REDO and goes on in the
+// 64-bit kernel, from the tree it has.  Artificial arcs leave the problem when they leave the
 // tree: they are never priced.
 #include <mutex>
 #include <type_traits>

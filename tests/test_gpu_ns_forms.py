@@ -130,3 +130,40 @@ def test_large_matrices(pd, ctx, na, nb):
         got = pd.pd_w1_approx(ctx, A, B, 0.1, pd.opts(warm_start=start, **kw))
         assert got["cert_failures"] == exp["cert_failures"] == 0
         assert got["opt_quanta"] == exp["opt_quanta"]
+
+
+def _grid(side, top):
+    """A square grid, arcs both ways between neighbours, costs up to top."""
+    rng = np.random.default_rng(side)
+    n = side * side
+    u = np.arange(n)
+    r, d = u[u % side < side - 1], u[u < n - side]
+    t, h = np.r_[r, r + 1, d, d + side], np.r_[r + 1, r, d + side, d]
+    o = np.lexsort((h, t))
+    sup = np.zeros(n, np.int64)
+    at = rng.permutation(n)[: n // 4 * 2]
+    k = len(at) // 2
+    sup[at[:k]] = rng.integers(1, 9, k)
+    sup[at[k:]] = -sup[at[:k]]
+    a = dict(row_ptr=np.r_[0, np.cumsum(np.bincount(t, minlength=n))], head=h[o].astype(np.int32),
+             cost=rng.integers(1, top + 1, len(t))[o], supply=sup)
+    return {x: torch.from_numpy(v).cuda() for x, v in a.items()}
+
+
+# Routes of more than 32 bits of cost: the 32-bit kernel's tree, from each of its
+# layouts, is where the 64-bit kernel goes on.
+@pytest.mark.parametrize("side", [30, 100, 130])
+def test_a_handed_back_tree_goes_on(pd, ctx, side):
+    big = _grid(side, 1 << 25)
+    opt, r = pd.pd_mcf_solve(ctx, big)
+    exp = pd.pd_mcf_solve(ctx, big, pd.opts(ns_smem=0))[0]
+    assert opt == exp and opt == pd.pd_mcf_solve(ctx, big, pd.opts(max_rounds=r["pivots"]))[0]
+    with pytest.raises(pd.PDError) as e:  # pivots of both kernels count
+        pd.pd_mcf_solve(ctx, big, pd.opts(max_rounds=r["pivots"] - 1))
+    assert e.value.status == pd.PD_ETIMEOUT
+
+
+# ... which takes 1.7 times as long as a solve that fits, and 4.2 times from a cold start
+def test_a_handed_back_solve_is_not_done_twice(pd, ctx):
+    ms = [min(pd.pd_mcf_solve(ctx, _grid(30, top))[1]["ns_kernel_ms"] for _ in range(4)) for top in (1 << 25, 1 << 10)]
+    assert ms[0] < 2.8 * ms[1], ms
