@@ -1495,7 +1495,7 @@ pd_status ns_solve_network(Ctx* c, const pd_network& net, const pd_opts& o, Solv
     PD_TRY_CUDA(c, cudaMemsetAsync(sm, 0, 8 * sizeof(unsigned long long), st));
     if (m > 0 && packed) {
         k_arc_pack<<<grid_for(32 * (n + 1), 256), 256, 0, st>>>(net.row_ptr, net.head, net.cost, n, m,
-                                                                ns_chunk_stride(m), (uint32_t*)tail, c32, sm,
+                                                                ns_chunk_stride(n, m), (uint32_t*)tail, c32, sm,
                                                                 sm + 1); pd::count_launch();
     } else if (m > 0) {
         k_arc_tails<<<grid_for(m, 256), 256, 0, st>>>(net.row_ptr, n, m, tail); pd::count_launch();

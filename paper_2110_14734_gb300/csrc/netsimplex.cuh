@@ -86,14 +86,17 @@ cudaError_t s32_kernel_setup();  // as ns_kernel_setup
 // chunks of NS_CHUNK arcs, the last one padded, chunk c at place c * stride mod
 // their number; bad += costs outside [0, 2^31), *cmax = the largest.  n < 65535.
 //
-// Neighbouring rows belong to neighbouring nodes, and so do the arcs of a
-// pricing block if they stay in order.  In a large network many blocks then hold no
-// arc worth entering, and the kernel has to price again; spread out, every block
-// samples the whole network.  In a small one the order is worth more: cycles
-// stay short.  19.5 M arcs (10,000 nodes): 1,964 ms in order, 912 spread; 1.9 M
-// arcs: 98 and 102.  Rows of a cost matrix stay in order too: 100,000 lower-star
-// points 278 ms, spread 291 (path nodes a pivot 51, spread 79); 20,000: 119 and
-// 113; 2,000 uniform points: 25.7 and 25.1.
+// Neighbouring rows belong to neighbouring nodes, and so do the arcs of a pricing
+// block if they stay in order.  Spread out, every block samples the whole network.
+// What that does to the pivots depends on the network (in order / spread, s each):
+// mixtures of 5,000 + 5,000 points (5.0 M arcs) 0.39 / 0.12, 9,000 + 9,000 (5.1 M)
+// 0.88 / 0.37; Gaussians of 5,000 + 5,000 (5.9 M) 0.23 / 0.27, 10,000 + 10,000 (39 M)
+// 2.5 / 2.8, 14,500 + 14,500 (7.5 M) 1.4 / 2.1; a mixture of 1.9 M arcs 0.098 / 0.102.
+// So spread from NS_SPREAD_ARCS on, where what is gained is the larger part, but only
+// up to the nodes of k_simplex32: beyond them longer cycles cost too much (Gaussians
+// of 24,432 nodes and 5.0 M arcs 2.9 / 5.0, 32,714 and 8.0 M 16.5 / 52.9).  Rows of a cost
+// matrix stay in order too: 100,000 lower-star points 278 ms, spread 291 (path nodes
+// a pivot 51, spread 79); 20,000: 119 and 113; 2,000 uniform points: 25.7 and 25.1.
 constexpr int64_t NS_CHUNK = 64;
 constexpr int64_t NS_SPREAD_ARCS = int64_t(1) << 22;
 PD_HD int64_t ns_chunks(int64_t m) { return (m + NS_CHUNK - 1) / NS_CHUNK; }
@@ -101,11 +104,11 @@ __global__ void k_arc_pack(const int64_t* __restrict__ rp, const int32_t* __rest
                            const int64_t* __restrict__ cost, int64_t n, int64_t m, int64_t stride,
                            uint32_t* __restrict__ th, int32_t* __restrict__ c32, unsigned long long* __restrict__ bad,
                            unsigned long long* __restrict__ cmax);
-// The stride of m arcs' chunks: 1 below NS_SPREAD_ARCS, else about the golden ratio
-// of their number and coprime to it.
-inline int64_t ns_chunk_stride(int64_t m) {
+// The stride of the chunks of m arcs between `nodes` nodes: 1, or (see above) about the
+// golden ratio of their number and coprime to it.
+inline int64_t ns_chunk_stride(int64_t nodes, int64_t m) {
     const int64_t n = ns_chunks(m);
-    if (m < NS_SPREAD_ARCS) return 1;
+    if (m < NS_SPREAD_ARCS || s32_layout(nodes + 1) == 0) return 1;
     int64_t s = (int64_t)(0.6180339887498949 * (double)n);
     for (;; s++) {
         int64_t a = n, b = s;

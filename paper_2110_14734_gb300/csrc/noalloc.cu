@@ -110,7 +110,7 @@ extern "C" pd_status pd_mcf_solve_noalloc(const pd_network* net, int64_t* opt_ou
     k_check_network<<<grid_for(n, 256), 256, 0, st>>>(net->row_ptr, net->head, n, m, flags); pd::count_launch();
     if (m > 0) {
         k_arc_pack<<<grid_for(32 * (n + 1), 256), 256, 0, st>>>(net->row_ptr, net->head, net->cost, n, m,
-                                                                ns_chunk_stride(m), th, c32,
+                                                                ns_chunk_stride(n, m), th, c32,
                                                                 flags + 1, flags + 2); pd::count_launch();
     }
     k_abs_sum<<<grid_for(n, 256), 256, 0, st>>>(net->supply, n, flags + 3); pd::count_launch();

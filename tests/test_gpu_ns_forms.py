@@ -167,3 +167,12 @@ def test_a_handed_back_tree_goes_on(pd, ctx, side):
 def test_a_handed_back_solve_is_not_done_twice(pd, ctx):
     ms = [min(pd.pd_mcf_solve(ctx, _grid(30, top))[1]["ns_kernel_ms"] for _ in range(4)) for top in (1 << 25, 1 << 10)]
     assert ms[0] < 2.8 * ms[1], ms
+
+
+# Lists of more nodes than the 32-bit kernel holds stay in order: 174,644 pivots
+# (2.9 s), spread over the pricing blocks 274,555 (5.0 s).
+def test_large_lists_stay_in_order(pd, ctx):
+    A, B = (torch.from_numpy(synth.gaussian_pd(15000, s)).cuda() for s in (1000, 1001))
+    r = pd.pd_w1_approx(ctx, A, B, 0.1, pd.opts(s_override=9, ns_transport=0, warm_start=0))
+    assert r["n_nodes"] > 23663 and r["n_arcs"] > 1 << 22
+    assert r["pivots"] < 220000
