@@ -497,27 +497,34 @@ constexpr int64_t RW_SMALL = 8192;
 // ---- the same minima through a uniform grid over each side ----------------
 // Large sides make the all-pairs scan quadratic (about 10^12 distance
 // evaluations at a million nodes a side).  Each side's nodes are bucketed into a
-// grid (a counting sort by cell), and every node of the other side searches square
-// rings of cells around its own cell.  After ring K every node not yet seen lies
-// beyond one of the square's sides that are not the grid's border, so its distance
-// is at least LB, the distance from the query to the nearest such side.  The
+// grid (a counting sort by cell), and every node of the other side searches
+// growing squares of cells around its own cell.  After a square of half side K every
+// node not yet seen lies beyond one of its sides that are not the grid's border, so
+// its distance is at least LB, the distance from the query to the nearest such side.  The
 // search stops when LB^2 >= the best squared distance found (the minimum is
 // exact), or when LB >= the query's diagonal cost c_make: every unseen node then
 // costs at least c_make, the relaxed flow takes min(c(u, nearest), c_make) either
 // way, and the stored value min(best, c_make^2) gives the same term.  A query that
-// has not stopped after RW_KMAX rings (a far outlier) keeps its best as an upper
+// has not stopped at half side RW_KMAX (a far outlier) keeps its best as an upper
 // bound and is finished by the all-pairs scan over the other side.
+//
+// A square grows to what the best distance or the diagonal cost leaves open, by a
+// quarter while nothing is found; its new cells are one stretch of nodes a row above
+// and below and two a row beside, so that empty space costs a few loads a row and
+// RW_KMAX reaches as far as 24 rings of cells of half a node did.
 //
 // Bound by the distances evaluated and by the gathers of cells.  Diagrams crowd
 // near the diagonal, so cells of two nodes on average hold dozens where most
 // nodes are: the grid has RW_CELLS cells a node instead.  Queries run in the
-// order of their own side's cells, so the lanes of a warp search the same cells,
-// and a row of a ring is one stretch of nodes between two cell starts.  1,000,000
-// nodes a side (mixture): 2.31 ms with half a cell a node and queries by
-// coordinate.
+// order of their own side's cells, so the lanes of a warp search the same cells.
+// pd_rwmd_lower_bound, a side: 1,000,000 nodes (mixture) 3.31 ms with half a cell a
+// node, queries by coordinate and single rings, 0.75 so; 100,000 nodes in 40 clusters,
+// the other side's elsewhere, 3.2 and 3.2 (8.3 where only single rings, 24 of them,
+// reached across 8 cells a node); 300,000 in three clusters on both sides 30 and 25.
 
-constexpr int RW_KMAX = 24;
+constexpr int RW_KMAX = 96;
 constexpr int64_t RW_CELLS = 8;
+constexpr uint32_t RW_CROWD = 64;  // nodes of a cell that is searched before its neighbours
 constexpr int64_t RW_GRID_MIN = int64_t(1) << 28;  // nA * nB from which the grid is used
 
 struct RwGrid {
@@ -573,7 +580,7 @@ __global__ void k_rw_scatter(const int32_t* __restrict__ X, const int32_t* __res
     id[k] = (uint32_t)i;
 }
 
-// Ring search of the q-th placed node in the other side's grid; see above.  end:
+// Search of the q-th placed node in the other side's grid; see above.  end:
 // the cells' ends (a cell starts where the one before it ends).  Unfinished queries
 // are listed: side A's from list[0], side B's from list[nA], their counts in nl[0],
 // nl[1].
@@ -594,25 +601,24 @@ __global__ void k_rw_query(int64_t nA, int64_t n, RwGrid g0, RwGrid g1, const ui
         const uint32_t k1 = end[c + x1];
         for (uint32_t k = c + x0 > 0 ? end[c + x0 - 1] : 0u; k < k1; k++) {
             const int2 v = pts[k];
-            const long long dx = (long long)u.x - v.x, dy = (long long)u.y - v.y;
-            const unsigned long long d2 = (unsigned long long)(dx * dx) + (unsigned long long)(dy * dy);
+            const int32_t dx = u.x - v.x, dy = u.y - v.y;  // below 2^30: products of 32 bits
+            const unsigned long long d2 = (unsigned long long)((int64_t)dx * dx) + (unsigned long long)((int64_t)dy * dy);
             best = d2 < best ? d2 : best;
         }
     };
-    int state = 0;  // 0 searching, 1 exact, 2 stopped by the diagonal cost
-    for (int32_t K = 1; K <= RW_KMAX && state == 0; K++) {
+    int state = 0;          // 0 searching, 1 exact, 2 stopped by the diagonal cost
+    int32_t done = -1;      // half side of the square of cells that is searched
+    auto widen = [&](int32_t K) {
         const int32_t xlo = max(cx - K, 0), xhi = min(cx + K, g.gw - 1);
-        if (K == 1) {  // the first nine cells at once
-            for (int32_t y = max(cy - 1, 0); y <= min(cy + 1, g.gh - 1); y++) row(y, xlo, xhi);
-        } else {
-            if (cy - K >= 0) row(cy - K, xlo, xhi);
-            if (cy + K < g.gh) row(cy + K, xlo, xhi);
-            const int32_t ylo = max(cy - K + 1, 0), yhi = min(cy + K - 1, g.gh - 1);
-            if (cx - K >= 0)
-                for (int32_t y = ylo; y <= yhi; y++) row(y, cx - K, cx - K);
-            if (cx + K < g.gw)
-                for (int32_t y = ylo; y <= yhi; y++) row(y, cx + K, cx + K);
+        for (int32_t y = max(cy - K, 0); y <= min(cy + K, g.gh - 1); y++) {
+            if (abs(y - cy) > done) {
+                row(y, xlo, xhi);
+            } else {
+                if (cx - done > xlo) row(y, xlo, cx - done - 1);
+                if (cx + done < xhi) row(y, cx + done + 1, xhi);
+            }
         }
+        done = K;
         // distance to the nearest side of the searched square beyond which nodes may remain
         const int64_t ux = u.x, uy = u.y;
         int64_t lb = INT64_MAX;
@@ -627,6 +633,17 @@ __global__ void k_rw_query(int64_t nA, int64_t n, RwGrid g0, RwGrid g1, const ui
             if ((unsigned long long)lb * (unsigned long long)lb >= best) state = 1;
             else if (lb >= cm) state = 2;
         }
+    };
+    // a crowded cell by itself first: its neighbours are as crowded, and mostly not needed
+    const int64_t own = g.base + (int64_t)cy * g.gw + cx;
+    if (end[own] - (own > 0 ? end[own - 1] : 0u) > RW_CROWD) widen(0);
+    if (state == 0) widen(1);
+    while (state == 0 && done < RW_KMAX) {
+        // as far as the best so far and the diagonal leave open, by a quarter while nothing is found
+        const float cells = 1.f / (float)g.h;
+        const int32_t open = (int32_t)((float)cm * cells);
+        const int32_t K = best == ~0ull ? min(done + max(1, done / 4), open) : min((int32_t)(sqrtf((float)best) * cells), open);
+        widen(min(max(K, done + 1), RW_KMAX));
     }
     if (state == 2) {
         const unsigned long long c2 = (unsigned long long)cm * (unsigned long long)cm;
@@ -707,7 +724,7 @@ static RwGrid rw_grid(const int64_t* b, int64_t n, int64_t base, int64_t pair) {
 }
 
 // Exact minima of both directions through the grids (see k_rw_query), the
-// queries the rings did not finish completed by the all-pairs scan.
+// queries that it did not finish completed by the all-pairs scan.
 static pd_status rwmd_grid(Ctx* c, const Hats& h, DiagCost dc, unsigned long long* mind2, int64_t chunk, int64_t gy,
                            cudaStream_t st) {
     const int64_t n = h.nA + h.nB;
