@@ -81,7 +81,8 @@ typedef struct {
     int32_t alpha;       /* cost-scaling divisor of the solver, >= 2 (default 8) */
     int32_t verify;      /* 1 = certify optimality of the final flow on the device */
     int64_t max_rounds;  /* solver watchdog: push/relabel rounds over all phases (0 = default) */
-    int64_t time_limit_ms;  /* solver watchdog: device wall-clock limit of one solve (0 = 60000) */
+    int64_t time_limit_ms;  /* solver watchdog: device wall-clock limit of one solve (0 = 60000); a simplex that
+                               leaves the range of 32-bit potentials goes on with the limit anew */
     int64_t update_every;   /* relabels between global price updates (0 = number of nodes, -1 = never) */
     int32_t seq_threshold;  /* cost scaling: at most this many active nodes, one block finishes them (-1 = 64) */
     int32_t solver;         /* 0 = network simplex (default), 1 = cost scaling with push/relabel */
